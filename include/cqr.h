@@ -199,8 +199,9 @@ int cqr_factor(int64_t m, int64_t n, double* A, int64_t lda, int panel_b, double
  *   Arguments 1-9 as in cqr_factor.  Argument 10 is a plain variant (enum
  *   cqr_variant) without flags: CQR_LOOKAHEAD, CQR_ADAPTIVE and CQR_EMULATED
  *   are refused with -10.  There is no workspace argument: the scratch is a
- *   file-scope device array of CQR_NOALLOC_SCRATCH_BYTES (64 MiB) that every
- *   GPU which loads the library holds until the process exits.  Under the
+ *   file-scope device array of CQR_NOALLOC_SCRATCH_BYTES (64 MiB), and 16 MiB
+ *   more for the finer split sums of short matrices, that every GPU which
+ *   loads the library holds until the process exits.  Under the
  *   CUDA runtime's lazy module loading (the default) the array is created on
  *   a device by the first cqr_factor_noalloc call there, so make that first
  *   call during initialisation.
@@ -210,8 +211,8 @@ int cqr_factor(int64_t m, int64_t n, double* A, int64_t lda, int panel_b, double
  *   stream   CUDA stream (arg 12)
  * Returns the same argument codes as cqr_factor, or
  * CQR_ERR_NOALLOC_TOO_LARGE when the sizes need more scratch than the array
- * holds (compare cqr_workspace_size() with CQR_NOALLOC_SCRATCH_BYTES); nothing
- * is launched then.  It calls no cudaMalloc, cudaFree or allocating library
+ * holds (a cqr_workspace_size() up to CQR_NOALLOC_SCRATCH_BYTES fits; for
+ * short matrices up to 16 MiB more); nothing is launched then.  It calls no cudaMalloc, cudaFree or allocating library
  * routine.  The first call on each device looks up the array's device
  * address (cudaGetSymbolAddress) with that device current; make that first
  * call before any stream capture.  All calls share the one array and it keeps

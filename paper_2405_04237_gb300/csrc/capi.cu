@@ -4,6 +4,7 @@
 // caller's stream; nothing here computes on the host, allocates, or waits.
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 #include <vector>
 
@@ -18,6 +19,7 @@ inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct Layout {
   size_t status, skip, panel, W, S1, S2, rinv, Z, R1, R2, part, oz, total;
+  size_t nominal;  // total with the partials of tn_nominal_doubles (mCQR2GS, CQR2GS, CQR2, sCQR3 without flags)
 };
 
 // Substitution block width of the emulated variant: its coupling products
@@ -57,21 +59,19 @@ Layout make_layout(i64 m, i64 n, int b, int variant, bool emulated = false, bool
   L.Z = take(variant == CQR_MCQR2GS ? sizeof(double) * n * b : 0);
   L.R1 = take((variant == CQR_CQR2GS || variant == CQR_SCQR3) ? sizeof(double) * n * n : 0);
   L.R2 = take((variant == CQR_CQR2GS || variant == CQR_SCQR3) ? sizeof(double) * n * n : 0);
-  size_t pd = tn_partial_doubles(m, (int)pw, (int)pw, 1);
-  if (!whole) {
+  auto partials = [&](size_t (*need)(i64, int, int, int)) {
+    size_t d = need(m, (int)pw, (int)pw, 1);
+    if (whole) return d;
     for (i64 j = 0; j * b < n; ++j) {
       const i64 w = n - (j + 1) * b;  // trailing width after panel j
-      if (w > 0) {
-        size_t d = tn_partial_doubles(m, b, (int)w, 0);
-        if (d > pd) pd = d;
-      }
+      if (w > 0) d = std::max(d, need(m, b, (int)w, 0));
       const i64 jb = (j + 1) * b;  // mCQR2GS re-orthogonalisation against jb columns
-      if (variant == CQR_MCQR2GS && jb < n) {
-        size_t d = tn_partial_doubles(m, (int)jb, b, 0);
-        if (d > pd) pd = d;
-      }
+      if (variant == CQR_MCQR2GS && jb < n) d = std::max(d, need(m, (int)jb, b, 0));
     }
-  }
+    return d;
+  };
+  size_t pd = partials(tn_partial_doubles);
+  L.nominal = align256(off + sizeof(double) * partials(tn_nominal_doubles));
   if (halving && variant == CQR_MCQR2GS) {
     // every width of the chain b, h(b), h(h(b)), ..., 1 at every position it
     // can start from (a multiple of itself), after a panel of any wider width
@@ -1066,7 +1066,7 @@ int cqr_factor_batched(int batch, const int64_t* m, const int64_t* n, const int6
 // by the first call there (the symbol lookup below loads the module).
 namespace {
 
-__device__ __align__(256) unsigned char g_noalloc_scratch[CQR_NOALLOC_SCRATCH_BYTES];
+__device__ __align__(256) unsigned char g_noalloc_scratch[CQR_NOALLOC_SCRATCH_BYTES + kNoallocSlack];
 
 std::mutex g_noalloc_mu;
 void* g_noalloc_addr[64] = {};  // device address of g_noalloc_scratch, per device
@@ -1103,7 +1103,8 @@ int cqr_factor_noalloc(int64_t m, int64_t n, double* A, int64_t lda, int panel_b
   if (!R) return -8;
   if (ldr < n) return -9;
   const Layout L = make_layout(m, n, b, variant);
-  if (L.total > (size_t)CQR_NOALLOC_SCRATCH_BYTES) return CQR_ERR_NOALLOC_TOO_LARGE;
+  if (L.nominal > (size_t)CQR_NOALLOC_SCRATCH_BYTES || L.total > (size_t)CQR_NOALLOC_SCRATCH_BYTES + kNoallocSlack)
+    return CQR_ERR_NOALLOC_TOO_LARGE;
   void* scratch = noalloc_scratch();
   if (!scratch) return CQR_ERR_CUDA;
   cudaStream_t st = (cudaStream_t)stream;

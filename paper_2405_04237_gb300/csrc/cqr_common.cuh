@@ -27,13 +27,13 @@ constexpr int kSMs = 152;
 
 // ---------------------------------------------------------------------------
 // Split-m transposed product  C (p x q) = X^T Y  summed over m rows.
-// Stage 1: S persistent blocks split the flattened (output tile, row block)
-// items into S equal contiguous ranges and write one partial tile per
+// Stage 1: S persistent blocks split the rows (Gram) or the flattened (output
+// tile, row block) items into S equal contiguous ranges and write one partial tile per
 // (block, tile) segment.  Stage 2 adds each entry's segments in ascending
 // row order.  With sym != 0, X == Y and only entries on or above the
 // diagonal are formed (syrk); the reduce mirrors them.
 struct TnPlan {
-  int tp, tq;        // output tile (8..64; sym: padded width)
+  int tp, tq;        // output tile (4..64; sym: padded width)
   int tiles_p, tiles_q;
   int ntiles;
   int S;             // persistent blocks
@@ -41,9 +41,61 @@ struct TnPlan {
 };
 TnPlan tn_plan(i64 m, int p, int q, int sym);
 size_t tn_partial_doubles(i64 m, int p, int q, int sym);  // S * p * q
+// The same for a split into blocks of about 8192 (Gram) or 4096 staged
+// doubles whatever m is: what cqr_factor_noalloc counts against its array.
+// A finer split of a short matrix takes at most kNoallocSlack bytes more.
+size_t tn_nominal_doubles(i64 m, int p, int q, int sym);
+constexpr size_t kNoallocSlack = (size_t)16 << 20;
 // C (ldc) := X^T Y.  `part` must hold tn_partial_doubles() doubles.
 cudaError_t tn_product(i64 m, int p, int q, const double* X, i64 ldx, const double* Y, i64 ldy, int sym,
                        double* part, double* C, i64 ldc, const int* status, cudaStream_t st);
+// Stage 1 of the Gram matrix alone (b <= 128): writes partial triangles
+// part[s][r + c * b], r <= c, and returns how many (0 for m <= 0).
+i64 gram_partials(i64 m, int b, const double* X, i64 ldx, double* part, const int* status, cudaStream_t st);
+
+#ifdef __CUDACC__
+// Upper-triangle enumeration, column by column: u -> (i, j), 0 <= i <= j.
+__host__ __device__ inline void decode_upper(int u, int& i, int& j) {
+  int jj = (int)((sqrtf(8.0f * (float)u + 1.0f) - 1.0f) * 0.5f);
+  while ((jj + 1) * (jj + 2) / 2 <= u) ++jj;
+  while (jj * (jj + 1) / 2 > u) --jj;
+  j = jj;
+  i = u - jj * (jj + 1) / 2;
+}
+
+// Ascending sum of nseg values in 16 contiguous parts, one per thread row of
+// a 16 x 16 block: thread (x, y) sums part y of output x (get(k) is the k-th
+// value), and the parts are added in order.  A dependent FP64 add takes 64
+// clocks, so one thread adding 456 partials in a row took 14 us.
+template <class Get>
+__device__ __forceinline__ double split_sum16(i64 nseg, bool live, double* red, Get get) {
+  const int x = threadIdx.x & 15, y = threadIdx.x >> 4;
+  double s = 0.0;
+  if (live) {
+    i64 k = y * nseg / 16;
+    const i64 k1 = (y + 1) * nseg / 16;
+    for (; k + 8 <= k1; k += 8) {  // eight loads in flight
+      double v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = get(k + j);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) s += v[j];
+    }
+    double v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = k + j < k1 ? get(k + j) : 0.0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (k + j < k1) s += v[j];
+  }
+  red[y * 17 + x] = s;
+  __syncthreads();
+  double v = 0.0;
+  if (y == 0)
+    for (int k = 0; k < 16; ++k) v += red[k * 17 + x];
+  return v;
+}
+#endif
 
 // FP64-accurate C = X^T Y on the FP8 tensor cores (k_ozaki.cu): the m-row
 // sum of the projections with the Ozaki splitting.  `ws` must hold

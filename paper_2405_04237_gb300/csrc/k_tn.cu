@@ -26,15 +26,7 @@ constexpr int kSyrkThreads = 512;  // 16 warps
 // row block; with three resident blocks the others keep the FP64 pipe busy
 // meanwhile (projection: 1.195 -> 1.213 TFLOP/s on GB300 against two).
 constexpr int kMaxResident = 3;
-
-// Upper-triangle enumeration, column by column: u -> (i, j), 0 <= i <= j.
-__host__ __device__ inline void decode_upper(int u, int& i, int& j) {
-  int jj = (int)((sqrtf(8.0f * (float)u + 1.0f) - 1.0f) * 0.5f);
-  while ((jj + 1) * (jj + 2) / 2 <= u) ++jj;
-  while (jj * (jj + 1) / 2 > u) --jj;
-  j = jj;
-  i = u - jj * (jj + 1) / 2;
-}
+constexpr int kFullRows = 32;  // staged rows of a 64 x 64 tile
 
 // [begin, end) of the items of persistent block c when T items are split
 // over P blocks.
@@ -48,23 +40,79 @@ __host__ __device__ inline i64 owner_of(i64 i, i64 T, i64 P) { return ((i + 1) *
 __device__ inline double2 lds2(const double* p) { return *reinterpret_cast<const double2*>(p); }
 
 // ---------------------------------------------------------------------------
-// Gram (syrk) kernel for b <= 128, 512 threads (16 warps: four per warp
-// scheduler, so every scheduler's share of the FP64 pipe gets the same
-// work).  The upper triangle is cut into cnt = T(T+1)/2 tiles of 4 x 4
-// (T = ceil(b/4)).  The largest power of two M <= cnt of them are "main"
-// tiles: thread t owns main tile t % M on the rows r = t / M (mod 512 / M)
-// of each staged row block.  The E = cnt - M other tiles are "extra": each
-// is owned by 512 / E threads (whole warps when E <= 16) that split the
-// rows round-robin.  Every thread thus carries one main and at most one
-// extra accumulator and runs the same instruction stream as its warp.
+// Fixed-order sums of per-thread 4 x 4 accumulators inside a block.  The
+// accumulators lie in shared memory entry-major (red[e * T + thread], entry
+// e = u * 4 + v).  Output o = e * ntile + tile is the sum over k < nv of
+// red[e * T + tile * st + k * sk].  A dependent FP64 add takes 64 clocks and
+// a warp's add costs the same with one live lane as with 32, so the outputs
+// are spread over all T threads: where there are fewer than T / 2 of them
+// every output is cut into S parts, summed by S threads and then over the
+// parts.  (One thread per tile adding all its values in a row took 200-330
+// us per Gram matrix for b <= 16, most of the time of a small
+// factorisation; spread it takes 1-2 us.)
+template <int T, class Store>
+__device__ __forceinline__ void block_sums(const double* red, double* scratch, int ntile, int nv, int st, int sk,
+                                           Store store) {
+  const int t = threadIdx.x;
+  const int O = 16 * ntile;
+  const int S = 2 * O <= T ? T / O : 1;
+  if (S == 1) {
+    for (int o = t; o < O; o += T) {
+      const int e = o / ntile, tile = o - e * ntile;
+      const double* p = red + e * T + tile * st;
+      double x = 0.0;
+      for (int k = 0; k < nv; ++k) x += p[k * sk];
+      store(tile, e, x);
+    }
+  } else {
+    const int s = t / O, o = t - s * O;
+    const int e = o / ntile, tile = o - e * ntile;
+    if (s < S) {
+      const double* p = red + e * T + tile * st;
+      const int k1 = (s + 1) * nv / S;
+      double x = 0.0;
+      for (int k = s * nv / S; k < k1; ++k) x += p[k * sk];
+      scratch[s * O + o] = x;
+    }
+    __syncthreads();
+    if (t < O) {
+      double x = scratch[t];
+      for (int q = 1; q < S; ++q) x += scratch[q * O + t];
+      store(tile, e, x);  // s == 0 here: (tile, e) is output t
+    }
+  }
+}
+
+__device__ __forceinline__ void spill_acc(double* red, int T, const double (&acc)[4][4]) {
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+#pragma unroll
+    for (int v = 0; v < 4; ++v) red[(u * 4 + v) * T + threadIdx.x] = acc[u][v];
+}
+
+__device__ __forceinline__ void cp_async8_zfill(double* dst, const double* src, bool ok) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(ok ? 8 : 0) : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// Gram (syrk) kernel for b <= 128, T threads.  The upper triangle is cut into
+// cnt = n4(n4+1)/2 tiles of 4 x 4 (n4 = ceil(b/4)).  M of them are "main"
+// tiles: thread t < M * RG owns main tile t % M on the rows r = t / M (mod
+// RG) of each staged row block.  The E = cnt - M other tiles are "extra":
+// each is owned by T / E threads that split the rows round-robin.  Where
+// cnt * (T / cnt) threads fill the block to 93 %, every tile is a main tile
+// (no second accumulator to sum at the end); otherwise M is the largest
+// power of two <= cnt and every thread carries one main and at most one
+// extra accumulator, so no lane idles.
 struct SyrkArgs {
   const double* X;
   i64 ldx, m;
   int b, bp;       // width, padded width (multiple of 4)
   int M, RG;       // main tiles, row groups
   int E, tpt;      // extra tiles, threads per extra tile
-  int rb;          // rows per block
-  i64 nb, P;       // row blocks, persistent blocks
+  int rb;          // rows per staged block
+  i64 P;           // persistent blocks; block c owns rows [c m / P, (c + 1) m / P)
   double* part;    // [P][b*b]
   const int* status;
 };
@@ -80,17 +128,8 @@ __device__ __forceinline__ void syrk_tile_row(const double* row, int i, int j, d
     for (int v = 0; v < 4; ++v) acc[u][v] = fma(xv[u], yv[v], acc[u][v]);
 }
 
-__device__ __forceinline__ void syrk_store_tile(double* P, int b, int i, int j, const double (&v)[4][4]) {
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-      const int r = 4 * i + u, c = 4 * j + w;
-      if (r <= c && c < b) P[r + c * b] = v[u][w];
-    }
-}
-
-__global__ void __launch_bounds__(kSyrkThreads) syrk_partial_kernel(SyrkArgs a) {
+template <int T>
+__global__ void __launch_bounds__(T) syrk_partial_kernel(SyrkArgs a) {
   extern __shared__ __align__(16) double sm[];
   if (a.status && *a.status) return;
   const int t = threadIdx.x;
@@ -108,86 +147,76 @@ __global__ void __launch_bounds__(kSyrkThreads) syrk_partial_kernel(SyrkArgs a) 
 #pragma unroll
     for (int v = 0; v < 4; ++v) am[u][v] = ae[u][v] = 0.0;
 
-  i64 ib, ie;
-  item_range(blockIdx.x, a.nb, a.P, ib, ie);
+  i64 rbeg, rend;
+  item_range(blockIdx.x, a.m, a.P, rbeg, rend);
   const int rb = a.rb;
-  for (i64 blk = ib; blk < ie; ++blk) {
-    const i64 r0 = blk * rb;
-    const int nrow = (int)imin64(rb, a.m - r0);
-    // stage X[r0:r0+rb, 0:bp] row-major; zero beyond m and beyond b.
-    // Asynchronous copies: every load of the block is in flight before the
-    // one wait, instead of one memory latency per loop iteration.
-    for (int e = t; e < rb * a.bp; e += kSyrkThreads) {
+  for (i64 r0 = rbeg; r0 < rend; r0 += rb) {
+    const int nrow = (int)imin64(rb, rend - r0);
+    // stage X[r0:r0+nrow, 0:bp] row-major; zero beyond b.  Asynchronous
+    // copies: every load of the block is in flight before the one wait,
+    // instead of one memory latency per loop iteration.
+    for (int e = t; e < rb * a.bp; e += T) {
       const int r = e % rb, c = e / rb;
       const bool ok = r < nrow && c < a.b;
-      const unsigned dst = (unsigned)__cvta_generic_to_shared(sm + r * sp + c);
-      const double* src = ok ? a.X + (r0 + r) + (i64)c * a.ldx : a.X;
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(ok ? 8 : 0) : "memory");
+      cp_async8_zfill(sm + r * sp + c, ok ? a.X + (r0 + r) + (i64)c * a.ldx : a.X, ok);
     }
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
     __syncthreads();
+    if (g < a.RG) {
 #pragma unroll 2
-    for (int r = g; r < nrow; r += a.RG) syrk_tile_row(sm + r * sp, mi, mj, am);
+      for (int r = g; r < nrow; r += a.RG) syrk_tile_row(sm + r * sp, mi, mj, am);
+    }
     if (extra)
       for (int r = ek; r < nrow; r += a.tpt) syrk_tile_row(sm + r * sp, ei, ej, ae);
     __syncthreads();
   }
   // fixed-order sums: main tiles over the row groups, extra tiles over their threads
   double* P = a.part + (i64)blockIdx.x * a.b * a.b;
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int v = 0; v < 4; ++v) sm[(u * 4 + v) * kSyrkThreads + t] = am[u][v];
+  const int b = a.b, M = a.M;
+  auto store = [P, b](int id, int e, double x) {
+    int i, j;
+    decode_upper(id, i, j);
+    const int r = 4 * i + (e >> 2), c = 4 * j + (e & 3);
+    if (r <= c && c < b) P[r + c * b] = x;
+  };
+  double* scratch = sm + 16 * T;
+  spill_acc(sm, T, am);
   __syncthreads();
-  if (t < a.M) {
-    double sum[4][4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        double x = 0.0;
-        for (int gg = 0; gg < a.RG; ++gg) x += sm[(u * 4 + v) * kSyrkThreads + gg * a.M + t];
-        sum[u][v] = x;
-      }
-    syrk_store_tile(P, a.b, mi, mj, sum);
-  }
+  block_sums<T>(sm, scratch, M, a.RG, 1, M, store);
   if (a.E > 0) {
     __syncthreads();
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-      for (int v = 0; v < 4; ++v) sm[(u * 4 + v) * kSyrkThreads + t] = ae[u][v];
+    spill_acc(sm, T, ae);
     __syncthreads();
-    if (extra && ek == 0) {
-      double sum[4][4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          double x = 0.0;
-          for (int k = 0; k < a.tpt; ++k) x += sm[(u * 4 + v) * kSyrkThreads + t + k];
-          sum[u][v] = x;
-        }
-      syrk_store_tile(P, a.b, ei, ej, sum);
-    }
+    block_sums<T>(sm, scratch, a.E, a.tpt, a.tpt, 1, [store, M](int id, int e, double x) { store(M + id, e, x); });
   }
 }
 
-// W[r + c*ldw] = sum_{s<P} part[s][r + c*b] for r <= c, mirrored.
-__global__ void syrk_reduce_kernel(const double* part, int b, i64 P, double* W, i64 ldw, const int* status) {
+// W[r + c*ldw] = sum_{s<P} part[s][r + c*b] for r <= c, mirrored.  16 entries
+// of the upper triangle (column by column) per block of 256 threads.
+__global__ void __launch_bounds__(256) syrk_reduce_kernel(const double* part, int b, i64 P, double* W, i64 ldw,
+                                                          const int* status) {
+  __shared__ double red[16 * 17];
   if (status && *status) return;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= b * b) return;
-  const int r = e % b, c = e / b;
-  if (r > c) return;
-  double s = 0.0;
-  for (i64 k = 0; k < P; ++k) s += part[k * b * b + e];
-  W[r + (i64)c * ldw] = s;
-  if (r != c) W[c + (i64)r * ldw] = s;
+  const int u = blockIdx.x * 16 + (threadIdx.x & 15);
+  const bool live = u < b * (b + 1) / 2;
+  int r = 0, c = 0;
+  if (live) decode_upper(u, r, c);
+  const double* p = part + r + c * b;
+  const i64 bb = (i64)b * b;
+  const double s = split_sum16(P, live, red, [p, bb](i64 k) { return p[k * bb]; });
+  if (threadIdx.x < 16 && live) {
+    W[r + (i64)c * ldw] = s;
+    if (r != c) W[c + (i64)r * ldw] = s;
+  }
 }
 
 // ---------------------------------------------------------------------------
-// General C = X^T Y (no symmetry).  Tile TP x TQ, 256 threads.
+// General C = X^T Y (no symmetry).  Tile tp x tq (multiples of 4, at most
+// 64), 256 threads: ntg = tp tq / 16 micro-tiles of 4 x 4, G = 256 / ntg row
+// groups; thread t < ntg * G owns micro-tile t % ntg on the rows r = t / ntg
+// (mod G).  The 64 x 64 tile (every product of two multiples of 64) has its
+// sizes at compile time: the address arithmetic of the run-time form costs
+// it 0.8 % (projections at 2^18 x 1024, b = 128: 395.0 -> 392.0 ms).
 struct TnArgs {
   const double* X;
   i64 ldx;
@@ -195,40 +224,26 @@ struct TnArgs {
   i64 ldy;
   i64 m;
   int p, q;
+  int tp, tq, rb;
   int tiles_p;
   i64 nb, T, P;  // row blocks per tile, total items, persistent blocks
-  double* part;  // [P + ntiles][TP*TQ]
+  double* part;  // [P + ntiles][tp * tq]
   const int* status;
 };
 
-template <int TP, int TQ>
-struct TnShape {
-  static constexpr int NP = TP / 4, NQ = TQ / 4;
-  static constexpr int NTG = NP * NQ;
-  static constexpr int G = kTnThreads / NTG;
-  static constexpr int RB0 = 4096 / (TP + TQ);
-  static constexpr int UNIT = G > 8 ? G : 8;
-  static constexpr int RB = (RB0 / UNIT) * UNIT;
-  static constexpr int SP = TP + 2, SQ = TQ + 2;
-  static constexpr int TILE_D = RB * (SP + SQ);
-  static constexpr int RED_D = 16 * kTnThreads;
-  static constexpr int SMEM_D = TILE_D > RED_D ? TILE_D : RED_D;
-  static_assert(TP % 4 == 0 && TQ % 4 == 0, "4 x 4 micro-tiles");
-  static_assert(NTG * G == kTnThreads, "every thread owns one micro-tile of one row group");
-  static_assert(RB >= G, "every row group gets rows");
-  static_assert(SMEM_D * (int)sizeof(double) <= 48 * 1024, "static shared memory limit");
-};
-
-template <int TP, int TQ>
+template <bool kFull>
 __global__ void __launch_bounds__(kTnThreads) tn_partial_kernel(TnArgs a) {
-  using Sh = TnShape<TP, TQ>;
-  __shared__ __align__(16) double sm[Sh::SMEM_D];
+  extern __shared__ __align__(16) double sm[];
   if (a.status && *a.status) return;
   const int t = threadIdx.x;
-  const int g = t / Sh::NTG, u = t - g * Sh::NTG;
-  const int mi = u % Sh::NP, mj = u / Sh::NP;
+  const int atp = kFull ? 64 : a.tp, atq = kFull ? 64 : a.tq;
+  const int NP = atp >> 2, ntg = NP * (atq >> 2), G = kTnThreads / ntg;
+  const int g = t / ntg, u = t - g * ntg;
+  const int mj = u / NP, mi = u - mj * NP;
+  const int SP = atp + 2, SQ = atq + 2;
+  const int rb = kFull ? kFullRows : a.rb;
   double* Xs = sm;
-  double* Ys = sm + Sh::RB * Sh::SP;
+  double* Ys = sm + rb * SP;
 
   i64 ib, ie;
   item_range(blockIdx.x, a.T, a.P, ib, ie);
@@ -236,179 +251,185 @@ __global__ void __launch_bounds__(kTnThreads) tn_partial_kernel(TnArgs a) {
   while (item < ie) {
     const i64 tile = item / a.nb;
     const i64 tile_end = imin64(ie, (tile + 1) * a.nb);
-    const int p0 = (int)(tile % a.tiles_p) * TP, q0 = (int)(tile / a.tiles_p) * TQ;
+    const int p0 = (int)(tile % a.tiles_p) * atp, q0 = (int)(tile / a.tiles_p) * atq;
     double acc[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
     for (; item < tile_end; ++item) {
-      const i64 r0 = (item - tile * a.nb) * Sh::RB;
-      const int nrow = (int)imin64(Sh::RB, a.m - r0);
-      // asynchronous staging (zero-filled beyond m, p, q): all loads in flight before one wait
-      for (int e = t; e < Sh::RB * TP; e += kTnThreads) {
-        const int r = e % Sh::RB, c = e / Sh::RB;
+      const i64 r0 = (item - tile * a.nb) * rb;
+      const int nrow = (int)imin64(rb, a.m - r0);
+      // asynchronous staging (zero-filled beyond p, q): all loads in flight before one wait
+      for (int e = t; e < rb * atp; e += kTnThreads) {
+        const int r = e % rb, c = e / rb;
         const bool ok = r < nrow && p0 + c < a.p;
-        const unsigned dst = (unsigned)__cvta_generic_to_shared(Xs + r * Sh::SP + c);
-        const double* src = ok ? a.X + (r0 + r) + (i64)(p0 + c) * a.ldx : a.X;
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(ok ? 8 : 0) : "memory");
+        cp_async8_zfill(Xs + r * SP + c, ok ? a.X + (r0 + r) + (i64)(p0 + c) * a.ldx : a.X, ok);
       }
-      for (int e = t; e < Sh::RB * TQ; e += kTnThreads) {
-        const int r = e % Sh::RB, c = e / Sh::RB;
+      for (int e = t; e < rb * atq; e += kTnThreads) {
+        const int r = e % rb, c = e / rb;
         const bool ok = r < nrow && q0 + c < a.q;
-        const unsigned dst = (unsigned)__cvta_generic_to_shared(Ys + r * Sh::SQ + c);
-        const double* src = ok ? a.Y + (r0 + r) + (i64)(q0 + c) * a.ldy : a.Y;
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(ok ? 8 : 0) : "memory");
+        cp_async8_zfill(Ys + r * SQ + c, ok ? a.Y + (r0 + r) + (i64)(q0 + c) * a.ldy : a.Y, ok);
       }
       asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
       __syncthreads();
-      const double* xi = Xs + 4 * mi;
-      const double* yj = Ys + 4 * mj;
+      if (g < G) {
+        const double* xi = Xs + 4 * mi;
+        const double* yj = Ys + 4 * mj;
 #pragma unroll 2
-      for (int r = g; r < nrow; r += Sh::G) {
-        const double2 p0v = lds2(xi + r * Sh::SP), p1v = lds2(xi + r * Sh::SP + 2);
-        const double2 q0v = lds2(yj + r * Sh::SQ), q1v = lds2(yj + r * Sh::SQ + 2);
-        const double xv[4] = {p0v.x, p0v.y, p1v.x, p1v.y};
-        const double yv[4] = {q0v.x, q0v.y, q1v.x, q1v.y};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fma(xv[i], yv[j], acc[i][j]);
-      }
-      __syncthreads();
-    }
-    if (Sh::G > 1) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) sm[(i * 4 + j) * kTnThreads + t] = acc[i][j];
-      __syncthreads();
-      if (g == 0) {
-        for (int gg = 1; gg < Sh::G; ++gg) {
-          const int tt = gg * Sh::NTG + u;
+        for (int r = g; r < nrow; r += G) {
+          const double2 p0v = lds2(xi + r * SP), p1v = lds2(xi + r * SP + 2);
+          const double2 q0v = lds2(yj + r * SQ), q1v = lds2(yj + r * SQ + 2);
+          const double xv[4] = {p0v.x, p0v.y, p1v.x, p1v.y};
+          const double yv[4] = {q0v.x, q0v.y, q1v.x, q1v.y};
 #pragma unroll
           for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] += sm[(i * 4 + j) * kTnThreads + tt];
+            for (int j = 0; j < 4; ++j) acc[i][j] = fma(xv[i], yv[j], acc[i][j]);
         }
       }
       __syncthreads();
     }
-    if (g == 0) {
-      // segment id = persistent block + tile (unique, increasing in rows)
-      double* Pp = a.part + ((i64)blockIdx.x + tile) * (TP * TQ);
+    // segment id = persistent block + tile (unique, increasing in rows)
+    double* Pp = a.part + ((i64)blockIdx.x + tile) * (atp * atq);
+      if (G > 1) {
+      spill_acc(sm, kTnThreads, acc);
+      __syncthreads();
+      block_sums<kTnThreads>(sm, sm + 16 * kTnThreads, ntg, G, 1, ntg, [Pp, atp, NP](int id, int e, double x) {
+        const int j = id / NP, i = id - j * NP;
+        Pp[(4 * i + (e >> 2)) + (4 * j + (e & 3)) * atp] = x;
+      });
+      __syncthreads();
+    } else if (g == 0) {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) Pp[(4 * mi + i) + (4 * mj + j) * TP] = acc[i][j];
+        for (int j = 0; j < 4; ++j) Pp[(4 * mi + i) + (4 * mj + j) * atp] = acc[i][j];
     }
   }
 }
 
 // C[r + c*ldc] = sum over the segments of tile(r, c), ascending rows.
-__global__ void tn_reduce_kernel(const double* part, int p, int q, int TP, int TQ, int tiles_p, i64 nb, i64 T,
-                                 i64 P, double* C, i64 ldc, const int* status) {
+__global__ void __launch_bounds__(256) tn_reduce_kernel(const double* part, int p, int q, int TP, int TQ, int tiles_p,
+                                                        i64 nb, i64 T, i64 P, double* C, i64 ldc, const int* status) {
+  __shared__ double red[16 * 17];
   if (status && *status) return;
-  const i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (i64)p * q) return;
+  const i64 e = (i64)blockIdx.x * 16 + (threadIdx.x & 15);
+  const bool live = e < (i64)p * q;
   const int r = (int)(e % p), c = (int)(e / p);
-  if (T == 0) {  // no rows: the empty sum
-    C[r + (i64)c * ldc] = 0.0;
-    return;
+  i64 nseg = 0;  // T == 0, no rows: the empty sum
+  const double* src = part;
+  const i64 tt = (i64)TP * TQ;
+  if (live && T > 0) {
+    const i64 tile = (i64)(r / TP) + (i64)(c / TQ) * tiles_p;
+    const i64 c_lo = owner_of(tile * nb, T, P);
+    const i64 c_hi = owner_of((tile + 1) * nb - 1, T, P);
+    nseg = c_hi - c_lo + 1;
+    src = part + (c_lo + tile) * tt + (r % TP) + (c % TQ) * TP;
   }
-  const i64 tile = (i64)(r / TP) + (i64)(c / TQ) * tiles_p;
-  const int loc = (r % TP) + (c % TQ) * TP;
-  const i64 c_lo = owner_of(tile * nb, T, P);
-  const i64 c_hi = owner_of((tile + 1) * nb - 1, T, P);
-  double s = 0.0;
-  for (i64 blk = c_lo; blk <= c_hi; ++blk) s += part[(blk + tile) * (TP * TQ) + loc];
-  C[r + (i64)c * ldc] = s;
+  const double s = split_sum16(nseg, live, red, [src, tt](i64 k) { return src[k * tt]; });
+  if (threadIdx.x < 16 && live) C[r + (i64)c * ldc] = s;
 }
 
 // ---------------------------------------------------------------------------
-inline int pick_tile(int d) { return d <= 8 ? 8 : d <= 16 ? 16 : d <= 32 ? 32 : 64; }
-
 struct SyrkPlan {
-  int bp, M, RG, E, tpt, rb;
+  int T, bp, M, RG, E, tpt, rb, P;
   size_t smem;
 };
-SyrkPlan syrk_plan(int b) {
+
+// Row count x tile count below which the 128-thread kernel is used.
+constexpr i64 kSyrkSmall = 1200000;
+
+constexpr i64 kPartCap = 730000;
+
+int g_occ_syrk[2][129];
+
+SyrkPlan syrk_plan(i64 m, int b) {
   SyrkPlan s;
   const int n4 = (b + 3) / 4;
   s.bp = 4 * n4;
   const int cnt = n4 * (n4 + 1) / 2;
-  s.M = 1;
-  while (s.M * 2 <= cnt && s.M * 2 <= kSyrkThreads) s.M *= 2;
-  s.RG = kSyrkThreads / s.M;
+  const bool small = cnt <= 256 && m * cnt < kSyrkSmall;
+  s.T = small ? 128 : kSyrkThreads;
+  if (cnt <= s.T && (s.T / cnt) * cnt * 100 >= s.T * 93) {
+    s.M = cnt;
+  } else {
+    s.M = 1;
+    while (s.M * 2 <= cnt && s.M * 2 <= s.T) s.M *= 2;
+  }
+  s.RG = s.T / s.M;
   s.E = cnt - s.M;
-  s.tpt = s.E > 0 ? kSyrkThreads / s.E : 0;
-  // about 8192 staged doubles (the size of the reduction area) per row
-  // block, a multiple of the row groups
-  const int per = 8192 / (s.bp + 2);
+  s.tpt = s.E > 0 ? s.T / s.E : 0;
+  // staged doubles per row block: half the reduction area of the large
+  // kernel, twice that of the small one
+  const int per = (small ? 4096 : 8192) / (s.bp + 2);
   s.rb = per >= s.RG ? per / s.RG * s.RG : s.RG;
-  const size_t tile = (size_t)s.rb * (s.bp + 2), red = (size_t)16 * kSyrkThreads;
+  // Blocks: at least 32 rows each, at most kMaxResident per SM, and for the
+  // widths where that many partial triangles would take longer to add up
+  // than they save, about kPartCap doubles of them.
+  const i64 min_rows = 32;
+  i64 want = (m + min_rows - 1) / min_rows;
+  if (want < 1) want = 1;
+  if (small) {
+    const i64 cap = kPartCap / ((i64)b * b);
+    const i64 most = cap > kSMs ? cap : (i64)kSMs;
+    if (want > most) want = most;
+  }
+  const size_t tile = (size_t)s.rb * (s.bp + 2), red = (size_t)17 * s.T;
   s.smem = (tile > red ? tile : red) * sizeof(double);
+  int& occ = g_occ_syrk[small ? 0 : 1][b];
+  if (occ == 0) {
+    int o = 0;
+    if (small) {
+      cudaFuncSetAttribute(syrk_partial_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, syrk_partial_kernel<128>, 128, s.smem);
+    } else {
+      cudaFuncSetAttribute(syrk_partial_kernel<kSyrkThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, syrk_partial_kernel<kSyrkThreads>, kSyrkThreads, s.smem);
+    }
+    occ = o > 0 ? o : 1;
+  }
+  const i64 slots = (i64)kSMs * min(occ, kMaxResident);
+  s.P = (int)(want < slots ? want : slots);
   return s;
 }
 
-int g_occ_syrk[129];
-int g_occ_tn[4][4];
-
-int syrk_occupancy(int b, const SyrkPlan& s) {
-  if (g_occ_syrk[b] == 0) {
-    cudaFuncSetAttribute(syrk_partial_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-    int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, syrk_partial_kernel, kSyrkThreads, s.smem);
-    g_occ_syrk[b] = occ > 0 ? occ : 1;
-  }
-  return g_occ_syrk[b];
-}
-
-template <int TP, int TQ>
-int tn_occ_impl() {
-  int occ = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, tn_partial_kernel<TP, TQ>, kTnThreads, 0);
-  return occ > 0 ? occ : 1;
-}
-inline int tidx(int t) { return t == 8 ? 0 : t == 16 ? 1 : t == 32 ? 2 : 3; }
-
-template <int TP>
-int tn_occ_q(int tq) {
-  switch (tq) {
-    case 8: return tn_occ_impl<TP, 8>();
-    case 16: return tn_occ_impl<TP, 16>();
-    case 32: return tn_occ_impl<TP, 32>();
-    default: return tn_occ_impl<TP, 64>();
-  }
-}
-int tn_occupancy(int tp, int tq) {
-  int& o = g_occ_tn[tidx(tp)][tidx(tq)];
-  if (o == 0) {
-    switch (tp) {
-      case 8: o = tn_occ_q<8>(tq); break;
-      case 16: o = tn_occ_q<16>(tq); break;
-      case 32: o = tn_occ_q<32>(tq); break;
-      default: o = tn_occ_q<64>(tq); break;
+// Tile of the general product: of the cuts of p and q into equal tiles of at
+// most 64, the one that wastes the fewest lanes (tile padding and threads
+// beyond ntg * G); among equals the largest tile.
+void tn_tile(int p, int q, int& tp, int& tq) {
+  const int kp = (p + 63) / 64, kq = (q + 63) / 64;
+  double best = -1.0;
+  tp = tq = 64;
+  for (int ip = kp; ip <= kp + 2; ++ip)
+    for (int iq = kq; iq <= kq + 2; ++iq) {
+      const int a = ((p + ip - 1) / ip + 3) / 4 * 4, b = ((q + iq - 1) / iq + 3) / 4 * 4;
+      const int np = (p + a - 1) / a, nq = (q + b - 1) / b;
+      const int ntg = (a / 4) * (b / 4);
+      const double util = (double)p * q / ((double)np * a * nq * b) * ((double)(kTnThreads / ntg * ntg) / kTnThreads);
+      if (util > best * 1.001) {
+        best = util;
+        tp = a;
+        tq = b;
+      }
     }
-  }
-  return o;
 }
 
-int tn_rb(int tp, int tq) {
-  const int ntg = (tp / 4) * (tq / 4);
-  const int G = kTnThreads / ntg;
-  const int unit = G > 8 ? G : 8;
-  return ((4096 / (tp + tq)) / unit) * unit;
+size_t tn_smem(int tp, int tq, int rb) {
+  const size_t tile = (size_t)rb * (tp + tq + 4), red = (size_t)17 * kTnThreads;
+  return (tile > red ? tile : red) * sizeof(double);
 }
 
-template <int TP>
-void launch_tn_q(int tq, dim3 grid, cudaStream_t st, const TnArgs& a) {
-  switch (tq) {
-    case 8: tn_partial_kernel<TP, 8><<<grid, kTnThreads, 0, st>>>(a); break;
-    case 16: tn_partial_kernel<TP, 16><<<grid, kTnThreads, 0, st>>>(a); break;
-    case 32: tn_partial_kernel<TP, 32><<<grid, kTnThreads, 0, st>>>(a); break;
-    default: tn_partial_kernel<TP, 64><<<grid, kTnThreads, 0, st>>>(a); break;
+int g_occ_tn = 0;  // run-time form, at the largest shared-memory size
+
+int tn_occupancy() {
+  if (g_occ_tn == 0) {
+    cudaFuncSetAttribute(tn_partial_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 48 * 1024);
+    int o = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, tn_partial_kernel<false>, kTnThreads, 48 * 1024);
+    g_occ_tn = o > 0 ? o : 1;
   }
+  return g_occ_tn;
 }
 
 }  // namespace
@@ -416,25 +437,31 @@ void launch_tn_q(int tq, dim3 grid, cudaStream_t st, const TnArgs& a) {
 TnPlan tn_plan(i64 m, int p, int q, int sym) {
   TnPlan P{};
   if (sym && p <= 128) {
-    SyrkPlan s = syrk_plan(p);
+    const SyrkPlan s = syrk_plan(m, p);
     P.tp = P.tq = s.bp;
     P.tiles_p = P.tiles_q = 1;
     P.ntiles = 1;
     P.rb = s.rb;
-    const i64 nb = (m + s.rb - 1) / s.rb;
-    i64 slots = (i64)kSMs * min(syrk_occupancy(p, s), kMaxResident);
-    P.S = (int)(nb < slots ? (nb > 0 ? nb : 1) : slots);
+    P.S = s.P;
     return P;
   }
-  P.tp = pick_tile(p);
-  P.tq = pick_tile(q);
+  tn_tile(p, q, P.tp, P.tq);
   P.tiles_p = (p + P.tp - 1) / P.tp;
   P.tiles_q = (q + P.tq - 1) / P.tq;
   P.ntiles = P.tiles_p * P.tiles_q;
-  P.rb = tn_rb(P.tp, P.tq);
-  const i64 nb = (m + P.rb - 1) / P.rb;
-  const i64 T = nb * P.ntiles;
-  i64 slots = (i64)kSMs * min(tn_occupancy(P.tp, P.tq), kMaxResident);
+  // Rows per item: about 4096 staged doubles, but where m is too short for
+  // every block to get that many, an even share (rounded up to the row
+  // groups, so that no block gets a second item), at least 32.
+  const i64 slots = (i64)kSMs * min(tn_occupancy(), kMaxResident);
+  const int G = kTnThreads / ((P.tp / 4) * (P.tq / 4));
+  i64 rb = 4096 / (P.tp + P.tq);
+  if (rb > G) rb = rb / G * G;
+  i64 even = (m * P.ntiles + slots - 1) / slots;
+  if (even < 32) even = 32;
+  if (even > G) even = (even + G - 1) / G * G;
+  if (rb > even) rb = even;
+  P.rb = (int)rb;
+  const i64 T = (m + P.rb - 1) / P.rb * P.ntiles;
   P.S = (int)(T < slots ? (T > 0 ? T : 1) : slots);
   return P;
 }
@@ -455,6 +482,61 @@ size_t tn_partial_doubles(i64 m, int p, int q, int sym) {
   TnPlan P = tn_plan(m, p, q, sym);
   if (sym) return (size_t)P.S * p * p;
   return (size_t)(P.S + P.ntiles) * P.tp * P.tq;
+}
+
+size_t tn_nominal_doubles(i64 m, int p, int q, int sym) {
+  if (p <= 0 || q <= 0) return 0;
+  if (sym && p > 128) {
+    size_t mx = 0;
+    for (int i = 0; i < p; i += 128)
+      for (int j = i; j < p; j += 128) {
+        const int pi = p - i < 128 ? p - i : 128, pj = p - j < 128 ? p - j : 128;
+        const size_t d = tn_nominal_doubles(m, pi, pj, i == j);
+        if (d > mx) mx = d;
+      }
+    return mx;
+  }
+  if (sym) {  // 512 threads, about 8192 staged doubles a block, one block per SM
+    const int n4 = (p + 3) / 4, cnt = n4 * (n4 + 1) / 2;
+    int M = 1;
+    while (M * 2 <= cnt && M * 2 <= kSyrkThreads) M *= 2;
+    const int RG = kSyrkThreads / M, per = 8192 / (4 * n4 + 2);
+    const i64 rb = per >= RG ? per / RG * RG : RG;
+    const i64 nb = (m + rb - 1) / rb;
+    return (size_t)(nb < kSMs ? nb : kSMs) * p * p;
+  }
+  auto tile = [](int d) { return d <= 8 ? 8 : d <= 16 ? 16 : d <= 32 ? 32 : 64; };
+  const int tp = tile(p), tq = tile(q);
+  const int G = kTnThreads / ((tp / 4) * (tq / 4)), unit = G > 8 ? G : 8;
+  const i64 rb = (4096 / (tp + tq)) / unit * unit;
+  const i64 nt = (i64)((p + tp - 1) / tp) * ((q + tq - 1) / tq), T = (m + rb - 1) / rb * nt;
+  return (size_t)((T < kSMs * kMaxResident ? T : kSMs * kMaxResident) + nt) * tp * tq;
+}
+
+i64 gram_partials(i64 m, int b, const double* X, i64 ldx, double* part, const int* status, cudaStream_t st) {
+  if (m <= 0) return 0;
+  const SyrkPlan s = syrk_plan(m, b);
+  SyrkArgs a;
+  a.X = X;
+  a.ldx = ldx;
+  a.m = m;
+  a.b = b;
+  a.bp = s.bp;
+  a.M = s.M;
+  a.RG = s.RG;
+  a.E = s.E;
+  a.tpt = s.tpt;
+  a.rb = s.rb;
+  a.P = s.P;
+  a.part = part;
+  a.status = status;
+  prof_begin(kGram, st);
+  if (s.T == 128)
+    syrk_partial_kernel<128><<<s.P, 128, s.smem, st>>>(a);
+  else
+    syrk_partial_kernel<kSyrkThreads><<<s.P, kSyrkThreads, s.smem, st>>>(a);
+  prof_end(kGram, (double)m * b * (b + 1), st);
+  return s.P;
 }
 
 cudaError_t tn_product(i64 m, int p, int q, const double* X, i64 ldx, const double* Y, i64 ldy, int sym,
@@ -478,37 +560,14 @@ cudaError_t tn_product(i64 m, int p, int q, const double* X, i64 ldx, const doub
     }
     return cudaSuccess;
   }
-  TnPlan P = tn_plan(m, p, q, sym);
   if (sym) {
-    SyrkPlan s = syrk_plan(p);
-    SyrkArgs a;
-    a.X = X;
-    a.ldx = ldx;
-    a.m = m;
-    a.b = p;
-    a.bp = s.bp;
-    a.M = s.M;
-    a.RG = s.RG;
-    a.E = s.E;
-    a.tpt = s.tpt;
-    a.rb = s.rb;
-    a.nb = (m + s.rb - 1) / s.rb;
-    a.P = P.S;
-    a.part = part;
-    a.status = status;
-    if (m > 0) {
-      prof_begin(kGram, st);
-      syrk_partial_kernel<<<P.S, kSyrkThreads, s.smem, st>>>(a);
-      prof_end(kGram, (double)m * p * (p + 1), st);
-    }
-    const int thr = 256;
-    const int blocks = (p * p + thr - 1) / thr;
-    const i64 nsum = m > 0 ? P.S : 0;  // m == 0: the empty sum, W = 0
+    const i64 nsum = gram_partials(m, p, X, ldx, part, status, st);  // m == 0: none, the empty sum W = 0
     prof_begin(kReduce, st);
-    syrk_reduce_kernel<<<blocks, thr, 0, st>>>(part, p, nsum, C, ldc, status);
+    syrk_reduce_kernel<<<(p * (p + 1) / 2 + 15) / 16, 256, 0, st>>>(part, p, nsum, C, ldc, status);
     prof_end(kReduce, (double)nsum * p * (p + 1) / 2, st);
     return cudaGetLastError();
   }
+  const TnPlan P = tn_plan(m, p, q, sym);
   TnArgs a;
   a.X = X;
   a.ldx = ldx;
@@ -517,6 +576,9 @@ cudaError_t tn_product(i64 m, int p, int q, const double* X, i64 ldx, const doub
   a.m = m;
   a.p = p;
   a.q = q;
+  a.tp = P.tp;
+  a.tq = P.tq;
+  a.rb = P.rb;
   a.tiles_p = P.tiles_p;
   a.nb = (m + P.rb - 1) / P.rb;
   a.T = a.nb * P.ntiles;
@@ -524,21 +586,17 @@ cudaError_t tn_product(i64 m, int p, int q, const double* X, i64 ldx, const doub
   a.part = part;
   a.status = status;
   if (m > 0) {
-    dim3 grid((unsigned)P.S);
     prof_begin(kProjection, st);
-    switch (P.tp) {
-      case 8: launch_tn_q<8>(P.tq, grid, st, a); break;
-      case 16: launch_tn_q<16>(P.tq, grid, st, a); break;
-      case 32: launch_tn_q<32>(P.tq, grid, st, a); break;
-      default: launch_tn_q<64>(P.tq, grid, st, a); break;
-    }
+    const size_t smem = tn_smem(P.tp, P.tq, P.rb);
+    if (P.tp == 64 && P.tq == 64 && P.rb == kFullRows)
+      tn_partial_kernel<true><<<(unsigned)P.S, kTnThreads, smem, st>>>(a);
+    else
+      tn_partial_kernel<false><<<(unsigned)P.S, kTnThreads, smem, st>>>(a);
     prof_end(kProjection, 2.0 * (double)m * p * q, st);
   }
   const i64 pq = (i64)p * q;
-  const int thr = 256;
-  const unsigned blocks = (unsigned)((pq + thr - 1) / thr);
   prof_begin(kReduce, st);
-  tn_reduce_kernel<<<blocks, thr, 0, st>>>(part, p, q, P.tp, P.tq, P.tiles_p, a.nb, m > 0 ? a.T : 0,
+  tn_reduce_kernel<<<(unsigned)((pq + 15) / 16), 256, 0, st>>>(part, p, q, P.tp, P.tq, P.tiles_p, a.nb, m > 0 ? a.T : 0,
                                            m > 0 ? a.P : 1, C, ldc, status);
   prof_end(kReduce, m > 0 ? (double)(P.S + P.ntiles) / P.ntiles * pq : 0.0, st);
   return cudaGetLastError();
