@@ -29,6 +29,9 @@ constexpr int kTrsmEmuB = 32;
 
 // Offsets of the words cqr_read_status and cqr_read_panel_width read.
 constexpr size_t kStatusOffset = 0, kPanelOffset = 512;
+// The status word and gram_chol's counter share the first 256 bytes, which
+// one memset clears at the start of a call.
+constexpr size_t kCounterOffset = 64, kClearBytes = 256;
 
 // Panel width after a rejected panel (adaptive width): the largest divisor
 // of b that is <= b/2, so that it still divides the remaining width.
@@ -121,6 +124,7 @@ Layout make_layout(i64 m, i64 n, int b, int variant, bool emulated = false, bool
 
 struct Work {
   int* status;
+  unsigned int* counter;  // gram_chol's block counter (zero between launches)
   int* skip;  // second-pass decision of the runtime repetition choice; panel test of the adaptive width
   double *W, *S1, *S2, *rinv, *Z, *R1, *R2, *part;
   void* oz;   // emulated projections and updates (null: native FP64)
@@ -130,6 +134,7 @@ Work bind(void* ws, const Layout& L) {
   char* p = (char*)ws;
   Work w;
   w.status = (int*)(p + L.status);
+  w.counter = (unsigned int*)(p + L.status + kCounterOffset);
   w.skip = (int*)(p + L.skip);
   w.W = (double*)(p + L.W);
   w.S1 = (double*)(p + L.S1);
@@ -193,9 +198,10 @@ cudaError_t cqr_panel(i64 m, int b, double* X, i64 ldx, double* U, i64 ldu, cons
   int* skip = second_pass_rule ? w.skip : nullptr;
   if (w.oz)  // emulated variant: the Gram W = X^T X on the tensor cores too (exactly symmetric)
     TRY(tn_product_emulated(m, b, b, X, ldx, X, ldx, w.oz, w.W, b, w.status, st));
+  if (w.oz)
+    TRY(chol_factor(b, w.W, b, U, ldu, w.rinv, col0, w.status, shift, m, st, skip));
   else
-    TRY(tn_product(m, b, b, X, ldx, X, ldx, 1, w.part, w.W, b, w.status, st));
-  TRY(chol_factor(b, w.W, b, U, ldu, w.rinv, col0, w.status, shift, m, st, skip));
+    TRY(gram_chol(m, b, X, ldx, w.part, w.W, b, U, ldu, w.rinv, col0, w.status, shift, w.counter, st, skip));
   TRY(trsm_any(m, b, X, ldx, U, ldu, w.rinv, w.status, st, skip, w.oz));
   return cudaSuccess;
 }
@@ -383,8 +389,8 @@ cudaError_t mcqr2gs_halving_run(i64 m, i64 n, int b, double* Q, i64 ldq, double*
       TracePhase ph("panel_test", pc);
       int rej = 0;
       TRY(cudaMemsetAsync(w.skip, 0, sizeof(int), st));
-      TRY(tn_product(m, bw, bw, Aj, ldq, Aj, ldq, 1, w.part, w.W, bw, w.status, st));
-      TRY(chol_factor(bw, w.W, bw, w.S1, bw, w.rinv, (int)c0, w.status, 0, m, st, nullptr, w.skip));
+      TRY(gram_chol(m, bw, Aj, ldq, w.part, w.W, bw, w.S1, bw, w.rinv, (int)c0, w.status, 0, w.counter, st, nullptr,
+                    w.skip));
       TRY(cudaMemcpyAsync(&rej, w.skip, sizeof(int), cudaMemcpyDeviceToHost, st));
       TRY(cudaStreamSynchronize(st));
       if (!rej) break;
@@ -616,7 +622,7 @@ int cqr_factor(int64_t m, int64_t n, double* A, int64_t lda, int panel_b, double
   Work w = bind(workspace, L);
   if (emulated) w.oz = (char*)workspace + L.oz;
   cudaGetLastError();  // clear stale errors from earlier, unrelated calls
-  if (cudaMemsetAsync(w.status, 0, sizeof(int), st) != cudaSuccess) return CQR_ERR_CUDA;
+  if (cudaMemsetAsync(w.status, 0, kClearBytes, st) != cudaSuccess) return CQR_ERR_CUDA;
   if (Q != A && cudaMemcpy2DAsync(Q, sizeof(double) * ldq, A, sizeof(double) * lda, sizeof(double) * m, n,
                                   cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return CQR_ERR_CUDA;
@@ -695,7 +701,7 @@ int cqr_factor_host(int64_t m, int64_t n, const double* A, int64_t lda, int pane
   // Alg. 9 overlaps; the other variants copy in, factor and copy out
   const bool overlap = variant == CQR_MCQR2GS;
   const i64 first = overlap ? b : n;
-  if (cudaMemsetAsync(w.status, 0, sizeof(int), st) != cudaSuccess) return CQR_ERR_CUDA;
+  if (cudaMemsetAsync(w.status, 0, kClearBytes, st) != cudaSuccess) return CQR_ERR_CUDA;
   if (cudaMemset2DAsync(Rd, sizeof(double) * ldrd, 0, sizeof(double) * n, n, st) != cudaSuccess) return CQR_ERR_CUDA;
   if (copy_cols(Qd, ldqd, A, lda, m, 0, first, cudaMemcpyHostToDevice, st) != cudaSuccess) return CQR_ERR_CUDA;
   // the copy stream starts behind the first panel's copy (which it does not
@@ -1024,7 +1030,9 @@ int cqr_factor_batched(int batch, const int64_t* m, const int64_t* n, const int6
   if (cudaMemsetAsync(status, 0, sizeof(int) * batch, st) != cudaSuccess || cudaEventRecord(pool->fork, st) != cudaSuccess)
     rc = CQR_ERR_CUDA;
   for (int k = 0; k < ns && rc == 0; ++k)
-    if (cudaStreamWaitEvent(pool->s[k], pool->fork, 0) != cudaSuccess) rc = CQR_ERR_CUDA;
+    if (cudaStreamWaitEvent(pool->s[k], pool->fork, 0) != cudaSuccess ||
+        cudaMemsetAsync((char*)workspace + slice * k, 0, kClearBytes, pool->s[k]) != cudaSuccess)
+      rc = CQR_ERR_CUDA;
   for (int q = 0; q < batch && rc == 0; ++q) {
     const int i = order[q];
     int k = 0;
@@ -1111,7 +1119,7 @@ int cqr_factor_noalloc(int64_t m, int64_t n, double* A, int64_t lda, int panel_b
   const Work w = bind(scratch, L);
   cudaGetLastError();
   // The array keeps the previous call's contents: the status word must start at 0.
-  if (cudaMemsetAsync(w.status, 0, sizeof(int), st) != cudaSuccess) return CQR_ERR_CUDA;
+  if (cudaMemsetAsync(w.status, 0, kClearBytes, st) != cudaSuccess) return CQR_ERR_CUDA;
   if (Q != A && cudaMemcpy2DAsync(Q, sizeof(double) * ldq, A, sizeof(double) * lda, sizeof(double) * m, n,
                                   cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return CQR_ERR_CUDA;

@@ -1,0 +1,114 @@
+// Cholesky factorisation of a small Gram matrix inside one block: shared by
+// the single-matrix kernels (k_chol.cu) and the persistent batched kernel.
+#pragma once
+#include <cuda_runtime.h>
+
+namespace cqr {
+
+// sqrt(d) and 1/sqrt(d) of a positive normal d by Newton's iteration.  The
+// FP64 pipe of an SM takes 64 clocks for every warp instruction, also for a
+// single live lane, so the chain of FP64 operations per column is what the
+// factorisation of a small matrix costs (sqrt() and 1/x take 600 and 354
+// clocks).  Here the reciprocal square root starts from the FP32 one of the
+// scaled mantissa m = d 2^(-2k) in [1, 4), and its Newton step is evaluated
+// in pairs of FP32 numbers (residual 1 - m r0^2 to 2^-46), which leaves r a
+// relative error of about 2^-44 for one FP64 addition; one correction step
+// u = u0 + (m - u0^2) r / 2 with an exact (fused) residual then gives the
+// root itself (Markstein, IBM J. Res. Dev. 34 (1990): a correction with the
+// fused residual rounds correctly but for near-ties; an exact root comes out
+// exact).
+__device__ __forceinline__ void sqrt_rsqrt(double d, double& u, double& r) {
+  const int hi = __double2hiint(d), lo = __double2loint(d);
+  const int ex = (hi >> 20) - 1023;
+  if (ex == -1023) {  // subnormal
+    u = sqrt(d);
+    r = 1.0 / u;
+    return;
+  }
+  const int k = ex >> 1, odd = ex & 1;
+  const int mh = hi - (k << 21);  // m = d 2^(-2k)
+  const double md = __hiloint2double(mh, lo);
+  const float f = __uint_as_float((unsigned)((127 + odd) << 23) | ((unsigned)(hi & 0xFFFFF) << 3) |
+                                  ((unsigned)lo >> 29));
+  const float fl = __uint2float_rn((unsigned)lo & 0x1FFFFFFFu) * (odd ? 0x1p-51f : 0x1p-52f);  // m = f + fl
+  const float r0 = rsqrtf(f);
+  const float ph = __fmul_rn(r0, r0), pl = __fmaf_rn(r0, r0, -ph);
+  float t = __fmaf_rn(-f, ph, 1.0f);
+  t = __fmaf_rn(-f, pl, t);
+  t = __fmaf_rn(-fl, ph, t);                                      // 1 - m r0^2
+  const float c = r0 * t * __fmaf_rn(0.375f, t, 0.5f);            // r0 ((1 - t)^(-1/2) - 1)
+  const double rm = (double)r0 + (double)c;
+  const double hr = __hiloint2double(__double2hiint(rm) - (1 << 20), __double2loint(rm));  // rm / 2
+  const double u0 = md * rm;
+  const double um = fma(fma(-u0, u0, md), hr, u0);
+  u = __hiloint2double(__double2hiint(um) + (k << 20), __double2loint(um));
+  r = __hiloint2double(__double2hiint(rm) - (k << 20), __double2loint(rm));
+}
+
+// ---------------------------------------------------------------------------
+// The rows of a trapezoid in shared memory: Ws (row-major, ld) holds the
+// upper triangle of a kb x kb diagonal block and nx further columns of the
+// same rows; on return row j of both is row j of the factor (the diagonal in
+// dg).  T threads, one barrier per row.  In step j the pivot warps (32
+// columns each) apply the update of row j - 1 to row j, take the square root
+// of its diagonal (each warp for itself) and scale it, while the other warps
+// apply the update of row j - 1 to the rows below; U_jc = w / u is w r
+// corrected with the fused residual, so exact quotients stay exact.  The
+// elements of the rows below are enumerated from the last row up (tab), so
+// the live ones are always a prefix and no lane idles.  Returns the row
+// that broke down, or -1.  Scratch in shared memory: urow (2 x us, us >= kb
+// + nx), tab (an entry per element), broken.  kb + nx <= 32 (T / 32 - 1).
+template <int T>
+__device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* urow, int us, double* dg,
+                              unsigned short* tab, int* broken) {
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  if (t == 0) *broken = -1;
+  for (int row = warp; row < kb; row += T / 32) {
+    const int k = kb - 1 - row, start = k * (k + 1) / 2 + k * nx;
+    for (int c = row + lane; c < kb + nx; c += 32) tab[start + c - row] = (unsigned short)((row << 8) | c);
+  }
+  __syncthreads();
+  const int np = (kb + nx - 1 + 31) / 32 > 0 ? (kb + nx - 1 + 31) / 32 : 1;
+  for (int j = 0; j < kb; ++j) {
+    int bad = 0;
+    const double* prev = urow + ((j + 1) & 1) * us;
+    double* cur = urow + (j & 1) * us;
+    if (warp < np) {
+      const int c = j + 1 + 32 * warp + lane;
+      double* row = Ws + j * ld;
+      const bool live = c < kb + nx;
+      double d = row[j], w = live ? row[c] : 0.0;
+      if (j > 0) {
+        const double pj = prev[j];
+        d = fma(-pj, pj, d);
+        if (live) w = fma(-pj, prev[c], w);
+      }
+      // d > 0 and finite, in integers (an FP64 comparison takes 64 clocks of the chain)
+      const int dh = __double2hiint(d);
+      if (dh < 0x7FF00000 && (dh > 0 || (dh == 0 && __double2loint(d) != 0))) {
+        double u, r;
+        sqrt_rsqrt(d, u, r);
+        if (live) {
+          const double q0 = w * r;
+          const double q = fma(fma(-q0, u, w), r, q0);
+          cur[c] = q;
+          row[c] = q;
+        }
+        if (t == 0) dg[j] = u;
+      } else {
+        bad = 1;
+        if (t == 0) *broken = j;
+      }
+    } else if (j > 0) {
+      const int k = kb - 1 - j, len = k * (k + 1) / 2 + k * nx;  // rows j+1 .. kb-1
+      for (int e = t - 32 * np; e < len; e += T - 32 * np) {
+        const int i = tab[e] >> 8, c = tab[e] & 255;
+        Ws[i * ld + c] = fma(-prev[i], prev[c], Ws[i * ld + c]);
+      }
+    }
+    if (__syncthreads_or(bad)) break;
+  }
+  return *broken;
+}
+
+}  // namespace cqr

@@ -137,6 +137,13 @@ cudaError_t nn_product_t(i64 M, int N, int K, const double* A, i64 lda, const do
 // else 0.  The kernel returns early, writing nothing, if *status != 0.
 cudaError_t chol_factor(int b, double* W, i64 ldw, double* U, i64 ldu, double* rinv, int col0, int* status,
                         int shift_fro, i64 m, cudaStream_t st, int* skip = nullptr, int* reject = nullptr);
+// W = X^T X (m x b panel X) and its Cholesky factorisation: tn_product() and
+// chol_factor(), with the partials' sum and the factorisation in one launch
+// for b <= 64.  `counter` must be zero when the stream reaches the call; it
+// is left zero.  W (upper triangle) is scratch.
+cudaError_t gram_chol(i64 m, int b, const double* X, i64 ldx, double* part, double* W, i64 ldw, double* U, i64 ldu,
+                      double* rinv, int col0, int* status, int shift_fro, unsigned int* counter, cudaStream_t st,
+                      int* skip = nullptr, int* reject = nullptr);
 
 // ---------------------------------------------------------------------------
 // Row-wise forward substitution  X := X U^{-1}  (X m x b, b <= kTrsmMaxB),
