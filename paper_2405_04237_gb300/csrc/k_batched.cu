@@ -2,17 +2,25 @@
 // (n <= 128) in ONE cooperative launch.
 //
 // Work split.  The grid holds one CTA of kBT threads per SM, all resident
-// (cooperative launch).  CTAs form groups of G consecutive blocks; group g
-// factors, one after the other, the matrices of its list (a static
-// largest-first schedule computed on the host).  Inside a group the rows of
-// the current matrix are split into G contiguous ranges, one per CTA: this
+// (cooperative launch).  CTAs form groups of consecutive blocks; a group
+// factors, one after the other, the matrices of its list (a static schedule
+// computed on the host).  By default the groups are the nodes of a binary
+// tree over the CTAs: all CTAs first factor the root's matrices together,
+// then each half its own, each quarter, and so on down to single CTAs, so a
+// batch of uneven matrices ends at about the same time on every SM (with
+// groups of 8 the largest matrix of a batch, 200000 x 128, alone took 3.5
+// times the batch's work divided by the chip); a given group size makes one
+// level of equal groups.  Inside a group of G CTAs the rows of the current
+// matrix are split into G contiguous ranges, one per CTA: this
 // is the paper's 1-D row-block distribution (Alg. 2, Alg. 8) with the G
 // CTAs as the ranks.  Every step that sums over the m rows ends with each
 // CTA writing its partial sum to its own slot, a group barrier, and every
 // CTA adding the G slots in rank order and doing the small dense work (the
 // b x b Cholesky, the triangular products) redundantly -- the "Allreduce +
 // redundant Cholesky" of Alg. 2 -- so all CTAs of a group hold bitwise
-// identical factors without a second barrier.
+// identical factors without a second barrier.  In groups of more than
+// kDirectSum CTAs each one first adds its share of the entries over all
+// slots, and a second barrier publishes the sums.
 //
 // Passes.  One panel step of Alg. 9 reads the rows it needs once per pass,
 // in sub-blocks of 64 to 256 rows (more when fewer columns are loaded)
@@ -44,6 +52,8 @@
 #include <mutex>
 #include <vector>
 
+#include "block_sums.cuh"
+#include "chol_device.cuh"
 #include "cqr.h"
 #include "cqr_common.cuh"
 
@@ -73,17 +83,33 @@ struct BMat {
   int n, b;     // width, starting panel width
 };
 
+// Groups of the launch: level l cuts the N CTAs into cnt[l] groups of equal
+// size (to within one), group g = CTAs [g N / cnt, (g + 1) N / cnt).  Every
+// CTA walks the levels in order; the groups of a level lie inside those of
+// the level before.
+constexpr int kBLevels = 12;  // 1, 2, 4, .. and N itself: grids of up to 1024 CTAs
+struct BLevels {
+  int n;
+  int cnt[kBLevels];
+  int off[kBLevels];   // node of the level's group 0 (node = entry of gstart, barrier counter)
+};
+
+// Slots added directly by every CTA.  Adding G slots costs b (b + 1) / 2 G
+// FP64 adds on every SM (2 per clock): 2 us at b = 64, G = 8, 40 us at G =
+// 152, against about 3 us for a second barrier.
+constexpr int kDirectSum = 8;
+
 struct BArgs {
   const BMat* mats;
-  const int* order;    // matrices of group g: order[gstart[g] .. gstart[g+1])
+  const int* order;    // matrices of node v: order[gstart[v] .. gstart[v+1])
   const int* gstart;
+  BLevels lev;
   int* status;         // per matrix
   int* bfinal;         // per matrix: width of its last panel
   double* part;        // [2][gridDim.x][kBSlot]
-  double* s1;          // [groups][kBNMax * kBNMax]: S1 of the current panel (column-major)
-  unsigned int* bar;   // [groups] barrier counters (zero at launch)
+  double* s1;          // [gridDim.x][kBNMax * kBNMax]: S1 of the current panel (column-major), at the group's first CTA
+  unsigned int* bar;   // [nodes] barrier counters (zero at launch)
   int* abort;          // launch-wide abort flag (zero at launch)
-  int G;               // CTAs per group
   int nmax, bmax;      // shared-memory layout
   int halve;           // adaptive panel width
   unsigned long long wait_ns;
@@ -149,19 +175,25 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
 }
 
+struct Group {
+  int node, g;   // node over all levels, index within the level
+  int lo, G;     // first CTA, CTAs
+  int rank;
+};
+
 // Group barrier, bounded in time.  Returns false (for every thread of the
 // CTA) when the wait expired or another CTA raised the abort flag.
-__device__ bool group_barrier(const BArgs& a, int group, int rank, unsigned int* count, int* ok) {
+__device__ __noinline__ bool group_barrier(const BArgs& a, const Group& gr, unsigned int* count, int* ok) {
   __syncthreads();
   if (threadIdx.x == 0) {
     const unsigned int c = ++(*count);
     int good = 1;
     __threadfence();  // this CTA's partial sums and R columns before the arrival
-    const bool skip = group == a.hook_group && rank == a.hook_rank && (int)c == a.hook_barrier;
-    if (!skip) atomicAdd(&a.bar[group], 1u);
-    const unsigned int target = c * (unsigned int)a.G;
+    const bool skip = gr.g == a.hook_group && gr.rank == a.hook_rank && (int)c == a.hook_barrier;
+    if (!skip) atomicAdd(&a.bar[gr.node], 1u);
+    const unsigned int target = c * (unsigned int)gr.G;
     const unsigned long long t0 = bglobal_ns();
-    while (ld_acquire(&a.bar[group]) < target) {
+    while (ld_acquire(&a.bar[gr.node]) < target) {
       if (*(volatile int*)a.abort) {
         good = 0;
         break;
@@ -258,38 +290,19 @@ __device__ __forceinline__ void tn_accumulate(const TnMap& mp, const Smem& s, in
   }
 }
 
-// In-CTA sums of the accumulators in a fixed order (row groups, then the
-// threads of an extra tile in thread order), written tile-major (16 doubles
-// per tile, entry u * 4 + v) to this CTA's slot.
+// In-CTA sums of the accumulators in a fixed order (block_sums), written
+// tile-major (16 doubles per tile, entry u * 4 + v) to this CTA's slot.
 __device__ void tn_flush(const TnMap& mp, const Smem& s, double (&am)[4][4], double (&ae)[4][4], double* slot) {
-  const int t = threadIdx.x;
   __syncthreads();
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int v = 0; v < 4; ++v) s.red[(size_t)t * 16 + u * 4 + v] = am[u][v];
+  spill_acc(s.red, kBT, am);
   __syncthreads();
-  if (t < mp.M) {
-    for (int e = 0; e < 16; ++e) {
-      double sum = 0.0;
-      for (int g = 0; g < mp.RG; ++g) sum += s.red[(size_t)(g * mp.M + t) * 16 + e];
-      slot[(size_t)t * 16 + e] = sum;
-    }
-  }
+  block_sums<kBT>(s.red, s.red, mp.M, mp.RG, 1, mp.M, [slot](int id, int e, double x) { slot[id * 16 + e] = x; });
   __syncthreads();
   if (mp.E > 0) {
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-      for (int v = 0; v < 4; ++v) s.red[(size_t)t * 16 + u * 4 + v] = ae[u][v];
+    spill_acc(s.red, kBT, ae);
     __syncthreads();
-    if (t < mp.E * mp.tpt && t % mp.tpt == 0) {
-      for (int e = 0; e < 16; ++e) {
-        double sum = 0.0;
-        for (int k = 0; k < mp.tpt; ++k) sum += s.red[(size_t)(t + k) * 16 + e];
-        slot[(size_t)(mp.M + t / mp.tpt) * 16 + e] = sum;
-      }
-    }
+    double* slot_e = slot + (size_t)mp.M * 16;
+    block_sums<kBT>(s.red, s.red, mp.E, mp.tpt, mp.tpt, 1, [slot_e](int id, int e, double x) { slot_e[id * 16 + e] = x; });
     __syncthreads();
   }
 }
@@ -481,45 +494,77 @@ __device__ __forceinline__ double slot_sum(const double* slots, int G, int sym, 
   return v;
 }
 
+// Where the reduced sums of a pass are found: G slots to add, in rank order.
+struct Sums {
+  const double* p;
+  int G;
+};
+
+// Entries of a partial in a slot: whole 4 x 4 tiles.
+__device__ __forceinline__ int gram_entries(int b) { return 8 * (b / 4) * (b / 4 + 1); }
+
+// After a pass: waits until every CTA of the group has written its partial
+// (n entries) and tells where to read the sums.  Large groups: CTA r adds
+// entries [r n / G, (r + 1) n / G) of all slots (up to 16 threads an entry,
+// their parts added in order), writes them to `res` and meets the others
+// again.
+__device__ __noinline__ bool exchange(const BArgs& a, const Group& gr, const Smem& s, const double* slots, double* res, int n,
+                         unsigned int* count, int* ok, Sums* out) {
+  if (!group_barrier(a, gr, count, ok)) return false;
+  out->p = slots;
+  out->G = gr.G;
+  if (gr.G <= kDirectSum) return true;
+  const int t = threadIdx.x;
+  const int e0 = (int)((i64)n * gr.rank / gr.G), len = (int)((i64)n * (gr.rank + 1) / gr.G) - e0;
+  int parts = 1;
+  while (parts < 16 && 2 * parts * len <= kBT) parts *= 2;
+  if (len > 0 && parts > 1) {
+    const int x = t % len, y = t / len;
+    if (y < parts) {
+      const double* p = slots + e0 + x;
+      double v = 0.0;
+      const int k1 = (y + 1) * gr.G / parts;
+#pragma unroll 4
+      for (int k = y * gr.G / parts; k < k1; ++k) v += p[(size_t)k * kBSlot];
+      s.red[y * len + x] = v;
+    }
+    __syncthreads();
+    if (t < len) {
+      double v = s.red[t];
+      for (int y = 1; y < parts; ++y) v += s.red[y * len + t];
+      res[e0 + t] = v;
+    }
+  } else {
+    for (int x = t; x < len; x += kBT) {
+      const double* p = slots + e0 + x;
+      double v = 0.0;
+#pragma unroll 4
+      for (int k = 0; k < gr.G; ++k) v += p[(size_t)k * kBSlot];
+      res[e0 + x] = v;
+    }
+  }
+  out->p = res;
+  out->G = 1;
+  return group_barrier(a, gr, count, ok);
+}
+
 // W = sum of the slots (upper triangle), then the right-looking Cholesky
 // W = U^T U in shared memory.  Returns the local breakdown column or -1;
 // *rej (when the panel test is on and b > 1) = breakdown or
 // (max U_jj / min U_jj)^2 > 1/(64 u).  Leaves U with zero diagonal and
 // lower triangle in s.U, the diagonal in s.dg and its reciprocals in s.rv.
-__device__ int reduce_cholesky(const Smem& s, const double* slots, int G, int b, bool test, int* rej,
+__device__ __noinline__ int reduce_cholesky(const Smem& s, const double* slots, int G, int b, bool test, int* rej,
                                int* sh_broken) {
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nw = kBT / 32;
+  const int t = threadIdx.x;
   double* U = s.U;
   for (int e = t; e < b * b; e += kBT) {
     const int a = e / b, c = e % b;
     U[e] = a <= c ? slot_sum(slots, G, 1, 0, a, c) : 0.0;
   }
-  if (t == 0) *sh_broken = -1;
-  __syncthreads();
-  for (int j = 0; j < b; ++j) {
-    if (warp == 0) {
-      const double d = U[(size_t)j * b + j];
-      if (d > 0.0 && isfinite(d)) {
-        const double u = sqrt(d);
-        for (int c = j + 1 + lane; c < b; c += 32) U[(size_t)j * b + c] /= u;
-        if (lane == 0) {
-          U[(size_t)j * b + j] = u;
-          s.dg[j] = u;
-          s.rv[j] = 1.0 / u;
-        }
-      } else if (lane == 0) {
-        *sh_broken = j;
-      }
-    }
-    __syncthreads();
-    if (*sh_broken >= 0) break;
-    for (int a = j + 1 + warp; a < b; a += nw) {
-      const double ua = U[(size_t)j * b + a];
-      for (int c = a + lane; c < b; c += 32) U[(size_t)a * b + c] = fma(-ua, U[(size_t)j * b + c], U[(size_t)a * b + c]);
-    }
-    __syncthreads();
-  }
-  const int broken = *sh_broken;
+  // scratch of the factorisation in the staging area (free between passes)
+  double* urow = s.red;
+  const int broken = chol_trapezoid<kBT>(U, b, b, 0, urow, kBNMax, s.dg,
+                                         reinterpret_cast<unsigned short*>(urow + 2 * kBNMax), sh_broken);
   if (test && t == 0) {
     int r = 0;
     if (b > 1) {
@@ -538,13 +583,16 @@ __device__ int reduce_cholesky(const Smem& s, const double* slots, int G, int b,
   }
   __syncthreads();
   if (broken < 0)  // the solve's form: zero diagonal (its reciprocal is in rv)
-    for (int e = t; e < b; e += kBT) U[(size_t)e * b + e] = 0.0;
+    for (int e = t; e < b; e += kBT) {
+      U[(size_t)e * b + e] = 0.0;
+      s.rv[e] = 1.0 / s.dg[e];
+    }
   __syncthreads();
   return broken;
 }
 
 // M = sum of the slots: a p x q transposed product, row-major in s.M.
-__device__ void reduce_tn(const Smem& s, const double* slots, int G, int p, int q) {
+__device__ __noinline__ void reduce_tn(const Smem& s, const double* slots, int G, int p, int q) {
   for (int e = threadIdx.x; e < p * q; e += kBT) {
     const int a = e / q, c = e % q;
     s.M[e] = slot_sum(slots, G, 0, p / 4, a, c);
@@ -563,39 +611,59 @@ __device__ int halved(int b) {
   return 1;
 }
 
-__global__ void __launch_bounds__(kBT, 1) batched_mcqr2gs_kernel(BArgs a) {
+__global__ void __launch_bounds__(kBT, 1) batched_mcqr2gs_kernel(const __grid_constant__ BArgs a) {
   extern __shared__ __align__(16) double bsm[];
   __shared__ unsigned int bar_count;
   __shared__ int bar_ok, sh_broken, sh_rej;
+  __shared__ Group gr;  // state that outlives the passes stays out of the registers
+  __shared__ BMat mt;
   const Smem s = carve(bsm, a.nmax, a.bmax);
   const int t = threadIdx.x;
-  const int group = blockIdx.x / a.G, rank = blockIdx.x % a.G;
-  if (t == 0) bar_count = 0;
-  __syncthreads();
-  double* slots[2] = {a.part + (size_t)(0 * gridDim.x + group * a.G) * kBSlot,
-                      a.part + (size_t)(1 * gridDim.x + group * a.G) * kBSlot};
-  int phase = 0;  // partial buffer parity
-  double* s1g = a.s1 + (size_t)group * kBNMax * kBNMax;
-  const int l0 = a.gstart[group], l1 = a.gstart[group + 1];
   bool alive = true;
+  for (int lev = 0; lev < a.lev.n; ++lev) {
+  __syncthreads();
+  if (t == 0) {
+    const int N = gridDim.x, cnt = a.lev.cnt[lev];
+    gr.g = ((blockIdx.x + 1) * cnt - 1) / N;
+    gr.node = a.lev.off[lev] + gr.g;
+    gr.lo = (int)((i64)gr.g * N / cnt);
+    gr.G = (int)((i64)(gr.g + 1) * N / cnt) - gr.lo;
+    gr.rank = blockIdx.x - gr.lo;
+    bar_count = 0;
+  }
+  __syncthreads();
+  const int rank = gr.rank, G = gr.G;
+  const int l0 = a.gstart[gr.node], l1 = a.gstart[gr.node + 1];
+  if (l0 == l1) continue;
+  // partial buffers: two by phase parity, or (large groups) one and the sums' place
+  const bool two = G > kDirectSum;
+  double* slots[2] = {a.part + (size_t)gr.lo * kBSlot, a.part + (size_t)(gridDim.x + gr.lo) * kBSlot};
+  int phase = 0;
+  auto cur = [&]() { return slots[two ? 0 : (phase & 1)]; };
+  auto meet = [&](int entries, Sums* out) {
+    return exchange(a, gr, s, cur(), slots[1], entries, &bar_count, &bar_ok, out);
+  };
+  double* s1g = a.s1 + (size_t)gr.lo * kBNMax * kBNMax;
   int li = l0;
   for (; li < l1 && alive; ++li) {
-    if (*(volatile int*)a.abort) {
+    if (__syncthreads_or(*(volatile int*)a.abort)) {  // one decision for the CTA
       alive = false;
       break;
     }
     const int mi = a.order[li];
-    const BMat mt = a.mats[mi];
+    if (t == 0) mt = a.mats[mi];
+    __syncthreads();
     const int n = mt.n;
-    const i64 R0 = (i64)rank * mt.m / a.G, R1 = (i64)(rank + 1) * mt.m / a.G;
+    const i64 R0 = (i64)rank * mt.m / G, R1 = (i64)(rank + 1) * mt.m / G;
     const bool oop = mt.Q != mt.A;
     // zero R (column slices of this rank)
-    for (int c = rank; c < n; c += a.G)
+    for (int c = rank; c < n; c += G)
       for (int e = t; e < n; e += kBT) mt.R[e + (i64)c * n] = 0.0;
     int bw = mt.b, bprev = 0;
     bool failed = false;  // a breakdown: the group leaves this matrix
     for (int c0 = 0; c0 < n && alive && !failed;) {
-      double* my = slots[phase & 1] + (size_t)rank * kBSlot;
+      double* my = cur() + (size_t)rank * kBSlot;
+      Sums sums{};
       // ---- the first CholeskyQR's Gram (with the update of step 4 for c0 > 0)
       {
         PassSpec P{};
@@ -627,12 +695,12 @@ __global__ void __launch_bounds__(kBT, 1) batched_mcqr2gs_kernel(BArgs a) {
         }
         run_pass(P, s, R0, R1, my);
       }
-      if (!(alive = group_barrier(a, group, rank, &bar_count, &bar_ok))) break;
-      int broken = reduce_cholesky(s, slots[phase & 1], a.G, bw, a.halve != 0, &sh_rej, &sh_broken);
+      if (!(alive = meet(gram_entries(bw), &sums))) break;
+      int broken = reduce_cholesky(s, sums.p, sums.G, bw, a.halve != 0, &sh_rej, &sh_broken);
       ++phase;
       while (a.halve && bw > 1 && sh_rej) {  // rejected panel: its Gram again at the narrower width
         bw = halved(bw);
-        my = slots[phase & 1] + (size_t)rank * kBSlot;
+        my = cur() + (size_t)rank * kBSlot;
         PassSpec P{};
         P.src = mt.Q;
         P.lds = mt.lda;
@@ -642,8 +710,8 @@ __global__ void __launch_bounds__(kBT, 1) batched_mcqr2gs_kernel(BArgs a) {
         P.g0 = c0;
         P.gb = bw;
         run_pass(P, s, R0, R1, my);
-        if (!(alive = group_barrier(a, group, rank, &bar_count, &bar_ok))) break;
-        broken = reduce_cholesky(s, slots[phase & 1], a.G, bw, true, &sh_rej, &sh_broken);
+        if (!(alive = meet(gram_entries(bw), &sums))) break;
+        broken = reduce_cholesky(s, sums.p, sums.G, bw, true, &sh_rej, &sh_broken);
         ++phase;
       }
       if (!alive) break;
@@ -662,7 +730,7 @@ __global__ void __launch_bounds__(kBT, 1) batched_mcqr2gs_kernel(BArgs a) {
       __syncthreads();  // S1 saved from the unscaled factor
       prescale_rows(s, bw);
       {
-        my = slots[phase & 1] + (size_t)rank * kBSlot;
+        my = cur() + (size_t)rank * kBSlot;
         PassSpec P{};
         P.src = mt.Q;
         P.lds = mt.lda;
@@ -688,12 +756,12 @@ __global__ void __launch_bounds__(kBT, 1) batched_mcqr2gs_kernel(BArgs a) {
         }
         run_pass(P, s, R0, R1, my);
       }
-      if (!(alive = group_barrier(a, group, rank, &bar_count, &bar_ok))) break;
+      if (!(alive = meet(c0 == 0 ? gram_entries(bw) : c0 * bw, &sums))) break;
       if (c0 > 0) {
-        reduce_tn(s, slots[phase & 1], a.G, c0, bw);  // Z (c0 x bw) in M
+        reduce_tn(s, sums.p, sums.G, c0, bw);  // Z (c0 x bw) in M
         ++phase;
         // ---- RO: P -= Q_{1:j-1} Z, then the Gram of P
-        my = slots[phase & 1] + (size_t)rank * kBSlot;
+        my = cur() + (size_t)rank * kBSlot;
         PassSpec P{};
         P.src = mt.Q;
         P.lds = mt.lda;
@@ -713,9 +781,9 @@ __global__ void __launch_bounds__(kBT, 1) batched_mcqr2gs_kernel(BArgs a) {
         P.g0 = c0;
         P.gb = bw;
         run_pass(P, s, R0, R1, my);
-        if (!(alive = group_barrier(a, group, rank, &bar_count, &bar_ok))) break;
+        if (!(alive = meet(gram_entries(bw), &sums))) break;
       }
-      broken = reduce_cholesky(s, slots[phase & 1], a.G, bw, false, &sh_rej, &sh_broken);  // S2
+      broken = reduce_cholesky(s, sums.p, sums.G, bw, false, &sh_rej, &sh_broken);  // S2
       ++phase;
       if (broken >= 0) {
         if (rank == 0 && t == 0) atomicCAS(&a.status[mi], 0, c0 + broken + 1);
@@ -734,10 +802,10 @@ __global__ void __launch_bounds__(kBT, 1) batched_mcqr2gs_kernel(BArgs a) {
           s1p[e] = s1g[(size_t)c * bw + i];
         }
         __syncthreads();
-        const int ncol = (bw - rank + a.G - 1) / a.G;  // this rank's columns c = rank + G * k
+        const int ncol = (bw - rank + G - 1) / G;  // this rank's columns c = rank + G * k
         const int per = c0 + bw;                       // rows of R above and on the diagonal block
         for (int e = t; e < ncol * per; e += kBT) {
-          const int c = rank + a.G * (e / per), r = e % per;
+          const int c = rank + G * (e / per), r = e % per;
           const double* s1c = s1p + c * (c + 1) / 2;  // S1[0..c][c]
           if (r >= c0) {  // R_jj entry (r - c0, c), on or above the diagonal
             const int rr = r - c0;
@@ -758,7 +826,7 @@ __global__ void __launch_bounds__(kBT, 1) batched_mcqr2gs_kernel(BArgs a) {
       __syncthreads();  // the R products used the unscaled factor
       prescale_rows(s, bw);
       {
-        my = slots[phase & 1] + (size_t)rank * kBSlot;
+        my = cur() + (size_t)rank * kBSlot;
         PassSpec P{};
         P.src = mt.Q;
         P.lds = mt.lda;
@@ -783,10 +851,10 @@ __global__ void __launch_bounds__(kBT, 1) batched_mcqr2gs_kernel(BArgs a) {
         run_pass(P, s, R0, R1, my);
       }
       if (wn > 0) {
-        if (!(alive = group_barrier(a, group, rank, &bar_count, &bar_ok))) break;
-        reduce_tn(s, slots[phase & 1], a.G, bw, wn);  // Y (bw x wn) in M
+        if (!(alive = meet(bw * wn, &sums))) break;
+        reduce_tn(s, sums.p, sums.G, bw, wn);  // Y (bw x wn) in M
         ++phase;
-        for (int c = rank; c < wn; c += a.G)
+        for (int c = rank; c < wn; c += G)
           for (int r = t; r < bw; r += kBT) mt.R[(c0 + r) + (i64)(c0 + bw + c) * n] = s.M[(size_t)r * wn + c];
       }
       bprev = bw;
@@ -797,8 +865,13 @@ __global__ void __launch_bounds__(kBT, 1) batched_mcqr2gs_kernel(BArgs a) {
     // the next matrix reuses M, U and the slots only after its first barrier
     __syncthreads();
   }
-  if (!alive && rank == 0 && t == 0) {  // this group's unfinished matrices
-    for (int k = li; k < l1; ++k) atomicCAS(&a.status[a.order[k]], 0, CQR_STATUS_TIMEOUT);
+  if (!alive) {  // this group's unfinished matrices, and those of this CTA's later groups
+    if (rank == 0 && t == 0)
+      for (int k = li; k < l1; ++k) atomicCAS(&a.status[a.order[k]], 0, CQR_STATUS_TIMEOUT);
+  } else {
+    // the group's slots and S1 may be another group's at the next level
+    alive = group_barrier(a, gr, &bar_count, &bar_ok);
+  }
   }
 }
 
@@ -814,11 +887,21 @@ __global__ void blob_copy_kernel(const __grid_constant__ Blob blob, unsigned cha
     dst[e] = blob.bytes[e];
 }
 
+// Costs of the schedule's estimate.
+constexpr double kEstRate = 7.6e9;       // FP64 flop/s of one SM inside a pass
+constexpr double kEstStage = 0.05e-9;     // seconds per staged entry
+constexpr double kEstPass = 8e-6;        // a pass: barrier, launch of the loads, in-CTA sums
+constexpr double kEstBarrier = 3e-6;
+constexpr double kEstCholCol = 0.45e-6;  // one column of a Cholesky factorisation
+
 inline size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct BLayout {
   size_t mats, order, gstart, bfinal, part, s1, bar, abort, total;
 };
+
+// 1 + 2 + 4 + .. (all below the grid) and the grid's single CTAs
+int max_nodes(int grid) { return 3 * grid; }
 
 BLayout blayout(int batch, int grid) {
   BLayout L{};
@@ -830,11 +913,11 @@ BLayout blayout(int batch, int grid) {
   };
   L.mats = take(sizeof(BMat) * (size_t)batch);
   L.order = take(sizeof(int) * (size_t)batch);
-  L.gstart = take(sizeof(int) * (size_t)(grid + 1));
+  L.gstart = take(sizeof(int) * (size_t)(max_nodes(grid) + 1));
   L.bfinal = take(sizeof(int) * (size_t)batch);
   L.part = take(sizeof(double) * 2 * (size_t)grid * kBSlot);
   L.s1 = take(sizeof(double) * (size_t)grid * kBNMax * kBNMax);
-  L.bar = take(sizeof(unsigned int) * (size_t)grid);
+  L.bar = take(sizeof(unsigned int) * (size_t)max_nodes(grid));
   L.abort = take(sizeof(int));
   L.total = off;
   return L;
@@ -872,30 +955,169 @@ bool batched_persistent_eligible(int batch, const int64_t* m, const int64_t* n, 
 
 size_t batched_persistent_workspace(int batch) { return blayout(batch, persistent_grid_impl()).total; }
 
+namespace {
+
 // Rough device time of one matrix on a group of G CTAs (for the static
-// largest-first schedule): its FLOPs at G SMs' FP64 rate, plus per-phase
-// costs (barrier, slot sums, the b x b Cholesky on one SM).
-static double est_seconds(i64 m, int n, int b, int G) {
+// schedule): its multiply-adds at the FP64 rate of G SMs, the staging of its
+// row blocks, and per pass the barrier, the slots' sum and the Cholesky's
+// chain of dependent operations.
+double est_seconds(i64 m, int n, int b, int G) {
   const int k = n / b;
-  const double flops = 4.0 * (double)m * n * n;
-  const double rate = (double)G * 8.0e9;
-  const double chol = (double)b * b * b / 6.0 / 4.0e9 + 4e-6;
-  return flops / rate + (4.0 * k) * (6e-6 + chol);
+  const double flops = 4.0 * (double)m * n * n / G / kEstRate;
+  const double rows = (double)m / G * (double)n * (4 * k - 1) * kEstStage;
+  const double sum = (G > kDirectSum ? kEstBarrier : 0.0) + 0.25e-9 * b * b * (G > kDirectSum ? 1 : G);
+  return flops + rows + 4.0 * k * (kEstPass + sum) + 2.0 * k * b * kEstCholCol;
 }
+
+// The static schedule: matrices (order) of every node.
+struct BSchedule {
+  BLevels lev;
+  int nodes;
+  std::vector<int> order, gstart;
+};
+
+void finish(BSchedule& S, const std::vector<std::vector<int>>& lists) {
+  S.nodes = (int)lists.size();
+  for (const auto& l : lists) {
+    S.gstart.push_back((int)S.order.size());
+    S.order.insert(S.order.end(), l.begin(), l.end());
+  }
+  S.gstart.push_back((int)S.order.size());
+}
+
+// Equal groups of G CTAs: largest estimated time first, each to the group
+// with the least work so far.
+BSchedule schedule_uniform(int batch, const int64_t* m, const int64_t* n, const int* b, int grid, int G) {
+  BSchedule S{};
+  const int groups = grid / G;
+  S.lev.n = 1;
+  S.lev.cnt[0] = groups;
+  std::vector<std::pair<double, int>> by;
+  for (int i = 0; i < batch; ++i) by.push_back({est_seconds(m[i], (int)n[i], b[i], G), i});
+  std::stable_sort(by.begin(), by.end(),
+                   [](const std::pair<double, int>& x, const std::pair<double, int>& y) { return x.first > y.first; });
+  std::vector<double> load((size_t)groups, 0.0);
+  std::vector<std::vector<int>> lists((size_t)groups);
+  for (const auto& e : by) {
+    int g = 0;
+    for (int h = 1; h < groups; ++h)
+      if (load[h] < load[g]) g = h;
+    load[g] += e.first;
+    lists[g].push_back(e.second);
+  }
+  finish(S, lists);
+  return S;
+}
+
+// The tree schedule.  A CTA's finishing time is the sum of the loads of the
+// nodes it belongs to (the members of a node arrive together, so nobody
+// waits).  For a bound on that time, the matrices are placed by decreasing
+// work, each on the smallest groups that keep the bound (fewer CTAs waste
+// less on barriers and sums), there on the least loaded one.  The bounds
+// tried grow from the largest of the mean work per CTA and the longest
+// matrix on the whole grid; on a bound that cannot be kept the next is
+// tried, and the last takes the best place for every matrix.
+BSchedule schedule_tree(int batch, const int64_t* m, const int64_t* n, const int* b, int grid) {
+  BSchedule S{};
+  BLevels& L = S.lev;
+  int nodes = 0;
+  for (int c = 1;; c *= 2) {
+    const bool last = c >= grid || L.n == kBLevels - 1;
+    L.cnt[L.n] = last ? grid : c;
+    L.off[L.n] = nodes;
+    nodes += L.cnt[L.n++];
+    if (last) break;
+  }
+  auto lo_of = [&](int l, int g) { return (int)((i64)g * grid / L.cnt[l]); };
+  // estimated times per matrix and level (the level's smallest group)
+  std::vector<double> est((size_t)batch * L.n);
+  std::vector<int> by((size_t)batch);
+  double mean = 0.0, longest = 0.0;
+  for (int i = 0; i < batch; ++i) {
+    by[i] = i;
+    double best = 0.0;
+    for (int l = 0; l < L.n; ++l) {
+      const double t = est[(size_t)i * L.n + l] = est_seconds(m[i], (int)n[i], b[i], grid / L.cnt[l]);
+      if (l == 0 || t < best) best = t;
+    }
+    mean += est[(size_t)i * L.n + L.n - 1] / grid;
+    longest = std::max(longest, best);
+  }
+  std::stable_sort(by.begin(), by.end(), [&](int x, int y) {
+    return est[(size_t)x * L.n + L.n - 1] > est[(size_t)y * L.n + L.n - 1];
+  });
+  std::vector<double> cta((size_t)grid);     // load of each CTA
+  std::vector<double> peak((size_t)nodes);   // largest load of the node's CTAs
+  std::vector<int> place((size_t)batch);
+  double bound = std::max(mean, longest);
+  for (int attempt = 0;; ++attempt, bound *= 1.08) {
+    const bool last = attempt == 12;
+    std::fill(cta.begin(), cta.end(), 0.0);
+    std::fill(peak.begin(), peak.end(), 0.0);
+    bool ok = true;
+    for (int q = 0; q < batch && ok; ++q) {
+      const int i = by[q];
+      int pl = -1, pg = -1;
+      double at = 0.0;
+      for (int l = L.n - 1; l >= 0 && pl < 0; --l) {
+        int g = 0;
+        for (int h = 1; h < L.cnt[l]; ++h)
+          if (peak[L.off[l] + h] < peak[L.off[l] + g]) g = h;
+        at = peak[L.off[l] + g] + est[(size_t)i * L.n + l];
+        if (at <= bound) {
+          pl = l;
+          pg = g;
+        }
+      }
+      if (pl < 0 && last) {
+        for (int l = 0; l < L.n; ++l) {
+          int g = 0;
+          for (int h = 1; h < L.cnt[l]; ++h)
+            if (peak[L.off[l] + h] < peak[L.off[l] + g]) g = h;
+          const double t = peak[L.off[l] + g] + est[(size_t)i * L.n + l];
+          if (pl < 0 || t < at) {
+            at = t;
+            pl = l;
+            pg = g;
+          }
+        }
+      }
+      if (pl < 0) {
+        ok = false;
+        break;
+      }
+      place[i] = L.off[pl] + pg;
+      // the node's CTAs wait for the slowest of them, then run the matrix
+      const int c0 = lo_of(pl, pg), c1 = lo_of(pl, pg + 1);
+      for (int c = c0; c < c1; ++c) cta[c] += est[(size_t)i * L.n + pl];
+      for (int l = 0; l < L.n; ++l) {
+        const int g0 = ((c0 + 1) * L.cnt[l] - 1) / grid, g1 = (c1 * L.cnt[l] - 1) / grid;
+        for (int g = g0; g <= g1; ++g) {
+          double v = 0.0;
+          for (int c = lo_of(l, g); c < lo_of(l, g + 1); ++c) v = std::max(v, cta[c]);
+          peak[L.off[l] + g] = v;
+        }
+      }
+    }
+    if (ok) break;
+  }
+  std::vector<std::vector<int>> lists((size_t)nodes);
+  for (int i : by) lists[place[i]].push_back(i);
+  finish(S, lists);
+  return S;
+}
+
+}  // namespace
 
 cudaError_t batched_persistent_run(int batch, const int64_t* m, const int64_t* n, const int64_t* lda,
                                    const int* b, double* const* A, double* const* Q, double* const* R,
                                    int* status, void* workspace, int G, bool halve, cudaStream_t st) {
   const int grid = persistent_grid_impl();
-  if (G < 1 || grid % G) return cudaErrorInvalidValue;
-  const int groups = grid / G;
+  if (G < 0 || (G > 0 && grid % G)) return cudaErrorInvalidValue;
   const BLayout L = blayout(batch, grid);
   char* ws = (char*)workspace;
-  // descriptors and the static schedule (largest estimated time first, each
-  // to the group with the least work so far)
   std::vector<BMat> mats((size_t)batch);
   int nmax = 4, bmax = 4;
-  std::vector<std::pair<double, int>> by;
   for (int i = 0; i < batch; ++i) {
     mats[i].A = A[i];
     mats[i].Q = Q[i];
@@ -906,26 +1128,8 @@ cudaError_t batched_persistent_run(int batch, const int64_t* m, const int64_t* n
     mats[i].b = b[i];
     nmax = std::max(nmax, (int)n[i]);
     bmax = std::max(bmax, b[i]);
-    by.push_back({est_seconds(m[i], (int)n[i], b[i], G), i});
   }
-  std::stable_sort(by.begin(), by.end(), [](const std::pair<double, int>& x, const std::pair<double, int>& y) {
-    return x.first > y.first;
-  });
-  std::vector<double> load((size_t)groups, 0.0);
-  std::vector<std::vector<int>> lists((size_t)groups);
-  for (const auto& e : by) {
-    int g = 0;
-    for (int h = 1; h < groups; ++h)
-      if (load[h] < load[g]) g = h;
-    load[g] += e.first;
-    lists[g].push_back(e.second);
-  }
-  std::vector<int> order, gstart((size_t)grid + 1, batch);
-  for (int g = 0; g < groups; ++g) {
-    gstart[g] = (int)order.size();
-    for (int i : lists[g]) order.push_back(i);
-  }
-  for (int g = groups; g <= grid; ++g) gstart[g] = batch;
+  const BSchedule S = G > 0 ? schedule_uniform(batch, m, n, b, grid, G) : schedule_tree(batch, m, n, b, grid);
   // descriptor table, schedule: kernel-parameter blobs into the workspace
   auto upload = [&](size_t off, const void* src, size_t bytes) -> cudaError_t {
     const unsigned char* p = (const unsigned char*)src;
@@ -942,10 +1146,10 @@ cudaError_t batched_persistent_run(int batch, const int64_t* m, const int64_t* n
   };
   if (batch > 0) {
     TRY_RET(upload(L.mats, mats.data(), sizeof(BMat) * (size_t)batch));
-    TRY_RET(upload(L.order, order.data(), sizeof(int) * (size_t)batch));
+    TRY_RET(upload(L.order, S.order.data(), sizeof(int) * (size_t)batch));
   }
-  TRY_RET(upload(L.gstart, gstart.data(), sizeof(int) * ((size_t)grid + 1)));
-  TRY_RET(cudaMemsetAsync(ws + L.bar, 0, sizeof(unsigned int) * (size_t)grid, st));
+  TRY_RET(upload(L.gstart, S.gstart.data(), sizeof(int) * ((size_t)S.nodes + 1)));
+  TRY_RET(cudaMemsetAsync(ws + L.bar, 0, sizeof(unsigned int) * (size_t)S.nodes, st));
   TRY_RET(cudaMemsetAsync(ws + L.abort, 0, sizeof(int), st));
   TRY_RET(cudaMemsetAsync(status, 0, sizeof(int) * (size_t)batch, st));
   BArgs a{};
@@ -958,7 +1162,7 @@ cudaError_t batched_persistent_run(int batch, const int64_t* m, const int64_t* n
   a.s1 = (double*)(ws + L.s1);
   a.bar = (unsigned int*)(ws + L.bar);
   a.abort = (int*)(ws + L.abort);
-  a.G = G;
+  a.lev = S.lev;
   a.nmax = nmax;
   a.bmax = bmax;
   a.halve = halve ? 1 : 0;
