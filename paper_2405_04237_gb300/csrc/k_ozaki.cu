@@ -6,10 +6,17 @@
 //
 // Splitting.  For C = X^T Y, rows are cut into sub-chunks of kSub = 4096.
 // Within a sub-chunk every column c of X (and of Y) gets a power-of-two
-// scale 2^e_c with |x| < 2^e_c, and each entry becomes the 56-bit fixed-point
-// integer |x| * 2^(56 - e_c) (truncated below 2^-56 of the scale) split into
-// 14 unsigned nibbles n_0..n_13 (n_i has weight 16^i); digit i of x is
-// sign(x) * n_i, an integer in [-15, 15] that e4m3 represents exactly.  For
+// scale 2^e_c with |x| < 2^e_c, and each entry becomes the fixed-point
+// integer X = x * 2^(54 - e_c) (rounded, |X| <= 2^54), written in base 32
+// with eleven balanced digits: X = sum_i d_i 32^i, -16 <= d_i <= 15 (16 for
+// the top digit).  An integer of magnitude up to 16 is exact in e4m3: the
+// code is the sign and |d|, read as |d| 2^-9 (e4m3's subnormals and the two
+// binades above them are evenly spaced), so no table is needed and every
+// product carries a factor 2^-18.  Balanced digits need 11 planes and 66
+// plane pairs where sign-magnitude nibbles needed 14 and 105, and the pairs
+// left out have no common sign: the error against exact sums is that of the
+// nibbles for X^T Y and 30 to 80 times smaller for the diagonal of X^T X,
+// whose neglected nibble products were all positive.  For
 // C -= X Y the contraction runs over the columns of X: each row of X gets its
 // own scale over (at most kSub of) its entries and takes a column's place;
 // Y (K x N) is split by columns.
@@ -19,35 +26,34 @@
 // stored tile-major: for each tile, each stage, each plane i, the T x 32
 // digits in the tensor cores' canonical K-major layout without swizzling
 // (8-column groups of 256 bytes, each two 8 x 16-byte core matrices holding
-// indices 0..15, then 16..31).  The 14 planes of one stage of one tile are
-// thus one contiguous run (56 KiB for X, 14 KiB for Y), and a stage arrives
+// indices 0..15, then 16..31).  The 11 planes of one stage of one tile are
+// thus one contiguous run (44 KiB for X, 11 KiB for Y), and a stage arrives
 // in shared memory with two bulk asynchronous copies (for a Gram matrix
 // X^T X, whose Y tiles are 32-column slices of the X planes, one copy for X
 // and one per plane for Y).
 //
-// Products.  x_a y_b = 2^(e_a + e_b - 112) sum_{i,j} d^x_i d^y_j 16^(i+j).
-// The 105 plane pairs with i + j >= 13 (the 14 most significant weight
+// Products.  x_a y_b = 2^(e_a + e_b - 108) sum_{i,j} d^x_i d^y_j 32^(i+j).
+// The 66 plane pairs with i + j >= 10 (the 11 most significant weight
 // levels) are multiplied with tcgen05.mma kind::f8f6f4 (e4m3 x e4m3 -> f32)
-// into one TMEM accumulator per level: TMEM region r (32 columns, r = 0..15)
-// holds level r + 11.  The Y planes of one stage lie in shared memory one
+// into one TMEM accumulator per level: TMEM region r (32 columns, r = 0..10)
+// holds level r + 10.  The Y planes of one stage lie in shared memory one
 // after the other, so planes j0 .. j0+n-1 form one operand of N = 32 n rows,
 // and one instruction A_i x [Y_j0; ...; Y_j0+n-1] (128 x 32n x 32) adds pair
-// (i, j0 + v) into region i + j0 + v - 11 for v < n.  22 such instructions
-// (N = 32 .. 256) cover the 105 pairs, plus 6 pairs of levels 11 and 12,
-// whose regions are never read.  Per level the sum over at most 4096
-// contraction indices is below 14 * 225 * 4096 < 2^24 in magnitude, so the
-// FP32 accumulation is exact (an integer).  The dropped levels weigh at most
-// about 2^-52.5 of the scales' product per index, so below 2^-50.5 of the
-// product of the two largest magnitudes.
+// (i, j0 + v) into region i + j0 + v - 10 for v < n.  14 such instructions
+// (N = 32 .. 256) cover the 66 pairs.  Per level the sum over at most 4096
+// contraction indices is below 11 * 256 * 4096 < 2^24 in magnitude, so the
+// FP32 accumulation is exact (an integer times 2^-18).  The dropped levels
+// weigh at most about 2^-51.6 of the scales' product per index, with signs
+// that cancel (rms 2^-55).
 //
 // Schedule.  A block of 4 warps computes a 128 x 32 tile of C over its
 // contraction range (a sub-chunk of a projection, all of K for an update).
-// Three shared-memory stages of 70 KiB rotate: one thread issues the bulk
+// Four shared-memory stages of 55 KiB rotate: one thread issues the bulk
 // copies of a stage (completion counted in bytes on the stage's "full"
-// mbarrier), one thread issues its 22 MMAs and commits them to the stage's
-// "empty" mbarrier, which frees the stage for the copy three stages later.
-// At the end every thread reads the 14 level sums of its row from TMEM,
-// combines levels 13..19 and 20..26 exactly in 64-bit integers (below 2^49),
+// mbarrier), one thread issues its 14 MMAs and commits them to the stage's
+// "empty" mbarrier, which frees the stage for the copy four stages later.
+// At the end every thread reads the 11 level sums of its row from TMEM,
+// combines levels 10..15 and 16..20 exactly in 64-bit integers (below 2^50),
 // builds the two scaled doubles with integer operations and adds them (one
 // rounding), so the FP64 pipe does one operation per element (two for an
 // update, which subtracts the tile from C).  Every wait is bounded in time
@@ -67,9 +73,10 @@ namespace cqr {
 namespace {
 
 constexpr int kSub = 4096;          // rows per sub-chunk (exact FP32 level sums)
-constexpr int kPlanes = 14;         // nibbles: 56 bits
-constexpr int kLevelLo = 13;        // lowest weight level i + j kept
+constexpr int kPlanes = 11;         // balanced base-32 digits of a 54-bit magnitude and its sign
+constexpr int kLevelLo = 10;        // lowest weight level i + j kept
 constexpr int kLevels = 2 * kPlanes - 1 - kLevelLo;
+constexpr int kLowLevels = 6;       // levels of the low 64-bit group; the others form the high one
 constexpr int kStage = 32;          // contraction indices per stage (one MMA K step for 8-bit types)
 constexpr int kStagesPerSub = kSub / kStage;
 constexpr int kExpZero = -100000;   // scale of an all-zero column
@@ -78,18 +85,19 @@ constexpr int kExpBad = 100000;     // a column holding Inf or NaN
 constexpr int kTcM = 128;           // rows of the tile (X side, TMEM lanes)
 constexpr int kTcN = 32;            // columns of the tile (Y side)
 constexpr int kTcThreads = 128;
-constexpr int kTcRing = 3;
-constexpr int kTcABytes = kPlanes * kTcM * kStage;    // 57344
-constexpr int kTcBBytes = kPlanes * kTcN * kStage;    // 14336
-constexpr int kTcStageBytes = kTcABytes + kTcBBytes;  // 71680
+constexpr int kTcRing = 4;
+constexpr int kTcABytes = kPlanes * kTcM * kStage;    // 45056
+constexpr int kTcBBytes = kPlanes * kTcN * kStage;    // 11264
+constexpr int kTcStageBytes = kTcABytes + kTcBBytes;  // 56320
 constexpr int kTcSmem = kTcRing * kTcStageBytes + 1024;  // + alignment slack
-constexpr uint32_t kTcCols = 512;   // TMEM columns: 16 regions of kTcN, levels 11..26
+constexpr uint32_t kTcCols = 512;   // TMEM columns: the levels' regions (352), rounded up to a power of 2
 constexpr int kMaxDynSmem = 227 * 1024 - 1024;  // opt-in dynamic shared memory per block, less static use
 static_assert(kTcSmem <= kMaxDynSmem, "projection ring fits in shared memory");
 static_assert(kTcCols >= 32 && kTcCols <= 512 && (kTcCols & (kTcCols - 1)) == 0, "TMEM allocation: power of 2, 32..512");
-constexpr int kRegionLo = 11;       // level of TMEM region 0
-static_assert((2 * kPlanes - 1 - kRegionLo) * kTcN == (int)kTcCols, "level regions fill the TMEM allocation");
-static_assert(kLevelLo == 13 && kLevels == 14, "the MMA schedule and the two groups of seven levels");
+constexpr int kRegionLo = kLevelLo;  // level of TMEM region 0
+static_assert(kLevels * kTcN <= (int)kTcCols, "level regions fit in the TMEM allocation");
+static_assert(kLevelLo == 10 && kLevels == 11, "the MMA schedule and the groups of six and five levels");
+static_assert((long long)kLevels * 256 * kSub < (1 << 24), "exact FP32 level sums");
 // Instruction descriptor of tcgen05.mma kind::f8f6f4 without N: D f32 (bits
 // 4-5 = 1), A and B e4m3 (bits 7-9, 10-12 = 0), both K-major (bits 15, 16 =
 // 0), M >> 4 at bits 24-28; N >> 3 goes to bits 17-22.
@@ -98,52 +106,69 @@ constexpr unsigned long long kWaitNs = 2000000000ull;  // bound of every mbarrie
 
 inline int round_up(int x, int t) { return (x + t - 1) / t * t; }
 
-// 56-bit magnitude |x| * 2^(56 - e) (truncated) of one FP64 value (raw bits b)
-// against scale e; zero for zeros, subnormals and a bad column.
-__device__ __forceinline__ unsigned long long magnitude(unsigned long long b, int e) {
+// x * 2^(54 - e) rounded to an integer, plus 16 in every base-32 digit, of one
+// FP64 value (raw bits b) against scale e: the fields of 5 bits (the top one
+// 6) are the balanced digits plus 16.  Zeros, subnormals and the entries of a
+// bad column count as 0.
+constexpr unsigned long long kDigitBias = 16ull * (((1ull << 50) - 1) / 31) + (16ull << 50);
+
+__device__ __forceinline__ unsigned long long biased_digits(unsigned long long b, int e) {
   const int E = (int)((b >> 52) & 0x7FF);
-  if (E == 0 || E == 0x7FF || e == kExpBad) return 0ull;
+  if (E == 0 || E == 0x7FF || e == kExpBad) return kDigitBias;
   const unsigned long long M = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-  const int sh = E - 1019 - e;  // |x| 2^(56-e) = M 2^(E - 1075 + 56 - e)
-  return sh >= 0 ? (M << sh) : (sh > -64 ? (M >> (-sh)) : 0ull);
+  const int sh = E - 1021 - e;  // |x| 2^(54-e) = M 2^(E - 1075 + 54 - e), sh <= 1
+  const int s = min(-sh, 63);
+  const unsigned long long mag = sh >= 0 ? M << sh : (M + (1ull << (s - 1))) >> s;
+  return (long long)b < 0 ? kDigitBias - mag : kDigitBias + mag;
 }
 
-// e4m3 codes of four nibbles (one per byte of n, each 0..15): 0, 1, ..., 7
-// come from two lookup words, 8..15 (0x50 + n - 8) from two more, chosen per
-// byte by bit 3 of the nibble.
-__device__ __forceinline__ uint32_t e4m3_of_nibbles(uint32_t n) {
-  const uint32_t v = n & 0x07070707u;
-  const uint32_t u = v | (v >> 4);
-  const uint32_t sel = __byte_perm(u, 0u, 0x4420);  // selector nibbles v0, v1, v2, v3
-  const uint32_t lo = __byte_perm(0x44403800u, 0x4E4C4A48u, sel);
-  const uint32_t hi = __byte_perm(0x53525150u, 0x57565554u, sel);
-  const uint32_t mask = ((n >> 3) & 0x01010101u) * 0xFFu;
-  return (lo & ~mask) | (hi & mask);
+// e4m3 codes, sign and magnitude, of four digits given as bytes u = d + 16
+// (0 .. 31; kTop: 0 .. 32).
+template <bool kTop>
+__device__ __forceinline__ uint32_t e4m3_of_digits(uint32_t u) {
+  const uint32_t six = kTop ? (u >> 1) & 0x10101010u : 0u;  // d = 16
+  const uint32_t t = ~(u | six) & 0x10101010u;              // d < 0
+  const uint32_t n = t >> 4;
+  return ((u & 0x0F0F0F0Fu) ^ (t - n)) + n + (t << 3) + six;
+}
+
+// 20 bits as four bytes of 5 bits
+__device__ __forceinline__ uint32_t bytes_of_fields(uint32_t x) {
+  const uint32_t y = (x & 0x3FFu) | ((x << 6) & 0x3FF0000u);
+  return (y & 0x1F001Fu) | ((y << 3) & 0x1F001F00u);
+}
+
+// out[i] = byte i of w[0..3] (i < N)
+template <int N>
+__device__ __forceinline__ void transpose4(const uint32_t (&w)[4], uint32_t* out) {
+  const uint32_t a = __byte_perm(w[0], w[1], 0x5140), c = __byte_perm(w[2], w[3], 0x5140);
+  out[0] = __byte_perm(a, c, 0x5410);
+  out[1] = __byte_perm(a, c, 0x7632);
+  const uint32_t b = __byte_perm(w[0], w[1], 0x7362), d = __byte_perm(w[2], w[3], 0x7362);
+  out[2] = __byte_perm(b, d, 0x5410);
+  if (N == 4) out[3] = __byte_perm(b, d, 0x7632);
 }
 
 // Digits of four FP64 values (raw bits b[0..3]) against scale e: byte k of
-// word i is the e4m3 code of digit i of value k, sign(x_k) * nibble i.  The
-// four 56-bit magnitudes are transposed bytewise with byte permutes, so that
-// every step below works on four values at once.
+// word i is the e4m3 code of digit i of value k.  Every step after the fixed-
+// point conversion works on four digits at once.
 __device__ __forceinline__ void digits4(const unsigned long long (&b)[4], int e, uint32_t (&w)[kPlanes]) {
-  uint32_t lo[4], hi[4], sgn = 0;
+  uint32_t f0[4], f1[4], f2[4], u[kPlanes];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const unsigned long long m = magnitude(b[k], e);
-    lo[k] = (uint32_t)m;
-    hi[k] = (uint32_t)(m >> 32);
-    sgn |= (uint32_t)(b[k] >> 63) << (8 * k + 7);
+    const unsigned long long v = biased_digits(b[k], e);
+    f0[k] = bytes_of_fields((uint32_t)v & 0xFFFFFu);
+    f1[k] = bytes_of_fields((uint32_t)(v >> 20) & 0xFFFFFu);
+    const uint32_t x = (uint32_t)(v >> 40);  // fields 8, 9 (5 bits) and 10 (6 bits)
+    const uint32_t y = (x & 0x3FFu) | ((x << 6) & 0x3F0000u);
+    f2[k] = (y & 0x3F001Fu) | ((y << 3) & 0x1F00u);
   }
+  transpose4<4>(f0, u);
+  transpose4<4>(f1, u + 4);
+  transpose4<3>(f2, u + 8);
 #pragma unroll
-  for (int j = 0; j < kPlanes / 2; ++j) {  // byte j of the four magnitudes
-    const uint32_t* src = j < 4 ? lo : hi;
-    const uint32_t sel = (uint32_t)(j & 3) | ((uint32_t)((j & 3) + 4) << 4);
-    const uint32_t t01 = __byte_perm(src[0], src[1], sel);
-    const uint32_t t23 = __byte_perm(src[2], src[3], sel);
-    const uint32_t bj = __byte_perm(t01, t23, 0x5410);
-    w[2 * j] = e4m3_of_nibbles(bj & 0x0F0F0F0Fu) | sgn;
-    w[2 * j + 1] = e4m3_of_nibbles((bj >> 4) & 0x0F0F0F0Fu) | sgn;
-  }
+  for (int i = 0; i < kPlanes - 1; ++i) w[i] = e4m3_of_digits<false>(u[i]);
+  w[kPlanes - 1] = e4m3_of_digits<true>(u[kPlanes - 1]);
 }
 
 // Byte offset, within one (stage, plane) block, of the 16 indices
@@ -159,7 +184,8 @@ __device__ __forceinline__ i64 plane_off(i64 col, int half) {
 // that for each stage and plane its digits form one contiguous 256-byte run
 // (8 columns x 32 indices).  Lane l of warp w handles column 8g + (l & 7),
 // half (l >> 3) & 1 (indices 0..15 or 16..31 of a stage) of stages
-// 16 it + 2 w + (l >> 4), it = 0..7: every warp store writes two whole
+// 16 it + 2 w + (l >> 4), it = 0..7 (only those below nst, rounded up to 16,
+// for the short Y of an update): every warp store writes two whole
 // 256-byte runs.  Two passes over the sub-chunk: the column maxima (scales),
 // then the digits; the second pass re-reads from L2 (at most two blocks, 2 x
 // 256 KiB, per SM).  Tiles of T columns (T a multiple of 8); plane block
@@ -187,19 +213,20 @@ __device__ __forceinline__ void load16(const double* xc, i64 row, i64 m, bool co
 }
 
 __global__ void __launch_bounds__(256, 2) ozaki_split_kernel(const double* X, i64 ldx, i64 m, i64 r0, int c, int T,
-                                                             uint8_t* planes, int* exps, const int* status) {
+                                                             int nst, uint8_t* planes, int* exps, const int* status) {
   if (status && *status) return;
   const int g = blockIdx.x, s = blockIdx.y, t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int cl = lane & 7, half = (lane >> 3) & 1, so = lane >> 4;
   const int col = 8 * g + cl;
   const bool colok = col < c;
   const i64 base = r0 + (i64)s * kSub;
+  const int iters = (nst + 15) / 16;
   const double* xc = X + (i64)(colok ? col : 0) * ldx;
   // pass 1: the column's largest exponent (zeros and subnormals do not set the scale) and Inf/NaN
   int emax = -2000;
   bool bad = false;
 #pragma unroll 1
-  for (int it = 0; it < 8; ++it) {
+  for (int it = 0; it < iters; ++it) {
     const int st = 16 * it + 2 * warp + so;
     unsigned long long bits[16];
     load16(xc, base + st * kStage + 16 * half, m, colok, bits);
@@ -240,7 +267,7 @@ __global__ void __launch_bounds__(256, 2) ozaki_split_kernel(const double* X, i6
   const int ntile = (c + T - 1) / T;
   uint8_t* dst0 = planes + ((i64)s * ntile + col / T) * kStagesPerSub * kPlanes * T * kStage + plane_off(col % T, half);
 #pragma unroll 1
-  for (int it = 0; it < 8; ++it) {
+  for (int it = 0; it < iters; ++it) {
     const int st = 16 * it + 2 * warp + so;
     unsigned long long bits[16];
     load16(xc, base + st * kStage + 16 * half, m, colok, bits);
@@ -375,49 +402,47 @@ __device__ __forceinline__ void tc_mma(uint32_t d, uint64_t ad, uint64_t bd, int
 }
 
 // The MMA schedule of one stage: (plane i of X, first plane j0 of Y, count n).
-// The first two write regions 2..9 and 10..15 (levels 13..26, every region
-// the epilogue reads) without overlap, so in the first stage of a tile they
-// run with acc = 0 and initialise the accumulators; regions 0 and 1 (levels
-// 11 and 12) only ever collect what is never read.
+// The first two write every region (levels 10..20) without overlap, so in the
+// first stage of a tile they run with acc = 0 and initialise the accumulators.
+// An instruction reads 4 KiB of X and n KiB of Y from shared memory (128 B per
+// clock) for 16 n clocks of arithmetic, so the splits are even: 5 + 4 rather
+// than 8 + 1.
 struct TcMma {
   int i, j0, n;
 };
-#define CQR_TC_SCHEDULE                                                                         \
-  {13, 0, 8}, {13, 8, 6},                                              /* i = 13: regions 2..9, 10..15 */ \
-      {11, 0, 8}, {12, 0, 8},                                          /* i = 11, 12 with all of j = 0..7 */ \
-      {3, 8, 6}, {4, 8, 6}, {5, 8, 6}, {6, 8, 6}, {7, 8, 6}, {8, 8, 6}, /* j = 8..13 for 3 <= i <= 12 */ \
-      {9, 8, 6}, {10, 8, 6}, {11, 8, 6}, {12, 8, 6},                                                    \
-      {6, 7, 1}, {7, 6, 2}, {8, 5, 3}, {9, 4, 4}, {10, 3, 5}, /* j <= 7 with i + j >= 13, i <= 10 */     \
-      {2, 11, 3}, {1, 12, 2}, {0, 13, 1}                      /* j >= 11 with i + j >= 13, i <= 2 */
-__device__ constexpr TcMma kTcSchedule[22] = {CQR_TC_SCHEDULE};
+constexpr int kTcMmas = 14;
+#define CQR_TC_SCHEDULE                                                  \
+  {10, 0, 6}, {10, 6, 5},                       /* i = 10: every level */ \
+      {9, 1, 5}, {9, 6, 5}, {8, 2, 5}, {8, 7, 4}, /* j >= 10 - i */       \
+      {7, 3, 8}, {6, 4, 7}, {5, 5, 6}, {4, 6, 5}, {3, 7, 4}, {2, 8, 3}, {1, 9, 2}, {0, 10, 1}
+__device__ constexpr TcMma kTcSchedule[kTcMmas] = {CQR_TC_SCHEDULE};
 
 // Compile-time check of the same entries: every digit pair (i, j) of a kept
-// level (i + j >= 13) exactly once, no pair twice, every instruction within
-// the planes, N = 32 n <= 256, every region in TMEM, and the first two
-// instructions writing each read region (levels 13..26) exactly once and
-// nothing else (they run with the accumulate flag off).
-constexpr TcMma kTcScheduleCheck[22] = {CQR_TC_SCHEDULE};
+// level exactly once and no other, every instruction within the planes,
+// N = 32 n <= 256, every region in TMEM, and the first two instructions
+// writing each region exactly once (they run with the accumulate flag off).
+constexpr TcMma kTcScheduleCheck[kTcMmas] = {CQR_TC_SCHEDULE};
 constexpr bool tc_schedule_ok() {
   int count[kPlanes][kPlanes] = {};
-  int first[kTcCols / kTcN] = {};
-  for (int u = 0; u < 22; ++u) {
+  int first[kLevels] = {};
+  for (int u = 0; u < kTcMmas; ++u) {
     const TcMma e = kTcScheduleCheck[u];
     if (e.i < 0 || e.i >= kPlanes || e.j0 < 0 || e.n < 1 || e.j0 + e.n > kPlanes || kTcN * e.n > 256) return false;
     for (int v = 0; v < e.n; ++v) {
       const int j = e.j0 + v, region = e.i + j - kRegionLo;
-      if (region < 0 || region >= (int)(kTcCols / kTcN)) return false;
+      if (region < 0 || region >= kLevels) return false;
       ++count[e.i][j];
       if (u < 2) ++first[region];
     }
   }
   for (int i = 0; i < kPlanes; ++i)
     for (int j = 0; j < kPlanes; ++j)
-      if (count[i][j] > 1 || (i + j >= kLevelLo && count[i][j] != 1)) return false;
-  for (int r = 0; r < (int)(kTcCols / kTcN); ++r)
-    if (first[r] != (r >= kLevelLo - kRegionLo ? 1 : 0)) return false;
+      if (count[i][j] != (i + j >= kLevelLo ? 1 : 0)) return false;
+  for (int r = 0; r < kLevels; ++r)
+    if (first[r] != 1) return false;
   return true;
 }
-static_assert(tc_schedule_ok(), "MMA schedule: kept pairs once, regions in range, first two initialise the read regions");
+static_assert(tc_schedule_ok(), "MMA schedule: kept pairs once, regions in range, first two initialise the regions");
 #undef CQR_TC_SCHEDULE
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -443,6 +468,52 @@ __device__ __forceinline__ double scaled_int(long long g, int e) {
   if (E <= 0 || E >= 2047) return ldexp((double)g, e);
   const unsigned long long mant = (a << (52 - msb)) & 0xFFFFFFFFFFFFFull;
   return __longlong_as_double((long long)(sgn | ((unsigned long long)E << 52) | mant));
+}
+
+// Contraction length up to which every level sum is below 2^22 units (11
+// pairs x 256 x K < 2^22): then the FP32 value f (a multiple of 2^-18) is read
+// exactly as bits(f + 48) - bits(48), one full-rate FP32 add and integer
+// arithmetic, instead of a quarter-rate conversion.
+constexpr int kMagicMaxK = 1312;
+static_assert(kLevels * 256 * kMagicMaxK < (1 << 22), "level sums below 2^22");
+constexpr float kMagicF = 48.0f;        // 1.5 * 2^5: steps of 2^-18
+constexpr int kMagicBits = 0x42400000;  // its encoding
+
+// The level sums of columns c0 .. c0+7 of this thread's TMEM lane.
+__device__ __forceinline__ void load_levels(uint32_t lane_base, int c0, uint32_t (&v)[kLevels][8]) {
+#pragma unroll
+  for (int l = 0; l < kLevels; ++l) tc_ld8(lane_base + (uint32_t)((kLevelLo - kRegionLo + l) * kTcN + c0), v[l]);
+  tc_wait_ld();
+}
+
+// g0 = sum_{l < 6} s_l 32^l and g1 = sum_{l >= 6} s_l 32^(l - 6) of column j's
+// level sums s_l (integers).  kMagic (|s_l| < 2^22): neighbouring levels first
+// combine in unsigned 32-bit arithmetic (the offsets cancel modulo 2^32 and
+// |s_l + 32 s_l+1| < 2^28, so the two's-complement reading is the value).
+template <bool kMagic>
+__device__ __forceinline__ void group_sums(const uint32_t (&v)[kLevels][8], int j, long long& g0, long long& g1) {
+  if (kMagic) {
+    uint32_t b[kLevels];
+#pragma unroll
+    for (int l = 0; l < kLevels; ++l) b[l] = __float_as_uint(__fadd_rn(__uint_as_float(v[l][j]), kMagicF));
+    const uint32_t off = 33u * (uint32_t)kMagicBits;  // modulo 2^32
+    auto two = [&](int l) { return (long long)(int)(b[l] + 32u * b[l + 1] - off); };
+    g0 = two(0) + (two(2) << 10) + (two(4) << 20);
+    g1 = two(6) + (two(8) << 10) + ((long long)(int)(b[10] - (uint32_t)kMagicBits) << 20);
+  } else {
+    auto lev = [&](int l) { return (long long)__float2int_rz(__uint_as_float(v[l][j]) * 262144.0f); };
+    g0 = g1 = 0;
+#pragma unroll
+    for (int l = kLowLevels - 1; l >= 0; --l) g0 = g0 * 32 + lev(l);
+#pragma unroll
+    for (int l = kLevels - 1; l >= kLowLevels; --l) g1 = g1 * 32 + lev(l);
+  }
+}
+
+// sum_L S_L 32^L = 32^10 (g0 + 2^30 g1), times 2^(ex + ey - 108); one rounding
+__device__ __forceinline__ double group_value(long long g0, long long g1, int exy) {
+  const int e2 = exy - 108 + 5 * kLevelLo;
+  return scaled_int(g1, e2 + 5 * kLowLevels) + scaled_int(g0, e2);
 }
 
 struct OzArgs {
@@ -537,7 +608,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) ozaki_tc_kernel(OzArgs a) {
     for (int st = issued - kTcRing < 0 ? 0 : issued - kTcRing; st < issued; ++st)
       mbar_wait(smem_u32(&full_bar[st % kTcRing]), (uint32_t)((st / kTcRing) & 1), a.wait_ns);
   } else if (warp == 1 && lane == 0) {
-    // MMA issuer: the 22 instructions of each stage (the 105 pairs, level L = i + j into region L - 11)
+    // MMA issuer: the 14 instructions of each stage (the 66 pairs, level L = i + j into region L - 10)
     for (int st = 0; st < nst; ++st) {
       const int slot = st % kTcRing;
       if (!mbar_wait(smem_u32(&full_bar[slot]), (uint32_t)((st / kTcRing) & 1), a.wait_ns)) {
@@ -549,7 +620,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) ozaki_tc_kernel(OzArgs a) {
       const uint32_t sa = smem_u32(ring + slot * kTcStageBytes), sb = sa + kTcABytes;
       const uint64_t ad0 = tc_desc(sa), bd0 = tc_desc(sb);
 #pragma unroll
-      for (int u = 0; u < 22; ++u) {
+      for (int u = 0; u < kTcMmas; ++u) {
         const TcMma e = kTcSchedule[u];
         const uint64_t ad = ad0 + (uint64_t)((e.i * kTcM * kStage) >> 4);
         const uint64_t bd = bd0 + (uint64_t)((e.j0 * kTcN * kStage) >> 4);
@@ -572,21 +643,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) ozaki_tc_kernel(OzArgs a) {
 #pragma unroll
     for (int c0 = 0; c0 < kTcN; c0 += 8) {
       long long g[2][8];
+      uint32_t v[kLevels][8];
+      load_levels(lane_base, c0, v);
 #pragma unroll
-      for (int grp = 1; grp >= 0; --grp) {
-        uint32_t v[7][8];
-#pragma unroll
-        for (int l = 6; l >= 0; --l)
-          tc_ld8(lane_base + (uint32_t)((kLevelLo - kRegionLo + 7 * grp + l) * kTcN + c0), v[l]);
-        tc_wait_ld();
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          long long acc = 0;
-#pragma unroll
-          for (int l = 6; l >= 0; --l) acc = acc * 16 + __float2int_rz(__uint_as_float(v[l][j]));
-          g[grp][j] = acc;
-        }
-      }
+      for (int j = 0; j < 8; ++j) group_sums<false>(v, j, g[0][j], g[1][j]);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const int qc = q0 + c0 + j;
@@ -598,9 +658,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) ozaki_tc_kernel(OzArgs a) {
         } else if (exr == kExpZero || eyc == kExpZero) {
           v = 0.0;
         } else {
-          // sum_L S_L 16^L = 16^13 (g0 + 2^28 g1); value = that * 2^(ex + ey - 112)
-          const int e2 = exr + eyc - 112 + 4 * kLevelLo;
-          v = scaled_int(g[1][j], e2 + 28) + scaled_int(g[0][j], e2);  // one rounding
+          v = group_value(g[0][j], g[1][j], exr + eyc);
         }
         a.part[(i64)(a.s_off + s) * a.p * a.q + pr + (i64)qc * a.p] = v;
       }
@@ -612,20 +670,27 @@ __global__ void __launch_bounds__(kTcThreads, 1) ozaki_tc_kernel(OzArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// Updates C -= X Y as a persistent, warp-specialised kernel: block c takes
-// tiles c, c + G, c + 2G, ... (G = grid size; tile T is row tile T / tiles_q,
-// column tile T % tiles_q, so the blocks running together share row tiles).
-// Warp 0 streams the stages of all its tiles through a three-stage ring, warp
+// Updates C -= X Y as a persistent, warp-specialised kernel.  Warp 0 streams
+// the stages of the block's tiles into two rings of four slots, one for X (44
+// KiB each) and one for Y (11 KiB each), warp
 // 1 issues the MMAs of a tile into the one set of TMEM level regions, and
 // warps 2-5 (TMEM lane quarters 2, 3, 0, 1) run the epilogue in two phases:
 // first the level sums become the exact 64-bit group sums, kept in registers
 // (two per column of the thread's row), and the regions are handed back to
 // warp 1 at once; then, while the next tile's MMAs run, the group sums are
-// scaled, added and subtracted from C.  An update has only K / 32 stages per tile (4 for K = 128), so without
-// this overlap the fill and the epilogue would cost as much as the MMAs.
-constexpr int kUpRing = 3;
+// scaled, added and subtracted from C.
+//
+// Tile T is row tile T / tiles_q, column tile T % tiles_q.  The kernel is
+// bound by how fast stages reach shared memory, and X is four fifths of a
+// stage.  Contractions of up to four stages (K <= 128: every product with one
+// panel) therefore keep the row tile's X stages in their four slots while the
+// block, which takes a contiguous run of tiles, goes through its column
+// tiles.  Longer contractions stream X with Y, and block c takes tiles c,
+// c + G, c + 2G, ... (G = grid size), so that the blocks running together
+// share row tiles in L2.
+constexpr int kUpRing = 4;
 constexpr int kUpThreads = 192;
-constexpr int kUpSmem = 1024 + kUpRing * kTcStageBytes;
+constexpr int kUpSmem = 1024 + kUpRing * kTcStageBytes;  // X slots, then Y slots
 static_assert(kUpSmem <= kMaxDynSmem, "update ring fits in shared memory");
 static_assert(kUpThreads == 6 * 32, "producer, MMA issuer and one epilogue warp per TMEM lane quarter");
 
@@ -633,35 +698,11 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// Contraction length up to which every level sum of an update tile is below
-// 2^22 in magnitude (14 pairs x 225 x K < 2^22): then the FP32 integer f is
-// read exactly as bits(f + 1.5 * 2^23) - bits(1.5 * 2^23), one full-rate
-// FP32 add and integer arithmetic, instead of a quarter-rate conversion.
-constexpr int kMagicMaxK = 1312;
-static_assert(14 * 225 * kMagicMaxK < (1 << 22), "level sums below 2^22");
-constexpr float kMagicF = 12582912.0f;  // 1.5 * 2^23
-constexpr int kMagicBits = 0x4B400000;  // its encoding
-
-// g = sum_{l<7} s_l 16^l for the seven FP32 level sums v[0..6][j] (s_l
-// exact integers, |s_l| < 2^22): three partial sums in unsigned 32-bit
-// arithmetic (the offsets cancel modulo 2^32 and |s_0 + 16 s_1 + 256 s_2| <
-// 2^31, so the two's-complement reading is the value), then
-// g = lo + 2^12 mid + 2^24 s_6.
-__device__ __forceinline__ long long group_sum_magic(const uint32_t (&v)[7][8], int j) {
-  uint32_t b[7];
-#pragma unroll
-  for (int l = 0; l < 7; ++l) b[l] = __float_as_uint(__fadd_rn(__uint_as_float(v[l][j]), kMagicF));
-  const uint32_t off = 273u * (uint32_t)kMagicBits;  // modulo 2^32
-  const int lo = (int)(b[0] + 16u * b[1] + 256u * b[2] - off);
-  const int mid = (int)(b[3] + 16u * b[4] + 256u * b[5] - off);
-  const int top = (int)(b[6] - (uint32_t)kMagicBits);
-  return (long long)lo + ((long long)mid << 12) + ((long long)top << 24);
-}
-
 template <bool kMagic>
 __global__ void __launch_bounds__(kUpThreads, 1) ozaki_tc_update_kernel(OzArgs a, int ntiles) {
   extern __shared__ uint8_t up_raw[];
-  __shared__ __align__(8) uint64_t full_bar[kUpRing], empty_bar[kUpRing], acc_full, acc_empty, mma_done;
+  __shared__ __align__(8) uint64_t full_a[kUpRing], empty_a[kUpRing], full_b[kUpRing], empty_b[kUpRing];
+  __shared__ __align__(8) uint64_t acc_full, acc_empty, mma_done;
   __shared__ uint32_t tmem_slot;
   __shared__ int give_up;
   if (a.status && *a.status) return;  // uniform across the block, before any allocation
@@ -669,8 +710,10 @@ __global__ void __launch_bounds__(kUpThreads, 1) ozaki_tc_update_kernel(OzArgs a
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(up_raw) + 1023) & ~(uintptr_t)1023);
   if (t == 0) {
     for (int i = 0; i < kUpRing; ++i) {
-      mbar_init(smem_u32(&full_bar[i]), 1);
-      mbar_init(smem_u32(&empty_bar[i]), 1);
+      mbar_init(smem_u32(&full_a[i]), 1);
+      mbar_init(smem_u32(&empty_a[i]), 1);
+      mbar_init(smem_u32(&full_b[i]), 1);
+      mbar_init(smem_u32(&empty_b[i]), 1);
     }
     mbar_init(smem_u32(&acc_full), 1);
     mbar_init(smem_u32(&acc_empty), 4);  // one arrival per epilogue warp
@@ -688,69 +731,90 @@ __global__ void __launch_bounds__(kUpThreads, 1) ozaki_tc_update_kernel(OzArgs a
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
   const int nst = a.nst;
+  const bool keep_x = nst <= kUpRing;
+  // this block's tiles: t_first, t_first + t_step, .. below t_last
+  const int t_step = keep_x ? 1 : (int)gridDim.x;
+  const int t_first = keep_x ? (int)((i64)blockIdx.x * ntiles / gridDim.x) : (int)blockIdx.x;
+  const int t_last = keep_x ? (int)((i64)(blockIdx.x + 1) * ntiles / gridDim.x) : ntiles;
+  const uint32_t xs = smem_u32(ring), ys = xs + kUpRing * kTcABytes;
 
   if (warp == 0) {
     if (lane == 0) {  // producer
-      int g = 0;
+      int ga = 0, gb = 0;  // X and Y stages issued; X stage h goes to slot h % nst (kept) or h % kUpRing
+      const int xr = keep_x ? nst : kUpRing;
       bool stop = false;
-      for (int T = blockIdx.x; T < ntiles && !stop; T += gridDim.x) {
+      for (int T = t_first; T < t_last && !stop; T += t_step) {
         // tile-major planes: nst stages per X tile, kStagesPerSub per Y tile
         const uint8_t* gx = a.px + (i64)(T / a.tiles_q) * nst * kTcABytes;
         const uint8_t* gy = a.py + (i64)(T % a.tiles_q) * kStagesPerSub * kTcBBytes;
+        const bool load_x = !keep_x || T == t_first || T % a.tiles_q == 0;
         for (int st = 0; st < nst; ++st) {
-          const int slot = g % kUpRing;
-          if (g >= kUpRing && !mbar_wait(smem_u32(&empty_bar[slot]), (uint32_t)((g / kUpRing - 1) & 1), a.wait_ns)) {
+          const int sa = ga % xr, sb = gb % kUpRing;
+          if ((load_x && ga >= xr && !mbar_wait(smem_u32(&empty_a[sa]), (uint32_t)((ga / xr - 1) & 1), a.wait_ns)) ||
+              (gb >= kUpRing && !mbar_wait(smem_u32(&empty_b[sb]), (uint32_t)((gb / kUpRing - 1) & 1), a.wait_ns))) {
             atomicExch(&give_up, 1);
             stop = true;
             break;
           }
-          if (*(volatile int*)&give_up || g == a.withhold) {
+          if (*(volatile int*)&give_up || gb == a.withhold) {
             stop = true;
             break;
           }
-          const uint32_t fb = smem_u32(&full_bar[slot]);
-          const uint32_t sa = smem_u32(ring + slot * kTcStageBytes), sb = sa + kTcABytes;
-          mbar_expect_tx(fb, kTcStageBytes);
-          bulk_g2s(sa, gx + (i64)st * kTcABytes, kTcABytes, fb);
-          bulk_g2s(sb, gy + (i64)st * kTcBBytes, kTcBBytes, fb);
-          ++g;
+          if (load_x) {
+            const uint32_t fa = smem_u32(&full_a[sa]);
+            mbar_expect_tx(fa, kTcABytes);
+            bulk_g2s(xs + sa * kTcABytes, gx + (i64)st * kTcABytes, kTcABytes, fa);
+            ++ga;
+          }
+          const uint32_t fb = smem_u32(&full_b[sb]);
+          mbar_expect_tx(fb, kTcBBytes);
+          bulk_g2s(ys + sb * kTcBBytes, gy + (i64)st * kTcBBytes, kTcBBytes, fb);
+          ++gb;
         }
       }
       // every issued copy must have landed before the block leaves (bounded)
-      for (int h = g - kUpRing < 0 ? 0 : g - kUpRing; h < g; ++h)
-        mbar_wait(smem_u32(&full_bar[h % kUpRing]), (uint32_t)((h / kUpRing) & 1), a.wait_ns);
+      for (int h = ga - xr < 0 ? 0 : ga - xr; h < ga; ++h)
+        mbar_wait(smem_u32(&full_a[h % xr]), (uint32_t)((h / xr) & 1), a.wait_ns);
+      for (int h = gb - kUpRing < 0 ? 0 : gb - kUpRing; h < gb; ++h)
+        mbar_wait(smem_u32(&full_b[h % kUpRing]), (uint32_t)((h / kUpRing) & 1), a.wait_ns);
     }
   } else if (warp == 1) {
     if (lane == 0) {  // MMA issuer
-      int g = 0, k = 0;
+      int ga = 0, gb = 0, k = 0;  // X stage of the tile's first one (kept) or of this one; Y stage; tile
+      const int xr = keep_x ? nst : kUpRing;
       bool stop = false;
-      for (int T = blockIdx.x; T < ntiles && !stop; T += gridDim.x, ++k) {
+      for (int T = t_first; T < t_last && !stop; T += t_step, ++k) {
         if (k >= 1 && !mbar_wait(smem_u32(&acc_empty), (uint32_t)((k - 1) & 1), a.wait_ns)) {
           atomicExch(&give_up, 1);
           break;
         }
         tc_fence_after();
+        const bool free_x = !keep_x || T + 1 == t_last || (T + 1) % a.tiles_q == 0;
         for (int st = 0; st < nst; ++st) {
-          const int slot = g % kUpRing;
-          if (!mbar_wait(smem_u32(&full_bar[slot]), (uint32_t)((g / kUpRing) & 1), a.wait_ns) ||
+          const int ha = keep_x ? ga + st : ga;
+          const int sa = ha % xr, sb = gb % kUpRing;
+          if (!mbar_wait(smem_u32(&full_a[sa]), (uint32_t)((ha / xr) & 1), a.wait_ns) ||
+              !mbar_wait(smem_u32(&full_b[sb]), (uint32_t)((gb / kUpRing) & 1), a.wait_ns) ||
               *(volatile int*)&give_up) {
             atomicExch(&give_up, 1);
             stop = true;
             break;
           }
           tc_fence_after();
-          const uint32_t sa = smem_u32(ring + slot * kTcStageBytes), sb = sa + kTcABytes;
-          const uint64_t ad0 = tc_desc(sa), bd0 = tc_desc(sb);
+          const uint64_t ad0 = tc_desc(xs + sa * kTcABytes), bd0 = tc_desc(ys + sb * kTcBBytes);
 #pragma unroll
-          for (int u = 0; u < 22; ++u) {
+          for (int u = 0; u < kTcMmas; ++u) {
             const TcMma e = kTcSchedule[u];
             const uint64_t ad = ad0 + (uint64_t)((e.i * kTcM * kStage) >> 4);
             const uint64_t bd = bd0 + (uint64_t)((e.j0 * kTcN * kStage) >> 4);
             tc_mma(tmem + (uint32_t)((e.i + e.j0 - kRegionLo) * kTcN), ad, bd, e.n, (st > 0 || u >= 2) ? 1u : 0u);
           }
-          tc_commit(smem_u32(&empty_bar[slot]));
-          ++g;
+          if (free_x) tc_commit(smem_u32(&empty_a[sa]));
+          tc_commit(smem_u32(&empty_b[sb]));
+          if (!keep_x) ++ga;
+          ++gb;
         }
+        if (keep_x && free_x) ga += nst;
         tc_commit(smem_u32(&acc_full));
       }
       tc_commit(smem_u32(&mma_done));  // every MMA issued above has completed when this arrives
@@ -761,7 +825,7 @@ __global__ void __launch_bounds__(kUpThreads, 1) ozaki_tc_update_kernel(OzArgs a
     const int qw = warp & 3, r = 32 * qw + lane;
     const uint32_t lane_base = tmem + ((uint32_t)(32 * qw) << 16);
     int k = 0;
-    for (int T = blockIdx.x; T < ntiles; T += gridDim.x, ++k) {
+    for (int T = t_first; T < t_last; T += t_step, ++k) {
       const int p0 = (T / a.tiles_q) * kTcM, q0 = (T % a.tiles_q) * kTcN;
       const bool ok = mbar_wait(smem_u32(&acc_full), (uint32_t)(k & 1), a.wait_ns);
       if (!__all_sync(0xffffffffu, ok) || *(volatile int*)&give_up) {
@@ -769,30 +833,14 @@ __global__ void __launch_bounds__(kUpThreads, 1) ozaki_tc_update_kernel(OzArgs a
         break;
       }
       tc_fence_after();
-      // phase 1: level sums -> exact group sums g0 (levels 13..19), g1 (20..26), kept in registers
+      // phase 1: level sums -> exact group sums g0 (levels 10..15), g1 (16..20), kept in registers
       long long g0[kTcN], g1[kTcN];
 #pragma unroll
       for (int c0 = 0; c0 < kTcN; c0 += 8) {
+        uint32_t v[kLevels][8];
+        load_levels(lane_base, c0, v);
 #pragma unroll
-        for (int grp = 1; grp >= 0; --grp) {
-          uint32_t v[7][8];
-#pragma unroll
-          for (int l = 6; l >= 0; --l)
-            tc_ld8(lane_base + (uint32_t)((kLevelLo - kRegionLo + 7 * grp + l) * kTcN + c0), v[l]);
-          tc_wait_ld();
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            long long acc = 0;
-            if (kMagic) {
-              acc = group_sum_magic(v, j);
-            } else {
-#pragma unroll
-              for (int l = 6; l >= 0; --l) acc = acc * 16 + __float2int_rz(__uint_as_float(v[l][j]));
-            }
-            if (grp) g1[c0 + j] = acc;
-            else g0[c0 + j] = acc;
-          }
-        }
+        for (int j = 0; j < 8; ++j) group_sums<kMagic>(v, j, g0[c0 + j], g1[c0 + j]);
       }
       // hand the regions back to the MMA warp (the next tile's first stage overwrites them)
       tc_fence_before();
@@ -819,8 +867,7 @@ __global__ void __launch_bounds__(kUpThreads, 1) ozaki_tc_update_kernel(OzArgs a
             } else if (exr == kExpZero || eyc == kExpZero) {
               v = 0.0;
             } else {
-              const int e2 = exr + eyc - 112 + 4 * kLevelLo;
-              v = scaled_int(g1[h + j], e2 + 28) + scaled_int(g0[h + j], e2);  // one rounding
+              v = group_value(g0[h + j], g1[h + j], exr + eyc);
             }
             a.C[pr + (i64)qc * a.ldc] = cv[j] - v;
           }
@@ -834,15 +881,15 @@ __global__ void __launch_bounds__(kUpThreads, 1) ozaki_tc_update_kernel(OzArgs a
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcCols));
 }
 
-__global__ void ozaki_reduce_kernel(const double* part, i64 nsub, int p, int q, double* C, i64 ldc,
-                                    const int* status) {
+// C = sum of the sub-chunks' partials, 16 entries per block (split_sum16).
+__global__ void __launch_bounds__(256) ozaki_reduce_kernel(const double* part, i64 nsub, int p, int q, double* C,
+                                                           i64 ldc, const int* status) {
+  __shared__ double red[16 * 17];
   if (status && *status) return;
-  const i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (i64)p * q) return;
-  const int r = (int)(e % p), c = (int)(e / p);
-  double s = 0.0;
-  for (i64 k = 0; k < nsub; ++k) s += part[k * p * q + e];
-  C[r + (i64)c * ldc] = s;
+  const i64 pq = (i64)p * q, e = (i64)blockIdx.x * 16 + (threadIdx.x & 15);
+  const bool live = e < pq;
+  const double s = split_sum16(nsub, live, red, [=](i64 k) { return part[k * pq + e]; });
+  if (threadIdx.x < 16 && live) C[e % p + (e / p) * ldc] = s;
 }
 
 void up_attr() {
@@ -952,11 +999,11 @@ cudaError_t tn_product_emulated(i64 m, int p, int q, const double* X, i64 ldx, c
   for (i64 r0 = 0; r0 < m; r0 += ch) {
     const i64 nsub = ((m - r0 < ch ? m - r0 : ch) + kSub - 1) / kSub;
     prof_begin(kMisc, st);
-    ozaki_split_kernel<<<dim3((unsigned)((p + 7) / 8), (unsigned)nsub), 256, 0, st>>>(X, ldx, m, r0, p, kTcM, px, ex, status);
+    ozaki_split_kernel<<<dim3((unsigned)((p + 7) / 8), (unsigned)nsub), 256, 0, st>>>(X, ldx, m, r0, p, kTcM, kStagesPerSub, px, ex, status);
     prof_end(kMisc, 0.0, st);
     if (!same) {
       prof_begin(kMisc, st);
-      ozaki_split_kernel<<<dim3((unsigned)((q + 7) / 8), (unsigned)nsub), 256, 0, st>>>(Y, ldy, m, r0, q, kTcN, py, ey, status);
+      ozaki_split_kernel<<<dim3((unsigned)((q + 7) / 8), (unsigned)nsub), 256, 0, st>>>(Y, ldy, m, r0, q, kTcN, kStagesPerSub, py, ey, status);
       prof_end(kMisc, 0.0, st);
     }
     OzArgs a{};
@@ -980,7 +1027,7 @@ cudaError_t tn_product_emulated(i64 m, int p, int q, const double* X, i64 ldx, c
   }
   const i64 pq = (i64)p * q;
   prof_begin(kReduce, st);
-  ozaki_reduce_kernel<<<(unsigned)((pq + 255) / 256), 256, 0, st>>>(part, nsub_total, p, q, C, ldc, status);
+  ozaki_reduce_kernel<<<(unsigned)((pq + 15) / 16), 256, 0, st>>>(part, nsub_total, p, q, C, ldc, status);
   prof_end(kReduce, (double)nsub_total * pq, st);
   return cudaGetLastError();
 }
@@ -1022,7 +1069,7 @@ cudaError_t nn_update_emulated(i64 M, int N, int K, const double* X, i64 ldx, co
     const int kc = (int)(K - k0 < kSub ? K - k0 : kSub);
     const int nst = (kc + kStage - 1) / kStage;
     prof_begin(kMisc, st);
-    ozaki_split_kernel<<<dim3((unsigned)((N + 7) / 8), 1u), 256, 0, st>>>(Y, ldy, k0 + kc, k0, N, kTcN, py, ey, status);
+    ozaki_split_kernel<<<dim3((unsigned)((N + 7) / 8), 1u), 256, 0, st>>>(Y, ldy, k0 + kc, k0, N, kTcN, nst, py, ey, status);
     prof_end(kMisc, 0.0, st);
     for (i64 r0 = 0; r0 < M; r0 += rows) {
       const i64 live = M - r0 < rows ? M - r0 : rows;
