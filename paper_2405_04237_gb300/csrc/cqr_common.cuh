@@ -54,6 +54,47 @@ cudaError_t tn_product(i64 m, int p, int q, const double* X, i64 ldx, const doub
 i64 gram_partials(i64 m, int b, const double* X, i64 ldx, double* part, const int* status, cudaStream_t st);
 
 #ifdef __CUDACC__
+// Dependent launches.  A factorisation is a chain of kernels that each need
+// the one before; for small matrices the gap between two of them, 2-3 us, is
+// as long as the kernels.  launch() lets a kernel be set up and its blocks
+// start while the one before it on the stream still runs; stream_wait(), the
+// first statement of every kernel launched this way, waits until that one has
+// ended and its writes are visible (so all earlier ones have ended too), and
+// then allows the next kernel the same.  Only grids of at most one block per
+// SM, or with less work than kEarlyFlops, start early: blocks placed while
+// others still run land unevenly, and the persistent grids of large products
+// (three equal blocks per SM) lost 11 % by it (2^20 x 256: 231 -> 258 ms).
+__device__ __forceinline__ void stream_wait() {
+  asm volatile("griddepcontrol.wait;\ngriddepcontrol.launch_dependents;" ::: "memory");
+}
+
+constexpr double kEarlyFlops = 3e7;  // 25 us of FP64 work; the gap saved is 2-3 us
+
+struct Work64 {  // FP64 operations of a launch
+  double flops;
+};
+constexpr Work64 kAnyWork{1e300};
+
+template <class... P, class... A>
+cudaError_t launch(Work64 w, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = (i64)grid.x * grid.y * grid.z <= kSMs || w.flops <= kEarlyFlops ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+template <class... P, class... A>
+cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  return launch(kAnyWork, kernel, grid, block, smem, st, args...);
+}
+
 // Upper-triangle enumeration, column by column: u -> (i, j), 0 <= i <= j.
 __host__ __device__ inline void decode_upper(int u, int& i, int& j) {
   int jj = (int)((sqrtf(8.0f * (float)u + 1.0f) - 1.0f) * 0.5f);
@@ -186,7 +227,6 @@ cudaError_t batched_persistent_run(int batch, const int64_t* m, const int64_t* n
                                    int* status, void* workspace, int G, bool halve, cudaStream_t st);
 cudaError_t batched_persistent_panels(int batch, const void* workspace, int* host_b, cudaStream_t st);
 
-// ---------------------------------------------------------------------------
 // Launch accounting (prof.cu).  Every launch is wrapped in prof_begin /
 // prof_end with its kernel class and algorithmic FLOP count.
 enum KernelClass {

@@ -137,6 +137,7 @@ __device__ void chol_small(const CholArgs& a, SmallChol& s) {
 }
 
 __global__ void __launch_bounds__(kSmallT) chol_small_kernel(CholArgs a) {
+  stream_wait();
   __shared__ SmallChol s;
   if (a.status && *a.status) return;
   chol_small(a, s);
@@ -148,6 +149,7 @@ __global__ void __launch_bounds__(kSmallT) chol_small_kernel(CholArgs a) {
 // CholeskyQR.  `counter` is zero at entry and left zero.
 __global__ void __launch_bounds__(kSmallT) gram_chol_kernel(const double* part, i64 P, CholArgs a,
                                                             unsigned int* counter) {
+  stream_wait();
   __shared__ SmallChol s;
   __shared__ double red[16 * 17];
   __shared__ unsigned int order;
@@ -200,6 +202,7 @@ __device__ __forceinline__ void cluster_barrier() {
 }
 
 __global__ void __cluster_dims__(kClu, 1, 1) __launch_bounds__(kSmallT) chol_cluster_kernel(CholArgs a) {
+  stream_wait();
   extern __shared__ __align__(16) double pan[];  // [kCluTile][rem]: the tile's row panel
   __shared__ double Ws[kCluTile * kCluLd];
   __shared__ TrapWork s;
@@ -309,6 +312,7 @@ __global__ void __cluster_dims__(kClu, 1, 1) __launch_bounds__(kSmallT) chol_clu
 
 // M := copyltu(T - G): M_ac = T_ac - G_ac for a >= c, mirrored above.
 __global__ void backward_middle_kernel(int n, const double* T, const double* G, double* M) {
+  stream_wait();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n * n) return;
   const int a = e % n, c = e / n;
@@ -317,6 +321,7 @@ __global__ void backward_middle_kernel(int n, const double* T, const double* G, 
 }
 
 __global__ void diag_reciprocal_kernel(int n, const double* R, i64 ldr, double* rinv) {
+  stream_wait();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < n) rinv[j] = 1.0 / R[j + (i64)j * ldr];
 }
@@ -329,7 +334,7 @@ cudaError_t chol_factor(int b, double* W, i64 ldw, double* U, i64 ldu, double* r
   prof_begin(kCholesky, st);
   const CholArgs a{b, W, ldw, U, ldu, rinv, col0, status, shift_fro, m, skip, reject};
   if (b <= kSmallChol) {
-    chol_small_kernel<<<1, kSmallT, 0, st>>>(a);
+    launch(chol_small_kernel, 1, kSmallT, 0, st, a);
   } else {
     static bool attr = false;
     if (!attr) {
@@ -337,7 +342,7 @@ cudaError_t chol_factor(int b, double* W, i64 ldw, double* U, i64 ldu, double* r
                            (int)chol_cluster_smem(CQR_MAX_PANEL));
       attr = true;
     }
-    chol_cluster_kernel<<<kClu, kSmallT, chol_cluster_smem(b), st>>>(a);
+    launch(chol_cluster_kernel, kClu, kSmallT, chol_cluster_smem(b), st, a);
   }
   prof_end(kCholesky, (double)b * b * b / 3.0, st);
   return cudaGetLastError();
@@ -355,7 +360,7 @@ cudaError_t gram_chol(i64 m, int b, const double* X, i64 ldx, double* part, doub
   const i64 P = gram_partials(m, b, X, ldx, part, status, st);
   const CholArgs a{b, W, ldw, U, ldu, rinv, col0, status, shift_fro, m, skip, reject};
   prof_begin(kCholesky, st);
-  gram_chol_kernel<<<(b * (b + 1) / 2 + 15) / 16, kSmallT, 0, st>>>(part, P, a, counter);
+  launch(gram_chol_kernel, (b * (b + 1) / 2 + 15) / 16, kSmallT, 0, st, part, P, a, counter);
   prof_end(kCholesky, (double)b * b * b / 3.0, st);
   return cudaGetLastError();
 }
@@ -363,14 +368,14 @@ cudaError_t gram_chol(i64 m, int b, const double* X, i64 ldx, double* part, doub
 cudaError_t backward_middle(int n, const double* T, const double* G, double* M, cudaStream_t st) {
   const int thr = 256;
   prof_begin(kMisc, st);
-  backward_middle_kernel<<<(n * n + thr - 1) / thr, thr, 0, st>>>(n, T, G, M);
+  launch(backward_middle_kernel, (n * n + thr - 1) / thr, thr, 0, st, n, T, G, M);
   prof_end(kMisc, (double)n * n, st);
   return cudaGetLastError();
 }
 
 cudaError_t diag_reciprocal(int n, const double* R, i64 ldr, double* rinv, cudaStream_t st) {
   prof_begin(kMisc, st);
-  diag_reciprocal_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, R, ldr, rinv);
+  launch(diag_reciprocal_kernel, (n + 255) / 256, 256, 0, st, n, R, ldr, rinv);
   prof_end(kMisc, (double)n, st);
   return cudaGetLastError();
 }

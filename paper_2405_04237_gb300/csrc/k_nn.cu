@@ -5,9 +5,13 @@
 // products R = R2 R1 (Alg. 3 step 3, Alg. 7 step 3), R_jj = S2 S1 and
 // R_{1:j-1,j} += Z S1 of Alg. 9.
 //
-// Each block computes a TM x TN output tile (TM * TN = 4096, 256 threads,
-// one 4 x 4 register micro-tile per thread); K is staged through shared
-// memory in chunks.  With beta = 1 the accumulator starts from C and every
+// Each block computes a TM x TN output tile (256 threads, one MT x MT register
+// micro-tile per thread, TM * TN = 256 MT^2); K is staged through shared
+// memory in chunks.  MT is 4 where that fills the chip; smaller outputs take
+// 2 or 1, so that their multiply-adds (64 clocks each for a warp) are spread
+// over more SMs: a 64 x 64 x 64 product took 81 us in one block of 4 x 4
+// micro-tiles.  Every element sees the same operations in the same order
+// whatever the tile.  With beta = 1 the accumulator starts from C and every
 // term is one fused multiply-add (negated operand when alpha = -1), so the
 // update issues exactly one FP64 instruction per multiply-add.  Threads
 // whose four columns all lie beyond N skip the arithmetic (warp-uniform when
@@ -34,19 +38,36 @@ struct NnArgs {
   const int* status;
 };
 
-template <int TM, int TN>
+template <int TM, int TN, int MT>
 struct NnShape {
-  static constexpr int NTM = TM / 4;
+  static constexpr int NTM = TM / MT;
   static constexpr int KC = TM >= 256 ? 8 : 16;
   static constexpr int SA = TM + 2, SB = TN + 2;
-  static_assert(TM % 4 == 0 && TN % 4 == 0, "4 x 4 micro-tiles");
-  static_assert(NTM * (TN / 4) == kNnThreads, "one micro-tile per thread covers the TM x TN tile");
+  static_assert(TM % MT == 0 && TN % MT == 0, "MT x MT micro-tiles");
+  static_assert(NTM * (TN / MT) == kNnThreads, "one micro-tile per thread covers the TM x TN tile");
   static_assert(KC * (SA + SB) * (int)sizeof(double) <= 48 * 1024, "static shared memory limit");
 };
 
-template <int TM, int TN, bool NEG>
+// MT consecutive doubles of a shared-memory row
+template <int MT>
+__device__ __forceinline__ void lds_micro(const double* p, double (&v)[MT]) {
+  if constexpr (MT % 2 == 0) {
+#pragma unroll
+    for (int i = 0; i < MT; i += 2) {
+      const double2 x = *reinterpret_cast<const double2*>(p + i);
+      v[i] = x.x;
+      v[i + 1] = x.y;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < MT; ++i) v[i] = p[i];
+  }
+}
+
+template <int TM, int TN, int MT, bool NEG>
 __global__ void __launch_bounds__(kNnThreads) nn_kernel(NnArgs a) {
-  using Sh = NnShape<TM, TN>;
+  stream_wait();
+  using Sh = NnShape<TM, TN, MT>;
   __shared__ __align__(16) double As[Sh::KC * Sh::SA];
   __shared__ __align__(16) double Bs[Sh::KC * Sh::SB];
   if (a.status && *a.status) return;
@@ -56,23 +77,23 @@ __global__ void __launch_bounds__(kNnThreads) nn_kernel(NnArgs a) {
   const int n0 = tn_i * TN;
   const int t = threadIdx.x;
   const int mi = t % Sh::NTM, nj = t / Sh::NTM;
-  const bool cols_live = n0 + 4 * nj < a.N;
-  const bool rows_live = m0 + 4 * mi < a.M;
+  const bool cols_live = n0 + MT * nj < a.N;
+  const bool rows_live = m0 + MT * mi < a.M;
   const bool live = cols_live && rows_live;
 
   int klo = 0, khi = a.K;
   if (a.a_upper) klo = (int)(m0 < (i64)a.K ? m0 : (i64)a.K);
   if (a.b_upper) khi = min(a.K, n0 + TN);
 
-  double acc[4][4];
+  double acc[MT][MT];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < MT; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < MT; ++j) {
       double v = 0.0;
       if (a.beta) {
-        const i64 r = m0 + 4 * mi + i;
-        const int c = n0 + 4 * nj + j;
+        const i64 r = m0 + MT * mi + i;
+        const int c = n0 + MT * nj + j;
         if (r < a.M && c < a.N) v = a.C[r + (i64)c * a.ldc];
       }
       acc[i][j] = v;
@@ -108,36 +129,46 @@ __global__ void __launch_bounds__(kNnThreads) nn_kernel(NnArgs a) {
     if (live) {
 #pragma unroll 4
       for (int kk = 0; kk < Sh::KC; ++kk) {
-        const double2 a01 = *reinterpret_cast<const double2*>(&As[kk * Sh::SA + 4 * mi]);
-        const double2 a23 = *reinterpret_cast<const double2*>(&As[kk * Sh::SA + 4 * mi + 2]);
-        const double2 b01 = *reinterpret_cast<const double2*>(&Bs[kk * Sh::SB + 4 * nj]);
-        const double2 b23 = *reinterpret_cast<const double2*>(&Bs[kk * Sh::SB + 4 * nj + 2]);
-        const double av[4] = {a01.x, a01.y, a23.x, a23.y};
-        const double bv[4] = {b01.x, b01.y, b23.x, b23.y};
+        double av[MT], bv[MT];
+        lds_micro<MT>(&As[kk * Sh::SA + MT * mi], av);
+        lds_micro<MT>(&Bs[kk * Sh::SB + MT * nj], bv);
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < MT; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = NEG ? fma(-av[i], bv[j], acc[i][j]) : fma(av[i], bv[j], acc[i][j]);
+          for (int j = 0; j < MT; ++j) acc[i][j] = NEG ? fma(-av[i], bv[j], acc[i][j]) : fma(av[i], bv[j], acc[i][j]);
       }
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < MT; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const i64 r = m0 + 4 * mi + i;
-      const int c = n0 + 4 * nj + j;
+    for (int j = 0; j < MT; ++j) {
+      const i64 r = m0 + MT * mi + i;
+      const int c = n0 + MT * nj + j;
       if (r < a.M && c < a.N) a.C[r + (i64)c * a.ldc] = acc[i][j];
     }
 }
 
-template <int TM, int TN>
-void launch_nn(const NnArgs& a, bool neg, i64 blocks, cudaStream_t st) {
+template <int TM, int TN, int MT>
+void launch_nn(const NnArgs& a, bool neg, cudaStream_t st) {
+  const i64 blocks = ((a.M + TM - 1) / TM) * a.tiles_n;
+  const Work64 w{2.0 * (double)a.M * a.N * a.K};
   if (neg)
-    nn_kernel<TM, TN, true><<<(unsigned)blocks, kNnThreads, 0, st>>>(a);
+    launch(w, nn_kernel<TM, TN, MT, true>, (unsigned)blocks, kNnThreads, 0, st, a);
   else
-    nn_kernel<TM, TN, false><<<(unsigned)blocks, kNnThreads, 0, st>>>(a);
+    launch(w, nn_kernel<TM, TN, MT, false>, (unsigned)blocks, kNnThreads, 0, st, a);
+}
+
+// Column tile for N columns and micro-tiles of MT (the widest is 16 MT).
+int nn_tile_n(int N, int MT) {
+  int t = 8;
+  while (t < N && t < 16 * MT) t *= 2;
+  return t;
+}
+i64 nn_blocks(i64 M, int N, int MT) {
+  const int TN = nn_tile_n(N, MT), TM = 256 * MT * MT / TN;
+  return (M + TM - 1) / TM * ((N + TN - 1) / TN);
 }
 
 }  // namespace
@@ -168,16 +199,29 @@ cudaError_t nn_product_t(i64 M, int N, int K, const double* A, i64 lda, const do
   a.transb = transb;
   a.status = status;
   const bool neg = alpha < 0.0;
-  int TN = N <= 8 ? 8 : N <= 16 ? 16 : N <= 32 ? 32 : 64;
-  int TM = 4096 / TN;
+  // 4 x 4 micro-tiles from two blocks per SM on, 2 x 2 from one, else single entries
+  const int MT = nn_blocks(M, N, 4) >= 2 * kSMs ? 4 : nn_blocks(M, N, 2) >= kSMs ? 2 : 1;
+  const int TN = nn_tile_n(N, MT);
   a.tiles_n = (N + TN - 1) / TN;
-  const i64 blocks = ((M + TM - 1) / TM) * a.tiles_n;
   prof_begin(kUpdate, st);
-  switch (TN) {
-    case 8: launch_nn<512, 8>(a, neg, blocks, st); break;
-    case 16: launch_nn<256, 16>(a, neg, blocks, st); break;
-    case 32: launch_nn<128, 32>(a, neg, blocks, st); break;
-    default: launch_nn<64, 64>(a, neg, blocks, st); break;
+  if (MT == 4) {
+    switch (TN) {
+      case 8: launch_nn<512, 8, 4>(a, neg, st); break;
+      case 16: launch_nn<256, 16, 4>(a, neg, st); break;
+      case 32: launch_nn<128, 32, 4>(a, neg, st); break;
+      default: launch_nn<64, 64, 4>(a, neg, st); break;
+    }
+  } else if (MT == 2) {
+    switch (TN) {
+      case 8: launch_nn<128, 8, 2>(a, neg, st); break;
+      case 16: launch_nn<64, 16, 2>(a, neg, st); break;
+      default: launch_nn<32, 32, 2>(a, neg, st); break;
+    }
+  } else {
+    if (TN == 8)
+      launch_nn<32, 8, 1>(a, neg, st);
+    else
+      launch_nn<16, 16, 1>(a, neg, st);
   }
   prof_end(kUpdate, 2.0 * (double)M * N * K, st);
   return cudaGetLastError();

@@ -214,6 +214,7 @@ __device__ __forceinline__ void load16(const double* xc, i64 row, i64 m, bool co
 
 __global__ void __launch_bounds__(256, 2) ozaki_split_kernel(const double* X, i64 ldx, i64 m, i64 r0, int c, int T,
                                                              int nst, uint8_t* planes, int* exps, const int* status) {
+  stream_wait();
   if (status && *status) return;
   const int g = blockIdx.x, s = blockIdx.y, t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int cl = lane & 7, half = (lane >> 3) & 1, so = lane >> 4;
@@ -299,6 +300,7 @@ __global__ void __launch_bounds__(256, 2) ozaki_split_kernel(const double* X, i6
 __global__ void __launch_bounds__(128) ozaki_rowsplit_kernel(const double* X, i64 ldx, i64 m, i64 r0, int rows,
                                                              i64 k0, int kc, uint8_t* planes, int* exps,
                                                              const int* status) {
+  stream_wait();
   if (status && *status) return;
   const int row = blockIdx.x * 128 + threadIdx.x;
   if (row >= rows) return;
@@ -540,6 +542,7 @@ struct OzArgs {
 // together share the X planes of a sub-chunk in L2); the tile goes to the
 // sub-chunk's partial.
 __global__ void __launch_bounds__(kTcThreads, 1) ozaki_tc_kernel(OzArgs a) {
+  stream_wait();
   extern __shared__ uint8_t tc_raw[];
   __shared__ __align__(8) uint64_t full_bar[kTcRing], empty_bar[kTcRing], done_bar;
   __shared__ uint32_t tmem_slot;
@@ -700,6 +703,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 
 template <bool kMagic>
 __global__ void __launch_bounds__(kUpThreads, 1) ozaki_tc_update_kernel(OzArgs a, int ntiles) {
+  stream_wait();
   extern __shared__ uint8_t up_raw[];
   __shared__ __align__(8) uint64_t full_a[kUpRing], empty_a[kUpRing], full_b[kUpRing], empty_b[kUpRing];
   __shared__ __align__(8) uint64_t acc_full, acc_empty, mma_done;
@@ -884,6 +888,7 @@ __global__ void __launch_bounds__(kUpThreads, 1) ozaki_tc_update_kernel(OzArgs a
 // C = sum of the sub-chunks' partials, 16 entries per block (split_sum16).
 __global__ void __launch_bounds__(256) ozaki_reduce_kernel(const double* part, i64 nsub, int p, int q, double* C,
                                                            i64 ldc, const int* status) {
+  stream_wait();
   __shared__ double red[16 * 17];
   if (status && *status) return;
   const i64 pq = (i64)p * q, e = (i64)blockIdx.x * 16 + (threadIdx.x & 15);
@@ -999,11 +1004,11 @@ cudaError_t tn_product_emulated(i64 m, int p, int q, const double* X, i64 ldx, c
   for (i64 r0 = 0; r0 < m; r0 += ch) {
     const i64 nsub = ((m - r0 < ch ? m - r0 : ch) + kSub - 1) / kSub;
     prof_begin(kMisc, st);
-    ozaki_split_kernel<<<dim3((unsigned)((p + 7) / 8), (unsigned)nsub), 256, 0, st>>>(X, ldx, m, r0, p, kTcM, kStagesPerSub, px, ex, status);
+    launch(ozaki_split_kernel, dim3((unsigned)((p + 7) / 8), (unsigned)nsub), 256, 0, st, X, ldx, m, r0, p, kTcM, kStagesPerSub, px, ex, status);
     prof_end(kMisc, 0.0, st);
     if (!same) {
       prof_begin(kMisc, st);
-      ozaki_split_kernel<<<dim3((unsigned)((q + 7) / 8), (unsigned)nsub), 256, 0, st>>>(Y, ldy, m, r0, q, kTcN, kStagesPerSub, py, ey, status);
+      launch(ozaki_split_kernel, dim3((unsigned)((q + 7) / 8), (unsigned)nsub), 256, 0, st, Y, ldy, m, r0, q, kTcN, kStagesPerSub, py, ey, status);
       prof_end(kMisc, 0.0, st);
     }
     OzArgs a{};
@@ -1022,12 +1027,12 @@ cudaError_t tn_product_emulated(i64 m, int p, int q, const double* X, i64 ldx, c
     a.status = const_cast<int*>(status);
     take_fault(0, a);
     prof_begin(kProjection, st);
-    ozaki_tc_kernel<<<dim3((unsigned)tiles_q, (unsigned)tiles_p, (unsigned)nsub), kTcThreads, kTcSmem, st>>>(a);
+    launch(ozaki_tc_kernel, dim3((unsigned)tiles_q, (unsigned)tiles_p, (unsigned)nsub), kTcThreads, kTcSmem, st, a);
     prof_end(kProjection, 2.0 * (double)(nsub * kSub < m - r0 ? nsub * kSub : m - r0) * p * q, st);
   }
   const i64 pq = (i64)p * q;
   prof_begin(kReduce, st);
-  ozaki_reduce_kernel<<<(unsigned)((pq + 15) / 16), 256, 0, st>>>(part, nsub_total, p, q, C, ldc, status);
+  launch(ozaki_reduce_kernel, (unsigned)((pq + 15) / 16), 256, 0, st, part, nsub_total, p, q, C, ldc, status);
   prof_end(kReduce, (double)nsub_total * pq, st);
   return cudaGetLastError();
 }
@@ -1069,13 +1074,13 @@ cudaError_t nn_update_emulated(i64 M, int N, int K, const double* X, i64 ldx, co
     const int kc = (int)(K - k0 < kSub ? K - k0 : kSub);
     const int nst = (kc + kStage - 1) / kStage;
     prof_begin(kMisc, st);
-    ozaki_split_kernel<<<dim3((unsigned)((N + 7) / 8), 1u), 256, 0, st>>>(Y, ldy, k0 + kc, k0, N, kTcN, nst, py, ey, status);
+    launch(ozaki_split_kernel, dim3((unsigned)((N + 7) / 8), 1u), 256, 0, st, Y, ldy, k0 + kc, k0, N, kTcN, nst, py, ey, status);
     prof_end(kMisc, 0.0, st);
     for (i64 r0 = 0; r0 < M; r0 += rows) {
       const i64 live = M - r0 < rows ? M - r0 : rows;
       const int rws = (int)((live + kTcM - 1) / kTcM * kTcM);
       prof_begin(kMisc, st);
-      ozaki_rowsplit_kernel<<<(unsigned)(rws / 128), 128, 0, st>>>(X, ldx, M, r0, rws, k0, kc, px, ex, status);
+      launch(ozaki_rowsplit_kernel, (unsigned)(rws / 128), 128, 0, st, X, ldx, M, r0, rws, k0, kc, px, ex, status);
       prof_end(kMisc, 0.0, st);
       OzArgs a{};
       a.px = px;
@@ -1095,9 +1100,9 @@ cudaError_t nn_update_emulated(i64 M, int N, int K, const double* X, i64 ldx, co
       prof_begin(kUpdate, st);
       const unsigned grid = (unsigned)(ntiles < kSMs ? ntiles : kSMs);
       if (nst * kStage <= kMagicMaxK)
-        ozaki_tc_update_kernel<true><<<grid, kUpThreads, kUpSmem, st>>>(a, ntiles);
+        launch(ozaki_tc_update_kernel<true>, grid, kUpThreads, kUpSmem, st, a, ntiles);
       else
-        ozaki_tc_update_kernel<false><<<grid, kUpThreads, kUpSmem, st>>>(a, ntiles);
+        launch(ozaki_tc_update_kernel<false>, grid, kUpThreads, kUpSmem, st, a, ntiles);
       prof_end(kUpdate, 2.0 * (double)live * N * kc, st);
     }
   }

@@ -80,6 +80,7 @@ __device__ __forceinline__ void syrk_tile_row(const double* row, int i, int j, d
 
 template <int T>
 __global__ void __launch_bounds__(T) syrk_partial_kernel(SyrkArgs a) {
+  stream_wait();
   extern __shared__ __align__(16) double sm[];
   if (a.status && *a.status) return;
   const int t = threadIdx.x;
@@ -145,6 +146,7 @@ __global__ void __launch_bounds__(T) syrk_partial_kernel(SyrkArgs a) {
 // of the upper triangle (column by column) per block of 256 threads.
 __global__ void __launch_bounds__(256) syrk_reduce_kernel(const double* part, int b, i64 P, double* W, i64 ldw,
                                                           const int* status) {
+  stream_wait();
   __shared__ double red[16 * 17];
   if (status && *status) return;
   const int u = blockIdx.x * 16 + (threadIdx.x & 15);
@@ -183,6 +185,7 @@ struct TnArgs {
 
 template <bool kFull>
 __global__ void __launch_bounds__(kTnThreads) tn_partial_kernel(TnArgs a) {
+  stream_wait();
   extern __shared__ __align__(16) double sm[];
   if (a.status && *a.status) return;
   const int t = threadIdx.x;
@@ -262,6 +265,7 @@ __global__ void __launch_bounds__(kTnThreads) tn_partial_kernel(TnArgs a) {
 // C[r + c*ldc] = sum over the segments of tile(r, c), ascending rows.
 __global__ void __launch_bounds__(256) tn_reduce_kernel(const double* part, int p, int q, int TP, int TQ, int tiles_p,
                                                         i64 nb, i64 T, i64 P, double* C, i64 ldc, const int* status) {
+  stream_wait();
   __shared__ double red[16 * 17];
   if (status && *status) return;
   const i64 e = (i64)blockIdx.x * 16 + (threadIdx.x & 15);
@@ -482,9 +486,9 @@ i64 gram_partials(i64 m, int b, const double* X, i64 ldx, double* part, const in
   a.status = status;
   prof_begin(kGram, st);
   if (s.T == 128)
-    syrk_partial_kernel<128><<<s.P, 128, s.smem, st>>>(a);
+    launch(Work64{(double)m * b * (b + 1)}, syrk_partial_kernel<128>, s.P, 128, s.smem, st, a);
   else
-    syrk_partial_kernel<kSyrkThreads><<<s.P, kSyrkThreads, s.smem, st>>>(a);
+    launch(syrk_partial_kernel<kSyrkThreads>, s.P, kSyrkThreads, s.smem, st, a);
   prof_end(kGram, (double)m * b * (b + 1), st);
   return s.P;
 }
@@ -513,7 +517,7 @@ cudaError_t tn_product(i64 m, int p, int q, const double* X, i64 ldx, const doub
   if (sym) {
     const i64 nsum = gram_partials(m, p, X, ldx, part, status, st);  // m == 0: none, the empty sum W = 0
     prof_begin(kReduce, st);
-    syrk_reduce_kernel<<<(p * (p + 1) / 2 + 15) / 16, 256, 0, st>>>(part, p, nsum, C, ldc, status);
+    launch(Work64{(double)nsum * p * (p + 1) / 2}, syrk_reduce_kernel, (p * (p + 1) / 2 + 15) / 16, 256, 0, st, part, p, nsum, C, ldc, status);
     prof_end(kReduce, (double)nsum * p * (p + 1) / 2, st);
     return cudaGetLastError();
   }
@@ -539,14 +543,14 @@ cudaError_t tn_product(i64 m, int p, int q, const double* X, i64 ldx, const doub
     prof_begin(kProjection, st);
     const size_t smem = tn_smem(P.tp, P.tq, P.rb);
     if (P.tp == 64 && P.tq == 64 && P.rb == kFullRows)
-      tn_partial_kernel<true><<<(unsigned)P.S, kTnThreads, smem, st>>>(a);
+      launch(tn_partial_kernel<true>, (unsigned)P.S, kTnThreads, smem, st, a);
     else
-      tn_partial_kernel<false><<<(unsigned)P.S, kTnThreads, smem, st>>>(a);
+      launch(Work64{2.0 * (double)m * p * q}, tn_partial_kernel<false>, (unsigned)P.S, kTnThreads, smem, st, a);
     prof_end(kProjection, 2.0 * (double)m * p * q, st);
   }
   const i64 pq = (i64)p * q;
   prof_begin(kReduce, st);
-  tn_reduce_kernel<<<(unsigned)((pq + 15) / 16), 256, 0, st>>>(part, p, q, P.tp, P.tq, P.tiles_p, a.nb, m > 0 ? a.T : 0,
+  launch(Work64{(double)(P.S + P.ntiles) / P.ntiles * pq}, tn_reduce_kernel, (unsigned)((pq + 15) / 16), 256, 0, st, part, p, q, P.tp, P.tq, P.tiles_p, a.nb, m > 0 ? a.T : 0,
                                            m > 0 ? a.P : 1, C, ldc, status);
   prof_end(kReduce, m > 0 ? (double)(P.S + P.ntiles) / P.ntiles * pq : 0.0, st);
   return cudaGetLastError();

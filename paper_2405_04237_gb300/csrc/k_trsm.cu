@@ -59,6 +59,7 @@ __device__ __forceinline__ void load_common(int b, const double* U, i64 ldu, con
 
 __global__ void __launch_bounds__(kRows) trsm_rows_kernel(i64 m, int b, double* X, i64 ldx, const double* U, i64 ldu,
                                                           const double* rinv, const int* status, const int* skip) {
+  stream_wait();
   extern __shared__ __align__(16) double sm[];
   if (status && *status) return;
   if (skip && *skip) return;  // U = I: the solve would leave X unchanged
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(kRows) trsm_rows_kernel(i64 m, int b, double* 
 
 __global__ void __launch_bounds__(kRows) trsm_rows_t_kernel(i64 m, int b, double* X, i64 ldx, const double* U, i64 ldu,
                                                             const double* rinv) {
+  stream_wait();
   extern __shared__ __align__(16) double sm[];
   double* Ts = sm;
   double* Up = sm + (size_t)b * kRows;
@@ -169,7 +171,7 @@ cudaError_t trsm_rows(i64 m, int b, double* X, i64 ldx, const double* U, i64 ldu
   set_trsm_attr();
   const i64 blocks = (m + kRows - 1) / kRows;
   prof_begin(kTrsm, st);
-  trsm_rows_kernel<<<(unsigned)blocks, kRows, trsm_smem(b), st>>>(m, b, X, ldx, U, ldu, rinv, status, skip);
+  launch(Work64{(double)m * b * b}, trsm_rows_kernel, (unsigned)blocks, kRows, trsm_smem(b), st, m, b, X, ldx, U, ldu, rinv, status, skip);
   prof_end(kTrsm, (double)m * b * b, st);
   return cudaGetLastError();
 }
@@ -181,7 +183,7 @@ cudaError_t trsm_rows_transposed(i64 m, int b, double* X, i64 ldx, const double*
   set_trsm_attr();
   const i64 blocks = (m + kRows - 1) / kRows;
   prof_begin(kTrsm, st);
-  trsm_rows_t_kernel<<<(unsigned)blocks, kRows, trsm_smem(b), st>>>(m, b, X, ldx, U, ldu, rinv);
+  launch(Work64{(double)m * b * b}, trsm_rows_t_kernel, (unsigned)blocks, kRows, trsm_smem(b), st, m, b, X, ldx, U, ldu, rinv);
   prof_end(kTrsm, (double)m * b * b, st);
   return cudaGetLastError();
 }
