@@ -291,18 +291,21 @@ __device__ __forceinline__ void tn_accumulate(const TnMap& mp, const Smem& s, in
 }
 
 // In-CTA sums of the accumulators in a fixed order (block_sums), written
-// tile-major (16 doubles per tile, entry u * 4 + v) to this CTA's slot.
-__device__ void tn_flush(const TnMap& mp, const Smem& s, double (&am)[4][4], double (&ae)[4][4], double* slot) {
+// tile-major (16 doubles per tile, entry u * 4 + v) to this CTA's slot.  Of
+// the threads that share a tile only the first `rows` (the most rows a staged
+// sub-block of the pass held) can have a nonzero part.
+__device__ void tn_flush(const TnMap& mp, const Smem& s, int rows, double (&am)[4][4], double (&ae)[4][4],
+                         double* slot) {
   __syncthreads();
   spill_acc(s.red, kBT, am);
   __syncthreads();
-  block_sums<kBT>(s.red, s.red, mp.M, mp.RG, 1, mp.M, [slot](int id, int e, double x) { slot[id * 16 + e] = x; });
+  block_sums<kBT>(s.red, s.red, mp.M, min(mp.RG, rows), 1, mp.M, [slot](int id, int e, double x) { slot[id * 16 + e] = x; });
   __syncthreads();
   if (mp.E > 0) {
     spill_acc(s.red, kBT, ae);
     __syncthreads();
     double* slot_e = slot + (size_t)mp.M * 16;
-    block_sums<kBT>(s.red, s.red, mp.E, mp.tpt, mp.tpt, 1, [slot_e](int id, int e, double x) { slot_e[id * 16 + e] = x; });
+    block_sums<kBT>(s.red, s.red, mp.E, min(mp.tpt, rows), mp.tpt, 1, [slot_e](int id, int e, double x) { slot_e[id * 16 + e] = x; });
     __syncthreads();
   }
 }
@@ -315,11 +318,10 @@ __device__ void tn_flush(const TnMap& mp, const Smem& s, double (&am)[4][4], dou
 // starts from C and takes one fused multiply-add per term in ascending k.
 template <int TR, int TC>
 __device__ void nn_update_block(const Smem& s, int nr, int xc, int p, int cc, int q, const double* Mm) {
-  const int nrt = s.rb / TR;
+  const int nrt = (nr + TR - 1) / TR;  // blocks of padding rows are left out
   const int nblk = nrt * (q / TC);
   for (int bi = threadIdx.x; bi < nblk; bi += kBT) {
   const int r0 = (bi % nrt) * TR, c0 = (bi / nrt) * TC;
-  if (r0 >= nr) continue;  // padding rows only
   double acc[TR][TC];
 #pragma unroll
   for (int u = 0; u < TR; ++u)
@@ -351,7 +353,7 @@ __device__ void nn_update(const Smem& s, int nr, int xc, int p, int cc, int q, c
   const int cand[8][2] = {{4, 4}, {4, 3}, {4, 2}, {2, 3}, {4, 1}, {1, 3}, {2, 1}, {1, 1}};
   for (int k = 0; k < 8; ++k) {
     if (q % cand[k][1]) continue;
-    const int thr = (s.rb / cand[k][0]) * (q / cand[k][1]);
+    const int thr = ((nr + cand[k][0] - 1) / cand[k][0]) * (q / cand[k][1]);
     if (thr <= kBT && thr > best) {
       best = thr;
       pick = k;
@@ -374,29 +376,68 @@ __device__ void nn_update(const Smem& s, int nr, int xc, int p, int cc, int q, c
 // prescale_rows), s_c' -= s_c Ut_cc' for c' > c in ascending c, then
 // q_c = s_c / U_cc (by the reciprocal rv[c]) -- q_c U_cc' = s_c Ut_cc', so
 // this is the substitution q_c = (x_c - sum_{i<c} q_i U_ic) / U_cc with
-// the division moved past the products.  L lanes of one warp share a row;
-// lane l owns the columns c = l (mod L).  Rows >= nr (padding) are skipped.
-__device__ void trsm_rows_staged(const Smem& s, int tc, int b, int nr) {
-  int L = kBT / s.rb;  // lanes per row: every thread busy, at most 8, at most b
-  L = L > 8 ? 8 : L;
-  L = L > b ? b : L;
-  const int t = threadIdx.x;
-  const int r = t / L, l = t % L;
-  const bool active = t < s.rb * L && r < nr;
+// the division moved past the products.  L lanes of one warp share a row,
+// as many as nr rows leave (up to a warp: an FP64 instruction takes 64 clocks
+// for one live lane as for 32); lane l keeps the columns c = l (mod L) of a block of 8 L
+// columns in registers (s_c travels by a shuffle), so a step's multiply-adds
+// are independent; with the row in shared memory every one waited for the
+// store before it (b = 64, 3 rows: 74000 clocks a solve, 1150 a column).
+// Columns past b and the warps of padding rows are skipped.
+template <int L>
+__device__ __forceinline__ void trsm_rows_lanes(const Smem& s, int tc, int b, int nr) {
+  const int t = threadIdx.x, r = t / L, l = t % L;
+  if ((t & ~31) / L >= nr) return;  // whole warp
+  const bool live = r < nr;
   double* row = s.tile + (size_t)r * s.ts + tc;
-  for (int c = 0; c < b; ++c) {
-    __syncwarp();  // column c complete: its last update came at step c - 1
-    if (active) {
-      const double q = row[c];
-      const double* urow = s.U + (size_t)c * b;
-      for (int cp = (c + 1) / L * L + l; cp < b; cp += L)
-        if (cp > c) row[cp] = fma(-q, urow[cp], row[cp]);
+  for (int c0 = 0; c0 < b; c0 += 8 * L) {
+    const int rem = b - c0;  // lane columns c0 + k L + l with k L + l < rem
+    const double* U0 = s.U + c0 + l;
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = live && k * L + l < rem ? row[c0 + k * L + l] : 0.0;
+    for (int i = 0; i < c0; ++i) {  // solved blocks
+      const double q = live ? row[i] : 0.0;
+      const double* u = U0 + (size_t)i * b;
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (k * L < rem) v[k] = fma(-q, k * L + l < rem ? u[k * L] : 0.0, v[k]);
     }
+#pragma unroll
+    for (int kc = 0; kc < 8; ++kc) {
+      if (kc * L >= rem) break;
+#pragma unroll 2
+      for (int lc = 0; lc < L; ++lc) {
+        if (kc * L + lc >= rem) break;
+        const double q = __shfl_sync(0xffffffffu, v[kc], lc, L);
+        const double* u = U0 + (size_t)(c0 + kc * L + lc) * b;
+        if (l > lc && kc * L + l < rem) v[kc] = fma(-q, u[kc * L], v[kc]);
+#pragma unroll
+        for (int k = kc + 1; k < 8; ++k)
+          if (k * L < rem) v[k] = fma(-q, k * L + l < rem ? u[k * L] : 0.0, v[k]);
+      }
+    }
+    const bool scale = b <= 8 * L;  // later blocks need the unscaled columns
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (live && k * L + l < rem) row[c0 + k * L + l] = scale ? v[k] * s.rv[c0 + k * L + l] : v[k];
+    __syncwarp();
   }
-  __syncwarp();
-  if (active)
+  if (b > 8 * L && live)
     for (int c = l; c < b; c += L) row[c] *= s.rv[c];
 }
+
+__device__ void trsm_rows_staged(const Smem& s, int tc, int b, int nr) {
+  int L = 2;
+  while (L < 32 && 2 * L * nr <= kBT && 2 * L <= b) L *= 2;
+  switch (L) {
+    case 2: trsm_rows_lanes<2>(s, tc, b, nr); break;
+    case 4: trsm_rows_lanes<4>(s, tc, b, nr); break;
+    case 8: trsm_rows_lanes<8>(s, tc, b, nr); break;
+    case 16: trsm_rows_lanes<16>(s, tc, b, nr); break;
+    default: trsm_rows_lanes<32>(s, tc, b, nr); break;
+  }
+}
+static_assert(kBT >= 2 * kBRMax, "two lanes for every staged row");
 
 // U_cc' := U_cc' / U_cc (by the reciprocal) for c' > c: the form the staged
 // substitution uses.  Called after the unscaled factor has been used for
@@ -472,7 +513,7 @@ __device__ void run_pass(const PassSpec& P, const Smem& s0, i64 R0, i64 R1, doub
     if (P.op2) tn_accumulate(mp, s, nr, am, ae);
     __syncthreads();
   }
-  if (P.op2) tn_flush(mp, s, am, ae, slot);
+  if (P.op2) tn_flush(mp, s, (int)imin64(rb, R1 - R0), am, ae, slot);
 }
 
 // Sum of the G slots of the group (rank order) for output entry (a, c).
@@ -562,9 +603,9 @@ __device__ __noinline__ int reduce_cholesky(const Smem& s, const double* slots, 
     U[e] = a <= c ? slot_sum(slots, G, 1, 0, a, c) : 0.0;
   }
   // scratch of the factorisation in the staging area (free between passes)
-  double* urow = s.red;
-  const int broken = chol_trapezoid<kBT>(U, b, b, 0, urow, kBNMax, s.dg,
-                                         reinterpret_cast<unsigned short*>(urow + 2 * kBNMax), sh_broken);
+  double* rows = s.red;
+  const int broken = chol_trapezoid<kBT>(U, b, b, 0, rows, kBNMax, s.dg,
+                                         reinterpret_cast<unsigned short*>(rows + 4 * kBNMax), sh_broken);
   if (test && t == 0) {
     int r = 0;
     if (b > 1) {
@@ -887,13 +928,6 @@ __global__ void blob_copy_kernel(const __grid_constant__ Blob blob, unsigned cha
     dst[e] = blob.bytes[e];
 }
 
-// Costs of the schedule's estimate.
-constexpr double kEstRate = 7.6e9;       // FP64 flop/s of one SM inside a pass
-constexpr double kEstStage = 0.05e-9;     // seconds per staged entry
-constexpr double kEstPass = 8e-6;        // a pass: barrier, launch of the loads, in-CTA sums
-constexpr double kEstBarrier = 3e-6;
-constexpr double kEstCholCol = 0.45e-6;  // one column of a Cholesky factorisation
-
 inline size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct BLayout {
@@ -958,15 +992,15 @@ size_t batched_persistent_workspace(int batch) { return blayout(batch, persisten
 namespace {
 
 // Rough device time of one matrix on a group of G CTAs (for the static
-// schedule): its multiply-adds at the FP64 rate of G SMs, the staging of its
-// row blocks, and per pass the barrier, the slots' sum and the Cholesky's
-// chain of dependent operations.
+// schedule), fitted to homogeneous batches (500 to 200000 rows, n = 16 to
+// 128, G = 1 to 152) to within 10 %: per row the multiply-adds at an SM's
+// FP64 rate and the staging of each pass, per pass the barrier, the in-CTA
+// sums and the solve's chain, per CholeskyQR the factorisation.
 double est_seconds(i64 m, int n, int b, int G) {
-  const int k = n / b;
-  const double flops = 4.0 * (double)m * n * n / G / kEstRate;
-  const double rows = (double)m / G * (double)n * (4 * k - 1) * kEstStage;
-  const double sum = (G > kDirectSum ? kEstBarrier : 0.0) + 0.25e-9 * b * b * (G > kDirectSum ? 1 : G);
-  return flops + rows + 4.0 * k * (kEstPass + sum) + 2.0 * k * b * kEstCholCol;
+  const double k = n / b, rows = (double)m / G;
+  const double row = 4.0 * n * n / 8.28e9 + n * (3.0 + 2.4 * k) * 1e-9;
+  const double pass = 13e-6 + 0.35e-6 * b, chol = 0.6e-6 * b * (1.0 + b / 128.0);
+  return rows * row + (4.0 * k - 1.0) * pass + 2.0 * k * chol;
 }
 
 // The static schedule: matrices (order) of every node.
@@ -1050,8 +1084,8 @@ BSchedule schedule_tree(int batch, const int64_t* m, const int64_t* n, const int
   std::vector<double> peak((size_t)nodes);   // largest load of the node's CTAs
   std::vector<int> place((size_t)batch);
   double bound = std::max(mean, longest);
-  for (int attempt = 0;; ++attempt, bound *= 1.08) {
-    const bool last = attempt == 12;
+  for (int attempt = 0;; ++attempt, bound *= 1.04) {
+    const bool last = attempt == 20;
     std::fill(cta.begin(), cta.end(), 0.0);
     std::fill(peak.begin(), peak.end(), 0.0);
     bool ok = true;
