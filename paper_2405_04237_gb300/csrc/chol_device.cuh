@@ -5,6 +5,13 @@
 
 namespace cqr {
 
+// A normal float as a double, in integer operations (a conversion takes 64
+// clocks like every FP64 instruction).
+__device__ __forceinline__ double widen(float f) {
+  const unsigned b = __float_as_uint(f);
+  return __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));  // f > 0
+}
+
 // sqrt(d) and 1/sqrt(d) of a positive normal d by Newton's iteration.  The
 // FP64 pipe of an SM takes 64 clocks for every warp instruction, also for a
 // single live lane, so the chain of FP64 operations per column is what the
@@ -37,7 +44,7 @@ __device__ __forceinline__ void sqrt_rsqrt(double d, double& u, double& r) {
   t = __fmaf_rn(-f, pl, t);
   t = __fmaf_rn(-fl, ph, t);                                      // 1 - m r0^2
   const float c = r0 * t * __fmaf_rn(0.375f, t, 0.5f);            // r0 ((1 - t)^(-1/2) - 1)
-  const double rm = (double)r0 + (double)c;
+  const double rm = widen(r0) + (double)c;
   const double hr = __hiloint2double(__double2hiint(rm) - (1 << 20), __double2loint(rm));  // rm / 2
   const double u0 = md * rm;
   const double um = fma(fma(-u0, u0, md), hr, u0);
@@ -45,21 +52,47 @@ __device__ __forceinline__ void sqrt_rsqrt(double d, double& u, double& r) {
   r = __hiloint2double(__double2hiint(rm) - (k << 20), __double2loint(rm));
 }
 
+// 1/d of a positive normal d: the FP32 reciprocal r0 of the mantissa m (24
+// bits), then r0 (1 + e + e^2) with the residual e = 1 - m r0 (third order
+// Newton: relative error e^3 < 2^-66 before rounding).
+__device__ __forceinline__ double reciprocal(double d) {
+  const int hi = __double2hiint(d), lo = __double2loint(d);
+  const int ex = (hi >> 20) - 1023;
+  if (ex == -1023 || ex > 1020) return 1.0 / d;  // subnormal d or result
+  const double m = __hiloint2double(hi - (ex << 20), lo);
+  const double r0 = widen(__frcp_rn(__uint_as_float((127u << 23) | ((unsigned)(hi & 0xFFFFF) << 3) | ((unsigned)lo >> 29))));
+  const double e = fma(-m, r0, 1.0);
+  const double r = fma(r0, fma(e, e, e), r0);
+  return __hiloint2double(__double2hiint(r) - (ex << 20), __double2loint(r));
+}
+
 // ---------------------------------------------------------------------------
 // The rows of a trapezoid in shared memory: Ws (row-major, ld) holds the
 // upper triangle of a kb x kb diagonal block and nx further columns of the
 // same rows; on return row j of both is row j of the factor (the diagonal in
-// dg).  T threads, one barrier per row.  In step j the pivot warps (32
-// columns each) apply the update of row j - 1 to row j, take the square root
-// of its diagonal (each warp for itself) and scale it, while the other warps
-// apply the update of row j - 1 to the rows below; U_jc = w / u is w r
-// corrected with the fused residual, so exact quotients stay exact.  The
+// dg).  T threads, one barrier per row.  The rows are eliminated in the
+// square-root-free form (pivots d_j, rows w_jc, multipliers l_jc = w_jc / d_j,
+// W_ac -= l_ja w_jc) and scaled by 1 / sqrt(d_j) at the end, all at once: a
+// column's chain of dependent FP64 operations is then six long instead of
+// nine.  In step j the pivot warps (32
+// columns each) apply the update of row j - 1 to row j and take the
+// reciprocal of its diagonal (each warp for itself), while the other warps
+// apply the update of row j - 1 to the rows below; at the end U_jc = w / u is
+// w r corrected with the fused residual, so exact quotients stay exact.  The
 // elements of the rows below are enumerated from the last row up (tab), so
-// the live ones are always a prefix and no lane idles.  Returns the row
-// that broke down, or -1.  Scratch in shared memory: urow (2 x us, us >= kb
+// the live ones are always a prefix and no lane idles.  While they
+// are few, the warps that share a scheduler (warp mod 4) with a pivot warp
+// leave the update to the others: their FP64 instructions, 64 clocks each,
+// would come between those of the pivot's chain.  Returns the row
+// that broke down, or -1.  Scratch in shared memory: rows (4 x us, us >= kb
 // + nx), tab (an entry per element), broken.  kb + nx <= 32 (T / 32 - 1).
+
+// Elements per scheduler up to which the update fits behind the pivot's chain
+// (about 500 clocks: 8 warp instructions of 64).
+constexpr int kQuietLen = 256;
+
 template <int T>
-__device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* urow, int us, double* dg,
+__device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* rows, int us, double* dg,
                               unsigned short* tab, int* broken) {
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   if (t == 0) *broken = -1;
@@ -71,44 +104,66 @@ __device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* urow, 
   const int np = (kb + nx - 1 + 31) / 32 > 0 ? (kb + nx - 1 + 31) / 32 : 1;
   for (int j = 0; j < kb; ++j) {
     int bad = 0;
-    const double* prev = urow + ((j + 1) & 1) * us;
-    double* cur = urow + (j & 1) * us;
+    const double *pw = rows + ((j + 1) & 1) * 2 * us, *pl = pw + us;  // row j - 1: w, l
+    double *cw = rows + (j & 1) * 2 * us, *cl = cw + us;
     if (warp < np) {
       const int c = j + 1 + 32 * warp + lane;
       double* row = Ws + j * ld;
       const bool live = c < kb + nx;
       double d = row[j], w = live ? row[c] : 0.0;
       if (j > 0) {
-        const double pj = prev[j];
-        d = fma(-pj, pj, d);
-        if (live) w = fma(-pj, prev[c], w);
+        const double lj = pl[j];
+        d = fma(-lj, pw[j], d);
+        if (live) w = fma(-lj, pw[c], w);
       }
       // d > 0 and finite, in integers (an FP64 comparison takes 64 clocks of the chain)
       const int dh = __double2hiint(d);
       if (dh < 0x7FF00000 && (dh > 0 || (dh == 0 && __double2loint(d) != 0))) {
-        double u, r;
-        sqrt_rsqrt(d, u, r);
+        const double l = w * reciprocal(d);
         if (live) {
-          const double q0 = w * r;
-          const double q = fma(fma(-q0, u, w), r, q0);
-          cur[c] = q;
-          row[c] = q;
+          cl[c] = l;
+          cw[c] = w;
+          row[c] = w;
         }
-        if (t == 0) dg[j] = u;
+        if (t == 0) dg[j] = d;
       } else {
         bad = 1;
         if (t == 0) *broken = j;
       }
     } else if (j > 0) {
       const int k = kb - 1 - j, len = k * (k + 1) / 2 + k * nx;  // rows j+1 .. kb-1
-      for (int e = t - 32 * np; e < len; e += T - 32 * np) {
-        const int i = tab[e] >> 8, c = tab[e] & 255;
-        Ws[i * ld + c] = fma(-prev[i], prev[c], Ws[i * ld + c]);
+      int w = warp - np, nw = T / 32 - np;
+      if (np < 4 && len <= kQuietLen * (4 - np)) {
+        const int q = warp & 3;
+        w = q < np ? -1 : (warp >> 2) * (4 - np) + q - np;
+        nw = (T / 128) * (4 - np);
       }
+      if (w >= 0)
+        for (int e = 32 * w + lane; e < len; e += 32 * nw) {
+          const int i = tab[e] >> 8, c = tab[e] & 255;
+          Ws[i * ld + c] = fma(-pl[i], pw[c], Ws[i * ld + c]);
+        }
     }
     if (__syncthreads_or(bad)) break;
   }
-  return *broken;
+  const int jb = *broken, done = jb >= 0 ? jb : kb;
+  double* rs = rows;  // 1 / sqrt(d_j)
+  for (int j = t; j < done; j += T) {
+    double u, r;
+    sqrt_rsqrt(dg[j], u, r);
+    dg[j] = u;
+    rs[j] = r;
+  }
+  __syncthreads();
+  for (int e = t; e < done * (kb + nx); e += T) {
+    const int j = e / (kb + nx), c = e - j * (kb + nx);
+    if (c > j) {
+      const double w = Ws[j * ld + c], r = rs[j], q = w * r;
+      Ws[j * ld + c] = fma(fma(-q, dg[j], w), r, q);
+    }
+  }
+  __syncthreads();
+  return jb;
 }
 
 }  // namespace cqr

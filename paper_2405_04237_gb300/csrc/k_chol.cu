@@ -32,7 +32,7 @@ constexpr int kTrapMax = 96;             // most columns kb + nx
 constexpr int kTrapTab = 2560;           // most elements (64 x 64: 2080; 32 x (32 + 61): 2480)
 
 struct TrapWork {
-  double urow[2 * kTrapMax];
+  double rows[4 * kTrapMax];
   double dg[kSmallChol];
   unsigned short tab[kTrapTab];
   int broken;
@@ -85,7 +85,7 @@ __device__ void chol_small(const CholArgs& a, SmallChol& s) {
       for (int j = 0; j < b; ++j) s.Ws[j * kSmallLd + j] += sh;
     }
   }
-  const int jb = chol_trapezoid<kSmallT>(s.Ws, kSmallLd, b, 0, s.w.urow, kTrapMax, s.w.dg, s.w.tab, &s.w.broken);
+  const int jb = chol_trapezoid<kSmallT>(s.Ws, kSmallLd, b, 0, s.w.rows, kTrapMax, s.w.dg, s.w.tab, &s.w.broken);
   // A breakdown of a panel wider than one column under the panel test is a
   // rejection, not a failure of the factorisation.
   if (t == 0 && jb >= 0 && a.status && !(a.reject && b > 1)) atomicCAS(a.status, 0, a.col0 + jb + 1);
@@ -238,7 +238,7 @@ __global__ void __cluster_dims__(kClu, 1, 1) __launch_bounds__(kSmallT) chol_clu
         Ws[i * kCluLd + c] = (a.shift && c == i) ? w + sh_shift : w;
       }
     }
-    jb = chol_trapezoid<kSmallT>(Ws, kCluLd, kb, nx, s.urow, kTrapMax, s.dg, s.tab, &s.broken);
+    jb = chol_trapezoid<kSmallT>(Ws, kCluLd, kb, nx, s.rows, kTrapMax, s.dg, s.tab, &s.broken);
     const int rows = jb >= 0 ? jb : kb;  // finished rows
     bool far = false;
     for (int e = t; e < rows * (kb + nx); e += kSmallT) {
