@@ -406,6 +406,18 @@ int cqr_batched_panel_widths(int batch, const void* workspace, cqr_stream_t stre
  */
 int cqr_test_arm_barrier_expiry(int group, int rank, int barrier, long long wait_ns);
 
+/*
+ * cqr_colmajor: Q := A for an m x n row-major A, the layout conversion for
+ * callers whose matrices are row-major (not in the paper).
+ *   m, n       rows and columns, >= 1                                (args 1, 2)
+ *   A, lda     DEVICE m x n FP64, row-major, row stride lda >= n      (args 3, 4)
+ *   Q, ldq     DEVICE m x n FP64, column-major, ldq >= m; must not
+ *              overlap A                                             (args 5, 6)
+ *   stream     CUDA stream the copy is ordered on                    (arg 7)
+ * Returns 0, -i for argument i, or CQR_ERR_CUDA.
+ */
+int cqr_colmajor(int64_t m, int64_t n, const double* A, int64_t lda, double* Q, int64_t ldq, cqr_stream_t stream);
+
 /* cqr_status_string: static description of a status or return code. */
 const char* cqr_status_string(int status);
 

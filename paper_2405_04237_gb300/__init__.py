@@ -46,6 +46,35 @@ def colmajor(A: torch.Tensor) -> torch.Tensor:
     return A.t().contiguous().t()
 
 
+def _packed(A: torch.Tensor) -> torch.Tensor:
+    """colmajor() for the library's own use (only the data matter): a plain
+    row-major matrix is copied by the library's kernel."""
+    if A.dim() == 2 and A.stride(0) != 1 and _native_rowmajor(A):
+        out = empty_colmajor(A.shape[0], A.shape[1], A.device)
+        _copy_rowmajor(A, out, _stream())
+        return out
+    return colmajor(A)
+
+
+def _native_rowmajor(A: torch.Tensor) -> bool:
+    """Whether cqr_colmajor takes A: a plain row-major CUDA FP64 matrix on the
+    current device with nothing recorded on it (autograd, function transforms)."""
+    if type(A) not in (torch.Tensor, torch.nn.Parameter) or not A.is_cuda or A.dtype != torch.float64:
+        return False
+    if torch._C._functorch.is_functorch_wrapped_tensor(A) or A.is_neg():
+        return False
+    m, n = A.shape
+    return (m > 0 and n > 0 and A.stride(1) == 1 and A.stride(0) >= n
+            and A.device.index == torch.cuda.current_device()
+            and not (A.requires_grad and torch.is_grad_enabled()))
+
+
+def _copy_rowmajor(A: torch.Tensor, out: torch.Tensor, st) -> None:
+    rc = load().cqr_colmajor(A.shape[0], A.shape[1], _ptr(A), A.stride(0), _ptr(out), _ld(out), st)
+    if rc != 0:
+        raise CQRError(rc, "cqr_colmajor")
+
+
 def empty_colmajor(m: int, n: int, device, dtype=torch.float64) -> torch.Tensor:
     return torch.empty((n, m), dtype=dtype, device=device).t()
 
@@ -181,7 +210,10 @@ def factor(A: torch.Tensor, panel_b: int = 0, variant="mcqr2gs", *, inplace: boo
     L = load()
     m, n = A.shape
     var = _variant(variant)
-    Ac = colmajor(A)
+    # a row-major A goes straight into the new Q, which is then factored in place
+    direct = (out is None and not inplace and (stream is None or stream == torch.cuda.current_stream())
+              and not (A.stride(0) == 1 and (n <= 1 or A.stride(1) >= m)) and _native_rowmajor(A))
+    Ac = A if direct else _packed(A)
     if inplace and Ac.data_ptr() != A.data_ptr():
         raise ValueError("inplace=True needs a column-major A")
     if out is not None:
@@ -199,6 +231,9 @@ def factor(A: torch.Tensor, panel_b: int = 0, variant="mcqr2gs", *, inplace: boo
     elif workspace.numel() < ws_bytes:
         raise ValueError(f"workspace too small: {workspace.numel()} < {ws_bytes}")
     st = _stream(stream)
+    if direct:
+        _copy_rowmajor(A, Q, st)
+        Ac = Q
     rc = L.cqr_factor(m, n, _ptr(Ac), _ld(Ac), int(panel_b), _ptr(Q), _ld(Q), _ptr(R), _ld(R), flags,
                       _ptr(workspace), ctypes.c_size_t(workspace.numel()), st)
     if rc != 0:
@@ -285,9 +320,9 @@ def backward(Q: torch.Tensor, R: torch.Tensor, dQ: torch.Tensor | None, dR: torc
         raise ValueError("backward: Q (m x n), R (n x n), dQ like Q, dR like R")
     L = load()
     m, n = Q.shape
-    Qc, Rc = colmajor(Q), colmajor(R)
-    dQc = colmajor(dQ) if dQ is not None else None
-    dRc = colmajor(dR) if dR is not None else None
+    Qc, Rc = _packed(Q), _packed(R)
+    dQc = _packed(dQ) if dQ is not None else None
+    dRc = _packed(dR) if dR is not None else None
     dA = empty_colmajor(m, n, Q.device)
     ws_bytes = L.cqr_backward_workspace_size(m, n)
     ws = torch.empty(max(ws_bytes, 1), dtype=torch.uint8, device=Q.device)
@@ -339,7 +374,7 @@ def factor_batched(As, panel_b=None, variant="mcqr2gs", *, check: bool = True, s
         return []
     var = _variant(variant)
     dev = As[0].device
-    Acs = [colmajor(A) for A in As]
+    Acs = [_packed(A) for A in As]
     for A in Acs:
         _check_input(A)
     if inplace and any(Ac.data_ptr() != A.data_ptr() for Ac, A in zip(Acs, As)):

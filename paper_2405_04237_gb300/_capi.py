@@ -37,7 +37,7 @@ NOALLOC_SCRATCH_BYTES = 64 << 20
 
 EXPORTS = [
     "cqr_workspace_size", "cqr_default_panel", "cqr_factor", "cqr_read_status", "cqr_read_panel_width", "cqr_set_allocator",
-    "cqr_backward_workspace_size", "cqr_backward", "cqr_batched_workspace_size",
+    "cqr_backward_workspace_size", "cqr_backward", "cqr_colmajor", "cqr_batched_workspace_size",
     "cqr_factor_batched", "cqr_status_string", "cqr_probe_fp64_peak", "cqr_probe_fp64",
     "cqr_factor_noalloc", "cqr_factor_host", "cqr_test_arm_wait_expiry", "cqr_test_arm_barrier_expiry", "cqr_batched_panel_widths", "cqr_launch_count", "cqr_set_trace", "cqr_profile_enable", "cqr_profile_disable", "cqr_profile_read", "cqr_kernel_class_name",
 ]
@@ -84,6 +84,7 @@ def load(build_if_missing: bool = True):
             "cqr_factor_host": (c_int, [i64, i64, dp, i64, c_int, dp, i64, dp, i64, c_int, dp, i64, dp, i64, vp, sz, vp]),
             "cqr_backward_workspace_size": (sz, [i64, i64]),
             "cqr_backward": (c_int, [i64, i64, dp, i64, dp, i64, dp, i64, dp, i64, dp, i64, vp, sz, vp]),
+            "cqr_colmajor": (c_int, [i64, i64, dp, i64, dp, i64, vp]),
             "cqr_batched_workspace_size": (sz, [c_int, P64, P64, PI, c_int]),
             "cqr_factor_batched": (c_int, [c_int, P64, P64, P64, PI, PV, PV, PV, c_int, vp, vp, sz, vp]),
             "cqr_status_string": (ctypes.c_char_p, [c_int]),

@@ -227,6 +227,10 @@ cudaError_t batched_persistent_run(int batch, const int64_t* m, const int64_t* n
                                    int* status, void* workspace, int G, bool halve, cudaStream_t st);
 cudaError_t batched_persistent_panels(int batch, const void* workspace, int* host_b, cudaStream_t st);
 
+// Q (m x n, column-major, ldq) := A (row-major, lda) (k_transpose.cu).
+cudaError_t colmajor_copy(i64 m, i64 n, const double* A, i64 lda, double* Q, i64 ldq, cudaStream_t st);
+
+// ---------------------------------------------------------------------------
 // Launch accounting (prof.cu).  Every launch is wrapped in prof_begin /
 // prof_end with its kernel class and algorithmic FLOP count.
 enum KernelClass {
@@ -236,7 +240,7 @@ enum KernelClass {
   kCholesky = 3,
   kTrsm = 4,
   kUpdate = 5,     // C = beta C + alpha A B (GS / re-orthogonalisation updates, R products)
-  kMisc = 6,       // adjoint helpers, probes, digit splitting of the emulated products
+  kMisc = 6,       // adjoint helpers, layout copies, probes, digit splitting of the emulated products
   kBatched = 7,
   kNumClasses = 8
 };
