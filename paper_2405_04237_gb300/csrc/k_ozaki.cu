@@ -12,11 +12,14 @@
 // the top digit).  An integer of magnitude up to 16 is exact in e4m3: the
 // code is the sign and |d|, read as |d| 2^-9 (e4m3's subnormals and the two
 // binades above them are evenly spaced), so no table is needed and every
-// product carries a factor 2^-18.  Balanced digits need 11 planes and 66
+// product carries a factor 2^-18.  Balanced digits need 11 planes and 76
 // plane pairs where sign-magnitude nibbles needed 14 and 105, and the pairs
-// left out have no common sign: the error against exact sums is that of the
-// nibbles for X^T Y and 30 to 80 times smaller for the diagonal of X^T X,
-// whose neglected nibble products were all positive.  For
+// left out have no common sign: the error against exact sums (rms, in units
+// of 2^-53 |x| |y|) is 0.02 to 0.1 at K = 4096 to 64 where the nibbles' was
+// 0.1 to 0.8, and 0.13 for the diagonal of X^T X where it was 16 (their
+// neglected products were all positive).  With 66 pairs (levels from 10) it
+// is 0.1 to 0.5, and a factorisation of 60013 x 360 was 12 % further from
+// the exact Q than with the nibbles.  For
 // C -= X Y the contraction runs over the columns of X: each row of X gets its
 // own scale over (at most kSub of) its entries and takes a column's place;
 // Y (K x N) is split by columns.
@@ -33,27 +36,26 @@
 // and one per plane for Y).
 //
 // Products.  x_a y_b = 2^(e_a + e_b - 108) sum_{i,j} d^x_i d^y_j 32^(i+j).
-// The 66 plane pairs with i + j >= 10 (the 11 most significant weight
+// The 76 plane pairs with i + j >= 9 (the 12 most significant weight
 // levels) are multiplied with tcgen05.mma kind::f8f6f4 (e4m3 x e4m3 -> f32)
-// into one TMEM accumulator per level: TMEM region r (32 columns, r = 0..10)
-// holds level r + 10.  The Y planes of one stage lie in shared memory one
+// into one TMEM accumulator per level: TMEM region r (32 columns, r = 0..11)
+// holds level r + 9.  The Y planes of one stage lie in shared memory one
 // after the other, so planes j0 .. j0+n-1 form one operand of N = 32 n rows,
 // and one instruction A_i x [Y_j0; ...; Y_j0+n-1] (128 x 32n x 32) adds pair
-// (i, j0 + v) into region i + j0 + v - 10 for v < n.  14 such instructions
-// (N = 32 .. 256) cover the 66 pairs.  Per level the sum over at most 4096
+// (i, j0 + v) into region i + j0 + v - 9 for v < n.  16 such instructions
+// (N = 32 .. 256) cover the 76 pairs.  Per level the sum over at most 4096
 // contraction indices is below 11 * 256 * 4096 < 2^24 in magnitude, so the
 // FP32 accumulation is exact (an integer times 2^-18).  The dropped levels
-// weigh at most about 2^-51.6 of the scales' product per index, with signs
-// that cancel (rms 2^-55).
+// weigh at most about 2^-56.6 of the scales' product per index.
 //
 // Schedule.  A block of 4 warps computes a 128 x 32 tile of C over its
 // contraction range (a sub-chunk of a projection, all of K for an update).
 // Four shared-memory stages of 55 KiB rotate: one thread issues the bulk
 // copies of a stage (completion counted in bytes on the stage's "full"
-// mbarrier), one thread issues its 14 MMAs and commits them to the stage's
+// mbarrier), one thread issues its 16 MMAs and commits them to the stage's
 // "empty" mbarrier, which frees the stage for the copy four stages later.
-// At the end every thread reads the 11 level sums of its row from TMEM,
-// combines levels 10..15 and 16..20 exactly in 64-bit integers (below 2^50),
+// At the end every thread reads the 12 level sums of its row from TMEM,
+// combines levels 9..14 and 15..20 exactly in 64-bit integers (below 2^50),
 // builds the two scaled doubles with integer operations and adds them (one
 // rounding), so the FP64 pipe does one operation per element (two for an
 // update, which subtracts the tile from C).  Every wait is bounded in time
@@ -74,7 +76,7 @@ namespace {
 
 constexpr int kSub = 4096;          // rows per sub-chunk (exact FP32 level sums)
 constexpr int kPlanes = 11;         // balanced base-32 digits of a 54-bit magnitude and its sign
-constexpr int kLevelLo = 10;        // lowest weight level i + j kept
+constexpr int kLevelLo = 9;         // lowest weight level i + j kept
 constexpr int kLevels = 2 * kPlanes - 1 - kLevelLo;
 constexpr int kLowLevels = 6;       // levels of the low 64-bit group; the others form the high one
 constexpr int kStage = 32;          // contraction indices per stage (one MMA K step for 8-bit types)
@@ -84,20 +86,20 @@ constexpr int kExpBad = 100000;     // a column holding Inf or NaN
 
 constexpr int kTcM = 128;           // rows of the tile (X side, TMEM lanes)
 constexpr int kTcN = 32;            // columns of the tile (Y side)
-constexpr int kTcThreads = 128;
+constexpr int kTcThreads = 512;     // warp 0 copies, warp 1 issues, all 16 run the epilogue
 constexpr int kTcRing = 4;
 constexpr int kTcABytes = kPlanes * kTcM * kStage;    // 45056
 constexpr int kTcBBytes = kPlanes * kTcN * kStage;    // 11264
 constexpr int kTcStageBytes = kTcABytes + kTcBBytes;  // 56320
 constexpr int kTcSmem = kTcRing * kTcStageBytes + 1024;  // + alignment slack
-constexpr uint32_t kTcCols = 512;   // TMEM columns: the levels' regions (352), rounded up to a power of 2
+constexpr uint32_t kTcCols = 512;   // TMEM columns: the levels' regions (384), rounded up to a power of 2
 constexpr int kMaxDynSmem = 227 * 1024 - 1024;  // opt-in dynamic shared memory per block, less static use
 static_assert(kTcSmem <= kMaxDynSmem, "projection ring fits in shared memory");
 static_assert(kTcCols >= 32 && kTcCols <= 512 && (kTcCols & (kTcCols - 1)) == 0, "TMEM allocation: power of 2, 32..512");
 constexpr int kRegionLo = kLevelLo;  // level of TMEM region 0
 static_assert(kLevels * kTcN <= (int)kTcCols, "level regions fit in the TMEM allocation");
-static_assert(kLevelLo == 10 && kLevels == 11, "the MMA schedule and the groups of six and five levels");
-static_assert((long long)kLevels * 256 * kSub < (1 << 24), "exact FP32 level sums");
+static_assert(kLevelLo == 9 && kLevels == 2 * kLowLevels, "the MMA schedule and the groups of six levels");
+static_assert((long long)kPlanes * 256 * kSub < (1 << 24), "exact FP32 level sums");
 // Instruction descriptor of tcgen05.mma kind::f8f6f4 without N: D f32 (bits
 // 4-5 = 1), A and B e4m3 (bits 7-9, 10-12 = 0), both K-major (bits 15, 16 =
 // 0), M >> 4 at bits 24-28; N >> 3 goes to bits 17-22.
@@ -182,110 +184,95 @@ __device__ __forceinline__ i64 plane_off(i64 col, int half) {
 // planes.  Grid (ceil(c / 8), nsub), 256 threads: block (g, s) takes the
 // 8-column group g of the layout (columns 8g .. 8g+7) over sub-chunk s, so
 // that for each stage and plane its digits form one contiguous 256-byte run
-// (8 columns x 32 indices).  Lane l of warp w handles column 8g + (l & 7),
-// half (l >> 3) & 1 (indices 0..15 or 16..31 of a stage) of stages
-// 16 it + 2 w + (l >> 4), it = 0..7 (only those below nst, rounded up to 16,
-// for the short Y of an update): every warp store writes two whole
-// 256-byte runs.  Two passes over the sub-chunk: the column maxima (scales),
-// then the digits; the second pass re-reads from L2 (at most two blocks, 2 x
-// 256 KiB, per SM).  Tiles of T columns (T a multiple of 8); plane block
+// (8 columns x 32 indices).  Warp w takes stages 8 it + w, it = 0..15 (only
+// those below nst, for the short Y of an update); lane l handles rows 4 (l mod
+// 4) .. + 3 of both halves of the stage in column 8g + l / 4.  A warp load
+// thus touches 8 lines and a warp store writes 128 consecutive bytes of a run
+// (with 16 rows a lane, four columns' worth of lines per load, the kernel was
+// bound by the L1's line rate: 3.6 TB/s).  Two passes over the sub-chunk: the
+// column maxima (scales), then the digits; the second pass re-reads from L2.
+// Tiles of T columns (T a multiple of 8); plane block
 // (s, tile, st, i) starts at byte
 // (((s * ntile + tile) * kStagesPerSub + st) * kPlanes + i) * T * 32 with
 // ntile = ceil(c / T); exps: [s * c + col].  Columns past c of the last
 // group are written as zero digits (the tile padding; never read).
-// 16 consecutive entries xc[row .. row+15] (zero past m or for a column past
+constexpr int kSplitWarps = 8;
+
+// 4 consecutive entries xc[row .. row+3] (zero past m or for a column past
 // c); 16-byte loads when the address allows (an odd leading dimension puts
 // every other column off the 16-byte grid).
-__device__ __forceinline__ void load16(const double* xc, i64 row, i64 m, bool colok, unsigned long long (&bits)[16]) {
-  if (colok && row + 15 < m && ((reinterpret_cast<uintptr_t>(xc + row) & 15) == 0)) {
+__device__ __forceinline__ void load4(const double* xc, i64 row, i64 m, bool colok, unsigned long long (&bits)[4]) {
+  if (colok && row + 3 < m && ((reinterpret_cast<uintptr_t>(xc + row) & 15) == 0)) {
     const double2* p = reinterpret_cast<const double2*>(xc + row);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
+    for (int k = 0; k < 2; ++k) {
       const double2 v = __ldg(p + k);
       bits[2 * k] = (unsigned long long)__double_as_longlong(v.x);
       bits[2 * k + 1] = (unsigned long long)__double_as_longlong(v.y);
     }
   } else {
 #pragma unroll
-    for (int k = 0; k < 16; ++k)
+    for (int k = 0; k < 4; ++k)
       bits[k] = (unsigned long long)__double_as_longlong((colok && row + k < m) ? xc[row + k] : 0.0);
   }
 }
 
-__global__ void __launch_bounds__(256, 2) ozaki_split_kernel(const double* X, i64 ldx, i64 m, i64 r0, int c, int T,
-                                                             int nst, uint8_t* planes, int* exps, const int* status) {
+__global__ void __launch_bounds__(32 * kSplitWarps, 4) ozaki_split_kernel(const double* X, i64 ldx, i64 m, i64 r0,
+                                                                          int c, int T, int nst, uint8_t* planes,
+                                                                          int* exps, const int* status) {
   stream_wait();
   if (status && *status) return;
   const int g = blockIdx.x, s = blockIdx.y, t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int cl = lane & 7, half = (lane >> 3) & 1, so = lane >> 4;
+  const int cl = lane >> 2, quad = lane & 3;
   const int col = 8 * g + cl;
   const bool colok = col < c;
-  const i64 base = r0 + (i64)s * kSub;
-  const int iters = (nst + 15) / 16;
+  const i64 base = r0 + (i64)s * kSub + 4 * quad;
   const double* xc = X + (i64)(colok ? col : 0) * ldx;
   // pass 1: the column's largest exponent (zeros and subnormals do not set the scale) and Inf/NaN
-  int emax = -2000;
-  bool bad = false;
-#pragma unroll 1
-  for (int it = 0; it < iters; ++it) {
-    const int st = 16 * it + 2 * warp + so;
-    unsigned long long bits[16];
-    load16(xc, base + st * kStage + 16 * half, m, colok, bits);
+  int emax = 0;
+#pragma unroll 2
+  for (int st = warp; st < nst; st += kSplitWarps) {
+    unsigned long long b0[4], b1[4];
+    load4(xc, base + st * kStage, m, colok, b0);
+    load4(xc, base + st * kStage + 16, m, colok, b1);
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const int E = (int)((bits[k] >> 52) & 0x7FF);
-      if (E == 0x7FF) bad = true;
-      if (E != 0 && E > emax) emax = E;
-    }
+    for (int k = 0; k < 4; ++k)
+      emax = max(emax, max((int)(b0[k] >> 52) & 0x7FF, (int)(b1[k] >> 52) & 0x7FF));
   }
-  // lanes l, l ^ 8, l ^ 16, l ^ 24 hold the same column
-  emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 8));
-  emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 16));
-  int anyb = bad ? 1 : 0;
-  anyb |= __shfl_xor_sync(0xffffffffu, anyb, 8);
-  anyb |= __shfl_xor_sync(0xffffffffu, anyb, 16);
-  __shared__ int red_max[8][8], red_bad[8][8];
+  // lanes l, l ^ 1, l ^ 2, l ^ 3 hold the same column
+  emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 1));
+  emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 2));
+  __shared__ int red_max[kSplitWarps][8];
   __shared__ int e_col[8];
-  if (lane < 8) {
-    red_max[warp][lane] = emax;
-    red_bad[warp][lane] = anyb;
-  }
+  if (quad == 0) red_max[warp][cl] = emax;
   __syncthreads();
   if (t < 8) {
-    int E_max = -2000, B = 0;
-    for (int w = 0; w < 8; ++w) {
-      E_max = max(E_max, red_max[w][t]);
-      B |= red_bad[w][t];
-    }
-    // |x| < 2^(E - 1022) for biased exponent E; scale e with |x| < 2^e: e = E_max - 1022
-    const int e = B ? kExpBad : (E_max < 0 ? kExpZero : E_max - 1022);
+    int E = 0;
+    for (int w = 0; w < kSplitWarps; ++w) E = max(E, red_max[w][t]);
+    // |x| < 2^(E - 1022) for biased exponent E; scale e with |x| < 2^e: e = E - 1022
+    const int e = E == 0x7FF ? kExpBad : (E == 0 ? kExpZero : E - 1022);
     e_col[t] = e;
     if (8 * g + t < c) exps[(i64)s * c + 8 * g + t] = e;
   }
   __syncthreads();
   const int e = e_col[cl];
-  // pass 2: digits, one 16-byte granule per plane
+  // pass 2: digits, 4 bytes per plane and half
   const int ntile = (c + T - 1) / T;
-  uint8_t* dst0 = planes + ((i64)s * ntile + col / T) * kStagesPerSub * kPlanes * T * kStage + plane_off(col % T, half);
+  uint8_t* dst0 = planes + ((i64)s * ntile + col / T) * kStagesPerSub * kPlanes * T * kStage + plane_off(col % T, 0) +
+                  4 * quad;
 #pragma unroll 1
-  for (int it = 0; it < iters; ++it) {
-    const int st = 16 * it + 2 * warp + so;
-    unsigned long long bits[16];
-    load16(xc, base + st * kStage + 16 * half, m, colok, bits);
-    uint32_t words[kPlanes][4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const unsigned long long b4[4] = {bits[4 * q], bits[4 * q + 1], bits[4 * q + 2], bits[4 * q + 3]};
-      uint32_t w[kPlanes];
-      digits4(b4, e, w);
-#pragma unroll
-      for (int i = 0; i < kPlanes; ++i) words[i][q] = w[i];
-    }
+  for (int st = warp; st < nst; st += kSplitWarps) {
+    unsigned long long b0[4], b1[4];
+    load4(xc, base + st * kStage, m, colok, b0);
+    load4(xc, base + st * kStage + 16, m, colok, b1);
+    uint32_t w0[kPlanes], w1[kPlanes];
+    digits4(b0, e, w0);
+    digits4(b1, e, w1);
     uint8_t* dst = dst0 + (i64)st * kPlanes * T * kStage;
 #pragma unroll
     for (int i = 0; i < kPlanes; ++i) {
-      uint4 v = make_uint4(words[i][0], words[i][1], words[i][2], words[i][3]);
-      *reinterpret_cast<uint4*>(dst + (i64)i * T * kStage) = v;
+      *reinterpret_cast<uint32_t*>(dst + (i64)i * T * kStage) = w0[i];
+      *reinterpret_cast<uint32_t*>(dst + (i64)i * T * kStage + 128) = w1[i];
     }
   }
 }
@@ -404,7 +391,7 @@ __device__ __forceinline__ void tc_mma(uint32_t d, uint64_t ad, uint64_t bd, int
 }
 
 // The MMA schedule of one stage: (plane i of X, first plane j0 of Y, count n).
-// The first two write every region (levels 10..20) without overlap, so in the
+// The first three write every region (levels 9..20) without overlap, so in the
 // first stage of a tile they run with acc = 0 and initialise the accumulators.
 // An instruction reads 4 KiB of X and n KiB of Y from shared memory (128 B per
 // clock) for 16 n clocks of arithmetic, so the splits are even: 5 + 4 rather
@@ -412,16 +399,16 @@ __device__ __forceinline__ void tc_mma(uint32_t d, uint64_t ad, uint64_t bd, int
 struct TcMma {
   int i, j0, n;
 };
-constexpr int kTcMmas = 14;
-#define CQR_TC_SCHEDULE                                                  \
-  {10, 0, 6}, {10, 6, 5},                       /* i = 10: every level */ \
-      {9, 1, 5}, {9, 6, 5}, {8, 2, 5}, {8, 7, 4}, /* j >= 10 - i */       \
-      {7, 3, 8}, {6, 4, 7}, {5, 5, 6}, {4, 6, 5}, {3, 7, 4}, {2, 8, 3}, {1, 9, 2}, {0, 10, 1}
+constexpr int kTcMmas = 16, kTcInit = 3;
+#define CQR_TC_SCHEDULE                                                                \
+  {10, 0, 6}, {10, 6, 5}, {9, 0, 1},                              /* every level once */ \
+      {9, 1, 5}, {9, 6, 5}, {8, 1, 5}, {8, 6, 5}, {7, 2, 5}, {7, 7, 4}, /* j >= 9 - i */  \
+      {6, 3, 8}, {5, 4, 7}, {4, 5, 6}, {3, 6, 5}, {2, 7, 4}, {1, 8, 3}, {0, 9, 2}
 __device__ constexpr TcMma kTcSchedule[kTcMmas] = {CQR_TC_SCHEDULE};
 
 // Compile-time check of the same entries: every digit pair (i, j) of a kept
 // level exactly once and no other, every instruction within the planes,
-// N = 32 n <= 256, every region in TMEM, and the first two instructions
+// N = 32 n <= 256, every region in TMEM, and the first kTcInit instructions
 // writing each region exactly once (they run with the accumulate flag off).
 constexpr TcMma kTcScheduleCheck[kTcMmas] = {CQR_TC_SCHEDULE};
 constexpr bool tc_schedule_ok() {
@@ -434,7 +421,7 @@ constexpr bool tc_schedule_ok() {
       const int j = e.j0 + v, region = e.i + j - kRegionLo;
       if (region < 0 || region >= kLevels) return false;
       ++count[e.i][j];
-      if (u < 2) ++first[region];
+      if (u < kTcInit) ++first[region];
     }
   }
   for (int i = 0; i < kPlanes; ++i)
@@ -444,17 +431,17 @@ constexpr bool tc_schedule_ok() {
     if (first[r] != 1) return false;
   return true;
 }
-static_assert(tc_schedule_ok(), "MMA schedule: kept pairs once, regions in range, first two initialise the regions");
+static_assert(tc_schedule_ok(), "MMA schedule: kept pairs once, regions in range, the first ones initialise the regions");
 #undef CQR_TC_SCHEDULE
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// 8 consecutive 32-bit TMEM columns of this thread's lane
-__device__ __forceinline__ void tc_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+// 4 consecutive 32-bit TMEM columns of this thread's lane
+__device__ __forceinline__ void tc_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(taddr));
 }
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
@@ -477,14 +464,19 @@ __device__ __forceinline__ double scaled_int(long long g, int e) {
 // exactly as bits(f + 48) - bits(48), one full-rate FP32 add and integer
 // arithmetic, instead of a quarter-rate conversion.
 constexpr int kMagicMaxK = 1312;
-static_assert(kLevels * 256 * kMagicMaxK < (1 << 22), "level sums below 2^22");
+static_assert(kPlanes * 256 * kMagicMaxK < (1 << 22), "level sums below 2^22");
 constexpr float kMagicF = 48.0f;        // 1.5 * 2^5: steps of 2^-18
 constexpr int kMagicBits = 0x42400000;  // its encoding
 
-// The level sums of columns c0 .. c0+7 of this thread's TMEM lane.
-__device__ __forceinline__ void load_levels(uint32_t lane_base, int c0, uint32_t (&v)[kLevels][8]) {
+// Columns of the epilogue's register step; warps that read one TMEM lane
+// quarter (each takes kEpiCols columns of the tile), of 16 epilogue warps.
+constexpr int kEpiStep = 4, kEpiCols = 8;
+constexpr int kEpiWarps = 4 * (kTcN / kEpiCols);
+
+// The level sums of columns c0 .. c0+3 of this thread's TMEM lane.
+__device__ __forceinline__ void load_levels(uint32_t lane_base, int c0, uint32_t (&v)[kLevels][kEpiStep]) {
 #pragma unroll
-  for (int l = 0; l < kLevels; ++l) tc_ld8(lane_base + (uint32_t)((kLevelLo - kRegionLo + l) * kTcN + c0), v[l]);
+  for (int l = 0; l < kLevels; ++l) tc_ld4(lane_base + (uint32_t)((kLevelLo - kRegionLo + l) * kTcN + c0), v[l]);
   tc_wait_ld();
 }
 
@@ -493,7 +485,7 @@ __device__ __forceinline__ void load_levels(uint32_t lane_base, int c0, uint32_t
 // combine in unsigned 32-bit arithmetic (the offsets cancel modulo 2^32 and
 // |s_l + 32 s_l+1| < 2^28, so the two's-complement reading is the value).
 template <bool kMagic>
-__device__ __forceinline__ void group_sums(const uint32_t (&v)[kLevels][8], int j, long long& g0, long long& g1) {
+__device__ __forceinline__ void group_sums(const uint32_t (&v)[kLevels][kEpiStep], int j, long long& g0, long long& g1) {
   if (kMagic) {
     uint32_t b[kLevels];
 #pragma unroll
@@ -501,7 +493,7 @@ __device__ __forceinline__ void group_sums(const uint32_t (&v)[kLevels][8], int 
     const uint32_t off = 33u * (uint32_t)kMagicBits;  // modulo 2^32
     auto two = [&](int l) { return (long long)(int)(b[l] + 32u * b[l + 1] - off); };
     g0 = two(0) + (two(2) << 10) + (two(4) << 20);
-    g1 = two(6) + (two(8) << 10) + ((long long)(int)(b[10] - (uint32_t)kMagicBits) << 20);
+    g1 = two(6) + (two(8) << 10) + (two(10) << 20);
   } else {
     auto lev = [&](int l) { return (long long)__float2int_rz(__uint_as_float(v[l][j]) * 262144.0f); };
     g0 = g1 = 0;
@@ -512,7 +504,7 @@ __device__ __forceinline__ void group_sums(const uint32_t (&v)[kLevels][8], int 
   }
 }
 
-// sum_L S_L 32^L = 32^10 (g0 + 2^30 g1), times 2^(ex + ey - 108); one rounding
+// sum_L S_L 32^L = 32^9 (g0 + 2^30 g1), times 2^(ex + ey - 108); one rounding
 __device__ __forceinline__ double group_value(long long g0, long long g1, int exy) {
   const int e2 = exy - 108 + 5 * kLevelLo;
   return scaled_int(g1, e2 + 5 * kLowLevels) + scaled_int(g0, e2);
@@ -553,7 +545,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) ozaki_tc_kernel(OzArgs a) {
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tc_raw) + 1023) & ~(uintptr_t)1023);
   // scales of the epilogue, fetched first so that their latency hides behind the contraction
   __shared__ int ey_s[kTcN];
-  const int r = 32 * warp + lane;  // tile row = TMEM lane
+  const int r = 32 * (warp & 3) + lane;  // tile row = TMEM lane
   const int pr = p0 + r;
   const bool live = pr < a.p;
   const int exr = live ? a.ex[(i64)s * a.p + pr] : kExpZero;
@@ -611,7 +603,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) ozaki_tc_kernel(OzArgs a) {
     for (int st = issued - kTcRing < 0 ? 0 : issued - kTcRing; st < issued; ++st)
       mbar_wait(smem_u32(&full_bar[st % kTcRing]), (uint32_t)((st / kTcRing) & 1), a.wait_ns);
   } else if (warp == 1 && lane == 0) {
-    // MMA issuer: the 14 instructions of each stage (the 66 pairs, level L = i + j into region L - 10)
+    // MMA issuer: the 16 instructions of each stage (the 76 pairs, level L = i + j into region L - 9)
     for (int st = 0; st < nst; ++st) {
       const int slot = st % kTcRing;
       if (!mbar_wait(smem_u32(&full_bar[slot]), (uint32_t)((st / kTcRing) & 1), a.wait_ns)) {
@@ -627,7 +619,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) ozaki_tc_kernel(OzArgs a) {
         const TcMma e = kTcSchedule[u];
         const uint64_t ad = ad0 + (uint64_t)((e.i * kTcM * kStage) >> 4);
         const uint64_t bd = bd0 + (uint64_t)((e.j0 * kTcN * kStage) >> 4);
-        tc_mma(tmem + (uint32_t)((e.i + e.j0 - kRegionLo) * kTcN), ad, bd, e.n, (st > 0 || u >= 2) ? 1u : 0u);
+        tc_mma(tmem + (uint32_t)((e.i + e.j0 - kRegionLo) * kTcN), ad, bd, e.n, (st > 0 || u >= kTcInit) ? 1u : 0u);
       }
       tc_commit(smem_u32(&empty_bar[slot]));
     }
@@ -641,29 +633,29 @@ __global__ void __launch_bounds__(kTcThreads, 1) ozaki_tc_kernel(OzArgs a) {
   if (failed) {
     if (t == 0 && a.status) atomicCAS(a.status, 0, CQR_STATUS_TIMEOUT);
   } else {
-    // epilogue: row r of the tile (TMEM lane r), 8 columns at a time
-    const uint32_t lane_base = tmem + ((uint32_t)(32 * warp) << 16);
+    // epilogue: row r of the tile (TMEM lane r), this warp's columns
+    const uint32_t lane_base = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+    const int cw = kEpiCols * (warp >> 2);
 #pragma unroll
-    for (int c0 = 0; c0 < kTcN; c0 += 8) {
-      long long g[2][8];
-      uint32_t v[kLevels][8];
+    for (int c0 = cw; c0 < cw + kEpiCols; c0 += kEpiStep) {
+      uint32_t v[kLevels][kEpiStep];
       load_levels(lane_base, c0, v);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) group_sums<false>(v, j, g[0][j], g[1][j]);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
+      for (int j = 0; j < kEpiStep; ++j) {
         const int qc = q0 + c0 + j;
         if (!live || qc >= a.q) continue;
         const int eyc = ey_s[c0 + j];
-        double v;
+        double x;
         if (exr == kExpBad || eyc == kExpBad) {
-          v = __longlong_as_double(0x7ff8000000000000LL);
+          x = __longlong_as_double(0x7ff8000000000000LL);
         } else if (exr == kExpZero || eyc == kExpZero) {
-          v = 0.0;
+          x = 0.0;
         } else {
-          v = group_value(g[0][j], g[1][j], exr + eyc);
+          long long g0, g1;
+          group_sums<false>(v, j, g0, g1);
+          x = group_value(g0, g1, exr + eyc);
         }
-        a.part[(i64)(a.s_off + s) * a.p * a.q + pr + (i64)qc * a.p] = v;
+        a.part[(i64)(a.s_off + s) * a.p * a.q + pr + (i64)qc * a.p] = x;
       }
     }
   }
@@ -677,11 +669,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) ozaki_tc_kernel(OzArgs a) {
 // the stages of the block's tiles into two rings of four slots, one for X (44
 // KiB each) and one for Y (11 KiB each), warp
 // 1 issues the MMAs of a tile into the one set of TMEM level regions, and
-// warps 2-5 (TMEM lane quarters 2, 3, 0, 1) run the epilogue in two phases:
+// warps 2-17 (TMEM lane quarter warp mod 4, eight columns each) run the
+// epilogue in two phases:
 // first the level sums become the exact 64-bit group sums, kept in registers
 // (two per column of the thread's row), and the regions are handed back to
 // warp 1 at once; then, while the next tile's MMAs run, the group sums are
-// scaled, added and subtracted from C.
+// scaled, added and subtracted from C, whose entries were fetched before the
+// wait for the MMAs.  The epilogue is about 120 instructions per entry, long
+// chains of integer operations: with one warp per lane quarter (one per
+// scheduler) it took 27000 clocks a tile, five times the MMAs.
 //
 // Tile T is row tile T / tiles_q, column tile T % tiles_q.  The kernel is
 // bound by how fast stages reach shared memory, and X is four fifths of a
@@ -692,10 +688,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) ozaki_tc_kernel(OzArgs a) {
 // c + G, c + 2G, ... (G = grid size), so that the blocks running together
 // share row tiles in L2.
 constexpr int kUpRing = 4;
-constexpr int kUpThreads = 192;
+constexpr int kUpThreads = 64 + 32 * kEpiWarps;
 constexpr int kUpSmem = 1024 + kUpRing * kTcStageBytes;  // X slots, then Y slots
 static_assert(kUpSmem <= kMaxDynSmem, "update ring fits in shared memory");
-static_assert(kUpThreads == 6 * 32, "producer, MMA issuer and one epilogue warp per TMEM lane quarter");
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
@@ -720,7 +715,7 @@ __global__ void __launch_bounds__(kUpThreads, 1) ozaki_tc_update_kernel(OzArgs a
       mbar_init(smem_u32(&empty_b[i]), 1);
     }
     mbar_init(smem_u32(&acc_full), 1);
-    mbar_init(smem_u32(&acc_empty), 4);  // one arrival per epilogue warp
+    mbar_init(smem_u32(&acc_empty), kEpiWarps);  // one arrival per epilogue warp
     mbar_init(smem_u32(&mma_done), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     give_up = 0;
@@ -811,7 +806,7 @@ __global__ void __launch_bounds__(kUpThreads, 1) ozaki_tc_update_kernel(OzArgs a
             const TcMma e = kTcSchedule[u];
             const uint64_t ad = ad0 + (uint64_t)((e.i * kTcM * kStage) >> 4);
             const uint64_t bd = bd0 + (uint64_t)((e.j0 * kTcN * kStage) >> 4);
-            tc_mma(tmem + (uint32_t)((e.i + e.j0 - kRegionLo) * kTcN), ad, bd, e.n, (st > 0 || u >= 2) ? 1u : 0u);
+            tc_mma(tmem + (uint32_t)((e.i + e.j0 - kRegionLo) * kTcN), ad, bd, e.n, (st > 0 || u >= kTcInit) ? 1u : 0u);
           }
           if (free_x) tc_commit(smem_u32(&empty_a[sa]));
           tc_commit(smem_u32(&empty_b[sb]));
@@ -825,57 +820,55 @@ __global__ void __launch_bounds__(kUpThreads, 1) ozaki_tc_update_kernel(OzArgs a
       mbar_wait(smem_u32(&mma_done), 0, a.wait_ns);
     }
   } else {
-    // epilogue: TMEM lane quarter qw, tile row r
-    const int qw = warp & 3, r = 32 * qw + lane;
+    // epilogue: TMEM lane quarter qw, tile row r, columns cw .. cw + 7
+    const int qw = warp & 3, r = 32 * qw + lane, cw = kEpiCols * ((warp - 2) >> 2);
     const uint32_t lane_base = tmem + ((uint32_t)(32 * qw) << 16);
     int k = 0;
     for (int T = t_first; T < t_last; T += t_step, ++k) {
-      const int p0 = (T / a.tiles_q) * kTcM, q0 = (T % a.tiles_q) * kTcN;
+      const int pr = (T / a.tiles_q) * kTcM + r, q0 = (T % a.tiles_q) * kTcN + cw;
+      const bool live = pr < a.p;
+      double* C = a.C + pr + (i64)q0 * a.ldc;
+      const int exr = live ? a.ex[pr] : kExpZero;
+      int eyc[kEpiCols];
+      double cv[kEpiCols];
+#pragma unroll
+      for (int j = 0; j < kEpiCols; ++j) {
+        const bool ok = live && q0 + j < a.q;
+        eyc[j] = ok ? a.ey[q0 + j] : kExpZero;
+        cv[j] = ok ? C[(i64)j * a.ldc] : 0.0;
+      }
       const bool ok = mbar_wait(smem_u32(&acc_full), (uint32_t)(k & 1), a.wait_ns);
       if (!__all_sync(0xffffffffu, ok) || *(volatile int*)&give_up) {
         atomicExch(&give_up, 1);
         break;
       }
       tc_fence_after();
-      // phase 1: level sums -> exact group sums g0 (levels 10..15), g1 (16..20), kept in registers
-      long long g0[kTcN], g1[kTcN];
+      // phase 1: level sums -> exact group sums g0 (levels 9..14), g1 (15..20), kept in registers
+      long long g0[kEpiCols], g1[kEpiCols];
 #pragma unroll
-      for (int c0 = 0; c0 < kTcN; c0 += 8) {
-        uint32_t v[kLevels][8];
-        load_levels(lane_base, c0, v);
+      for (int c0 = 0; c0 < kEpiCols; c0 += kEpiStep) {
+        uint32_t v[kLevels][kEpiStep];
+        load_levels(lane_base, cw + c0, v);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) group_sums<kMagic>(v, j, g0[c0 + j], g1[c0 + j]);
+        for (int j = 0; j < kEpiStep; ++j) group_sums<kMagic>(v, j, g0[c0 + j], g1[c0 + j]);
       }
       // hand the regions back to the MMA warp (the next tile's first stage overwrites them)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&acc_empty));
-      // phase 2 (overlaps the next tile's MMAs): scale, add the two groups, subtract from C,
-      // 16 columns at a time
-      const int pr = p0 + r;
-      if (pr < a.p) {
-        const int exr = a.ex[pr];
+      // phase 2 (overlaps the next tile's MMAs): scale, add the two groups, subtract from C
 #pragma unroll
-        for (int h = 0; h < kTcN; h += 16) {
-          double cv[16];
-#pragma unroll
-          for (int j = 0; j < 16; ++j) cv[j] = q0 + h + j < a.q ? a.C[pr + (i64)(q0 + h + j) * a.ldc] : 0.0;
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int qc = q0 + h + j;
-            if (qc >= a.q) continue;
-            const int eyc = a.ey[qc];
-            double v;
-            if (exr == kExpBad || eyc == kExpBad) {
-              v = __longlong_as_double(0x7ff8000000000000LL);
-            } else if (exr == kExpZero || eyc == kExpZero) {
-              v = 0.0;
-            } else {
-              v = group_value(g0[h + j], g1[h + j], exr + eyc);
-            }
-            a.C[pr + (i64)qc * a.ldc] = cv[j] - v;
-          }
+      for (int j = 0; j < kEpiCols; ++j) {
+        if (!live || q0 + j >= a.q) continue;
+        double v;
+        if (exr == kExpBad || eyc[j] == kExpBad) {
+          v = __longlong_as_double(0x7ff8000000000000LL);
+        } else if (exr == kExpZero || eyc[j] == kExpZero) {
+          v = 0.0;
+        } else {
+          v = group_value(g0[j], g1[j], exr + eyc[j]);
         }
+        C[(i64)j * a.ldc] = cv[j] - v;
       }
     }
   }
