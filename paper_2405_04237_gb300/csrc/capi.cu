@@ -169,7 +169,9 @@ cudaError_t trsm_any(i64 m, int b, double* X, i64 ldx, const double* U, i64 ldu,
       TRY(nn_update_emulated(m, cb, c0, X, ldx, U + (i64)c0 * ldu, ldu, X + (i64)c0 * ldx, ldx, oz, status, st));
     else if (c0 > 0)
       TRY(nn_product(m, cb, c0, X, ldx, U + (i64)c0 * ldu, ldu, X + (i64)c0 * ldx, ldx, -1.0, 1, 0, 0, status, st));
-    TRY(trsm_rows(m, cb, X + (i64)c0 * ldx, ldx, U + c0 + (i64)c0 * ldu, ldu, rinv + c0, status, st, skip));
+    // behind a tensor-core kernel, which fills every SM's shared memory, an early start costs more than it saves
+    // (60013 x 360: 8.11 -> 8.43 ms)
+    TRY(trsm_rows(m, cb, X + (i64)c0 * ldx, ldx, U + c0 + (i64)c0 * ldu, ldu, rinv + c0, status, st, skip, !oz));
   }
   return cudaSuccess;
 }

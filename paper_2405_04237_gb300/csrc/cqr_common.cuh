@@ -60,20 +60,22 @@ i64 gram_partials(i64 m, int b, const double* X, i64 ldx, double* part, const in
 // start while the one before it on the stream still runs; stream_wait(), the
 // first statement of every kernel launched this way, waits until that one has
 // ended and its writes are visible (so all earlier ones have ended too), and
-// then allows the next kernel the same.  Only grids of at most one block per
-// SM, or with less work than kEarlyFlops, start early: blocks placed while
-// others still run land unevenly, and the persistent grids of large products
-// (three equal blocks per SM) lost 11 % by it (2^20 x 256: 231 -> 258 ms).
+// then allows the next kernel the same.  Only launches of at most kEarlyFlops
+// FP64 operations start early: blocks placed while others still run land
+// unevenly, and the persistent grids of large products (three equal blocks per
+// SM) lost 11 % by it (2^20 x 256: 231 -> 258 ms).
 __device__ __forceinline__ void stream_wait() {
   asm volatile("griddepcontrol.wait;\ngriddepcontrol.launch_dependents;" ::: "memory");
 }
 
-constexpr double kEarlyFlops = 3e7;  // 25 us of FP64 work; the gap saved is 2-3 us
+// 80 us of FP64 work: a line at 3e6 costs 20000 x 64 5 % (859 against 812 us),
+// larger launches no longer gain.
+constexpr double kEarlyFlops = 1e8;
 
 struct Work64 {  // FP64 operations of a launch
   double flops;
 };
-constexpr Work64 kAnyWork{1e300};
+constexpr Work64 kNotEarly{1e300};
 
 template <class... P, class... A>
 cudaError_t launch(Work64 w, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
@@ -86,13 +88,13 @@ cudaError_t launch(Work64 w, void (*kernel)(P...), dim3 grid, dim3 block, size_t
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = attr;
-  cfg.numAttrs = (i64)grid.x * grid.y * grid.z <= kSMs || w.flops <= kEarlyFlops ? 1 : 0;
+  cfg.numAttrs = w.flops <= kEarlyFlops ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
 template <class... P, class... A>
 cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
-  return launch(kAnyWork, kernel, grid, block, smem, st, args...);
+  return launch(kNotEarly, kernel, grid, block, smem, st, args...);
 }
 
 // Upper-triangle enumeration, column by column: u -> (i, j), 0 <= i <= j.
@@ -195,8 +197,9 @@ cudaError_t gram_chol(i64 m, int b, const double* X, i64 ldx, double* part, doub
 // (b = 128: 0.78 -> 1.13 TFLOP/s on GB300).
 constexpr int kTrsmMaxB = 64;
 // With `skip` non-null and *skip set on the device, the launch does nothing.
+// early = false: no early start (see launch()).
 cudaError_t trsm_rows(i64 m, int b, double* X, i64 ldx, const double* U, i64 ldu, const double* rinv,
-                      const int* status, cudaStream_t st, const int* skip = nullptr);
+                      const int* status, cudaStream_t st, const int* skip = nullptr, bool early = true);
 
 // Row-wise back substitution  X := X U^{-T}  (X m x b, b <= kTrsmMaxB): solves
 // Abar U^T = B for the adjoint.  rinv as above.

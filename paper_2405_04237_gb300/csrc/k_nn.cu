@@ -7,11 +7,14 @@
 //
 // Each block computes a TM x TN output tile (256 threads, one MT x MT register
 // micro-tile per thread, TM * TN = 256 MT^2); K is staged through shared
-// memory in chunks.  MT is 4 where that fills the chip; smaller outputs take
-// 2 or 1, so that their multiply-adds (64 clocks each for a warp) are spread
-// over more SMs: a 64 x 64 x 64 product took 81 us in one block of 4 x 4
-// micro-tiles.  Every element sees the same operations in the same order
-// whatever the tile.  With beta = 1 the accumulator starts from C and every
+// memory in chunks.  MT is 2 from one block per SM on, else 1, so that the
+// multiply-adds (64 clocks each for a warp) are spread over the SMs: a 64 x 64
+// x 64 product took 81 us in one block of 4 x 4 micro-tiles.  The FP64 pipe is
+// so slow that 2 x 2 already hides the shared-memory loads, and its smaller
+// blocks even out the last wave and the partial tiles: against 4 x 4, CQR2GS
+// 30011 x 90 takes 1717 instead of 1814 us, 60000 x 256 14.94 instead of 15.40
+// ms, 2^18 x 256 58.47 instead of 58.59 ms.  Every element sees the same
+// operations in the same order whatever the tile.  With beta = 1 the accumulator starts from C and every
 // term is one fused multiply-add (negated operand when alpha = -1), so the
 // update issues exactly one FP64 instruction per multiply-add.  Threads
 // whose four columns all lie beyond N skip the arithmetic (warp-uniform when
@@ -41,7 +44,7 @@ struct NnArgs {
 template <int TM, int TN, int MT>
 struct NnShape {
   static constexpr int NTM = TM / MT;
-  static constexpr int KC = TM >= 256 ? 8 : 16;
+  static constexpr int KC = 16;
   static constexpr int SA = TM + 2, SB = TN + 2;
   static_assert(TM % MT == 0 && TN % MT == 0, "MT x MT micro-tiles");
   static_assert(NTM * (TN / MT) == kNnThreads, "one micro-tile per thread covers the TM x TN tile");
@@ -51,16 +54,12 @@ struct NnShape {
 // MT consecutive doubles of a shared-memory row
 template <int MT>
 __device__ __forceinline__ void lds_micro(const double* p, double (&v)[MT]) {
-  if constexpr (MT % 2 == 0) {
-#pragma unroll
-    for (int i = 0; i < MT; i += 2) {
-      const double2 x = *reinterpret_cast<const double2*>(p + i);
-      v[i] = x.x;
-      v[i + 1] = x.y;
-    }
+  if constexpr (MT == 2) {
+    const double2 x = *reinterpret_cast<const double2*>(p);
+    v[0] = x.x;
+    v[1] = x.y;
   } else {
-#pragma unroll
-    for (int i = 0; i < MT; ++i) v[i] = p[i];
+    v[0] = p[0];
   }
 }
 
@@ -199,19 +198,11 @@ cudaError_t nn_product_t(i64 M, int N, int K, const double* A, i64 lda, const do
   a.transb = transb;
   a.status = status;
   const bool neg = alpha < 0.0;
-  // 4 x 4 micro-tiles from two blocks per SM on, 2 x 2 from one, else single entries
-  const int MT = nn_blocks(M, N, 4) >= 2 * kSMs ? 4 : nn_blocks(M, N, 2) >= kSMs ? 2 : 1;
+  const int MT = nn_blocks(M, N, 2) >= kSMs ? 2 : 1;
   const int TN = nn_tile_n(N, MT);
   a.tiles_n = (N + TN - 1) / TN;
   prof_begin(kUpdate, st);
-  if (MT == 4) {
-    switch (TN) {
-      case 8: launch_nn<512, 8, 4>(a, neg, st); break;
-      case 16: launch_nn<256, 16, 4>(a, neg, st); break;
-      case 32: launch_nn<128, 32, 4>(a, neg, st); break;
-      default: launch_nn<64, 64, 4>(a, neg, st); break;
-    }
-  } else if (MT == 2) {
+  if (MT == 2) {
     switch (TN) {
       case 8: launch_nn<128, 8, 2>(a, neg, st); break;
       case 16: launch_nn<64, 16, 2>(a, neg, st); break;

@@ -165,13 +165,13 @@ void set_trsm_attr() {
 }  // namespace
 
 cudaError_t trsm_rows(i64 m, int b, double* X, i64 ldx, const double* U, i64 ldu, const double* rinv,
-                      const int* status, cudaStream_t st, const int* skip) {
+                      const int* status, cudaStream_t st, const int* skip, bool early) {
   if (m <= 0 || b <= 0) return cudaSuccess;
   if (b > kTrsmMaxB) return cudaErrorInvalidValue;
   set_trsm_attr();
   const i64 blocks = (m + kRows - 1) / kRows;
   prof_begin(kTrsm, st);
-  launch(Work64{(double)m * b * b}, trsm_rows_kernel, (unsigned)blocks, kRows, trsm_smem(b), st, m, b, X, ldx, U, ldu, rinv, status, skip);
+  launch(early ? Work64{(double)m * b * b} : kNotEarly, trsm_rows_kernel, (unsigned)blocks, kRows, trsm_smem(b), st, m, b, X, ldx, U, ldu, rinv, status, skip);
   prof_end(kTrsm, (double)m * b * b, st);
   return cudaGetLastError();
 }

@@ -1,5 +1,5 @@
-"""The product kernel's micro-tiles (4 x 4, 2 x 2, single entries) on both sides
-of the lines between them, through factorisations whose updates and R products
+"""The product kernel's micro-tiles (2 x 2, single entries) on both sides of the
+line between them, through factorisations whose updates and R products
 fall there, and the same calls captured into a CUDA graph: the launches that
 start before the one ahead of them has ended give the eager result bit for bit.
 
