@@ -110,17 +110,19 @@ struct BArgs {
   double* s1;          // [gridDim.x][kBNMax * kBNMax]: S1 of the current panel (column-major), at the group's first CTA
   unsigned int* bar;   // [nodes] barrier counters (zero at launch)
   int* abort;          // launch-wide abort flag (zero at launch)
-  int nmax, bmax;      // shared-memory layout
+  int nmax, bmax, two_tiles;  // shared-memory layout
   int halve;           // adaptive panel width
   unsigned long long wait_ns;
   int hook_group, hook_rank, hook_barrier;  // test hook: that CTA skips that barrier's arrival
 };
 
 // Shared memory (doubles): tile [kBR][ts] (ts = nmax + 1, odd) or the
-// reduction scratch [kBT][16]; U [bmax * bmax] row-major (zero diagonal and
+// reduction scratch [kBT][16]; a second tile where it fits (the next rows are
+// fetched while the current ones are computed on); U [bmax * bmax] row-major (zero diagonal and
 // lower triangle once factored); dg, rv [bmax]; M [nmax^2/4] (Y or Z).
 struct Smem {
   double* tile;
+  double* next;  // second tile, or null
   double* red;
   double* U;
   double* dg;
@@ -136,15 +138,18 @@ __host__ __device__ inline size_t region0_doubles(int nmax) {
   return t > r ? t : r;
 }
 __host__ __device__ inline size_t mdoubles(int nmax) { return (size_t)nmax * nmax / 4 + 1; }
-size_t bsmem_bytes(int nmax, int bmax) {
-  return sizeof(double) * (region0_doubles(nmax) + (size_t)bmax * bmax + 2 * (size_t)bmax + mdoubles(nmax));
+size_t bsmem_bytes(int nmax, int bmax, bool two_tiles) {
+  return sizeof(double) * ((two_tiles ? 2 : 1) * region0_doubles(nmax) + (size_t)bmax * bmax + 2 * (size_t)bmax +
+                           mdoubles(nmax));
 }
+constexpr size_t kBSmemMax = 226 * 1024;  // opt-in shared memory per block, less the kernel's static use
 
-__device__ Smem carve(double* sm, int nmax, int bmax) {
+__device__ Smem carve(double* sm, int nmax, int bmax, int two_tiles) {
   Smem s;
   s.tile = sm;
   s.red = sm;
-  s.U = sm + region0_doubles(nmax);
+  s.next = two_tiles ? sm + region0_doubles(nmax) : nullptr;
+  s.U = sm + (two_tiles ? 2 : 1) * region0_doubles(nmax);
   s.dg = s.U + (size_t)bmax * bmax;
   s.rv = s.dg + bmax;
   s.M = s.rv + bmax;
@@ -427,9 +432,15 @@ __device__ __forceinline__ void trsm_rows_lanes(const Smem& s, int tc, int b, in
 }
 
 __device__ void trsm_rows_staged(const Smem& s, int tc, int b, int nr) {
-  int L = 2;
-  while (L < 32 && 2 * L * nr <= kBT && 2 * L <= b) L *= 2;
+  // Narrow panels: half the threads, as fewer lanes a row waste less of the
+  // triangle (36 against 48 FP64 instructions a row at b = 8: 8000 x 16 on one
+  // CTA 2.12 -> 1.97 ms).  Wide ones need all of them to hide the shuffles
+  // (8000 x 128, b = 64: 72 against 78 ms).
+  const int threads = b <= 16 ? kBT / 2 : kBT;
+  int L = 1;
+  while (L < 32 && 2 * L * nr <= threads && 2 * L <= b) L *= 2;
   switch (L) {
+    case 1: trsm_rows_lanes<1>(s, tc, b, nr); break;
     case 2: trsm_rows_lanes<2>(s, tc, b, nr); break;
     case 4: trsm_rows_lanes<4>(s, tc, b, nr); break;
     case 8: trsm_rows_lanes<8>(s, tc, b, nr); break;
@@ -437,7 +448,7 @@ __device__ void trsm_rows_staged(const Smem& s, int tc, int b, int nr) {
     default: trsm_rows_lanes<32>(s, tc, b, nr); break;
   }
 }
-static_assert(kBT >= 2 * kBRMax, "two lanes for every staged row");
+static_assert(kBT >= kBRMax, "a lane for every staged row");
 
 // U_cc' := U_cc' / U_cc (by the reciprocal) for c' > c: the form the staged
 // substitution uses.  Called after the unscaled factor has been used for
@@ -491,17 +502,24 @@ __device__ void run_pass(const PassSpec& P, const Smem& s0, i64 R0, i64 R1, doub
     for (int v = 0; v < 4; ++v) am[u][v] = ae[u][v] = 0.0;
   const int w = P.hi - P.lo;
   const int rb = s.rb;
-  for (i64 r0 = R0; r0 < R1; r0 += rb) {
+  // stages rows r0 .. (zero beyond the range) in `tile`: asynchronous copies,
+  // coalesced along the rows of each column, all in flight together
+  auto stage = [&](double* tile, i64 r0) {
     const int nr = (int)imin64(rb, R1 - r0);
-    // stage rows (zero beyond nr): asynchronous copies, coalesced along the
-    // rows of each column, all in flight before the one wait
     for (int e = t; e < rb * w; e += kBT) {
       const int r = e % rb, c = e / rb;
       const bool ok = r < nr;
-      cp_async8(s.tile + (size_t)r * s.ts + c, ok ? P.src + (r0 + r) + (i64)(P.lo + c) * P.lds : P.src, ok);
+      cp_async8(tile + (size_t)r * s.ts + c, ok ? P.src + (r0 + r) + (i64)(P.lo + c) * P.lds : P.src, ok);
     }
+  };
+  double* spare = s.next;
+  if (spare && R0 < R1) stage(s.tile, R0);
+  for (i64 r0 = R0; r0 < R1; r0 += rb) {
+    const int nr = (int)imin64(rb, R1 - r0);
+    if (!spare) stage(s.tile, r0);
     cp_async_wait_all();
     __syncthreads();
+    if (spare && r0 + rb < R1) stage(spare, r0 + rb);  // its last use ended at the barrier below
     if (P.op1 == 1) trsm_rows_staged(s, P.t0 - P.lo, P.tb, nr);
     if (P.op1 == 2) nn_update(s, nr, P.x0u - P.lo, P.pu, P.c0u - P.lo, P.qu, P.Mm);
     __syncthreads();
@@ -512,6 +530,11 @@ __device__ void run_pass(const PassSpec& P, const Smem& s0, i64 R0, i64 R1, doub
     }
     if (P.op2) tn_accumulate(mp, s, nr, am, ae);
     __syncthreads();
+    if (spare) {
+      double* done = s.tile;
+      s.tile = spare;
+      spare = done;
+    }
   }
   if (P.op2) tn_flush(mp, s, (int)imin64(rb, R1 - R0), am, ae, slot);
 }
@@ -658,7 +681,7 @@ __global__ void __launch_bounds__(kBT, 1) batched_mcqr2gs_kernel(const __grid_co
   __shared__ int bar_ok, sh_broken, sh_rej;
   __shared__ Group gr;  // state that outlives the passes stays out of the registers
   __shared__ BMat mt;
-  const Smem s = carve(bsm, a.nmax, a.bmax);
+  const Smem s = carve(bsm, a.nmax, a.bmax, a.two_tiles);
   const int t = threadIdx.x;
   bool alive = true;
   for (int lev = 0; lev < a.lev.n; ++lev) {
@@ -1212,7 +1235,9 @@ cudaError_t batched_persistent_run(int batch, const int64_t* m, const int64_t* n
       g_bhook_group = -1;
     }
   }
-  const size_t smem = bsmem_bytes(nmax, bmax);
+  const bool two_tiles = bsmem_bytes(nmax, bmax, true) <= kBSmemMax;
+  a.two_tiles = two_tiles ? 1 : 0;
+  const size_t smem = bsmem_bytes(nmax, bmax, two_tiles);
   TRY_RET(cudaFuncSetAttribute(batched_mcqr2gs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int occ = 0;
   TRY_RET(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, batched_mcqr2gs_kernel, kBT, smem));
