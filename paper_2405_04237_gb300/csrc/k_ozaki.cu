@@ -55,10 +55,10 @@
 // mbarrier), one thread issues its 16 MMAs and commits them to the stage's
 // "empty" mbarrier, which frees the stage for the copy four stages later.
 // At the end every thread reads the 12 level sums of its row from TMEM,
-// combines levels 9..14 and 15..20 exactly in 64-bit integers (below 2^50),
-// builds the two scaled doubles with integer operations and adds them (one
-// rounding), so the FP64 pipe does one operation per element (two for an
-// update, which subtracts the tile from C).  Every wait is bounded in time
+// combines levels 9..14 and 15..20 exactly in 64-bit integers (below 2^51)
+// and rounds the two to a double in integer operations (group_value), so the
+// FP64 pipe does nothing for a projection and one subtraction per entry of an
+// update.  Every wait is bounded in time
 // (kWaitNs of the global nanosecond timer, 2 s: a stage arrives within
 // microseconds); on expiry the block records CQR_STATUS_TIMEOUT, waits
 // (bounded) for its copies in flight, frees its TMEM and returns.  A
@@ -181,28 +181,30 @@ __device__ __forceinline__ i64 plane_off(i64 col, int half) {
 
 // ---------------------------------------------------------------------------
 // Column splitting: X (rows r0 .. r0 + nsub*kSub of an m x c matrix) ->
-// planes.  Grid (ceil(c / 8), nsub), 256 threads: block (g, s) takes the
+// planes.  Grid (ceil(c / 8), nsub), 512 threads: block (g, s) takes the
 // 8-column group g of the layout (columns 8g .. 8g+7) over sub-chunk s, so
 // that for each stage and plane its digits form one contiguous 256-byte run
-// (8 columns x 32 indices).  Warp w takes stages 8 it + w, it = 0..15 (only
+// (8 columns x 32 indices).  Warp w takes stages 16 it + w, it = 0..7 (only
 // those below nst, for the short Y of an update); lane l handles rows 4 (l mod
 // 4) .. + 3 of both halves of the stage in column 8g + l / 4.  A warp load
 // thus touches 8 lines and a warp store writes 128 consecutive bytes of a run
 // (with 16 rows a lane, four columns' worth of lines per load, the kernel was
 // bound by the L1's line rate: 3.6 TB/s).  Two passes over the sub-chunk: the
-// column maxima (scales), then the digits; the second pass re-reads from L2.
+// column maxima (scales), then the digits; the second pass re-reads from L2
+// (two blocks an SM: 256 KiB each, 80 MB over the chip).
 // Tiles of T columns (T a multiple of 8); plane block
 // (s, tile, st, i) starts at byte
 // (((s * ntile + tile) * kStagesPerSub + st) * kPlanes + i) * T * 32 with
 // ntile = ceil(c / T); exps: [s * c + col].  Columns past c of the last
 // group are written as zero digits (the tile padding; never read).
-constexpr int kSplitWarps = 8;
+constexpr int kSplitWarps = 16;
 
 // 4 consecutive entries xc[row .. row+3] (zero past m or for a column past
-// c); 16-byte loads when the address allows (an odd leading dimension puts
-// every other column off the 16-byte grid).
-__device__ __forceinline__ void load4(const double* xc, i64 row, i64 m, bool colok, unsigned long long (&bits)[4]) {
-  if (colok && row + 3 < m && ((reinterpret_cast<uintptr_t>(xc + row) & 15) == 0)) {
+// c); 16-byte loads when `vec` (an odd leading dimension puts every other
+// column off the 16-byte grid).
+__device__ __forceinline__ void load4(const double* xc, i64 row, i64 m, bool colok, bool vec,
+                                      unsigned long long (&bits)[4]) {
+  if (vec && colok && row + 3 < m) {
     const double2* p = reinterpret_cast<const double2*>(xc + row);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
@@ -217,7 +219,7 @@ __device__ __forceinline__ void load4(const double* xc, i64 row, i64 m, bool col
   }
 }
 
-__global__ void __launch_bounds__(32 * kSplitWarps, 4) ozaki_split_kernel(const double* X, i64 ldx, i64 m, i64 r0,
+__global__ void __launch_bounds__(32 * kSplitWarps, 2) ozaki_split_kernel(const double* X, i64 ldx, i64 m, i64 r0,
                                                                           int c, int T, int nst, uint8_t* planes,
                                                                           int* exps, const int* status) {
   stream_wait();
@@ -228,13 +230,14 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 4) ozaki_split_kernel(const 
   const bool colok = col < c;
   const i64 base = r0 + (i64)s * kSub + 4 * quad;
   const double* xc = X + (i64)(colok ? col : 0) * ldx;
+  const bool vec = (ldx & 1) == 0 && (reinterpret_cast<uintptr_t>(X + r0) & 15) == 0;  // rows are multiples of 4
   // pass 1: the column's largest exponent (zeros and subnormals do not set the scale) and Inf/NaN
   int emax = 0;
 #pragma unroll 2
   for (int st = warp; st < nst; st += kSplitWarps) {
     unsigned long long b0[4], b1[4];
-    load4(xc, base + st * kStage, m, colok, b0);
-    load4(xc, base + st * kStage + 16, m, colok, b1);
+    load4(xc, base + st * kStage, m, colok, vec, b0);
+    load4(xc, base + st * kStage + 16, m, colok, vec, b1);
 #pragma unroll
     for (int k = 0; k < 4; ++k)
       emax = max(emax, max((int)(b0[k] >> 52) & 0x7FF, (int)(b1[k] >> 52) & 0x7FF));
@@ -263,8 +266,8 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 4) ozaki_split_kernel(const 
 #pragma unroll 1
   for (int st = warp; st < nst; st += kSplitWarps) {
     unsigned long long b0[4], b1[4];
-    load4(xc, base + st * kStage, m, colok, b0);
-    load4(xc, base + st * kStage + 16, m, colok, b1);
+    load4(xc, base + st * kStage, m, colok, vec, b0);
+    load4(xc, base + st * kStage + 16, m, colok, vec, b1);
     uint32_t w0[kPlanes], w1[kPlanes];
     digits4(b0, e, w0);
     digits4(b1, e, w1);
@@ -333,6 +336,56 @@ __global__ void __launch_bounds__(128) ozaki_rowsplit_kernel(const double* X, i6
         *reinterpret_cast<uint4*>(dst + (i64)i * kTcM * kStage) = v;
       }
     }
+  }
+}
+
+// The same for contractions of up to four stages (kc <= 128), in one pass: a
+// block of nst warps takes 32 rows, warp w the 32 columns of stage w, which
+// each lane keeps in registers between the maximum and the digits.  (Two
+// passes re-read the rows from DRAM: the blocks in flight hold more than L2.)
+constexpr int kRowStages = 4;
+
+__global__ void __launch_bounds__(32 * kRowStages) ozaki_rowsplit_short_kernel(const double* X, i64 ldx, i64 m, i64 r0,
+                                                                               i64 k0, int kc, uint8_t* planes,
+                                                                               int* exps, const int* status) {
+  stream_wait();
+  if (status && *status) return;
+  __shared__ int red[kRowStages][32];
+  const int lane = threadIdx.x & 31, st = threadIdx.x >> 5, nst = blockDim.x >> 5;
+  const int row = blockIdx.x * 32 + lane;
+  const i64 r = r0 + row;
+  const bool live = r < m;
+  const double* xr = X + (live ? r : 0) + (k0 + st * kStage) * ldx;
+  const int w = min(kStage, kc - st * kStage);  // live columns of the stage
+  unsigned long long b[kStage];
+  int emax = 0;
+#pragma unroll
+  for (int k = 0; k < kStage; ++k)
+    b[k] = (unsigned long long)__double_as_longlong(live && k < w ? xr[(i64)k * ldx] : 0.0);
+#pragma unroll
+  for (int k = 0; k < kStage; ++k) emax = max(emax, (int)(b[k] >> 52) & 0x7FF);
+  red[st][lane] = emax;
+  __syncthreads();
+  for (int q = 0; q < nst; ++q) emax = max(emax, red[q][lane]);
+  const int e = emax == 0x7FF ? kExpBad : (emax == 0 ? kExpZero : emax - 1022);
+  if (st == 0) exps[row] = e;
+  uint8_t* dst0 = planes + ((i64)(row / kTcM) * nst + st) * kTcABytes + plane_off(row % kTcM, 0);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t words[kPlanes][4];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const int o = 16 * h + 4 * g;
+      const unsigned long long b4[4] = {b[o], b[o + 1], b[o + 2], b[o + 3]};
+      uint32_t d[kPlanes];
+      digits4(b4, e, d);
+#pragma unroll
+      for (int i = 0; i < kPlanes; ++i) words[i][g] = d[i];
+    }
+#pragma unroll
+    for (int i = 0; i < kPlanes; ++i)
+      *reinterpret_cast<uint4*>(dst0 + 128 * h + (i64)i * kTcM * kStage) =
+          make_uint4(words[i][0], words[i][1], words[i][2], words[i][3]);
   }
 }
 
@@ -446,19 +499,6 @@ __device__ __forceinline__ void tc_ld4(uint32_t taddr, uint32_t (&r)[4]) {
 }
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// g * 2^e for an integer |g| < 2^53 (exact), built with integer operations;
-// outside the normal range it falls back to the FP64 library ldexp.
-__device__ __forceinline__ double scaled_int(long long g, int e) {
-  if (g == 0) return 0.0;
-  const unsigned long long sgn = g < 0 ? 0x8000000000000000ull : 0ull;
-  const unsigned long long a = g < 0 ? (unsigned long long)(-g) : (unsigned long long)g;
-  const int msb = 63 - __clzll((long long)a);
-  const int E = msb + e + 1023;
-  if (E <= 0 || E >= 2047) return ldexp((double)g, e);
-  const unsigned long long mant = (a << (52 - msb)) & 0xFFFFFFFFFFFFFull;
-  return __longlong_as_double((long long)(sgn | ((unsigned long long)E << 52) | mant));
-}
-
 // Contraction length up to which every level sum is below 2^22 units (11
 // pairs x 256 x K < 2^22): then the FP32 value f (a multiple of 2^-18) is read
 // exactly as bits(f + 48) - bits(48), one full-rate FP32 add and integer
@@ -492,8 +532,8 @@ __device__ __forceinline__ void group_sums(const uint32_t (&v)[kLevels][kEpiStep
     for (int l = 0; l < kLevels; ++l) b[l] = __float_as_uint(__fadd_rn(__uint_as_float(v[l][j]), kMagicF));
     const uint32_t off = 33u * (uint32_t)kMagicBits;  // modulo 2^32
     auto two = [&](int l) { return (long long)(int)(b[l] + 32u * b[l + 1] - off); };
-    g0 = two(0) + (two(2) << 10) + (two(4) << 20);
-    g1 = two(6) + (two(8) << 10) + (two(10) << 20);
+    g0 = two(4) * 1048576 + (two(2) * 1024 + two(0));
+    g1 = two(10) * 1048576 + (two(8) * 1024 + two(6));
   } else {
     auto lev = [&](int l) { return (long long)__float2int_rz(__uint_as_float(v[l][j]) * 262144.0f); };
     g0 = g1 = 0;
@@ -504,10 +544,31 @@ __device__ __forceinline__ void group_sums(const uint32_t (&v)[kLevels][kEpiStep
   }
 }
 
-// sum_L S_L 32^L = 32^9 (g0 + 2^30 g1), times 2^(ex + ey - 108); one rounding
+// sum_L S_L 32^L = 32^9 (g0 + 2^30 g1), times 2^(ex + ey - 108), rounded to
+// double in integer operations (|g0| < 2^51, |g1| < 2^46): the FP64 pipe takes
+// 64 clocks an instruction, and the epilogue of an update tile is bound by its
+// issue slots and that pipe together.  The 77-bit sum is cut to its sign and
+// a 64-bit window with at least 57 significant bits where low bits are cut
+// off; outside the normal range the library's ldexp.
 __device__ __forceinline__ double group_value(long long g0, long long g1, int exy) {
-  const int e2 = exy - 108 + 5 * kLevelLo;
-  return scaled_int(g1, e2 + 5 * kLowLevels) + scaled_int(g0, e2);
+  const long long h = g1 + (g0 >> 30);
+  const uint32_t l = (uint32_t)g0 & 0x3FFFFFFFu;  // sum = h 2^30 + l
+  const bool neg = h < 0;
+  const uint32_t lo = neg ? (0u - l) & 0x3FFFFFFFu : l;
+  const unsigned long long hi = (unsigned long long)(neg ? -h - (l != 0u) : h);  // |sum| = hi 2^30 + lo, hi < 2^47
+  const uint32_t top = (uint32_t)(hi >> 32);
+  const int k = top >= 256u ? 17 : (top >= 4u ? 24 : 30);  // hi < 2^47, 2^40, 2^34
+  const unsigned long long w = (hi << k) | (lo >> (30 - k));
+  if (w == 0ull) return 0.0;
+  const int z = __clzll((long long)w);
+  const int E = exy - 108 + 5 * kLevelLo + (30 - k) + 63 - z + 1023;  // biased exponent
+  if (E <= 0 || E >= 2046) {
+    const double v = ldexp((double)w, exy - 108 + 5 * kLevelLo + 30 - k);
+    return neg ? -v : v;
+  }
+  const unsigned long long n = w << z;
+  const unsigned long long m = (n >> 11) + ((n >> 10) & 1ull);  // 2^52 .. 2^53
+  return __longlong_as_double((long long)(m + ((unsigned long long)(E - 1) << 52) + ((unsigned long long)neg << 63)));
 }
 
 struct OzArgs {
@@ -824,6 +885,7 @@ __global__ void __launch_bounds__(kUpThreads, 1) ozaki_tc_update_kernel(OzArgs a
     const int qw = warp & 3, r = 32 * qw + lane, cw = kEpiCols * ((warp - 2) >> 2);
     const uint32_t lane_base = tmem + ((uint32_t)(32 * qw) << 16);
     int k = 0;
+    bool stop = false;  // a warp that gave up still meets the others at the barrier of every tile
     for (int T = t_first; T < t_last; T += t_step, ++k) {
       const int pr = (T / a.tiles_q) * kTcM + r, q0 = (T % a.tiles_q) * kTcN + cw;
       const bool live = pr < a.p;
@@ -837,25 +899,32 @@ __global__ void __launch_bounds__(kUpThreads, 1) ozaki_tc_update_kernel(OzArgs a
         eyc[j] = ok ? a.ey[q0 + j] : kExpZero;
         cv[j] = ok ? C[(i64)j * a.ldc] : 0.0;
       }
-      const bool ok = mbar_wait(smem_u32(&acc_full), (uint32_t)(k & 1), a.wait_ns);
-      if (!__all_sync(0xffffffffu, ok) || *(volatile int*)&give_up) {
-        atomicExch(&give_up, 1);
-        break;
+      if (!stop) {
+        const bool ok = mbar_wait(smem_u32(&acc_full), (uint32_t)(k & 1), a.wait_ns);
+        if (!__all_sync(0xffffffffu, ok) || __any_sync(0xffffffffu, *(volatile int*)&give_up)) {
+          atomicExch(&give_up, 1);
+          stop = true;
+        }
       }
-      tc_fence_after();
       // phase 1: level sums -> exact group sums g0 (levels 9..14), g1 (15..20), kept in registers
       long long g0[kEpiCols], g1[kEpiCols];
+      if (!stop) {
+        tc_fence_after();
 #pragma unroll
-      for (int c0 = 0; c0 < kEpiCols; c0 += kEpiStep) {
-        uint32_t v[kLevels][kEpiStep];
-        load_levels(lane_base, cw + c0, v);
+        for (int c0 = 0; c0 < kEpiCols; c0 += kEpiStep) {
+          uint32_t v[kLevels][kEpiStep];
+          load_levels(lane_base, cw + c0, v);
 #pragma unroll
-        for (int j = 0; j < kEpiStep; ++j) group_sums<kMagic>(v, j, g0[c0 + j], g1[c0 + j]);
+          for (int j = 0; j < kEpiStep; ++j) group_sums<kMagic>(v, j, g0[c0 + j], g1[c0 + j]);
+        }
+        // hand the regions back to the MMA warp (the next tile's first stage overwrites them)
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&acc_empty));
       }
-      // hand the regions back to the MMA warp (the next tile's first stage overwrites them)
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&acc_empty));
+      // no warp's second phase takes issue slots from another's first one, which the MMAs wait for
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
+      if (stop) continue;
       // phase 2 (overlaps the next tile's MMAs): scale, add the two groups, subtract from C
 #pragma unroll
       for (int j = 0; j < kEpiCols; ++j) {
@@ -997,11 +1066,11 @@ cudaError_t tn_product_emulated(i64 m, int p, int q, const double* X, i64 ldx, c
   for (i64 r0 = 0; r0 < m; r0 += ch) {
     const i64 nsub = ((m - r0 < ch ? m - r0 : ch) + kSub - 1) / kSub;
     prof_begin(kMisc, st);
-    launch(ozaki_split_kernel, dim3((unsigned)((p + 7) / 8), (unsigned)nsub), 256, 0, st, X, ldx, m, r0, p, kTcM, kStagesPerSub, px, ex, status);
+    launch(ozaki_split_kernel, dim3((unsigned)((p + 7) / 8), (unsigned)nsub), 32 * kSplitWarps, 0, st, X, ldx, m, r0, p, kTcM, kStagesPerSub, px, ex, status);
     prof_end(kMisc, 0.0, st);
     if (!same) {
       prof_begin(kMisc, st);
-      launch(ozaki_split_kernel, dim3((unsigned)((q + 7) / 8), (unsigned)nsub), 256, 0, st, Y, ldy, m, r0, q, kTcN, kStagesPerSub, py, ey, status);
+      launch(ozaki_split_kernel, dim3((unsigned)((q + 7) / 8), (unsigned)nsub), 32 * kSplitWarps, 0, st, Y, ldy, m, r0, q, kTcN, kStagesPerSub, py, ey, status);
       prof_end(kMisc, 0.0, st);
     }
     OzArgs a{};
@@ -1067,13 +1136,16 @@ cudaError_t nn_update_emulated(i64 M, int N, int K, const double* X, i64 ldx, co
     const int kc = (int)(K - k0 < kSub ? K - k0 : kSub);
     const int nst = (kc + kStage - 1) / kStage;
     prof_begin(kMisc, st);
-    launch(ozaki_split_kernel, dim3((unsigned)((N + 7) / 8), 1u), 256, 0, st, Y, ldy, k0 + kc, k0, N, kTcN, nst, py, ey, status);
+    launch(ozaki_split_kernel, dim3((unsigned)((N + 7) / 8), 1u), 32 * kSplitWarps, 0, st, Y, ldy, k0 + kc, k0, N, kTcN, nst, py, ey, status);
     prof_end(kMisc, 0.0, st);
     for (i64 r0 = 0; r0 < M; r0 += rows) {
       const i64 live = M - r0 < rows ? M - r0 : rows;
       const int rws = (int)((live + kTcM - 1) / kTcM * kTcM);
       prof_begin(kMisc, st);
-      launch(ozaki_rowsplit_kernel, (unsigned)(rws / 128), 128, 0, st, X, ldx, M, r0, rws, k0, kc, px, ex, status);
+      if (nst <= kRowStages)
+        launch(ozaki_rowsplit_short_kernel, (unsigned)(rws / 32), 32 * nst, 0, st, X, ldx, M, r0, k0, kc, px, ex, status);
+      else
+        launch(ozaki_rowsplit_kernel, (unsigned)(rws / 128), 128, 0, st, X, ldx, M, r0, rws, k0, kc, px, ex, status);
       prof_end(kMisc, 0.0, st);
       OzArgs a{};
       a.px = px;
