@@ -111,33 +111,28 @@ inline int round_up(int x, int t) { return (x + t - 1) / t * t; }
 // x * 2^(54 - e) rounded to an integer, plus 16 in every base-32 digit, of one
 // FP64 value (raw bits b) against scale e: the fields of 5 bits (the top one
 // 6) are the balanced digits plus 16.  Zeros, subnormals and the entries of a
-// bad column count as 0.
+// bad column (e far above any exponent) count as 0.
 constexpr unsigned long long kDigitBias = 16ull * (((1ull << 50) - 1) / 31) + (16ull << 50);
 
 __device__ __forceinline__ unsigned long long biased_digits(unsigned long long b, int e) {
-  const int E = (int)((b >> 52) & 0x7FF);
-  if (E == 0 || E == 0x7FF || e == kExpBad) return kDigitBias;
-  const unsigned long long M = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-  const int sh = E - 1021 - e;  // |x| 2^(54-e) = M 2^(E - 1075 + 54 - e), sh <= 1
-  const int s = min(-sh, 63);
-  const unsigned long long mag = sh >= 0 ? M << sh : (M + (1ull << (s - 1))) >> s;
-  return (long long)b < 0 ? kDigitBias - mag : kDigitBias + mag;
+  const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
+  const int E = (int)((hi >> 20) & 0x7FFu);
+  // the mantissa with its leading one at bit 62; |x| 2^(54-e) = M 2^(E - 1031 - e), E <= e + 1022
+  const unsigned long long M =
+      ((unsigned long long)((__funnelshift_l(lo, hi, 10) & 0x3FFFFFFFu) | 0x40000000u) << 32) | (lo << 10);
+  const int s = E ? min(e + 1030 - E, 63) : 63;
+  const unsigned long long mag = ((M >> s) + 1) >> 1;
+  const unsigned long long neg = (unsigned long long)((long long)b >> 63);
+  return (mag ^ neg) + (kDigitBias - neg);
 }
 
 // e4m3 codes, sign and magnitude, of four digits given as bytes u = d + 16
 // (0 .. 31; kTop: 0 .. 32).
 template <bool kTop>
 __device__ __forceinline__ uint32_t e4m3_of_digits(uint32_t u) {
-  const uint32_t six = kTop ? (u >> 1) & 0x10101010u : 0u;  // d = 16
-  const uint32_t t = ~(u | six) & 0x10101010u;              // d < 0
-  const uint32_t n = t >> 4;
-  return ((u & 0x0F0F0F0Fu) ^ (t - n)) + n + (t << 3) + six;
-}
-
-// 20 bits as four bytes of 5 bits
-__device__ __forceinline__ uint32_t bytes_of_fields(uint32_t x) {
-  const uint32_t y = (x & 0x3FFu) | ((x << 6) & 0x3FF0000u);
-  return (y & 0x1F001Fu) | ((y << 3) & 0x1F001F00u);
+  const uint32_t six = kTop ? (u >> 1) & 0x10101010u : 0u;    // d = 16
+  const uint32_t n = (~(u | six) >> 4) & 0x01010101u;         // d < 0
+  return ((u & 0x0F0F0F0Fu) ^ (n * 15u)) + (n * 129u + six);  // 16 - u's low bits, sign bit
 }
 
 // out[i] = byte i of w[0..3] (i < N)
@@ -151,27 +146,46 @@ __device__ __forceinline__ void transpose4(const uint32_t (&w)[4], uint32_t* out
   if (N == 4) out[3] = __byte_perm(b, d, 0x7632);
 }
 
+// The 5-bit field at bit 5 I of four values given bytewise (w[q] = byte q of
+// each): one byte, or the upper bits of one and the lower of the next.
+template <int I>
+__device__ __forceinline__ uint32_t field(const uint32_t* w) {
+  constexpr int q = 5 * I / 8, r = 5 * I % 8;
+  constexpr uint32_t all = I == kPlanes - 1 ? 0x3F3F3F3Fu : 0x1F1F1F1Fu;
+  if (r <= 3) return (w[q] >> r) & all;
+  constexpr uint32_t low = 0x01010101u * ((1u << ((8 - r) & 7)) - 1u);
+  return ((w[q] >> r) & low) | ((w[q + 1] << ((8 - r) & 7)) & (all & ~low));
+}
+
 // Digits of four FP64 values (raw bits b[0..3]) against scale e: byte k of
-// word i is the e4m3 code of digit i of value k.  Every step after the fixed-
-// point conversion works on four digits at once.
+// word i is the e4m3 code of digit i of value k.  The fixed-point values are
+// transposed bytewise first, so that every later step works on four digits at
+// once: about 45 instructions a value in all (the splitting kernels are bound
+// by the integer pipes; extracting the fields of each value by itself took 70).
 __device__ __forceinline__ void digits4(const unsigned long long (&b)[4], int e, uint32_t (&w)[kPlanes]) {
-  uint32_t f0[4], f1[4], f2[4], u[kPlanes];
+  uint32_t lo[4], hi[4], v[8];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const unsigned long long v = biased_digits(b[k], e);
-    f0[k] = bytes_of_fields((uint32_t)v & 0xFFFFFu);
-    f1[k] = bytes_of_fields((uint32_t)(v >> 20) & 0xFFFFFu);
-    const uint32_t x = (uint32_t)(v >> 40);  // fields 8, 9 (5 bits) and 10 (6 bits)
-    const uint32_t y = (x & 0x3FFu) | ((x << 6) & 0x3F0000u);
-    f2[k] = (y & 0x3F001Fu) | ((y << 3) & 0x1F00u);
+    const unsigned long long x = biased_digits(b[k], e);
+    lo[k] = (uint32_t)x;
+    hi[k] = (uint32_t)(x >> 32);
   }
-  transpose4<4>(f0, u);
-  transpose4<4>(f1, u + 4);
-  transpose4<3>(f2, u + 8);
-#pragma unroll
-  for (int i = 0; i < kPlanes - 1; ++i) w[i] = e4m3_of_digits<false>(u[i]);
-  w[kPlanes - 1] = e4m3_of_digits<true>(u[kPlanes - 1]);
+  transpose4<4>(lo, v);
+  transpose4<3>(hi, v + 4);
+  v[7] = 0u;
+  w[0] = e4m3_of_digits<false>(field<0>(v));
+  w[1] = e4m3_of_digits<false>(field<1>(v));
+  w[2] = e4m3_of_digits<false>(field<2>(v));
+  w[3] = e4m3_of_digits<false>(field<3>(v));
+  w[4] = e4m3_of_digits<false>(field<4>(v));
+  w[5] = e4m3_of_digits<false>(field<5>(v));
+  w[6] = e4m3_of_digits<false>(field<6>(v));
+  w[7] = e4m3_of_digits<false>(field<7>(v));
+  w[8] = e4m3_of_digits<false>(field<8>(v));
+  w[9] = e4m3_of_digits<false>(field<9>(v));
+  w[10] = e4m3_of_digits<true>(field<10>(v));
 }
+static_assert(kPlanes == 11 && 5 * (kPlanes - 1) + 6 <= 56, "eleven fields in the first seven bytes");
 
 // Byte offset, within one (stage, plane) block, of the 16 indices
 // 16*half .. 16*half+15 of column col (canonical K-major layout).
