@@ -195,22 +195,20 @@ __device__ __forceinline__ i64 plane_off(i64 col, int half) {
 
 // ---------------------------------------------------------------------------
 // Column splitting: X (rows r0 .. r0 + nsub*kSub of an m x c matrix) ->
-// planes.  Grid (ceil(c / 8), nsub), 512 threads: block (g, s) takes the
-// 8-column group g of the layout (columns 8g .. 8g+7) over sub-chunk s, so
-// that for each stage and plane its digits form one contiguous 256-byte run
-// (8 columns x 32 indices).  Warp w takes stages 16 it + w, it = 0..7 (only
+// planes.  Grid (ceil(c / 4), nsub), 512 threads: block (g, s) takes columns
+// 4g .. 4g+3 over sub-chunk s.  Warp w takes stages 16 it + w, it = 0..7 (only
 // those below nst, for the short Y of an update); lane l handles rows 4 (l mod
-// 4) .. + 3 of both halves of the stage in column 8g + l / 4.  A warp load
-// thus touches 8 lines and a warp store writes 128 consecutive bytes of a run
-// (with 16 rows a lane, four columns' worth of lines per load, the kernel was
-// bound by the L1's line rate: 3.6 TB/s).  Two passes over the sub-chunk: the
-// column maxima (scales), then the digits; the second pass re-reads from L2
-// (two blocks an SM: 256 KiB each, 80 MB over the chip).
+// 8) .. + 3 of the stage in column 4g + l / 8.  A warp load thus reads whole
+// lines and a warp store writes two runs of 64 bytes of a plane (4 columns x
+// 16 indices each).  Two passes over the sub-chunk: the column maxima
+// (scales), then the digits; the second pass re-reads from L2 what two blocks
+// an SM leave there (128 KiB each, 40 MB over the chip).
 // Tiles of T columns (T a multiple of 8); plane block
 // (s, tile, st, i) starts at byte
 // (((s * ntile + tile) * kStagesPerSub + st) * kPlanes + i) * T * 32 with
 // ntile = ceil(c / T); exps: [s * c + col].  Columns past c of the last
 // group are written as zero digits (the tile padding; never read).
+constexpr int kSplitCols = 4;
 constexpr int kSplitWarps = 16;
 
 // 4 consecutive entries xc[row .. row+3] (zero past m or for a column past
@@ -239,59 +237,62 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 2) ozaki_split_kernel(const 
   stream_wait();
   if (status && *status) return;
   const int g = blockIdx.x, s = blockIdx.y, t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int cl = lane >> 2, quad = lane & 3;
-  const int col = 8 * g + cl;
+  const int cl = lane >> 3, quad = lane & 7;
+  const int col = kSplitCols * g + cl;
   const bool colok = col < c;
   const i64 base = r0 + (i64)s * kSub + 4 * quad;
   const double* xc = X + (i64)(colok ? col : 0) * ldx;
   const bool vec = (ldx & 1) == 0 && (reinterpret_cast<uintptr_t>(X + r0) & 15) == 0;  // rows are multiples of 4
   // pass 1: the column's largest exponent (zeros and subnormals do not set the scale) and Inf/NaN
   int emax = 0;
-#pragma unroll 2
+#pragma unroll 4
   for (int st = warp; st < nst; st += kSplitWarps) {
-    unsigned long long b0[4], b1[4];
-    load4(xc, base + st * kStage, m, colok, vec, b0);
-    load4(xc, base + st * kStage + 16, m, colok, vec, b1);
+    unsigned long long b[4];
+    load4(xc, base + st * kStage, m, colok, vec, b);
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      emax = max(emax, max((int)(b0[k] >> 52) & 0x7FF, (int)(b1[k] >> 52) & 0x7FF));
+    for (int k = 0; k < 4; ++k) emax = max(emax, (int)(b[k] >> 52) & 0x7FF);
   }
-  // lanes l, l ^ 1, l ^ 2, l ^ 3 hold the same column
-  emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 1));
-  emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 2));
-  __shared__ int red_max[kSplitWarps][8];
-  __shared__ int e_col[8];
+  // the eight lanes of a column
+#pragma unroll
+  for (int o = 1; o < 8; o *= 2) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+  __shared__ int red_max[kSplitWarps][kSplitCols];
+  __shared__ int e_col[kSplitCols];
   if (quad == 0) red_max[warp][cl] = emax;
   __syncthreads();
-  if (t < 8) {
+  if (t < kSplitCols) {
     int E = 0;
     for (int w = 0; w < kSplitWarps; ++w) E = max(E, red_max[w][t]);
     // |x| < 2^(E - 1022) for biased exponent E; scale e with |x| < 2^e: e = E - 1022
     const int e = E == 0x7FF ? kExpBad : (E == 0 ? kExpZero : E - 1022);
     e_col[t] = e;
-    if (8 * g + t < c) exps[(i64)s * c + 8 * g + t] = e;
+    if (kSplitCols * g + t < c) exps[(i64)s * c + kSplitCols * g + t] = e;
   }
   __syncthreads();
   const int e = e_col[cl];
-  // pass 2: digits, 4 bytes per plane and half
+  // pass 2: digits, 4 bytes per plane; the stage after the next is fetched while this one's digits are formed
   const int ntile = (c + T - 1) / T;
-  uint8_t* dst0 = planes + ((i64)s * ntile + col / T) * kStagesPerSub * kPlanes * T * kStage + plane_off(col % T, 0) +
-                  4 * quad;
-  // the next stage's entries are fetched while this one's digits are formed
+  uint8_t* dst = planes +
+                 (((i64)s * ntile + col / T) * kStagesPerSub + warp) * kPlanes * T * kStage +
+                 plane_off(col % T, quad >> 2) + 4 * (quad & 3);
   unsigned long long b[2][4];
 #pragma unroll
-  for (int h = 0; h < 2; ++h) load4(xc, base + warp * kStage + 16 * h, m, colok && warp < nst, vec, b[h]);
+  for (int h = 0; h < 2; ++h) {
+    const int st = warp + h * kSplitWarps;
+    load4(xc, base + st * kStage, m, colok && st < nst, vec, b[h]);
+  }
 #pragma unroll 1
-  for (int st = warp; st < nst; st += kSplitWarps) {
-    uint8_t* dst = dst0 + (i64)st * kPlanes * T * kStage;
+  for (int st0 = warp; st0 < nst; st0 += 2 * kSplitWarps) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
+      const int st = st0 + h * kSplitWarps, next = st + 2 * kSplitWarps;
       uint32_t w[kPlanes];
       digits4(b[h], e, w);
-      const int next = st + kSplitWarps;
-      load4(xc, base + next * kStage + 16 * h, m, colok && next < nst, vec, b[h]);
+      load4(xc, base + next * kStage, m, colok && next < nst, vec, b[h]);
+      if (st < nst) {
 #pragma unroll
-      for (int i = 0; i < kPlanes; ++i) *reinterpret_cast<uint32_t*>(dst + (i64)i * T * kStage + 128 * h) = w[i];
+        for (int i = 0; i < kPlanes; ++i) *reinterpret_cast<uint32_t*>(dst + (i64)i * T * kStage) = w[i];
+      }
+      dst += (i64)kSplitWarps * kPlanes * T * kStage;
     }
   }
 }
@@ -1078,11 +1079,11 @@ cudaError_t tn_product_emulated(i64 m, int p, int q, const double* X, i64 ldx, c
   for (i64 r0 = 0; r0 < m; r0 += ch) {
     const i64 nsub = ((m - r0 < ch ? m - r0 : ch) + kSub - 1) / kSub;
     prof_begin(kMisc, st);
-    launch(ozaki_split_kernel, dim3((unsigned)((p + 7) / 8), (unsigned)nsub), 32 * kSplitWarps, 0, st, X, ldx, m, r0, p, kTcM, kStagesPerSub, px, ex, status);
+    launch(ozaki_split_kernel, dim3((unsigned)((p + kSplitCols - 1) / kSplitCols), (unsigned)nsub), 32 * kSplitWarps, 0, st, X, ldx, m, r0, p, kTcM, kStagesPerSub, px, ex, status);
     prof_end(kMisc, 0.0, st);
     if (!same) {
       prof_begin(kMisc, st);
-      launch(ozaki_split_kernel, dim3((unsigned)((q + 7) / 8), (unsigned)nsub), 32 * kSplitWarps, 0, st, Y, ldy, m, r0, q, kTcN, kStagesPerSub, py, ey, status);
+      launch(ozaki_split_kernel, dim3((unsigned)((q + kSplitCols - 1) / kSplitCols), (unsigned)nsub), 32 * kSplitWarps, 0, st, Y, ldy, m, r0, q, kTcN, kStagesPerSub, py, ey, status);
       prof_end(kMisc, 0.0, st);
     }
     OzArgs a{};
@@ -1148,7 +1149,7 @@ cudaError_t nn_update_emulated(i64 M, int N, int K, const double* X, i64 ldx, co
     const int kc = (int)(K - k0 < kSub ? K - k0 : kSub);
     const int nst = (kc + kStage - 1) / kStage;
     prof_begin(kMisc, st);
-    launch(ozaki_split_kernel, dim3((unsigned)((N + 7) / 8), 1u), 32 * kSplitWarps, 0, st, Y, ldy, k0 + kc, k0, N, kTcN, nst, py, ey, status);
+    launch(ozaki_split_kernel, dim3((unsigned)((N + kSplitCols - 1) / kSplitCols), 1u), 32 * kSplitWarps, 0, st, Y, ldy, k0 + kc, k0, N, kTcN, nst, py, ey, status);
     prof_end(kMisc, 0.0, st);
     for (i64 r0 = 0; r0 < M; r0 += rows) {
       const i64 live = M - r0 < rows ? M - r0 : rows;
