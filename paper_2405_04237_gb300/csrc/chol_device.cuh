@@ -96,9 +96,14 @@ __device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* rows, 
                               unsigned short* tab, int* broken) {
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   if (t == 0) *broken = -1;
-  for (int row = warp; row < kb; row += T / 32) {
-    const int k = kb - 1 - row, start = k * (k + 1) / 2 + k * nx;
-    for (int c = row + lane; c < kb + nx; c += 32) tab[start + c - row] = (unsigned short)((row << 8) | c);
+  const int total = kb * (kb + 1) / 2 + kb * nx;
+  for (int e = t; e < total; e += T) {  // row kb-1-k starts at k (k + 1) / 2 + k nx
+    const float h = (float)nx + 0.5f;
+    int k = (int)(sqrtf(h * h + 2.0f * (float)e) - h);
+    while ((k + 1) * (k + 2) / 2 + (k + 1) * nx <= e) ++k;
+    while (k * (k + 1) / 2 + k * nx > e) --k;
+    const int row = kb - 1 - k;
+    tab[e] = (unsigned short)((row << 8) | (row + e - k * (k + 1) / 2 - k * nx));
   }
   __syncthreads();
   const int np = (kb + nx - 1 + 31) / 32 > 0 ? (kb + nx - 1 + 31) / 32 : 1;
@@ -155,9 +160,9 @@ __device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* rows, 
     rs[j] = r;
   }
   __syncthreads();
-  for (int e = t; e < done * (kb + nx); e += T) {
-    const int j = e / (kb + nx), c = e - j * (kb + nx);
-    if (c > j) {
+  for (int e = t; e < total; e += T) {
+    const int j = tab[e] >> 8, c = tab[e] & 255;
+    if (c > j && j < done) {
       const double w = Ws[j * ld + c], r = rs[j], q = w * r;
       Ws[j * ld + c] = fma(fma(-q, dg[j], w), r, q);
     }
