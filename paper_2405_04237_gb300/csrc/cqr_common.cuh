@@ -191,10 +191,9 @@ cudaError_t gram_chol(i64 m, int b, const double* X, i64 ldx, double* part, doub
 // ---------------------------------------------------------------------------
 // Row-wise forward substitution  X := X U^{-1}  (X m x b, b <= kTrsmMaxB),
 // using the reciprocals rinv of U's diagonal.  Wider panels are solved in
-// blocks of kTrsmMaxB columns with the coupling applied by the GEMM kernel:
-// 64 keeps two blocks (eight warps) per SM where a 128-wide tile of rows
-// and U would fill the shared memory with one block of four warps
-// (b = 128: 0.78 -> 1.13 TFLOP/s on GB300).
+// blocks of kTrsmMaxB columns with the coupling applied by the GEMM kernel: a
+// row of 64 columns fits in the registers of a thread, three blocks of four
+// warps per SM.
 constexpr int kTrsmMaxB = 64;
 // With `skip` non-null and *skip set on the device, the launch does nothing.
 // early = false: no early start (see launch()).
