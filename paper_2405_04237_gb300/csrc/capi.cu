@@ -315,7 +315,7 @@ cudaError_t mcqr2gs_run(i64 m, i64 n, int b, double* Q, i64 ldq, double* R, i64 
     TracePhase ph("cqr2_first_panel", 0);
     TRY(cqr_panel(m, b, Q, ldq, w.S1, b, w, 0, 0, st));
     TRY(cqr_panel(m, b, Q, ldq, w.S2, b, w, 0, 0, st, adaptive));
-    TRY(nn_product(b, b, b, w.S2, b, w.S1, b, R, ldr, 1.0, 0, 1, 1, w.status, st));
+    TRY(r_products(0, b, w.S2, w.S1, nullptr, R, ldr, w.status, st));
     TRY(io_panel_out(io, m, Q, ldq, 0, b, st));
   }
   for (i64 j = 1; j < k; ++j) {
@@ -359,8 +359,7 @@ cudaError_t mcqr2gs_run(i64 m, i64 n, int b, double* Q, i64 ldq, double* R, i64 
     }
     {  // R_jj = S2 S1;  R_{1:j-1,j} += Z S1
       TracePhase ph("r_update", pj);
-      TRY(nn_product(b, b, b, w.S2, b, w.S1, b, R + jb + jb * ldr, ldr, 1.0, 0, 1, 1, w.status, st));
-      TRY(nn_product(jb, b, b, w.Z, jb, w.S1, b, R + jb * ldr, ldr, 1.0, 1, 0, 1, w.status, st));
+      TRY(r_products(jb, b, w.S2, w.S1, w.Z, R, ldr, w.status, st));
     }
   }
   return join_side(st, side, &pending);
@@ -414,8 +413,7 @@ cudaError_t mcqr2gs_halving_run(i64 m, i64 n, int b, double* Q, i64 ldq, double*
     }
     {  // R_jj = S2 S1;  R_{1:j-1,j} += Z S1
       TracePhase ph("r_update", pc);
-      TRY(nn_product(bw, bw, bw, w.S2, bw, w.S1, bw, R + c0 + c0 * ldr, ldr, 1.0, 0, 1, 1, w.status, st));
-      if (c0 > 0) TRY(nn_product(c0, bw, bw, w.Z, c0, w.S1, bw, R + c0 * ldr, ldr, 1.0, 1, 0, 1, w.status, st));
+      TRY(r_products(c0, bw, w.S2, w.S1, w.Z, R, ldr, w.status, st));
     }
     bprev = bw;
     c0 += bw;

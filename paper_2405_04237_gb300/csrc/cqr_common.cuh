@@ -165,6 +165,11 @@ cudaError_t nn_product(i64 M, int N, int K, const double* A, i64 lda, const doub
 cudaError_t nn_product_t(i64 M, int N, int K, const double* A, i64 lda, const double* B, i64 ldb, int transb,
                          double* C, i64 ldc, double alpha, int beta, int a_upper, int b_upper, const int* status,
                          cudaStream_t st);
+// R_jj = S2 S1 and, for jb > 0, R_{1:j-1,j} += Z S1 (Z is jb x b, leading
+// dimension jb) in one launch; R points to the n x n factor, panel j starts at
+// column jb.
+cudaError_t r_products(i64 jb, int b, const double* S2, const double* S1, const double* Z, double* R, i64 ldr,
+                       const int* status, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
 // One-block Cholesky  W = U^T U (b x b, U upper, positive diagonal).

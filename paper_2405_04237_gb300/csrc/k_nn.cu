@@ -3,7 +3,7 @@
 // P -= Q_{1:j-1} Z (Alg. 9 step 7), the blocked part of wide triangular
 // solves, the adjoint's Q copyltu(M) product, and the small triangular
 // products R = R2 R1 (Alg. 3 step 3, Alg. 7 step 3), R_jj = S2 S1 and
-// R_{1:j-1,j} += Z S1 of Alg. 9.
+// R_{1:j-1,j} += Z S1 of Alg. 9 (these two in one launch).
 //
 // Each block computes a TM x TN output tile (256 threads, one MT x MT register
 // micro-tile per thread, TM * TN = 256 MT^2); K is staged through shared
@@ -14,11 +14,12 @@
 // blocks even out the last wave and the partial tiles: against 4 x 4, CQR2GS
 // 30011 x 90 takes 1717 instead of 1814 us, 60000 x 256 14.94 instead of 15.40
 // ms, 2^18 x 256 58.47 instead of 58.59 ms.  Every element sees the same
-// operations in the same order whatever the tile.  With beta = 1 the accumulator starts from C and every
-// term is one fused multiply-add (negated operand when alpha = -1), so the
-// update issues exactly one FP64 instruction per multiply-add.  Threads
-// whose four columns all lie beyond N skip the arithmetic (warp-uniform when
-// N is a multiple of 8), so narrow outputs do not pay for padding.
+// operations in the same order whatever the tile.  With beta = 1 the
+// accumulator starts from C and every term is one fused multiply-add (negated
+// operand when alpha = -1), so the update issues exactly one FP64 instruction
+// per multiply-add.  Threads whose columns all lie beyond N skip the
+// arithmetic (warp-uniform when N is a multiple of 8), so narrow outputs do
+// not pay for padding.
 #include "cqr_common.cuh"
 
 namespace cqr {
@@ -39,6 +40,13 @@ struct NnArgs {
   int beta, a_upper, b_upper, transb;
   int tiles_n;
   const int* status;
+  // a second product with the same B, N and K in the blocks from `first` on (kPair)
+  const double* A2;
+  i64 lda2;
+  double* C2;
+  i64 ldc2, M2;
+  int beta2, a_upper2;
+  i64 first;
 };
 
 template <int TM, int TN, int MT>
@@ -63,14 +71,24 @@ __device__ __forceinline__ void lds_micro(const double* p, double (&v)[MT]) {
   }
 }
 
-template <int TM, int TN, int MT, bool NEG>
+template <int TM, int TN, int MT, bool NEG, bool kPair = false>
 __global__ void __launch_bounds__(kNnThreads) nn_kernel(NnArgs a) {
   stream_wait();
   using Sh = NnShape<TM, TN, MT>;
   __shared__ __align__(16) double As[Sh::KC * Sh::SA];
   __shared__ __align__(16) double Bs[Sh::KC * Sh::SB];
   if (a.status && *a.status) return;
-  const i64 bid = blockIdx.x;
+  i64 bid = blockIdx.x;
+  if (kPair && bid >= a.first) {
+    bid -= a.first;
+    a.A = a.A2;
+    a.lda = a.lda2;
+    a.C = a.C2;
+    a.ldc = a.ldc2;
+    a.M = a.M2;
+    a.beta = a.beta2;
+    a.a_upper = a.a_upper2;
+  }
   const int tn_i = (int)(bid % a.tiles_n);
   const i64 m0 = (bid / a.tiles_n) * TM;
   const int n0 = tn_i * TN;
@@ -150,13 +168,19 @@ __global__ void __launch_bounds__(kNnThreads) nn_kernel(NnArgs a) {
 }
 
 template <int TM, int TN, int MT>
-void launch_nn(const NnArgs& a, bool neg, cudaStream_t st) {
+void launch_nn(const NnArgs& a, bool neg, bool pair, cudaStream_t st) {
   const i64 blocks = ((a.M + TM - 1) / TM) * a.tiles_n;
-  const Work64 w{2.0 * (double)a.M * a.N * a.K};
-  if (neg)
+  const Work64 w{2.0 * (double)(a.M + a.M2) * a.N * a.K};
+  if (pair) {
+    NnArgs b = a;
+    b.first = blocks;
+    launch(w, nn_kernel<TM, TN, MT, false, true>, (unsigned)(blocks + ((a.M2 + TM - 1) / TM) * a.tiles_n), kNnThreads, 0,
+           st, b);
+  } else if (neg) {
     launch(w, nn_kernel<TM, TN, MT, true>, (unsigned)blocks, kNnThreads, 0, st, a);
-  else
+  } else {
     launch(w, nn_kernel<TM, TN, MT, false>, (unsigned)blocks, kNnThreads, 0, st, a);
+  }
 }
 
 // Column tile for N columns and micro-tiles of MT (the widest is 16 MT).
@@ -168,6 +192,27 @@ int nn_tile_n(int N, int MT) {
 i64 nn_blocks(i64 M, int N, int MT) {
   const int TN = nn_tile_n(N, MT), TM = 256 * MT * MT / TN;
   return (M + TM - 1) / TM * ((N + TN - 1) / TN);
+}
+
+// Tile by size, then the launch (the FP64 operations of a pair count together).
+void run_nn(NnArgs& a, bool neg, bool pair, cudaStream_t st) {
+  const int MT = nn_blocks(a.M + a.M2, a.N, 2) >= kSMs ? 2 : 1;
+  const int TN = nn_tile_n(a.N, MT);
+  a.tiles_n = (a.N + TN - 1) / TN;
+  prof_begin(kUpdate, st);
+  if (MT == 2) {
+    switch (TN) {
+      case 8: launch_nn<128, 8, 2>(a, neg, pair, st); break;
+      case 16: launch_nn<64, 16, 2>(a, neg, pair, st); break;
+      default: launch_nn<32, 32, 2>(a, neg, pair, st); break;
+    }
+  } else {
+    if (TN == 8)
+      launch_nn<32, 8, 1>(a, neg, pair, st);
+    else
+      launch_nn<16, 16, 1>(a, neg, pair, st);
+  }
+  prof_end(kUpdate, 2.0 * (double)(a.M + a.M2) * a.N * a.K, st);
 }
 
 }  // namespace
@@ -182,7 +227,7 @@ cudaError_t nn_product_t(i64 M, int N, int K, const double* A, i64 lda, const do
                          double* C, i64 ldc, double alpha, int beta, int a_upper, int b_upper, const int* status,
                          cudaStream_t st) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  NnArgs a;
+  NnArgs a{};
   a.A = A;
   a.lda = lda;
   a.B = B;
@@ -198,23 +243,33 @@ cudaError_t nn_product_t(i64 M, int N, int K, const double* A, i64 lda, const do
   a.transb = transb;
   a.status = status;
   const bool neg = alpha < 0.0;
-  const int MT = nn_blocks(M, N, 2) >= kSMs ? 2 : 1;
-  const int TN = nn_tile_n(N, MT);
-  a.tiles_n = (N + TN - 1) / TN;
-  prof_begin(kUpdate, st);
-  if (MT == 2) {
-    switch (TN) {
-      case 8: launch_nn<128, 8, 2>(a, neg, st); break;
-      case 16: launch_nn<64, 16, 2>(a, neg, st); break;
-      default: launch_nn<32, 32, 2>(a, neg, st); break;
-    }
-  } else {
-    if (TN == 8)
-      launch_nn<32, 8, 1>(a, neg, st);
-    else
-      launch_nn<16, 16, 1>(a, neg, st);
-  }
-  prof_end(kUpdate, 2.0 * (double)M * N * K, st);
+  run_nn(a, neg, false, st);
+  return cudaGetLastError();
+}
+
+cudaError_t r_products(i64 jb, int b, const double* S2, const double* S1, const double* Z, double* R, i64 ldr,
+                       const int* status, cudaStream_t st) {
+  if (b <= 0) return cudaSuccess;
+  NnArgs a{};
+  a.A = S2;
+  a.lda = b;
+  a.B = S1;
+  a.ldb = b;
+  a.C = R + jb + jb * ldr;
+  a.ldc = ldr;
+  a.M = b;
+  a.N = b;
+  a.K = b;
+  a.a_upper = 1;
+  a.b_upper = 1;
+  a.status = status;
+  a.A2 = Z;
+  a.lda2 = jb;
+  a.C2 = R + jb * ldr;
+  a.ldc2 = ldr;
+  a.M2 = jb;
+  a.beta2 = 1;
+  run_nn(a, false, jb > 0, st);
   return cudaGetLastError();
 }
 
