@@ -70,26 +70,33 @@ __device__ __forceinline__ double reciprocal(double d) {
 // The rows of a trapezoid in shared memory: Ws (row-major, ld) holds the
 // upper triangle of a kb x kb diagonal block and nx further columns of the
 // same rows; on return row j of both is row j of the factor (the diagonal in
-// dg).  T threads, one barrier per row.  The rows are eliminated in the
+// dg).  T threads, one barrier per two rows.  The rows are eliminated in the
 // square-root-free form (pivots d_j, rows w_jc, multipliers l_jc = w_jc / d_j,
-// W_ac -= l_ja w_jc) and scaled by 1 / sqrt(d_j) at the end, all at once: a
-// column's chain of dependent FP64 operations is then six long instead of
-// nine.  In step j the pivot warps (32
-// columns each) apply the update of row j - 1 to row j and take the
-// reciprocal of its diagonal (each warp for itself), while the other warps
-// apply the update of row j - 1 to the rows below; at the end U_jc = w / u is
-// w r corrected with the fused residual, so exact quotients stay exact.  The
-// elements of the rows below are enumerated from the last row up (tab), so
-// the live ones are always a prefix and no lane idles.  While they
-// are few, the warps that share a scheduler (warp mod 4) with a pivot warp
-// leave the update to the others: their FP64 instructions, 64 clocks each,
-// would come between those of the pivot's chain.  Returns the row
-// that broke down, or -1.  Scratch in shared memory: rows (4 x us, us >= kb
-// + nx), tab (an entry per element), broken.  kb + nx <= 32 (T / 32 - 1).
+// W_ac -= l_ja w_jc) and scaled by 1 / sqrt(d_j) at the end, all at once.  In
+// step j (even) the pivot warps apply the updates of rows j - 2 and j - 1 to
+// rows j and j + 1 and eliminate the two; lanes 0 and 1 of each hold columns
+// j and j + 1 (the pivots travel by shuffles), the others 30 further columns.
+// Meanwhile the other warps apply the updates of rows j - 2 and j - 1 to the
+// rows below.  A column's chain is six dependent FP64 operations (64 clocks
+// each), and two columns share a barrier and a round trip through shared
+// memory.  At the end U_jc = w / u is w r corrected with the fused residual,
+// so exact quotients stay exact.  The elements of the rows below are
+// enumerated from the last row up (tab), so the live ones are always a prefix
+// and no lane idles.  While they are few, the warps that share a scheduler
+// (warp mod 4) with a pivot warp leave the update to the others: their FP64
+// instructions would come between those of the pivot's chain.  Returns the row
+// that broke down, or -1.  Scratch in shared memory: rows (8 x us, us >= kb
+// + nx), tab (an entry per element), broken.  kb + nx <= 30 (T / 32 - 1).
 
-// Elements per scheduler up to which the update fits behind the pivot's chain
-// (about 500 clocks: 8 warp instructions of 64).
+// Elements per scheduler up to which the update fits behind the pivots' chain
+// (about 1100 clocks: 8 elements a lane, two instructions of 64 each).
 constexpr int kQuietLen = 256;
+
+__device__ __forceinline__ bool good_pivot(double d) {
+  // d > 0 and finite, in integers (an FP64 comparison takes 64 clocks of the chain)
+  const int hi = __double2hiint(d);
+  return hi < 0x7FF00000 && (hi > 0 || (hi == 0 && __double2loint(d) != 0));
+}
 
 template <int T>
 __device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* rows, int us, double* dg,
@@ -106,37 +113,61 @@ __device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* rows, 
     tab[e] = (unsigned short)((row << 8) | (row + e - k * (k + 1) / 2 - k * nx));
   }
   __syncthreads();
-  const int np = (kb + nx - 1 + 31) / 32 > 0 ? (kb + nx - 1 + 31) / 32 : 1;
-  for (int j = 0; j < kb; ++j) {
+  for (int j = 0; j < kb; j += 2) {
     int bad = 0;
-    const double *pw = rows + ((j + 1) & 1) * 2 * us, *pl = pw + us;  // row j - 1: w, l
-    double *cw = rows + (j & 1) * 2 * us, *cl = cw + us;
+    // rows j - 2, j - 1 (w, l each) and this step's
+    const double* pw = rows + ((j >> 1) + 1 & 1) * 4 * us;
+    double* cw = rows + (j >> 1 & 1) * 4 * us;
+    const double *pl = pw + us, *pw2 = pw + 2 * us, *pl2 = pw + 3 * us;
+    const int rest = kb + nx - j - 2;  // columns beyond the two pivots'
+    const int np = rest > 30 ? (rest + 29) / 30 : 1;
     if (warp < np) {
-      const int c = j + 1 + 32 * warp + lane;
-      double* row = Ws + j * ld;
+      const bool two = j + 1 < kb;
+      const int c = lane < 2 ? j + lane : j + 30 * warp + lane;
       const bool live = c < kb + nx;
-      double d = row[j], w = live ? row[c] : 0.0;
-      if (j > 0) {
-        const double lj = pl[j];
-        d = fma(-lj, pw[j], d);
-        if (live) w = fma(-lj, pw[c], w);
-      }
-      // d > 0 and finite, in integers (an FP64 comparison takes 64 clocks of the chain)
-      const int dh = __double2hiint(d);
-      if (dh < 0x7FF00000 && (dh > 0 || (dh == 0 && __double2loint(d) != 0))) {
-        const double l = w * reciprocal(d);
-        if (live) {
-          cl[c] = l;
-          cw[c] = w;
-          row[c] = w;
+      double *r1 = Ws + j * ld, *r2 = r1 + ld;
+      double w1 = live ? r1[c] : 0.0, w2 = live && two && c > j ? r2[c] : 0.0;
+      if (j > 0 && live) {
+        const double x1 = pw[c], x2 = pw2[c];
+        w1 = fma(-pl[j], x1, w1);
+        w1 = fma(-pl2[j], x2, w1);
+        if (two) {
+          w2 = fma(-pl[j + 1], x1, w2);
+          w2 = fma(-pl2[j + 1], x2, w2);
         }
-        if (t == 0) dg[j] = d;
+      }
+      const double d1 = __shfl_sync(0xffffffffu, w1, 0);
+      if (good_pivot(d1)) {
+        const double l1 = w1 * reciprocal(d1);
+        const bool own = live && (lane >= 2 || warp == 0);
+        if (own && c > j) {
+          cw[c] = w1;
+          cw[us + c] = l1;
+          r1[c] = w1;
+        }
+        if (t == 0) dg[j] = d1;
+        if (two) {
+          w2 = fma(-__shfl_sync(0xffffffffu, l1, 1), w1, w2);
+          const double d2 = __shfl_sync(0xffffffffu, w2, 1);
+          if (good_pivot(d2)) {
+            const double l2 = w2 * reciprocal(d2);
+            if (own && c > j + 1) {
+              cw[2 * us + c] = w2;
+              cw[3 * us + c] = l2;
+              r2[c] = w2;
+            }
+            if (t == 0) dg[j + 1] = d2;
+          } else {
+            bad = 1;
+            if (t == 0) *broken = j + 1;
+          }
+        }
       } else {
         bad = 1;
         if (t == 0) *broken = j;
       }
     } else if (j > 0) {
-      const int k = kb - 1 - j, len = k * (k + 1) / 2 + k * nx;  // rows j+1 .. kb-1
+      const int k = kb - 2 - j, len = k > 0 ? k * (k + 1) / 2 + k * nx : 0;  // rows j+2 .. kb-1
       int w = warp - np, nw = T / 32 - np;
       if (np < 4 && len <= kQuietLen * (4 - np)) {
         const int q = warp & 3;
@@ -146,7 +177,8 @@ __device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* rows, 
       if (w >= 0)
         for (int e = 32 * w + lane; e < len; e += 32 * nw) {
           const int i = tab[e] >> 8, c = tab[e] & 255;
-          Ws[i * ld + c] = fma(-pl[i], pw[c], Ws[i * ld + c]);
+          const double v = fma(-pl[i], pw[c], Ws[i * ld + c]);
+          Ws[i * ld + c] = fma(-pl2[i], pw2[c], v);
         }
     }
     if (__syncthreads_or(bad)) break;

@@ -628,7 +628,7 @@ __device__ __noinline__ int reduce_cholesky(const Smem& s, const double* slots, 
   // scratch of the factorisation in the staging area (free between passes)
   double* rows = s.red;
   const int broken = chol_trapezoid<kBT>(U, b, b, 0, rows, kBNMax, s.dg,
-                                         reinterpret_cast<unsigned short*>(rows + 4 * kBNMax), sh_broken);
+                                         reinterpret_cast<unsigned short*>(rows + 8 * kBNMax), sh_broken);
   if (test && t == 0) {
     int r = 0;
     if (b > 1) {

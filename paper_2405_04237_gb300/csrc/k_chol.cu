@@ -32,7 +32,7 @@ constexpr int kTrapMax = 96;             // most columns kb + nx
 constexpr int kTrapTab = 2560;           // most elements (64 x 64: 2080; 32 x (32 + 61): 2480)
 
 struct TrapWork {
-  double rows[4 * kTrapMax];
+  double rows[8 * kTrapMax];
   double dg[kSmallChol];
   unsigned short tab[kTrapTab];
   int broken;
