@@ -48,7 +48,7 @@
 // FP32 accumulation is exact (an integer times 2^-18).  The dropped levels
 // weigh at most about 2^-56.6 of the scales' product per index.
 //
-// Schedule.  A block of 4 warps computes a 128 x 32 tile of C over its
+// Schedule.  A block of 16 warps computes a 128 x 32 tile of C over its
 // contraction range (a sub-chunk of a projection, all of K for an update).
 // Four shared-memory stages of 55 KiB rotate: one thread issues the bulk
 // copies of a stage (completion counted in bytes on the stage's "full"
@@ -761,10 +761,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) ozaki_tc_kernel(OzArgs a) {
 // for 32 columns, the MMAs re-read X twice as often), nor does holding the
 // second phases back until all first ones are done.
 //
-// Tile T is row tile T / tiles_q, column tile T % tiles_q.  The kernel is
-// bound by how fast stages reach shared memory, and X is four fifths of a
-// stage.  Contractions of up to four stages (K <= 128: every product with one
-// panel) therefore keep the row tile's X stages in their four slots while the
+// Tile T is row tile T / tiles_q, column tile T % tiles_q.  X is four
+// fifths of a stage's bytes.  Contractions of up to four stages (K <= 128:
+// every product with one panel) therefore keep the row tile's X stages in their four slots while the
 // block, which takes a contiguous run of tiles, goes through its column
 // tiles.  Longer contractions stream X with Y, and block c takes tiles c,
 // c + G, c + 2G, ... (G = grid size), so that the blocks running together
