@@ -79,7 +79,12 @@ __device__ __forceinline__ double reciprocal(double d) {
 // Meanwhile the other warps apply the updates of rows j - 2 and j - 1 to the
 // rows below.  A column's chain is six dependent FP64 operations (64 clocks
 // each), and two columns share a barrier and a round trip through shared
-// memory.  At the end U_jc = w / u is w r corrected with the fused residual,
+// memory.  Every pivot warp reads rows j and j + 1 in columns j and j + 1, so
+// none of these four is written in step j: a warp's own entries are those
+// beyond column j + 1, the pivots go to dg, and the updated entry (j, j + 1)
+// stays with its thread until the next step, which reads rows j + 2 and below
+// only (two warps never touch one entry between two barriers, unless to read).
+// At the end U_jc = w / u is w r corrected with the fused residual,
 // so exact quotients stay exact.  The elements of the rows below are
 // enumerated from the last row up (tab), so the live ones are always a prefix
 // and no lane idles.  While they are few, the warps that share a scheduler
@@ -113,8 +118,11 @@ __device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* rows, 
     tab[e] = (unsigned short)((row << 8) | (row + e - k * (k + 1) / 2 - k * nx));
   }
   __syncthreads();
+  double* kept = nullptr;  // warp 0, lane 1: entry (j, j + 1) of the step before
+  double kept_w = 0.0;
   for (int j = 0; j < kb; j += 2) {
     int bad = 0;
+    if (kept) *kept = kept_w;
     // rows j - 2, j - 1 (w, l each) and this step's
     const double* pw = rows + ((j >> 1) + 1 & 1) * 4 * us;
     double* cw = rows + (j >> 1 & 1) * 4 * us;
@@ -143,7 +151,12 @@ __device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* rows, 
         if (own && c > j) {
           cw[c] = w1;
           cw[us + c] = l1;
-          r1[c] = w1;
+          if (c > j + 1) {
+            r1[c] = w1;
+          } else {
+            kept = r1 + c;
+            kept_w = w1;
+          }
         }
         if (t == 0) dg[j] = d1;
         if (two) {
@@ -183,6 +196,7 @@ __device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* rows, 
     }
     if (__syncthreads_or(bad)) break;
   }
+  if (kept) *kept = kept_w;
   const int jb = *broken, done = jb >= 0 ? jb : kb;
   double* rs = rows;  // 1 / sqrt(d_j)
   for (int j = t; j < done; j += T) {
