@@ -52,18 +52,20 @@ __device__ __forceinline__ void sqrt_rsqrt(double d, double& u, double& r) {
   r = __hiloint2double(__double2hiint(rm) - (k << 20), __double2loint(rm));
 }
 
-// 1/d of a positive normal d: the FP32 reciprocal r0 of the mantissa m (24
-// bits), then r0 (1 + e + e^2) with the residual e = 1 - m r0 (third order
-// Newton: relative error e^3 < 2^-66 before rounding).
-__device__ __forceinline__ double reciprocal(double d) {
+// w / d for a positive d as w times the reciprocal: the FP32 reciprocal r0 of
+// the mantissa m (24 bits), then r0 (1 + e + e^2) with the residual e = 1 - m
+// r0 (third order Newton: relative error e^3 < 2^-66 before rounding).  Where
+// d or 1/d is subnormal (1/d of a subnormal d overflows, 1/d below 2^-1022
+// loses bits), the library's division.
+__device__ __forceinline__ double over_pivot(double w, double d) {
   const int hi = __double2hiint(d), lo = __double2loint(d);
   const int ex = (hi >> 20) - 1023;
-  if (ex == -1023 || ex > 1020) return 1.0 / d;  // subnormal d or result
+  if (ex == -1023 || ex > 1020) return w / d;
   const double m = __hiloint2double(hi - (ex << 20), lo);
   const double r0 = widen(__frcp_rn(__uint_as_float((127u << 23) | ((unsigned)(hi & 0xFFFFF) << 3) | ((unsigned)lo >> 29))));
   const double e = fma(-m, r0, 1.0);
   const double r = fma(r0, fma(e, e, e), r0);
-  return __hiloint2double(__double2hiint(r) - (ex << 20), __double2loint(r));
+  return w * __hiloint2double(__double2hiint(r) - (ex << 20), __double2loint(r));
 }
 
 // ---------------------------------------------------------------------------
@@ -146,7 +148,7 @@ __device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* rows, 
       }
       const double d1 = __shfl_sync(0xffffffffu, w1, 0);
       if (good_pivot(d1)) {
-        const double l1 = w1 * reciprocal(d1);
+        const double l1 = over_pivot(w1, d1);
         const bool own = live && (lane >= 2 || warp == 0);
         if (own && c > j) {
           cw[c] = w1;
@@ -163,7 +165,7 @@ __device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* rows, 
           w2 = fma(-__shfl_sync(0xffffffffu, l1, 1), w1, w2);
           const double d2 = __shfl_sync(0xffffffffu, w2, 1);
           if (good_pivot(d2)) {
-            const double l2 = w2 * reciprocal(d2);
+            const double l2 = over_pivot(w2, d2);
             if (own && c > j + 1) {
               cw[2 * us + c] = w2;
               cw[3 * us + c] = l2;

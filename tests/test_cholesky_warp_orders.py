@@ -86,3 +86,18 @@ def test_breakdown_in_any_warp_order(trapezoid, T, kb, nx, row):
         r, U = trapezoid(T, order, W, nx)
         assert r == row
         assert np.abs(U[:row] - want).max() < 1e-13, order
+
+
+# The whole range of pivots: down to subnormal Gram entries (columns of norm 1e-158), up to the largest.  W keeps
+# log2(s) + 1074 bits there and every term of the elimination is rounded to 2^-1074: kb of them move an entry of U by
+# a multiple (the condition number, below 3, and a factor for the root) of kb 2^-1074 / s of its scale sqrt(s).
+@pytest.mark.parametrize("T,kb,nx", [(256, 16, 0), (256, 40, 0), (256, 32, 20), (512, 64, 0)])
+@pytest.mark.parametrize("e", [-1050, -1040, -1026, -1023, -1022, -600, 0, 600, 1020, 1021])
+def test_pivots_of_any_size(trapezoid, T, kb, nx, e):
+    s = np.ldexp(1.0, e)
+    W = _gram(kb, nx, seed=29) * s
+    scale = np.sqrt(np.longdouble(2.0) ** e)
+    want = _factor_rows(np.ldexp(W, -e)) * scale  # exact: a power of two
+    r, U = trapezoid(T, np.arange(T // 32), W, nx)
+    assert r == -1
+    assert np.abs(U - want).max() <= 8 * kb * (2.0 ** (-1074 - e) + 2.0 ** -53) * scale
