@@ -73,7 +73,7 @@ constexpr int kBRMax = 4 * kBR;     // rows per staged sub-block for narrow pass
 constexpr int kBNMax = 128;         // widest matrix of the persistent path
 constexpr int kBSlot = 8448;        // doubles per partial slot: the Gram of b = 128 (528 tiles x 16)
 constexpr unsigned long long kBWaitNs = 2000000000ull;
-static_assert(kBSlot >= 528 * 16 && kBSlot >= (kBNMax / 2) * (kBNMax / 2), "a slot holds any partial");
+static_assert(kBSlot >= 528 * 16 && kBSlot >= (kBNMax / 2 + 3) * (kBNMax / 2 + 3), "a slot holds any partial");
 
 struct BMat {
   const double* A;
@@ -224,7 +224,13 @@ __device__ __noinline__ bool group_barrier(const BArgs& a, const Group& gr, unsi
 // threads that split the rows round-robin; the remaining E are "extra"
 // tiles, each owned by kBT / E threads that also split the rows.  Every
 // thread thus has one main and at most one extra 4 x 4 accumulator, and the
-// threads of a warp run the same instruction stream.
+// threads of a warp run the same instruction stream.  Starting widths are
+// multiples of 4; a width halved on the device (12 -> 6, 4 -> 2 -> 1) need not
+// be: then the last tiles hang over the range, read the columns beyond it (or
+// up to two entries beyond the tile, still this kernel's shared memory) and
+// form entries that nobody uses.
+__host__ __device__ constexpr int tiles4(int n) { return (n + 3) / 4; }
+
 struct TnMap {
   int sym;        // Gram: upper tiles of a T x T grid
   int tp, cnt;    // tiles along p (TN), tile count
@@ -249,8 +255,8 @@ __device__ __forceinline__ void tile_ij(const TnMap& mp, int id, int& i, int& j)
 __device__ TnMap make_map(int sym, int p, int q, int xc, int yc) {
   TnMap mp;
   mp.sym = sym;
-  mp.tp = p / 4;
-  const int tq = q / 4;
+  mp.tp = tiles4(p);
+  const int tq = tiles4(q);
   mp.cnt = sym ? mp.tp * (mp.tp + 1) / 2 : mp.tp * tq;
   int M = 1;
   while (M * 2 <= mp.cnt && M * 2 <= kBT) M *= 2;
@@ -565,7 +571,8 @@ struct Sums {
 };
 
 // Entries of a partial in a slot: whole 4 x 4 tiles.
-__device__ __forceinline__ int gram_entries(int b) { return 8 * (b / 4) * (b / 4 + 1); }
+__device__ __forceinline__ int gram_entries(int b) { return 8 * tiles4(b) * (tiles4(b) + 1); }
+__device__ __forceinline__ int tn_entries(int p, int q) { return 16 * tiles4(p) * tiles4(q); }
 
 // After a pass: waits until every CTA of the group has written its partial
 // (n entries) and tells where to read the sums.  Large groups: CTA r adds
@@ -659,7 +666,7 @@ __device__ __noinline__ int reduce_cholesky(const Smem& s, const double* slots, 
 __device__ __noinline__ void reduce_tn(const Smem& s, const double* slots, int G, int p, int q) {
   for (int e = threadIdx.x; e < p * q; e += kBT) {
     const int a = e / q, c = e % q;
-    s.M[e] = slot_sum(slots, G, 0, p / 4, a, c);
+    s.M[e] = slot_sum(slots, G, 0, tiles4(p), a, c);
   }
   __syncthreads();
 }
@@ -820,7 +827,7 @@ __global__ void __launch_bounds__(kBT, 1) batched_mcqr2gs_kernel(const __grid_co
         }
         run_pass(P, s, R0, R1, my);
       }
-      if (!(alive = meet(c0 == 0 ? gram_entries(bw) : c0 * bw, &sums))) break;
+      if (!(alive = meet(c0 == 0 ? gram_entries(bw) : tn_entries(c0, bw), &sums))) break;
       if (c0 > 0) {
         reduce_tn(s, sums.p, sums.G, c0, bw);  // Z (c0 x bw) in M
         ++phase;
@@ -915,7 +922,7 @@ __global__ void __launch_bounds__(kBT, 1) batched_mcqr2gs_kernel(const __grid_co
         run_pass(P, s, R0, R1, my);
       }
       if (wn > 0) {
-        if (!(alive = meet(bw * wn, &sums))) break;
+        if (!(alive = meet(tn_entries(bw, wn), &sums))) break;
         reduce_tn(s, sums.p, sums.G, bw, wn);  // Y (bw x wn) in M
         ++phase;
         for (int c = rank; c < wn; c += G)
