@@ -1108,7 +1108,9 @@ int cqr_factor_noalloc(int64_t m, int64_t n, double* A, int64_t lda, int panel_b
   if (!R) return -8;
   if (ldr < n) return -9;
   const Layout L = make_layout(m, n, b, variant);
-  if (L.nominal > (size_t)CQR_NOALLOC_SCRATCH_BYTES || L.total > (size_t)CQR_NOALLOC_SCRATCH_BYTES + kNoallocSlack)
+  // tiles cut to a product's shape can need less than the nominal ones: what fits the declared size is taken
+  if (std::min(L.nominal, L.total) > (size_t)CQR_NOALLOC_SCRATCH_BYTES ||
+      L.total > (size_t)CQR_NOALLOC_SCRATCH_BYTES + kNoallocSlack)
     return CQR_ERR_NOALLOC_TOO_LARGE;
   void* scratch = noalloc_scratch();
   if (!scratch) return CQR_ERR_CUDA;
