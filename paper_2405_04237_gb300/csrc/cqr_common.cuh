@@ -25,6 +25,19 @@ __host__ __device__ __forceinline__ i64 imin64(i64 a, i64 b) { return a < b ? a 
 // is a constant (not a device query) to keep results reproducible.
 constexpr int kSMs = 152;
 
+// A value for each device of the process.  Function attributes (the opt-in
+// sizes of shared memory) and occupancies belong to the device that is current
+// when they are set or asked for, so what remembers them does too.
+constexpr int kMaxDevices = 64;
+template <class T>
+struct PerDevice {
+  T v[kMaxDevices] = {};
+  T& here() {
+    int d = 0;
+    return v[cudaGetDevice(&d) == cudaSuccess && d >= 0 && d < kMaxDevices ? d : 0];
+  }
+};
+
 // ---------------------------------------------------------------------------
 // Split-m transposed product  C (p x q) = X^T Y  summed over m rows.
 // Stage 1: S persistent blocks split the rows (Gram) or the flattened (output

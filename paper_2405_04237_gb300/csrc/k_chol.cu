@@ -336,11 +336,11 @@ cudaError_t chol_factor(int b, double* W, i64 ldw, double* U, i64 ldu, double* r
   if (b <= kSmallChol) {
     launch(chol_small_kernel, 1, kSmallT, 0, st, a);
   } else {
-    static bool attr = false;
-    if (!attr) {
+    static PerDevice<bool> attr;
+    if (bool& set = attr.here(); !set) {
       cudaFuncSetAttribute(chol_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)chol_cluster_smem(CQR_MAX_PANEL));
-      attr = true;
+      set = true;
     }
     launch(chol_cluster_kernel, kClu, kSmallT, chol_cluster_smem(b), st, a);
   }

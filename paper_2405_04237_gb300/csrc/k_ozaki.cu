@@ -972,19 +972,19 @@ __global__ void __launch_bounds__(256) ozaki_reduce_kernel(const double* part, i
 }
 
 void up_attr() {
-  static bool done = false;
-  if (!done) {
+  static PerDevice<bool> done;
+  if (bool& set = done.here(); !set) {
     cudaFuncSetAttribute(ozaki_tc_update_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUpSmem);
     cudaFuncSetAttribute(ozaki_tc_update_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUpSmem);
-    done = true;
+    set = true;
   }
 }
 
 void tc_attr() {
-  static bool done = false;
-  if (!done) {
+  static PerDevice<bool> done;
+  if (bool& set = done.here(); !set) {
     cudaFuncSetAttribute(ozaki_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
-    done = true;
+    set = true;
   }
 }
 

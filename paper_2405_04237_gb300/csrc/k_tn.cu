@@ -296,7 +296,10 @@ constexpr i64 kSyrkSmall = 1200000;
 
 constexpr i64 kPartCap = 730000;
 
-int g_occ_syrk[2][129];
+struct SyrkOcc {
+  int o[2][129];
+};
+PerDevice<SyrkOcc> g_occ_syrk;
 
 SyrkPlan syrk_plan(i64 m, int b) {
   SyrkPlan s;
@@ -331,7 +334,7 @@ SyrkPlan syrk_plan(i64 m, int b) {
   }
   const size_t tile = (size_t)s.rb * (s.bp + 2), red = (size_t)17 * s.T;
   s.smem = (tile > red ? tile : red) * sizeof(double);
-  int& occ = g_occ_syrk[small ? 0 : 1][b];
+  int& occ = g_occ_syrk.here().o[small ? 0 : 1][b];
   if (occ == 0) {
     int o = 0;
     if (small) {
@@ -374,16 +377,17 @@ size_t tn_smem(int tp, int tq, int rb) {
   return (tile > red ? tile : red) * sizeof(double);
 }
 
-int g_occ_tn = 0;  // run-time form, at the largest shared-memory size
+PerDevice<int> g_occ_tn;  // run-time form, at the largest shared-memory size
 
 int tn_occupancy() {
-  if (g_occ_tn == 0) {
+  int& occ = g_occ_tn.here();
+  if (occ == 0) {
     cudaFuncSetAttribute(tn_partial_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 48 * 1024);
     int o = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, tn_partial_kernel<false>, kTnThreads, 48 * 1024);
-    g_occ_tn = o > 0 ? o : 1;
+    occ = o > 0 ? o : 1;
   }
-  return g_occ_tn;
+  return occ;
 }
 
 }  // namespace
