@@ -57,11 +57,14 @@ def _packed(A: torch.Tensor) -> torch.Tensor:
 
 
 def _native_rowmajor(A: torch.Tensor) -> bool:
-    """Whether cqr_colmajor takes A: a plain row-major CUDA FP64 matrix on the
-    current device with nothing recorded on it (autograd, function transforms)."""
+    """Whether cqr_colmajor takes A: a plain row-major CUDA FP64 matrix in
+    memory of its own, on the current device, with nothing recorded on it."""
     if type(A) not in (torch.Tensor, torch.nn.Parameter) or not A.is_cuda or A.dtype != torch.float64:
         return False
-    if torch._C._functorch.is_functorch_wrapped_tensor(A) or A.is_neg():
+    try:
+        if A.is_neg() or A.data_ptr() == 0:  # negated views; zeros without storage
+            return False
+    except RuntimeError:  # wrapped by a function transform: no storage to point to
         return False
     m, n = A.shape
     return (m > 0 and n > 0 and A.stride(1) == 1 and A.stride(0) >= n
