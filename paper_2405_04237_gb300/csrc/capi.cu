@@ -1024,7 +1024,8 @@ int cqr_factor_batched(int batch, const int64_t* m, const int64_t* n, const int6
   }
   double load[kBatchStreams] = {0};
   int rc = 0;
-  if (cudaMemsetAsync(status, 0, sizeof(int) * batch, st) != cudaSuccess || cudaEventRecord(pool->fork, st) != cudaSuccess)
+  if (cudaMemsetAsync(status, 0, sizeof(int) * batch, st) != cudaSuccess ||
+      cudaEventRecord(pool->fork, st) != cudaSuccess)
     rc = CQR_ERR_CUDA;
   for (int k = 0; k < ns && rc == 0; ++k)
     if (cudaStreamWaitEvent(pool->s[k], pool->fork, 0) != cudaSuccess ||
@@ -1051,7 +1052,8 @@ int cqr_factor_batched(int batch, const int64_t* m, const int64_t* n, const int6
   }
   // join: the caller's stream waits for every pool stream (also after an error)
   for (int k = 0; k < ns; ++k) {
-    if (cudaEventRecord(pool->done[k], pool->s[k]) != cudaSuccess || cudaStreamWaitEvent(st, pool->done[k], 0) != cudaSuccess)
+    if (cudaEventRecord(pool->done[k], pool->s[k]) != cudaSuccess ||
+        cudaStreamWaitEvent(st, pool->done[k], 0) != cudaSuccess)
       rc = CQR_ERR_CUDA;
   }
   delete[] order;
@@ -1137,7 +1139,8 @@ const char* cqr_status_string(int status) {
   if (status == CQR_ERR_ALLOC)
     return "workspace = NULL: the allocator registered with cqr_set_allocator returned no 256-byte aligned memory";
   if (status == CQR_STATUS_TIMEOUT) return "a bounded wait inside a kernel expired";
-  if (status > 0) return "Cholesky breakdown: the Gram matrix is not numerically positive definite (status = column + 1)";
+  if (status > 0)
+    return "Cholesky breakdown: the Gram matrix is not numerically positive definite (status = column + 1)";
   return "invalid argument (status = -(argument position))";
 }
 

@@ -62,7 +62,8 @@ __device__ __forceinline__ double over_pivot(double w, double d) {
   const int ex = (hi >> 20) - 1023;
   if (ex == -1023 || ex > 1020) return w / d;
   const double m = __hiloint2double(hi - (ex << 20), lo);
-  const double r0 = widen(__frcp_rn(__uint_as_float((127u << 23) | ((unsigned)(hi & 0xFFFFF) << 3) | ((unsigned)lo >> 29))));
+  const float f = __uint_as_float((127u << 23) | ((unsigned)(hi & 0xFFFFF) << 3) | ((unsigned)lo >> 29));
+  const double r0 = widen(__frcp_rn(f));
   const double e = fma(-m, r0, 1.0);
   const double r = fma(r0, fma(e, e, e), r0);
   return w * __hiloint2double(__double2hiint(r) - (ex << 20), __double2loint(r));

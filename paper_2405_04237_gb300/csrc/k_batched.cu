@@ -310,13 +310,15 @@ __device__ void tn_flush(const TnMap& mp, const Smem& s, int rows, double (&am)[
   __syncthreads();
   spill_acc(s.red, kBT, am);
   __syncthreads();
-  block_sums<kBT>(s.red, s.red, mp.M, min(mp.RG, rows), 1, mp.M, [slot](int id, int e, double x) { slot[id * 16 + e] = x; });
+  block_sums<kBT>(s.red, s.red, mp.M, min(mp.RG, rows), 1, mp.M,
+                  [slot](int id, int e, double x) { slot[id * 16 + e] = x; });
   __syncthreads();
   if (mp.E > 0) {
     spill_acc(s.red, kBT, ae);
     __syncthreads();
     double* slot_e = slot + (size_t)mp.M * 16;
-    block_sums<kBT>(s.red, s.red, mp.E, min(mp.tpt, rows), mp.tpt, 1, [slot_e](int id, int e, double x) { slot_e[id * 16 + e] = x; });
+    block_sums<kBT>(s.red, s.red, mp.E, min(mp.tpt, rows), mp.tpt, 1,
+                    [slot_e](int id, int e, double x) { slot_e[id * 16 + e] = x; });
     __syncthreads();
   }
 }
@@ -332,28 +334,28 @@ __device__ void nn_update_block(const Smem& s, int nr, int xc, int p, int cc, in
   const int nrt = (nr + TR - 1) / TR;  // blocks of padding rows are left out
   const int nblk = nrt * (q / TC);
   for (int bi = threadIdx.x; bi < nblk; bi += kBT) {
-  const int r0 = (bi % nrt) * TR, c0 = (bi / nrt) * TC;
-  double acc[TR][TC];
-#pragma unroll
-  for (int u = 0; u < TR; ++u)
-#pragma unroll
-    for (int v = 0; v < TC; ++v) acc[u][v] = s.tile[(size_t)(r0 + u) * s.ts + cc + c0 + v];
-#pragma unroll 2
-  for (int k = 0; k < p; ++k) {
-    double x[TR], mv[TC];
-#pragma unroll
-    for (int u = 0; u < TR; ++u) x[u] = s.tile[(size_t)(r0 + u) * s.ts + xc + k];
-#pragma unroll
-    for (int v = 0; v < TC; ++v) mv[v] = Mm[(size_t)k * q + c0 + v];
+    const int r0 = (bi % nrt) * TR, c0 = (bi / nrt) * TC;
+    double acc[TR][TC];
 #pragma unroll
     for (int u = 0; u < TR; ++u)
 #pragma unroll
-      for (int v = 0; v < TC; ++v) acc[u][v] = fma(-x[u], mv[v], acc[u][v]);
-  }
+      for (int v = 0; v < TC; ++v) acc[u][v] = s.tile[(size_t)(r0 + u) * s.ts + cc + c0 + v];
+#pragma unroll 2
+    for (int k = 0; k < p; ++k) {
+      double x[TR], mv[TC];
 #pragma unroll
-  for (int u = 0; u < TR; ++u)
+      for (int u = 0; u < TR; ++u) x[u] = s.tile[(size_t)(r0 + u) * s.ts + xc + k];
 #pragma unroll
-    for (int v = 0; v < TC; ++v) s.tile[(size_t)(r0 + u) * s.ts + cc + c0 + v] = acc[u][v];
+      for (int v = 0; v < TC; ++v) mv[v] = Mm[(size_t)k * q + c0 + v];
+#pragma unroll
+      for (int u = 0; u < TR; ++u)
+#pragma unroll
+        for (int v = 0; v < TC; ++v) acc[u][v] = fma(-x[u], mv[v], acc[u][v]);
+    }
+#pragma unroll
+    for (int u = 0; u < TR; ++u)
+#pragma unroll
+      for (int v = 0; v < TC; ++v) s.tile[(size_t)(r0 + u) * s.ts + cc + c0 + v] = acc[u][v];
   }
 }
 
@@ -579,8 +581,8 @@ __device__ __forceinline__ int tn_entries(int p, int q) { return 16 * tiles4(p) 
 // entries [r n / G, (r + 1) n / G) of all slots (up to 16 threads an entry,
 // their parts added in order), writes them to `res` and meets the others
 // again.
-__device__ __noinline__ bool exchange(const BArgs& a, const Group& gr, const Smem& s, const double* slots, double* res, int n,
-                         unsigned int* count, int* ok, Sums* out) {
+__device__ __noinline__ bool exchange(const BArgs& a, const Group& gr, const Smem& s, const double* slots,
+                                      double* res, int n, unsigned int* count, int* ok, Sums* out) {
   if (!group_barrier(a, gr, count, ok)) return false;
   out->p = slots;
   out->G = gr.G;
@@ -692,257 +694,257 @@ __global__ void __launch_bounds__(kBT, 1) batched_mcqr2gs_kernel(const __grid_co
   const int t = threadIdx.x;
   bool alive = true;
   for (int lev = 0; lev < a.lev.n; ++lev) {
-  __syncthreads();
-  if (t == 0) {
-    const int N = gridDim.x, cnt = a.lev.cnt[lev];
-    gr.g = ((blockIdx.x + 1) * cnt - 1) / N;
-    gr.node = a.lev.off[lev] + gr.g;
-    gr.lo = (int)((i64)gr.g * N / cnt);
-    gr.G = (int)((i64)(gr.g + 1) * N / cnt) - gr.lo;
-    gr.rank = blockIdx.x - gr.lo;
-    bar_count = 0;
-  }
-  __syncthreads();
-  const int rank = gr.rank, G = gr.G;
-  const int l0 = a.gstart[gr.node], l1 = a.gstart[gr.node + 1];
-  if (l0 == l1) continue;
-  // partial buffers: two by phase parity, or (large groups) one and the sums' place
-  const bool two = G > kDirectSum;
-  double* slots[2] = {a.part + (size_t)gr.lo * kBSlot, a.part + (size_t)(gridDim.x + gr.lo) * kBSlot};
-  int phase = 0;
-  auto cur = [&]() { return slots[two ? 0 : (phase & 1)]; };
-  auto meet = [&](int entries, Sums* out) {
-    return exchange(a, gr, s, cur(), slots[1], entries, &bar_count, &bar_ok, out);
-  };
-  double* s1g = a.s1 + (size_t)gr.lo * kBNMax * kBNMax;
-  int li = l0;
-  for (; li < l1 && alive; ++li) {
-    if (__syncthreads_or(*(volatile int*)a.abort)) {  // one decision for the CTA
-      alive = false;
-      break;
-    }
-    const int mi = a.order[li];
-    if (t == 0) mt = a.mats[mi];
     __syncthreads();
-    const int n = mt.n;
-    const i64 R0 = (i64)rank * mt.m / G, R1 = (i64)(rank + 1) * mt.m / G;
-    const bool oop = mt.Q != mt.A;
-    // zero R (column slices of this rank)
-    for (int c = rank; c < n; c += G)
-      for (int e = t; e < n; e += kBT) mt.R[e + (i64)c * n] = 0.0;
-    int bw = mt.b, bprev = 0;
-    bool failed = false;  // a breakdown: the group leaves this matrix
-    for (int c0 = 0; c0 < n && alive && !failed;) {
-      double* my = cur() + (size_t)rank * kBSlot;
-      Sums sums{};
-      // ---- the first CholeskyQR's Gram (with the update of step 4 for c0 > 0)
-      {
-        PassSpec P{};
-        P.dst = mt.Q;
-        P.ldd = mt.lda;
-        P.op2 = 1;
-        P.g0 = c0;
-        P.gb = bw;
-        if (c0 == 0) {
-          P.src = oop ? mt.A : mt.Q;
-          P.lds = mt.lda;
-          P.lo = 0;
-          P.hi = oop ? n : bw;
-          P.st_lo = 0;
-          P.st_hi = oop ? n : 0;
-        } else {  // A_{j:k} -= Q_{j-1} Y, Y (bprev x (n - c0)) in M
+    if (t == 0) {
+      const int N = gridDim.x, cnt = a.lev.cnt[lev];
+      gr.g = ((blockIdx.x + 1) * cnt - 1) / N;
+      gr.node = a.lev.off[lev] + gr.g;
+      gr.lo = (int)((i64)gr.g * N / cnt);
+      gr.G = (int)((i64)(gr.g + 1) * N / cnt) - gr.lo;
+      gr.rank = blockIdx.x - gr.lo;
+      bar_count = 0;
+    }
+    __syncthreads();
+    const int rank = gr.rank, G = gr.G;
+    const int l0 = a.gstart[gr.node], l1 = a.gstart[gr.node + 1];
+    if (l0 == l1) continue;
+    // partial buffers: two by phase parity, or (large groups) one and the sums' place
+    const bool two = G > kDirectSum;
+    double* slots[2] = {a.part + (size_t)gr.lo * kBSlot, a.part + (size_t)(gridDim.x + gr.lo) * kBSlot};
+    int phase = 0;
+    auto cur = [&]() { return slots[two ? 0 : (phase & 1)]; };
+    auto meet = [&](int entries, Sums* out) {
+      return exchange(a, gr, s, cur(), slots[1], entries, &bar_count, &bar_ok, out);
+    };
+    double* s1g = a.s1 + (size_t)gr.lo * kBNMax * kBNMax;
+    int li = l0;
+    for (; li < l1 && alive; ++li) {
+      if (__syncthreads_or(*(volatile int*)a.abort)) {  // one decision for the CTA
+        alive = false;
+        break;
+      }
+      const int mi = a.order[li];
+      if (t == 0) mt = a.mats[mi];
+      __syncthreads();
+      const int n = mt.n;
+      const i64 R0 = (i64)rank * mt.m / G, R1 = (i64)(rank + 1) * mt.m / G;
+      const bool oop = mt.Q != mt.A;
+      // zero R (column slices of this rank)
+      for (int c = rank; c < n; c += G)
+        for (int e = t; e < n; e += kBT) mt.R[e + (i64)c * n] = 0.0;
+      int bw = mt.b, bprev = 0;
+      bool failed = false;  // a breakdown: the group leaves this matrix
+      for (int c0 = 0; c0 < n && alive && !failed;) {
+        double* my = cur() + (size_t)rank * kBSlot;
+        Sums sums{};
+        // ---- the first CholeskyQR's Gram (with the update of step 4 for c0 > 0)
+        {
+          PassSpec P{};
+          P.dst = mt.Q;
+          P.ldd = mt.lda;
+          P.op2 = 1;
+          P.g0 = c0;
+          P.gb = bw;
+          if (c0 == 0) {
+            P.src = oop ? mt.A : mt.Q;
+            P.lds = mt.lda;
+            P.lo = 0;
+            P.hi = oop ? n : bw;
+            P.st_lo = 0;
+            P.st_hi = oop ? n : 0;
+          } else {  // A_{j:k} -= Q_{j-1} Y, Y (bprev x (n - c0)) in M
+            P.src = mt.Q;
+            P.lds = mt.lda;
+            P.lo = c0 - bprev;
+            P.hi = n;
+            P.st_lo = c0;
+            P.st_hi = n;
+            P.op1 = 2;
+            P.x0u = c0 - bprev;
+            P.pu = bprev;
+            P.c0u = c0;
+            P.qu = n - c0;
+            P.Mm = s.M;
+          }
+          run_pass(P, s, R0, R1, my);
+        }
+        if (!(alive = meet(gram_entries(bw), &sums))) break;
+        int broken = reduce_cholesky(s, sums.p, sums.G, bw, a.halve != 0, &sh_rej, &sh_broken);
+        ++phase;
+        while (a.halve && bw > 1 && sh_rej) {  // rejected panel: its Gram again at the narrower width
+          bw = halved(bw);
+          my = cur() + (size_t)rank * kBSlot;
+          PassSpec P{};
           P.src = mt.Q;
           P.lds = mt.lda;
-          P.lo = c0 - bprev;
+          P.lo = c0;
+          P.hi = c0 + bw;
+          P.op2 = 1;
+          P.g0 = c0;
+          P.gb = bw;
+          run_pass(P, s, R0, R1, my);
+          if (!(alive = meet(gram_entries(bw), &sums))) break;
+          broken = reduce_cholesky(s, sums.p, sums.G, bw, true, &sh_rej, &sh_broken);
+          ++phase;
+        }
+        if (!alive) break;
+        if (broken >= 0) {
+          if (rank == 0 && t == 0) atomicCAS(&a.status[mi], 0, c0 + broken + 1);
+          failed = true;
+          break;
+        }
+        // S1 for the R products (rank 0; read after the next barrier)
+        if (rank == 0)
+          for (int e = t; e < bw * bw; e += kBT) {
+            const int i = e % bw, c = e / bw;
+            s1g[e] = i <= c ? su(s, bw, i, c) : 0.0;
+          }
+        // ---- T1: P = A_j S1^{-1}, then the Gram of P (c0 == 0) or Z = Q_{1:j-1}^T P
+        __syncthreads();  // S1 saved from the unscaled factor
+        prescale_rows(s, bw);
+        {
+          my = cur() + (size_t)rank * kBSlot;
+          PassSpec P{};
+          P.src = mt.Q;
+          P.lds = mt.lda;
+          P.dst = mt.Q;
+          P.ldd = mt.lda;
+          P.lo = 0;
+          P.hi = c0 + bw;
+          P.st_lo = c0;
+          P.st_hi = c0 + bw;
+          P.op1 = 1;
+          P.t0 = c0;
+          P.tb = bw;
+          if (c0 == 0) {
+            P.op2 = 1;
+            P.g0 = 0;
+            P.gb = bw;
+          } else {
+            P.op2 = 2;
+            P.x0 = 0;
+            P.px = c0;
+            P.y0 = c0;
+            P.qy = bw;
+          }
+          run_pass(P, s, R0, R1, my);
+        }
+        if (!(alive = meet(c0 == 0 ? gram_entries(bw) : tn_entries(c0, bw), &sums))) break;
+        if (c0 > 0) {
+          reduce_tn(s, sums.p, sums.G, c0, bw);  // Z (c0 x bw) in M
+          ++phase;
+          // ---- RO: P -= Q_{1:j-1} Z, then the Gram of P
+          my = cur() + (size_t)rank * kBSlot;
+          PassSpec P{};
+          P.src = mt.Q;
+          P.lds = mt.lda;
+          P.dst = mt.Q;
+          P.ldd = mt.lda;
+          P.lo = 0;
+          P.hi = c0 + bw;
+          P.st_lo = c0;
+          P.st_hi = c0 + bw;
+          P.op1 = 2;
+          P.x0u = 0;
+          P.pu = c0;
+          P.c0u = c0;
+          P.qu = bw;
+          P.Mm = s.M;
+          P.op2 = 1;
+          P.g0 = c0;
+          P.gb = bw;
+          run_pass(P, s, R0, R1, my);
+          if (!(alive = meet(gram_entries(bw), &sums))) break;
+        }
+        broken = reduce_cholesky(s, sums.p, sums.G, bw, false, &sh_rej, &sh_broken);  // S2
+        ++phase;
+        if (broken >= 0) {
+          if (rank == 0 && t == 0) atomicCAS(&a.status[mi], 0, c0 + broken + 1);
+          failed = true;
+          break;
+        }
+        // R_jj = S2 S1 and (c0 > 0) R_{1:j-1,j} += Z S1, column slices of this
+        // rank; S1's upper triangle staged (packed by columns) in the tile area
+        {
+          double* s1p = s.tile;
+          for (int e = t; e < bw * (bw + 1) / 2; e += kBT) {
+            int c = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+            while ((c + 1) * (c + 2) / 2 <= e) ++c;
+            while (c * (c + 1) / 2 > e) --c;
+            const int i = e - c * (c + 1) / 2;
+            s1p[e] = s1g[(size_t)c * bw + i];
+          }
+          __syncthreads();
+          const int ncol = (bw - rank + G - 1) / G;  // this rank's columns c = rank + G * k
+          const int per = c0 + bw;                       // rows of R above and on the diagonal block
+          for (int e = t; e < ncol * per; e += kBT) {
+            const int c = rank + G * (e / per), r = e % per;
+            const double* s1c = s1p + c * (c + 1) / 2;  // S1[0..c][c]
+            if (r >= c0) {  // R_jj entry (r - c0, c), on or above the diagonal
+              const int rr = r - c0;
+              if (rr > c) continue;
+              double v = 0.0;
+              for (int i = rr; i <= c; ++i) v = fma(su(s, bw, rr, i), s1c[i], v);
+              mt.R[(c0 + rr) + (i64)(c0 + c) * n] = v;
+            } else {
+              double v = mt.R[r + (i64)(c0 + c) * n];
+              for (int i = 0; i <= c; ++i) v = fma(s.M[(size_t)r * bw + i], s1c[i], v);
+              mt.R[r + (i64)(c0 + c) * n] = v;
+            }
+          }
+          __syncthreads();
+        }
+        // ---- T2: Q_j = P S2^{-1}, then Y = Q_j^T A_{j+1:k}
+        const int wn = n - c0 - bw;
+        __syncthreads();  // the R products used the unscaled factor
+        prescale_rows(s, bw);
+        {
+          my = cur() + (size_t)rank * kBSlot;
+          PassSpec P{};
+          P.src = mt.Q;
+          P.lds = mt.lda;
+          P.dst = mt.Q;
+          P.ldd = mt.lda;
+          P.lo = c0;
           P.hi = n;
           P.st_lo = c0;
-          P.st_hi = n;
-          P.op1 = 2;
-          P.x0u = c0 - bprev;
-          P.pu = bprev;
-          P.c0u = c0;
-          P.qu = n - c0;
-          P.Mm = s.M;
+          P.st_hi = c0 + bw;
+          P.op1 = 1;
+          P.t0 = c0;
+          P.tb = bw;
+          if (wn > 0) {
+            P.op2 = 2;
+            P.x0 = c0;
+            P.px = bw;
+            P.y0 = c0 + bw;
+            P.qy = wn;
+          } else {
+            P.hi = c0 + bw;
+          }
+          run_pass(P, s, R0, R1, my);
         }
-        run_pass(P, s, R0, R1, my);
-      }
-      if (!(alive = meet(gram_entries(bw), &sums))) break;
-      int broken = reduce_cholesky(s, sums.p, sums.G, bw, a.halve != 0, &sh_rej, &sh_broken);
-      ++phase;
-      while (a.halve && bw > 1 && sh_rej) {  // rejected panel: its Gram again at the narrower width
-        bw = halved(bw);
-        my = cur() + (size_t)rank * kBSlot;
-        PassSpec P{};
-        P.src = mt.Q;
-        P.lds = mt.lda;
-        P.lo = c0;
-        P.hi = c0 + bw;
-        P.op2 = 1;
-        P.g0 = c0;
-        P.gb = bw;
-        run_pass(P, s, R0, R1, my);
-        if (!(alive = meet(gram_entries(bw), &sums))) break;
-        broken = reduce_cholesky(s, sums.p, sums.G, bw, true, &sh_rej, &sh_broken);
-        ++phase;
+        if (wn > 0) {
+          if (!(alive = meet(tn_entries(bw, wn), &sums))) break;
+          reduce_tn(s, sums.p, sums.G, bw, wn);  // Y (bw x wn) in M
+          ++phase;
+          for (int c = rank; c < wn; c += G)
+            for (int r = t; r < bw; r += kBT) mt.R[(c0 + r) + (i64)(c0 + bw + c) * n] = s.M[(size_t)r * wn + c];
+        }
+        bprev = bw;
+        c0 += bw;
       }
       if (!alive) break;
-      if (broken >= 0) {
-        if (rank == 0 && t == 0) atomicCAS(&a.status[mi], 0, c0 + broken + 1);
-        failed = true;
-        break;
-      }
-      // S1 for the R products (rank 0; read after the next barrier)
-      if (rank == 0)
-        for (int e = t; e < bw * bw; e += kBT) {
-          const int i = e % bw, c = e / bw;
-          s1g[e] = i <= c ? su(s, bw, i, c) : 0.0;
-        }
-      // ---- T1: P = A_j S1^{-1}, then the Gram of P (c0 == 0) or Z = Q_{1:j-1}^T P
-      __syncthreads();  // S1 saved from the unscaled factor
-      prescale_rows(s, bw);
-      {
-        my = cur() + (size_t)rank * kBSlot;
-        PassSpec P{};
-        P.src = mt.Q;
-        P.lds = mt.lda;
-        P.dst = mt.Q;
-        P.ldd = mt.lda;
-        P.lo = 0;
-        P.hi = c0 + bw;
-        P.st_lo = c0;
-        P.st_hi = c0 + bw;
-        P.op1 = 1;
-        P.t0 = c0;
-        P.tb = bw;
-        if (c0 == 0) {
-          P.op2 = 1;
-          P.g0 = 0;
-          P.gb = bw;
-        } else {
-          P.op2 = 2;
-          P.x0 = 0;
-          P.px = c0;
-          P.y0 = c0;
-          P.qy = bw;
-        }
-        run_pass(P, s, R0, R1, my);
-      }
-      if (!(alive = meet(c0 == 0 ? gram_entries(bw) : tn_entries(c0, bw), &sums))) break;
-      if (c0 > 0) {
-        reduce_tn(s, sums.p, sums.G, c0, bw);  // Z (c0 x bw) in M
-        ++phase;
-        // ---- RO: P -= Q_{1:j-1} Z, then the Gram of P
-        my = cur() + (size_t)rank * kBSlot;
-        PassSpec P{};
-        P.src = mt.Q;
-        P.lds = mt.lda;
-        P.dst = mt.Q;
-        P.ldd = mt.lda;
-        P.lo = 0;
-        P.hi = c0 + bw;
-        P.st_lo = c0;
-        P.st_hi = c0 + bw;
-        P.op1 = 2;
-        P.x0u = 0;
-        P.pu = c0;
-        P.c0u = c0;
-        P.qu = bw;
-        P.Mm = s.M;
-        P.op2 = 1;
-        P.g0 = c0;
-        P.gb = bw;
-        run_pass(P, s, R0, R1, my);
-        if (!(alive = meet(gram_entries(bw), &sums))) break;
-      }
-      broken = reduce_cholesky(s, sums.p, sums.G, bw, false, &sh_rej, &sh_broken);  // S2
-      ++phase;
-      if (broken >= 0) {
-        if (rank == 0 && t == 0) atomicCAS(&a.status[mi], 0, c0 + broken + 1);
-        failed = true;
-        break;
-      }
-      // R_jj = S2 S1 and (c0 > 0) R_{1:j-1,j} += Z S1, column slices of this
-      // rank; S1's upper triangle staged (packed by columns) in the tile area
-      {
-        double* s1p = s.tile;
-        for (int e = t; e < bw * (bw + 1) / 2; e += kBT) {
-          int c = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-          while ((c + 1) * (c + 2) / 2 <= e) ++c;
-          while (c * (c + 1) / 2 > e) --c;
-          const int i = e - c * (c + 1) / 2;
-          s1p[e] = s1g[(size_t)c * bw + i];
-        }
-        __syncthreads();
-        const int ncol = (bw - rank + G - 1) / G;  // this rank's columns c = rank + G * k
-        const int per = c0 + bw;                       // rows of R above and on the diagonal block
-        for (int e = t; e < ncol * per; e += kBT) {
-          const int c = rank + G * (e / per), r = e % per;
-          const double* s1c = s1p + c * (c + 1) / 2;  // S1[0..c][c]
-          if (r >= c0) {  // R_jj entry (r - c0, c), on or above the diagonal
-            const int rr = r - c0;
-            if (rr > c) continue;
-            double v = 0.0;
-            for (int i = rr; i <= c; ++i) v = fma(su(s, bw, rr, i), s1c[i], v);
-            mt.R[(c0 + rr) + (i64)(c0 + c) * n] = v;
-          } else {
-            double v = mt.R[r + (i64)(c0 + c) * n];
-            for (int i = 0; i <= c; ++i) v = fma(s.M[(size_t)r * bw + i], s1c[i], v);
-            mt.R[r + (i64)(c0 + c) * n] = v;
-          }
-        }
-        __syncthreads();
-      }
-      // ---- T2: Q_j = P S2^{-1}, then Y = Q_j^T A_{j+1:k}
-      const int wn = n - c0 - bw;
-      __syncthreads();  // the R products used the unscaled factor
-      prescale_rows(s, bw);
-      {
-        my = cur() + (size_t)rank * kBSlot;
-        PassSpec P{};
-        P.src = mt.Q;
-        P.lds = mt.lda;
-        P.dst = mt.Q;
-        P.ldd = mt.lda;
-        P.lo = c0;
-        P.hi = n;
-        P.st_lo = c0;
-        P.st_hi = c0 + bw;
-        P.op1 = 1;
-        P.t0 = c0;
-        P.tb = bw;
-        if (wn > 0) {
-          P.op2 = 2;
-          P.x0 = c0;
-          P.px = bw;
-          P.y0 = c0 + bw;
-          P.qy = wn;
-        } else {
-          P.hi = c0 + bw;
-        }
-        run_pass(P, s, R0, R1, my);
-      }
-      if (wn > 0) {
-        if (!(alive = meet(tn_entries(bw, wn), &sums))) break;
-        reduce_tn(s, sums.p, sums.G, bw, wn);  // Y (bw x wn) in M
-        ++phase;
-        for (int c = rank; c < wn; c += G)
-          for (int r = t; r < bw; r += kBT) mt.R[(c0 + r) + (i64)(c0 + bw + c) * n] = s.M[(size_t)r * wn + c];
-      }
-      bprev = bw;
-      c0 += bw;
+      if (rank == 0 && t == 0) a.bfinal[mi] = bw;
+      // the next matrix reuses M, U and the slots only after its first barrier
+      __syncthreads();
     }
-    if (!alive) break;
-    if (rank == 0 && t == 0) a.bfinal[mi] = bw;
-    // the next matrix reuses M, U and the slots only after its first barrier
-    __syncthreads();
-  }
-  if (!alive) {  // this group's unfinished matrices, and those of this CTA's later groups
-    if (rank == 0 && t == 0)
-      for (int k = li; k < l1; ++k) atomicCAS(&a.status[a.order[k]], 0, CQR_STATUS_TIMEOUT);
-  } else {
-    // the group's slots and S1 may be another group's at the next level
-    alive = group_barrier(a, gr, &bar_count, &bar_ok);
-  }
+    if (!alive) {  // this group's unfinished matrices, and those of this CTA's later groups
+      if (rank == 0 && t == 0)
+        for (int k = li; k < l1; ++k) atomicCAS(&a.status[a.order[k]], 0, CQR_STATUS_TIMEOUT);
+    } else {
+      // the group's slots and S1 may be another group's at the next level
+      alive = group_barrier(a, gr, &bar_count, &bar_ok);
+    }
   }
 }
 

@@ -361,7 +361,8 @@ cudaError_t gram_chol(i64 m, int b, const double* X, i64 ldx, double* part, doub
   const CholArgs a{b, W, ldw, U, ldu, rinv, col0, status, shift_fro, m, skip, reject};
   prof_begin(kCholesky, st);
   // early only behind a Gram kernel that leaves SMs free (its blocks take 44 KB of shared memory each)
-  launch(P <= kSMs ? Work64{0.0} : kNotEarly, gram_chol_kernel, (b * (b + 1) / 2 + 15) / 16, kSmallT, 0, st, part, P, a, counter);
+  launch(P <= kSMs ? Work64{0.0} : kNotEarly, gram_chol_kernel, (b * (b + 1) / 2 + 15) / 16, kSmallT, 0, st, part, P, a,
+         counter);
   prof_end(kCholesky, (double)b * b * b / 3.0, st);
   return cudaGetLastError();
 }

@@ -174,8 +174,8 @@ void launch_nn(const NnArgs& a, bool neg, bool pair, cudaStream_t st) {
   if (pair) {
     NnArgs b = a;
     b.first = blocks;
-    launch(w, nn_kernel<TM, TN, MT, false, true>, (unsigned)(blocks + ((a.M2 + TM - 1) / TM) * a.tiles_n), kNnThreads, 0,
-           st, b);
+    launch(w, nn_kernel<TM, TN, MT, false, true>, (unsigned)(blocks + ((a.M2 + TM - 1) / TM) * a.tiles_n), kNnThreads,
+           0, st, b);
   } else if (neg) {
     launch(w, nn_kernel<TM, TN, MT, true>, (unsigned)blocks, kNnThreads, 0, st, a);
   } else {

@@ -95,7 +95,8 @@ constexpr int kTcSmem = kTcRing * kTcStageBytes + 1024;  // + alignment slack
 constexpr uint32_t kTcCols = 512;   // TMEM columns: the levels' regions (384), rounded up to a power of 2
 constexpr int kMaxDynSmem = 227 * 1024 - 1024;  // opt-in dynamic shared memory per block, less static use
 static_assert(kTcSmem <= kMaxDynSmem, "projection ring fits in shared memory");
-static_assert(kTcCols >= 32 && kTcCols <= 512 && (kTcCols & (kTcCols - 1)) == 0, "TMEM allocation: power of 2, 32..512");
+static_assert(kTcCols >= 32 && kTcCols <= 512 && (kTcCols & (kTcCols - 1)) == 0,
+              "TMEM allocation: power of 2, 32..512");
 constexpr int kRegionLo = kLevelLo;  // level of TMEM region 0
 static_assert(kLevels * kTcN <= (int)kTcCols, "level regions fit in the TMEM allocation");
 static_assert(kLevelLo == 9 && kLevels == 2 * kLowLevels, "the MMA schedule and the groups of six levels");
@@ -456,7 +457,8 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
 __device__ __forceinline__ void tc_mma(uint32_t d, uint64_t ad, uint64_t bd, int nb, uint32_t acc) {
   const uint32_t idesc = kTcIdescM | ((uint32_t)(kTcN * nb >> 3) << 17);
   asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
       "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
 }
 
@@ -501,7 +503,8 @@ constexpr bool tc_schedule_ok() {
     if (first[r] != 1) return false;
   return true;
 }
-static_assert(tc_schedule_ok(), "MMA schedule: kept pairs once, regions in range, the first ones initialise the regions");
+static_assert(tc_schedule_ok(),
+              "MMA schedule: kept pairs once, regions in range, the first ones initialise the regions");
 #undef CQR_TC_SCHEDULE
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -542,7 +545,8 @@ __device__ __forceinline__ void load_levels(uint32_t lane_base, int c0, uint32_t
 // combine in unsigned 32-bit arithmetic (the offsets cancel modulo 2^32 and
 // |s_l + 32 s_l+1| < 2^28, so the two's-complement reading is the value).
 template <bool kMagic>
-__device__ __forceinline__ void group_sums(const uint32_t (&v)[kLevels][kEpiStep], int j, long long& g0, long long& g1) {
+__device__ __forceinline__ void group_sums(const uint32_t (&v)[kLevels][kEpiStep], int j, long long& g0,
+                                           long long& g1) {
   if (kMagic) {
     uint32_t b[kLevels];
 #pragma unroll
@@ -1051,11 +1055,13 @@ cudaError_t tn_product_emulated(i64 m, int p, int q, const double* X, i64 ldx, c
   for (i64 r0 = 0; r0 < m; r0 += ch) {
     const i64 nsub = ((m - r0 < ch ? m - r0 : ch) + kSub - 1) / kSub;
     prof_begin(kMisc, st);
-    launch(ozaki_split_kernel, dim3((unsigned)((p + kSplitCols - 1) / kSplitCols), (unsigned)nsub), 32 * kSplitWarps, 0, st, X, ldx, m, r0, p, kTcM, kStagesPerSub, px, ex, status);
+    launch(ozaki_split_kernel, dim3((unsigned)((p + kSplitCols - 1) / kSplitCols), (unsigned)nsub), 32 * kSplitWarps,
+           0, st, X, ldx, m, r0, p, kTcM, kStagesPerSub, px, ex, status);
     prof_end(kMisc, 0.0, st);
     if (!same) {
       prof_begin(kMisc, st);
-      launch(ozaki_split_kernel, dim3((unsigned)((q + kSplitCols - 1) / kSplitCols), (unsigned)nsub), 32 * kSplitWarps, 0, st, Y, ldy, m, r0, q, kTcN, kStagesPerSub, py, ey, status);
+      launch(ozaki_split_kernel, dim3((unsigned)((q + kSplitCols - 1) / kSplitCols), (unsigned)nsub),
+             32 * kSplitWarps, 0, st, Y, ldy, m, r0, q, kTcN, kStagesPerSub, py, ey, status);
       prof_end(kMisc, 0.0, st);
     }
     OzArgs a{};
@@ -1121,14 +1127,16 @@ cudaError_t nn_update_emulated(i64 M, int N, int K, const double* X, i64 ldx, co
     const int kc = (int)(K - k0 < kSub ? K - k0 : kSub);
     const int nst = (kc + kStage - 1) / kStage;
     prof_begin(kMisc, st);
-    launch(ozaki_split_kernel, dim3((unsigned)((N + kSplitCols - 1) / kSplitCols), 1u), 32 * kSplitWarps, 0, st, Y, ldy, k0 + kc, k0, N, kTcN, nst, py, ey, status);
+    launch(ozaki_split_kernel, dim3((unsigned)((N + kSplitCols - 1) / kSplitCols), 1u), 32 * kSplitWarps, 0, st, Y, ldy,
+           k0 + kc, k0, N, kTcN, nst, py, ey, status);
     prof_end(kMisc, 0.0, st);
     for (i64 r0 = 0; r0 < M; r0 += rows) {
       const i64 live = M - r0 < rows ? M - r0 : rows;
       const int rws = (int)((live + kTcM - 1) / kTcM * kTcM);
       prof_begin(kMisc, st);
       if (nst <= kRowStages)
-        launch(ozaki_rowsplit_short_kernel, (unsigned)(rws / 32), 32 * nst, 0, st, X, ldx, M, r0, k0, kc, px, ex, status);
+        launch(ozaki_rowsplit_short_kernel, (unsigned)(rws / 32), 32 * nst, 0, st, X, ldx, M, r0, k0, kc, px, ex,
+               status);
       else
         launch(ozaki_rowsplit_kernel, (unsigned)(rws / 128), 128, 0, st, X, ldx, M, r0, rws, k0, kc, px, ex, status);
       prof_end(kMisc, 0.0, st);

@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(kTnThreads) tn_partial_kernel(TnArgs a) {
     }
     // segment id = persistent block + tile (unique, increasing in rows)
     double* Pp = a.part + ((i64)blockIdx.x + tile) * (atp * atq);
-      if (G > 1) {
+    if (G > 1) {
       spill_acc(sm, kTnThreads, acc);
       __syncthreads();
       block_sums<kTnThreads>(sm, sm + 16 * kTnThreads, ntg, G, 1, ntg, [Pp, atp, NP](int id, int e, double x) {
@@ -521,7 +521,8 @@ cudaError_t tn_product(i64 m, int p, int q, const double* X, i64 ldx, const doub
   if (sym) {
     const i64 nsum = gram_partials(m, p, X, ldx, part, status, st);  // m == 0: none, the empty sum W = 0
     prof_begin(kReduce, st);
-    launch(Work64{(double)nsum * p * (p + 1) / 2}, syrk_reduce_kernel, (p * (p + 1) / 2 + 15) / 16, 256, 0, st, part, p, nsum, C, ldc, status);
+    launch(Work64{(double)nsum * p * (p + 1) / 2}, syrk_reduce_kernel, (p * (p + 1) / 2 + 15) / 16, 256, 0, st, part, p,
+           nsum, C, ldc, status);
     prof_end(kReduce, (double)nsum * p * (p + 1) / 2, st);
     return cudaGetLastError();
   }
@@ -554,8 +555,8 @@ cudaError_t tn_product(i64 m, int p, int q, const double* X, i64 ldx, const doub
   }
   const i64 pq = (i64)p * q;
   prof_begin(kReduce, st);
-  launch(Work64{(double)(P.S + P.ntiles) / P.ntiles * pq}, tn_reduce_kernel, (unsigned)((pq + 15) / 16), 256, 0, st, part, p, q, P.tp, P.tq, P.tiles_p, a.nb, m > 0 ? a.T : 0,
-                                           m > 0 ? a.P : 1, C, ldc, status);
+  launch(Work64{(double)(P.S + P.ntiles) / P.ntiles * pq}, tn_reduce_kernel, (unsigned)((pq + 15) / 16), 256, 0, st,
+         part, p, q, P.tp, P.tq, P.tiles_p, a.nb, m > 0 ? a.T : 0, m > 0 ? a.P : 1, C, ldc, status);
   prof_end(kReduce, m > 0 ? (double)(P.S + P.ntiles) / P.ntiles * pq : 0.0, st);
   return cudaGetLastError();
 }

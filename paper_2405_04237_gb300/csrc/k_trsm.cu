@@ -61,7 +61,8 @@ __device__ __forceinline__ void store_row(const double (&x)[B], double* p, i64 l
 // U's upper triangle (zero elsewhere) into Us [B][B + 1] and its reciprocals,
 // zero beyond b.
 template <int B>
-__device__ __forceinline__ void load_factor(int b, const double* U, i64 ldu, const double* rinv, double* Us, double* rv) {
+__device__ __forceinline__ void load_factor(int b, const double* U, i64 ldu, const double* rinv, double* Us,
+                                            double* rv) {
   for (int e = threadIdx.x; e < B * B; e += kRows) {
     const int i = e % B, c = e / B;
     Us[i * (B + 1) + c] = i <= c && c < b ? U[i + (i64)c * ldu] : 0.0;
@@ -70,8 +71,9 @@ __device__ __forceinline__ void load_factor(int b, const double* U, i64 ldu, con
 }
 
 template <int B>
-__global__ void __launch_bounds__(kRows, kMinBlocks<B>) trsm_rows_kernel(i64 m, int b, double* X, i64 ldx, const double* U, i64 ldu,
-                                                          const double* rinv, const int* status, const int* skip) {
+__global__ void __launch_bounds__(kRows, kMinBlocks<B>)
+    trsm_rows_kernel(i64 m, int b, double* X, i64 ldx, const double* U, i64 ldu, const double* rinv, const int* status,
+                     const int* skip) {
   stream_wait();
   __shared__ double Us[B * (B + 1)], rv[B];
   if (status && *status) return;
@@ -92,8 +94,8 @@ __global__ void __launch_bounds__(kRows, kMinBlocks<B>) trsm_rows_kernel(i64 m, 
 }
 
 template <int B>
-__global__ void __launch_bounds__(kRows, kMinBlocks<B>) trsm_rows_t_kernel(i64 m, int b, double* X, i64 ldx, const double* U, i64 ldu,
-                                                            const double* rinv) {
+__global__ void __launch_bounds__(kRows, kMinBlocks<B>)
+    trsm_rows_t_kernel(i64 m, int b, double* X, i64 ldx, const double* U, i64 ldu, const double* rinv) {
   stream_wait();
   __shared__ double Us[B * (B + 1)], rv[B];
   const i64 r = (i64)blockIdx.x * kRows + threadIdx.x;
@@ -145,7 +147,8 @@ cudaError_t trsm_rows_transposed(i64 m, int b, double* X, i64 ldx, const double*
   const i64 blocks = (m + kRows - 1) / kRows;
   prof_begin(kTrsm, st);
   with_width(b, [&](auto B) {
-    launch(Work64{(double)m * b * b}, trsm_rows_t_kernel<B>, (unsigned)blocks, kRows, 0, st, m, b, X, ldx, U, ldu, rinv);
+    launch(Work64{(double)m * b * b}, trsm_rows_t_kernel<B>, (unsigned)blocks, kRows, 0, st, m, b, X, ldx, U, ldu,
+           rinv);
   });
   prof_end(kTrsm, (double)m * b * b, st);
   return cudaGetLastError();
