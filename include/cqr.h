@@ -78,11 +78,15 @@ enum cqr_variant {
  * (tcgen05, accumulators in TMEM) with an error-free splitting of the FP64
  * operands (Ozaki scheme): each operand is scaled by powers of two along
  * the contraction (per column and 4096-row sub-chunk for a Gram matrix or
- * projection, per row for an update) and cut into 14 signed 4-bit digits
- * (56 bits); the 105 most significant digit-plane pairs are multiplied
- * exactly (FP32 accumulation of integers < 2^24) and recombined with one
- * rounding.  Not FP64 arithmetic, but FP64-accurate: the truncation drops
- * terms below about 2^-52 of the scales' product.  The Cholesky
+ * projection, per row for an update), rounded to 54 bits and a sign, and
+ * written in eleven balanced base-32 digits; the 76 most significant
+ * digit-plane pairs are multiplied exactly (FP32 accumulation of integers
+ * < 2^24) and recombined with one rounding to the nearest double.  Not FP64
+ * arithmetic, but FP64-accurate: the pairs left out are below about 2^-56 of
+ * the scales' product, an operand's rounding below 2^-55 of its scale (the
+ * root-mean-square error of a product is below that of an FP64 dot product:
+ * 0.10 / 0.08 / 0.015 against 0.14 / 0.12 / 0.06 units of 2^-53 ||x|| ||y||
+ * for 64 / 128 / 4096 terms).  The Cholesky
  * factorisations and the substitutions of the triangular solves stay native
  * FP64; a solve runs in 32-column substitution blocks, and the products that
  * couple the blocks (X_2 -= X_1 U_12, m rows) are emulated like the other
@@ -212,10 +216,10 @@ int cqr_factor(int64_t m, int64_t n, double* A, int64_t lda, int panel_b, double
  * Returns the same argument codes as cqr_factor, or
  * CQR_ERR_NOALLOC_TOO_LARGE when the sizes need more scratch than the array
  * holds (a cqr_workspace_size() up to CQR_NOALLOC_SCRATCH_BYTES fits; for
- * short matrices up to 16 MiB more); nothing is launched then.  It calls no cudaMalloc, cudaFree or allocating library
- * routine.  The first call on each device looks up the array's device
- * address (cudaGetSymbolAddress) with that device current; make that first
- * call before any stream capture.  All calls share the one array and it keeps
+ * short matrices up to 16 MiB more); nothing is launched then.  It calls no
+ * cudaMalloc, cudaFree or allocating library routine.  The first call on
+ * each device looks up the array's device address (cudaGetSymbolAddress)
+ * with that device current; make that first call before any stream capture.  All calls share the one array and it keeps
  * the last call's contents (each call clears what must start at zero), so
  * calls whose work overlaps on the GPU -- on different streams, or from
  * different threads -- race and give wrong results; order them on one stream
@@ -316,8 +320,8 @@ size_t cqr_batched_workspace_size(int batch, const int64_t* m, const int64_t* n,
  * cqr_batched_workspace_size.  CQR_BATCH_POOL forces the stream-pool
  * schedule; CQR_BATCH_GROUP(G) sets the CTAs per matrix of the persistent
  * launch (G must divide the SM count; 0 = default, groups of several sizes
- * chosen from the matrices' sizes); CQR_HALVE (persistent path only) applies the adaptive panel width
- * on the device. */
+ * chosen from the matrices' sizes); CQR_HALVE (persistent path only)
+ * applies the adaptive panel width on the device. */
 #define CQR_BATCH_POOL 0x1000
 #define CQR_BATCH_GROUP(G) ((G) << 16)
 
@@ -330,15 +334,19 @@ size_t cqr_batched_workspace_size(int batch, const int64_t* m, const int64_t* n,
  *   unless CQR_BATCH_POOL): ONE cooperative kernel launch with one CTA per
  *   SM.  Groups of CTAs take whole matrices (a static schedule: by default
  *   groups of several sizes, large matrices on many CTAs and small ones on
- *   few, else groups of G); the G CTAs of a group split the matrix's rows (the row-block
- *   distribution of Alg. 2 / Alg. 8), write partial sums of every m-row
- *   product to their own slots, meet at a group barrier and add the slots
- *   in rank order, each factoring the b x b Gram matrix redundantly (the
- *   redundant Cholesky of Alg. 2).  Each pass over a sub-block of rows
+ *   few, else groups of G); the G CTAs of a group split the matrix's rows
+ *   (the row-block distribution of Alg. 2 / Alg. 8), write partial sums of
+ *   every m-row product to their own slots, meet at a group barrier and add
+ *   the slots in rank order, each factoring the b x b Gram matrix redundantly
+ *   (the redundant Cholesky of Alg. 2).  Each pass over a sub-block of rows
  *   fuses a streaming step with the next m-row product (update + Gram,
  *   solve + projection, re-orthogonalisation + Gram).  Results match the
  *   single-matrix path to rounding (a different summation order), not
- *   bitwise.  Every group-barrier wait is bounded (2 s); on expiry the
+ *   bitwise.  The size of its group sets a matrix's summation order: by
+ *   default it depends on the other matrices of the batch, so the last bits
+ *   of a result do too (the same batch gives the same bits on every call);
+ *   with CQR_BATCH_GROUP(G), G > 0, a matrix gives the same bits in every
+ *   batch.  Every group-barrier wait is bounded (2 s); on expiry the
  *   unfinished matrices get CQR_STATUS_TIMEOUT.  With CQR_HALVE a rejected
  *   panel (see CQR_HALVE) is retried at half width on the device; read the
  *   final widths with cqr_batched_panel_widths().

@@ -1,10 +1,10 @@
 // Internal declarations shared by the CUDA translation units of the library.
 //
-// Every kernel here computes in FP64 on the CUDA-core FMA pipe (DFMA).  On
-// GB300 that pipe delivers 2 FP64 FMA per clock per SM (about 1.19 TFLOP/s
-// over 152 SMs), while `mma.sync ... .f64` measures slower (about 1.04
+// Every native kernel computes in FP64 on the CUDA-core FMA pipe (DFMA).  On
+// GB300 that pipe delivers 2 FP64 FMA per clock per SM (1.2585 TFLOP/s over
+// 152 SMs at 2070 MHz), while `mma.sync ... .f64` measures slower (1.10
 // TFLOP/s) and would also waste half of every symmetric Gram product, so the
-// tensor cores are not used.  At 2 DFMA per clock an SM consumes only
+// tensor cores serve the emulated products (k_ozaki.cu) only.  At 2 DFMA per clock an SM consumes only
 // about 8 bytes of operands per FMA issued, far under its share of HBM
 // bandwidth, so every kernel is bound by the FP64 pipe; the designs aim at
 // (a) issuing no FP64 instruction that the algorithm does not need, and
@@ -41,8 +41,8 @@ struct PerDevice {
 // ---------------------------------------------------------------------------
 // Split-m transposed product  C (p x q) = X^T Y  summed over m rows.
 // Stage 1: S persistent blocks split the rows (Gram) or the flattened (output
-// tile, row block) items into S equal contiguous ranges and write one partial tile per
-// (block, tile) segment.  Stage 2 adds each entry's segments in ascending
+// tile, row block) items into S equal contiguous ranges and write one partial
+// tile per (block, tile) segment.  Stage 2 adds each entry's segments in ascending
 // row order.  With sym != 0, X == Y and only entries on or above the
 // diagonal are formed (syrk); the reduce mirrors them.
 struct TnPlan {
@@ -53,7 +53,10 @@ struct TnPlan {
   int rb;            // rows per row block
 };
 TnPlan tn_plan(i64 m, int p, int q, int sym);
-size_t tn_partial_doubles(i64 m, int p, int q, int sym);  // S * p * q
+// Doubles of the partials: S p q for a Gram matrix of up to 128 columns (the
+// largest 128-wide piece of a wider one), else (S + ntiles) tp tq, a tile per
+// segment.
+size_t tn_partial_doubles(i64 m, int p, int q, int sym);
 // The same for a split into blocks of about 8192 (Gram) or 4096 staged
 // doubles whatever m is: what cqr_factor_noalloc counts against its array.
 // A finer split of a short matrix takes at most kNoallocSlack bytes more.
@@ -185,14 +188,17 @@ cudaError_t r_products(i64 jb, int b, const double* S2, const double* S1, const 
                        const int* status, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
-// One-block Cholesky  W = U^T U (b x b, U upper, positive diagonal).
+// Cholesky factorisation  W = U^T U (b x b, U upper, positive diagonal): one
+// block up to 64 columns, a cluster of eight blocks above (W's upper triangle
+// is scratch there and is overwritten).
 // Writes U (ldu; strict lower triangle zeroed) and rinv[j] = 1 / U_jj.
 // On breakdown at local column j, status is set to col0 + j + 1 (first
 // breakdown wins) and U_jj onward are NaN.  `shift_fro` != 0 applies the
 // shifted-CholeskyQR shift s = sqrt(m) * 2^-53 * trace(W) first (Alg. 4).
 // With `skip` non-null the second-pass rule of the runtime repetition
 // choice applies: if every entry of U - I is within 8u, U := I exactly and
-// *skip = 1 (else 0).  With `reject` non-null the panel test of the adaptive
+// *skip = 1 (else 0; valid when the launch has ended -- the cluster sets it to
+// 1 first and takes it back).  With `reject` non-null the panel test of the adaptive
 // panel width applies: *reject = 1 when b > 1 and the factorisation broke
 // down (status then left untouched) or (max U_jj / min U_jj)^2 > 1/(64 u),
 // else 0.  The kernel returns early, writing nothing, if *status != 0.

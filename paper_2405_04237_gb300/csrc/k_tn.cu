@@ -291,9 +291,20 @@ struct SyrkPlan {
   size_t smem;
 };
 
-// Row count x tile count below which the 128-thread kernel is used.
+// Row count x tile count (the work) below which the 128-thread kernel is used,
+// for up to 256 tiles: its smaller blocks spread a short matrix over more SMs.
+// Times of a panel, two Gram matrices each, with 128 / 512 threads, us: work
+// 1e5: b = 8 66 / 67, 16 81 / 83, 24 99 / 102, 32 125 / 125, 48 213 / 215, 64
+// 320 / 321, 80 439 / 424; work 1.2e6: 209 / 206, 224 / 211, 220 / 213, 240 /
+// 226, 317 / 273, 402 / 365, 515 / 472.  So it gains up to 3 % below 3e5 and
+// costs 2 to 16 % from 6e5 up to the line, which lies too far up: at 3e5 it
+// would cost nothing.
 constexpr i64 kSyrkSmall = 1200000;
 
+// Doubles of partial triangles up to which the 128-thread kernel takes more
+// than one block per SM: 5.8 MB of a small call's workspace.  It binds for 41
+// to 69 columns.  A panel of 48 columns, work 1.2e6: 318 us, 372 with one block
+// per SM, 285 without a limit; 64 columns: 403, 393 and 383.
 constexpr i64 kPartCap = 730000;
 
 struct SyrkOcc {
@@ -321,9 +332,8 @@ SyrkPlan syrk_plan(i64 m, int b) {
   // kernel, twice that of the small one
   const int per = (small ? 4096 : 8192) / (s.bp + 2);
   s.rb = per >= s.RG ? per / s.RG * s.RG : s.RG;
-  // Blocks: at least 32 rows each, at most kMaxResident per SM, and for the
-  // widths where that many partial triangles would take longer to add up
-  // than they save, about kPartCap doubles of them.
+  // Blocks: at least 32 rows each, at most kMaxResident per SM, and above one
+  // per SM at most kPartCap doubles of partial triangles.
   const i64 min_rows = 32;
   i64 want = (m + min_rows - 1) / min_rows;
   if (want < 1) want = 1;
