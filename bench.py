@@ -422,9 +422,9 @@ def bench_emulated(P, A, Q, R, b, args, flops, t_native):
 
 # DRAM bytes per launch of the update kernel class, from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum) of every update launch of an
-# m = 2^18, n = 1024, b = 128 factorisation: 33.29 GB over 45 launches,
+# m = 2^18, n = 1024, b = 128 factorisation: 33.41 GB over 38 launches,
 # scaled by m (every launch that matters streams m-row operands).
-UPDATE_DRAM_BYTES_PER_LAUNCH_2P18 = 33.29e9 / 45
+UPDATE_DRAM_BYTES_PER_LAUNCH_2P18 = 33.41e9 / 38
 
 
 def update_traffic(m, n, b, dom, emulated):

@@ -320,7 +320,7 @@ size_t cqr_batched_workspace_size(int batch, const int64_t* m, const int64_t* n,
  * cqr_batched_workspace_size.  CQR_BATCH_POOL forces the stream-pool
  * schedule; CQR_BATCH_GROUP(G) sets the CTAs per matrix of the persistent
  * launch (G must divide the SM count; 0 = default, groups of several sizes
- * chosen from the matrices' sizes); CQR_HALVE (persistent path only)
+ * or equal groups, whichever the matrices' sizes make faster); CQR_HALVE (persistent path only)
  * applies the adaptive panel width on the device. */
 #define CQR_BATCH_POOL 0x1000
 #define CQR_BATCH_GROUP(G) ((G) << 16)
@@ -334,7 +334,8 @@ size_t cqr_batched_workspace_size(int batch, const int64_t* m, const int64_t* n,
  *   unless CQR_BATCH_POOL): ONE cooperative kernel launch with one CTA per
  *   SM.  Groups of CTAs take whole matrices (a static schedule: by default
  *   groups of several sizes, large matrices on many CTAs and small ones on
- *   few, else groups of G); the G CTAs of a group split the matrix's rows
+ *   few, or equal groups where these are estimated to be faster, else groups
+ *   of G); the G CTAs of a group split the matrix's rows
  *   (the row-block distribution of Alg. 2 / Alg. 8), write partial sums of
  *   every m-row product to their own slots, meet at a group barrier and add
  *   the slots in rank order, each factoring the b x b Gram matrix redundantly

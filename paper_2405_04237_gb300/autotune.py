@@ -134,8 +134,7 @@ def starting_panels(ns, k0):
 
 def autotune_batched(As, variant: str = "mcqr2gs", groups=(0, 4, 8, 19), panel_counts=(1, 2, 4), reps: int = 2,
                      use_cache: bool = True, verbose: bool = False):
-    """(G, panel_b list) for the persistent batched launch of these matrices; G = 0 is the default schedule
-    (groups of several sizes)."""
+    """(G, panel_b list) for the persistent batched launch of these matrices; G = 0 is the default schedule."""
     from . import batched_workspace_size, factor_batched
 
     ns = [int(A.shape[1]) for A in As]

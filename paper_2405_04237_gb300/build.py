@@ -34,7 +34,8 @@ def _sources():
 
 
 def _deps():
-    return _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
+    headers = [os.path.join(CSRC, "*.cuh"), os.path.join(CSRC, "*.h"), os.path.join(INCLUDE, "*.h")]
+    return _sources() + [f for pattern in headers for f in glob.glob(pattern)]
 
 
 def up_to_date() -> bool:

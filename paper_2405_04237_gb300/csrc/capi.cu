@@ -990,7 +990,7 @@ int cqr_factor_batched(int batch, const int64_t* m, const int64_t* n, const int6
   TracePhase ph("batched", batch);
   if (persistent) {
     const int grid = batched_persistent_grid();
-    const int G = md.G;  // 0: groups of several sizes, from the matrices' sizes
+    const int G = md.G;  // 0: chosen from the matrices' sizes
     if (G > 0 && grid % G) return -9;
     std::vector<int> b((size_t)batch);
     for (int i = 0; i < batch; ++i) b[i] = resolve_panel(n[i], panel_b[i], variant);

@@ -244,7 +244,7 @@ int probe_fp64(int kind, int iters, double* gflops, double* flop_per_clk_sm, dou
 // Persistent batched mCQR2GS (k_batched.cu): one cooperative launch over all
 // SMs, groups of G CTAs factoring whole matrices (n <= 128, n and b
 // multiples of 4).  `halve` applies the adaptive panel width on the device.
-// G == 0: groups of several sizes, chosen from the matrices' sizes.
+// G == 0: the schedule is chosen from the matrices' sizes (batched_schedule.h).
 bool batched_persistent_eligible(int batch, const int64_t* m, const int64_t* n, const int* b);
 size_t batched_persistent_workspace(int batch);
 int batched_persistent_grid();  // CTAs of the launch: one per SM

@@ -4,13 +4,14 @@
 // Work split.  The grid holds one CTA of kBT threads per SM, all resident
 // (cooperative launch).  CTAs form groups of consecutive blocks; a group
 // factors, one after the other, the matrices of its list (a static schedule
-// computed on the host).  By default the groups are the nodes of a binary
-// tree over the CTAs: all CTAs first factor the root's matrices together,
-// then each half its own, each quarter, and so on down to single CTAs, so a
-// batch of uneven matrices ends at about the same time on every SM (with
-// groups of 8 the largest matrix of a batch, 200000 x 128, alone took 3.5
-// times the batch's work divided by the chip); a given group size makes one
-// level of equal groups.  Inside a group of G CTAs the rows of the current
+// computed on the host, batched_schedule.h).  By default the groups are the
+// nodes of a binary tree over the CTAs: all CTAs first factor the root's
+// matrices together, then each half its own, each quarter, and so on down to
+// single CTAs, so a batch of uneven matrices ends at about the same time on
+// every SM (with groups of 8 the largest matrix of a batch, 200000 x 128, alone
+// took 3.5 times the batch's work divided by the chip) -- or, where that is
+// estimated to be faster, equal groups of 8, one level; a given group size
+// makes one level of equal groups, too.  Inside a group of G CTAs the rows of the current
 // matrix are split into G contiguous ranges, one per CTA: this
 // is the paper's 1-D row-block distribution (Alg. 2, Alg. 8) with the G
 // CTAs as the ranks.  Every step that sums over the m rows ends with each
@@ -52,6 +53,7 @@
 #include <mutex>
 #include <vector>
 
+#include "batched_schedule.h"
 #include "block_sums.cuh"
 #include "chol_device.cuh"
 #include "cqr.h"
@@ -81,17 +83,6 @@ struct BMat {
   double* R;
   i64 m, lda;   // ldq = lda, ldr = n
   int n, b;     // width, starting panel width
-};
-
-// Groups of the launch: level l cuts the N CTAs into cnt[l] groups of equal
-// size (to within one), group g = CTAs [g N / cnt, (g + 1) N / cnt).  Every
-// CTA walks the levels in order; the groups of a level lie inside those of
-// the level before.
-constexpr int kBLevels = 12;  // 1, 2, 4, .. and N itself: grids of up to 1024 CTAs
-struct BLevels {
-  int n;
-  int cnt[kBLevels];
-  int off[kBLevels];   // node of the level's group 0 (node = entry of gstart, barrier counter)
 };
 
 // Slots added directly by every CTA.  Adding G slots costs b (b + 1) / 2 G
@@ -1021,160 +1012,6 @@ bool batched_persistent_eligible(int batch, const int64_t* m, const int64_t* n, 
 
 size_t batched_persistent_workspace(int batch) { return blayout(batch, persistent_grid_impl()).total; }
 
-namespace {
-
-// Rough device time of one matrix on a group of G CTAs (for the static
-// schedule), fitted to homogeneous batches (500 to 200000 rows, n = 16 to
-// 128, G = 1 to 152) to within 10 %: per row the multiply-adds at an SM's
-// FP64 rate and the staging of each pass, per pass the barrier, the in-CTA
-// sums and the solve's chain, per CholeskyQR the factorisation.
-double est_seconds(i64 m, int n, int b, int G) {
-  const double k = n / b, rows = (double)m / G;
-  const double row = 4.0 * n * n / 8.28e9 + n * (3.0 + 2.4 * k) * 1e-9;
-  const double pass = 13e-6 + 0.35e-6 * b, chol = 0.6e-6 * b * (1.0 + b / 128.0);
-  return rows * row + (4.0 * k - 1.0) * pass + 2.0 * k * chol;
-}
-
-// The static schedule: matrices (order) of every node.
-struct BSchedule {
-  BLevels lev;
-  int nodes;
-  std::vector<int> order, gstart;
-};
-
-void finish(BSchedule& S, const std::vector<std::vector<int>>& lists) {
-  S.nodes = (int)lists.size();
-  for (const auto& l : lists) {
-    S.gstart.push_back((int)S.order.size());
-    S.order.insert(S.order.end(), l.begin(), l.end());
-  }
-  S.gstart.push_back((int)S.order.size());
-}
-
-// Equal groups of G CTAs: largest estimated time first, each to the group
-// with the least work so far.
-BSchedule schedule_uniform(int batch, const int64_t* m, const int64_t* n, const int* b, int grid, int G) {
-  BSchedule S{};
-  const int groups = grid / G;
-  S.lev.n = 1;
-  S.lev.cnt[0] = groups;
-  std::vector<std::pair<double, int>> by;
-  for (int i = 0; i < batch; ++i) by.push_back({est_seconds(m[i], (int)n[i], b[i], G), i});
-  std::stable_sort(by.begin(), by.end(),
-                   [](const std::pair<double, int>& x, const std::pair<double, int>& y) { return x.first > y.first; });
-  std::vector<double> load((size_t)groups, 0.0);
-  std::vector<std::vector<int>> lists((size_t)groups);
-  for (const auto& e : by) {
-    int g = 0;
-    for (int h = 1; h < groups; ++h)
-      if (load[h] < load[g]) g = h;
-    load[g] += e.first;
-    lists[g].push_back(e.second);
-  }
-  finish(S, lists);
-  return S;
-}
-
-// The tree schedule.  A CTA's finishing time is the sum of the loads of the
-// nodes it belongs to (the members of a node arrive together, so nobody
-// waits).  For a bound on that time, the matrices are placed by decreasing
-// work, each on the smallest groups that keep the bound (fewer CTAs waste
-// less on barriers and sums), there on the least loaded one.  The bounds
-// tried grow from the largest of the mean work per CTA and the longest
-// matrix on the whole grid; on a bound that cannot be kept the next is
-// tried, and the last takes the best place for every matrix.
-BSchedule schedule_tree(int batch, const int64_t* m, const int64_t* n, const int* b, int grid) {
-  BSchedule S{};
-  BLevels& L = S.lev;
-  int nodes = 0;
-  for (int c = 1;; c *= 2) {
-    const bool last = c >= grid || L.n == kBLevels - 1;
-    L.cnt[L.n] = last ? grid : c;
-    L.off[L.n] = nodes;
-    nodes += L.cnt[L.n++];
-    if (last) break;
-  }
-  auto lo_of = [&](int l, int g) { return (int)((i64)g * grid / L.cnt[l]); };
-  // estimated times per matrix and level (the level's smallest group)
-  std::vector<double> est((size_t)batch * L.n);
-  std::vector<int> by((size_t)batch);
-  double mean = 0.0, longest = 0.0;
-  for (int i = 0; i < batch; ++i) {
-    by[i] = i;
-    double best = 0.0;
-    for (int l = 0; l < L.n; ++l) {
-      const double t = est[(size_t)i * L.n + l] = est_seconds(m[i], (int)n[i], b[i], grid / L.cnt[l]);
-      if (l == 0 || t < best) best = t;
-    }
-    mean += est[(size_t)i * L.n + L.n - 1] / grid;
-    longest = std::max(longest, best);
-  }
-  std::stable_sort(by.begin(), by.end(), [&](int x, int y) {
-    return est[(size_t)x * L.n + L.n - 1] > est[(size_t)y * L.n + L.n - 1];
-  });
-  std::vector<double> cta((size_t)grid);     // load of each CTA
-  std::vector<double> peak((size_t)nodes);   // largest load of the node's CTAs
-  std::vector<int> place((size_t)batch);
-  double bound = std::max(mean, longest);
-  for (int attempt = 0;; ++attempt, bound *= 1.04) {
-    const bool last = attempt == 20;
-    std::fill(cta.begin(), cta.end(), 0.0);
-    std::fill(peak.begin(), peak.end(), 0.0);
-    bool ok = true;
-    for (int q = 0; q < batch && ok; ++q) {
-      const int i = by[q];
-      int pl = -1, pg = -1;
-      double at = 0.0;
-      for (int l = L.n - 1; l >= 0 && pl < 0; --l) {
-        int g = 0;
-        for (int h = 1; h < L.cnt[l]; ++h)
-          if (peak[L.off[l] + h] < peak[L.off[l] + g]) g = h;
-        at = peak[L.off[l] + g] + est[(size_t)i * L.n + l];
-        if (at <= bound) {
-          pl = l;
-          pg = g;
-        }
-      }
-      if (pl < 0 && last) {
-        for (int l = 0; l < L.n; ++l) {
-          int g = 0;
-          for (int h = 1; h < L.cnt[l]; ++h)
-            if (peak[L.off[l] + h] < peak[L.off[l] + g]) g = h;
-          const double t = peak[L.off[l] + g] + est[(size_t)i * L.n + l];
-          if (pl < 0 || t < at) {
-            at = t;
-            pl = l;
-            pg = g;
-          }
-        }
-      }
-      if (pl < 0) {
-        ok = false;
-        break;
-      }
-      place[i] = L.off[pl] + pg;
-      // the node's CTAs wait for the slowest of them, then run the matrix
-      const int c0 = lo_of(pl, pg), c1 = lo_of(pl, pg + 1);
-      for (int c = c0; c < c1; ++c) cta[c] += est[(size_t)i * L.n + pl];
-      for (int l = 0; l < L.n; ++l) {
-        const int g0 = ((c0 + 1) * L.cnt[l] - 1) / grid, g1 = (c1 * L.cnt[l] - 1) / grid;
-        for (int g = g0; g <= g1; ++g) {
-          double v = 0.0;
-          for (int c = lo_of(l, g); c < lo_of(l, g + 1); ++c) v = std::max(v, cta[c]);
-          peak[L.off[l] + g] = v;
-        }
-      }
-    }
-    if (ok) break;
-  }
-  std::vector<std::vector<int>> lists((size_t)nodes);
-  for (int i : by) lists[place[i]].push_back(i);
-  finish(S, lists);
-  return S;
-}
-
-}  // namespace
-
 cudaError_t batched_persistent_run(int batch, const int64_t* m, const int64_t* n, const int64_t* lda,
                                    const int* b, double* const* A, double* const* Q, double* const* R,
                                    int* status, void* workspace, int G, bool halve, cudaStream_t st) {
@@ -1195,7 +1032,7 @@ cudaError_t batched_persistent_run(int batch, const int64_t* m, const int64_t* n
     nmax = std::max(nmax, (int)n[i]);
     bmax = std::max(bmax, b[i]);
   }
-  const BSchedule S = G > 0 ? schedule_uniform(batch, m, n, b, grid, G) : schedule_tree(batch, m, n, b, grid);
+  const BSchedule S = G > 0 ? schedule_uniform(batch, m, n, b, grid, G) : schedule_default(batch, m, n, b, grid);
   // descriptor table, schedule: kernel-parameter blobs into the workspace
   auto upload = [&](size_t off, const void* src, size_t bytes) -> cudaError_t {
     const unsigned char* p = (const unsigned char*)src;
