@@ -54,13 +54,19 @@ __device__ __forceinline__ void sqrt_rsqrt(double d, double& u, double& r) {
 
 // w / d for a positive d as w times the reciprocal: the FP32 reciprocal r0 of
 // the mantissa m (24 bits), then r0 (1 + e + e^2) with the residual e = 1 - m
-// r0 (third order Newton: relative error e^3 < 2^-66 before rounding).  Where
-// d or 1/d is subnormal (1/d of a subnormal d overflows, 1/d below 2^-1022
-// loses bits), the library's division.
+// r0 (third order Newton: relative error e^3 < 2^-66 before rounding).  Where d
+// or 1/d is subnormal (1/d of a subnormal d overflows, 1/d below 2^-1022 loses
+// bits) both are scaled first; w^2 <= d W_cc keeps w 2^54 finite.
 __device__ __forceinline__ double over_pivot(double w, double d) {
-  const int hi = __double2hiint(d), lo = __double2loint(d);
-  const int ex = (hi >> 20) - 1023;
-  if (ex == -1023 || ex > 1020) return w / d;
+  int hi = __double2hiint(d), ex = (hi >> 20) - 1023;
+  if (ex == -1023 || ex > 1020) {
+    const double s = ex < 0 ? 0x1p54 : 0x1p-54;
+    w *= s;
+    d *= s;
+    hi = __double2hiint(d);
+    ex = (hi >> 20) - 1023;
+  }
+  const int lo = __double2loint(d);
   const double m = __hiloint2double(hi - (ex << 20), lo);
   const float f = __uint_as_float((127u << 23) | ((unsigned)(hi & 0xFFFFF) << 3) | ((unsigned)lo >> 29));
   const double r0 = widen(__frcp_rn(f));
@@ -85,8 +91,8 @@ __device__ __forceinline__ double over_pivot(double w, double d) {
 // memory.  Every pivot warp reads rows j and j + 1 in columns j and j + 1, so
 // none of these four is written in step j: a warp's own entries are those
 // beyond column j + 1, the pivots go to dg, and the updated entry (j, j + 1)
-// stays with its thread until the next step, which reads rows j + 2 and below
-// only (two warps never touch one entry between two barriers, unless to read).
+// waits for the end in the unused place (j + 1, j) below the diagonal (two
+// warps never touch one entry between two barriers, unless to read).
 // At the end U_jc = w / u is w r corrected with the fused residual,
 // so exact quotients stay exact.  The elements of the rows below are
 // enumerated from the last row up (tab), so the live ones are always a prefix
@@ -121,11 +127,8 @@ __device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* rows, 
     tab[e] = (unsigned short)((row << 8) | (row + e - k * (k + 1) / 2 - k * nx));
   }
   __syncthreads();
-  double* kept = nullptr;  // warp 0, lane 1: entry (j, j + 1) of the step before
-  double kept_w = 0.0;
   for (int j = 0; j < kb; j += 2) {
     int bad = 0;
-    if (kept) *kept = kept_w;
     // rows j - 2, j - 1 (w, l each) and this step's
     const double* pw = rows + ((j >> 1) + 1 & 1) * 4 * us;
     double* cw = rows + (j >> 1 & 1) * 4 * us;
@@ -135,7 +138,7 @@ __device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* rows, 
     if (warp < np) {
       const bool two = j + 1 < kb;
       const int c = lane < 2 ? j + lane : j + 30 * warp + lane;
-      const bool live = c < kb + nx;
+      const bool live = c < kb + nx && (lane != 1 || two || warp == 0);
       double *r1 = Ws + j * ld, *r2 = r1 + ld;
       double w1 = live ? r1[c] : 0.0, w2 = live && two && c > j ? r2[c] : 0.0;
       if (j > 0 && live) {
@@ -154,12 +157,7 @@ __device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* rows, 
         if (own && c > j) {
           cw[c] = w1;
           cw[us + c] = l1;
-          if (c > j + 1) {
-            r1[c] = w1;
-          } else {
-            kept = r1 + c;
-            kept_w = w1;
-          }
+          *(c > j + 1 || !two ? r1 + c : r2 + j) = w1;
         }
         if (t == 0) dg[j] = d1;
         if (two) {
@@ -199,7 +197,6 @@ __device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* rows, 
     }
     if (__syncthreads_or(bad)) break;
   }
-  if (kept) *kept = kept_w;
   const int jb = *broken, done = jb >= 0 ? jb : kb;
   double* rs = rows;  // 1 / sqrt(d_j)
   for (int j = t; j < done; j += T) {
@@ -212,7 +209,10 @@ __device__ int chol_trapezoid(double* Ws, int ld, int kb, int nx, double* rows, 
   for (int e = t; e < total; e += T) {
     const int j = tab[e] >> 8, c = tab[e] & 255;
     if (c > j && j < done) {
-      const double w = Ws[j * ld + c], r = rs[j], q = w * r;
+      double* from = Ws + j * ld + c;
+      if (c == j + 1 && c < kb && !(j & 1)) from = Ws + c * ld + j;  // entry (j, j + 1) of a pair of rows
+      const double w = *from, r = rs[j], q = w * r;
+      *from = 0.0;
       Ws[j * ld + c] = fma(fma(-q, dg[j], w), r, q);
     }
   }
